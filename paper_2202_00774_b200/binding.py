@@ -1,8 +1,9 @@
 """Python binding of the SDGP C ABI (``include/sdgp.h``): argument marshalling only.
 
 Tensors are torch CUDA tensors (device memory and streams come from torch); every
-computation happens inside ``libsdgp.so``. There is no fallback: a missing library or a
-non-OK status raises.
+computation happens inside ``libsdgp.so``. The calls of a training step are marshalled in
+C++ (``csrc/torch_binding.cpp``); ``lib()`` gives the plain C ABI through ctypes. There is no
+fallback: a missing library or a non-OK status raises.
 """
 from __future__ import annotations
 
@@ -25,6 +26,7 @@ EXPORTS = ["sdgp_prune", "sdgp_dgrad_linear", "sdgp_dgrad_conv2d", "sdgp_spmm_li
            "sdgp_status_string"]
 
 _lib = None
+_torch = None   # the C++ module, once loaded
 
 
 class SdgpError(RuntimeError):
@@ -93,6 +95,16 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def _load():
+    """The C++ module that calls the library with torch tensors (built first if its source is newer)."""
+    global _torch
+    lib()
+    _build.build_binding()
+    from . import _sdgp_torch
+    _torch = _sdgp_torch
+    return _torch
+
+
 def status_string(status: int) -> str:
     return lib().sdgp_status_string(int(status)).decode()
 
@@ -115,76 +127,46 @@ def _dev(t, name):
         raise ValueError("%s must be a contiguous CUDA tensor" % name)
 
 
+# Tensors must be contiguous CUDA tensors (ValueError otherwise); the work goes to torch's current stream.
+
+
 def sdgp_prune(dO, n, m, scheme, seed=0, dense=None, values=None, meta=None, mask=None):
     """``sdgp_prune`` of sdgp.h. ``dO`` is a 2-byte-element tensor whose last dimension is K;
     outputs are caller-allocated tensors (or None)."""
-    for t, name in ((dO, "dO"), (dense, "dense"), (values, "values"), (meta, "meta"), (mask, "mask")):
-        _dev(t, name)
-    K = dO.shape[-1] if dO.dim() else 0
-    rows = dO.numel() // K if K else 0
-    _check(lib().sdgp_prune(_ptr(dO), rows, K, n, m, scheme, seed, _ptr(dense), _ptr(values), _ptr(meta),
-                            _ptr(mask), _stream()), "sdgp_prune")
+    _check((_torch or _load()).prune(dO, n, m, scheme, seed, BF16, dense, values, meta, mask), "sdgp_prune")
 
 
 def sdgp_workspace_size_linear(rows, K, N, flags=FLAG_TWO_PASS) -> int:
-    return int(lib().sdgp_workspace_size_linear(rows, K, N, flags))
+    return (_torch or _load()).workspace_size_linear(rows, K, N, flags)
 
 
 def sdgp_workspace_size_conv2d(B, H, Wd, Cin, Cout, R, S, stride, pad, flags=FLAG_TWO_PASS) -> int:
-    return int(lib().sdgp_workspace_size_conv2d(B, H, Wd, Cin, Cout, R, S, stride, pad, flags))
+    return (_torch or _load()).workspace_size_conv2d(B, H, Wd, Cin, Cout, R, S, stride, pad, 0, flags)
 
 
 def sdgp_dgrad_linear(dO, W, dD, n, m, scheme, seed=0, workspace=None, flags=FLAG_TWO_PASS):
     """``sdgp_dgrad_linear``: dO [rows,K], W [K,N], dD [rows,N] (bf16 or 2-byte views)."""
-    for t, name in ((dO, "dO"), (W, "W"), (dD, "dD"), (workspace, "workspace")):
-        _dev(t, name)
-    rows, K = dO.shape
-    N = W.shape[1]
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(lib().sdgp_dgrad_linear(_ptr(dO), _ptr(W), _ptr(dD), rows, K, N, n, m, scheme, seed,
-                                   _ptr(workspace), ws_bytes, flags, _stream()), "sdgp_dgrad_linear")
+    _check((_torch or _load()).dgrad_linear(dO, W, dD, n, m, scheme, seed, BF16, workspace, flags), "sdgp_dgrad_linear")
 
 
 def sdgp_dgrad_linear_static(dO, W, dD, n, m, scheme, seed=0):
     """``sdgp_dgrad_linear_static``: like :func:`sdgp_dgrad_linear` in two-pass mode, but the
     scratch is the library's own fixed device array - for callers that cannot allocate a
     workspace. rows*K is limited to 8Mi elements; calls must not overlap on the GPU."""
-    for t, name in ((dO, "dO"), (W, "W"), (dD, "dD")):
-        _dev(t, name)
-    rows, K = dO.shape
-    N = W.shape[1]
-    _check(lib().sdgp_dgrad_linear_static(_ptr(dO), _ptr(W), _ptr(dD), rows, K, N, n, m, scheme, seed,
-                                          _stream()), "sdgp_dgrad_linear_static")
+    _check((_torch or _load()).dgrad_linear_static(dO, W, dD, n, m, scheme, seed), "sdgp_dgrad_linear_static")
 
 
 def sdgp_dgrad_conv2d(dO, W, dD, stride, pad, n, m, scheme, seed=0, workspace=None, flags=FLAG_TWO_PASS):
     """``sdgp_dgrad_conv2d``: dO NHWC [B,P,Q,Cout], W [Cout,R,S,Cin], dD NHWC [B,H,Wd,Cin]."""
-    for t, name in ((dO, "dO"), (W, "W"), (dD, "dD"), (workspace, "workspace")):
-        _dev(t, name)
-    B, H, Wd, Cin = dD.shape
-    Cout, R, S, _ = W.shape
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(lib().sdgp_dgrad_conv2d(_ptr(dO), _ptr(W), _ptr(dD), B, H, Wd, Cin, Cout, R, S, stride, pad, n, m,
-                                   scheme, seed, _ptr(workspace), ws_bytes, flags, _stream()),
-           "sdgp_dgrad_conv2d")
+    _check((_torch or _load()).dgrad_conv2d(dO, W, dD, stride, pad, 0, n, m, scheme, seed, BF16, workspace, flags), "sdgp_dgrad_conv2d")
 
 
 def sdgp_spmm_linear(values, meta, W, dD):
-    for t, name in ((values, "values"), (meta, "meta"), (W, "W"), (dD, "dD")):
-        _dev(t, name)
-    rows, N = dD.shape
-    K = W.shape[0]
-    _check(lib().sdgp_spmm_linear(_ptr(values), _ptr(meta), _ptr(W), _ptr(dD), rows, K, N, _stream()),
-           "sdgp_spmm_linear")
+    _check((_torch or _load()).spmm_linear(values, meta, W, dD, BF16), "sdgp_spmm_linear")
 
 
 def sdgp_spmm_conv2d(values, meta, W, dD, stride, pad):
-    for t, name in ((values, "values"), (meta, "meta"), (W, "W"), (dD, "dD")):
-        _dev(t, name)
-    B, H, Wd, Cin = dD.shape
-    Cout, R, S, _ = W.shape
-    _check(lib().sdgp_spmm_conv2d(_ptr(values), _ptr(meta), _ptr(W), _ptr(dD), B, H, Wd, Cin, Cout, R, S,
-                                  stride, pad, _stream()), "sdgp_spmm_conv2d")
+    _check((_torch or _load()).spmm_conv2d(values, meta, W, dD, stride, pad, BF16), "sdgp_spmm_conv2d")
 
 
 # ---- the same operations on tensors of an explicit element type (sdgp_dtype: BF16 or FP16) ----
@@ -192,42 +174,23 @@ def sdgp_spmm_conv2d(values, meta, W, dD, stride, pad):
 
 def sdgp_prune_typed(dO, n, m, scheme, seed, dtype, dense=None, values=None, meta=None, mask=None):
     """``sdgp_prune_typed``: :func:`sdgp_prune` for 2-byte elements of type ``dtype``."""
-    for t, name in ((dO, "dO"), (dense, "dense"), (values, "values"), (meta, "meta"), (mask, "mask")):
-        _dev(t, name)
-    K = dO.shape[-1] if dO.dim() else 0
-    rows = dO.numel() // K if K else 0
-    _check(lib().sdgp_prune_typed(_ptr(dO), rows, K, n, m, scheme, seed, dtype, _ptr(dense), _ptr(values),
-                                  _ptr(meta), _ptr(mask), _stream()), "sdgp_prune_typed")
+    _check((_torch or _load()).prune(dO, n, m, scheme, seed, dtype, dense, values, meta, mask), "sdgp_prune_typed")
 
 
 def sdgp_relu_backward_prune(dY, act, n, m, scheme, seed=0, dtype=BF16, grad=None, dense=None, values=None, meta=None,
                              mask=None):
     """``sdgp_relu_backward_prune``: dL/dO = dY where ``act`` > 0, pruned in the same pass. ``dY`` and ``act`` are
     2-byte-element tensors of the same shape whose last dimension is K; outputs are caller-allocated (or None)."""
-    for t, name in ((dY, "dY"), (act, "act"), (grad, "grad"), (dense, "dense"), (values, "values"), (meta, "meta"),
-                    (mask, "mask")):
-        _dev(t, name)
-    if dY.shape != act.shape:
-        raise ValueError("dY and act must have the same shape")
-    K = dY.shape[-1] if dY.dim() else 0
-    rows = dY.numel() // K if K else 0
-    _check(lib().sdgp_relu_backward_prune(_ptr(dY), _ptr(act), rows, K, n, m, scheme, seed, dtype, _ptr(grad), _ptr(dense),
-                                          _ptr(values), _ptr(meta), _ptr(mask), _stream()), "sdgp_relu_backward_prune")
+    _check((_torch or _load()).relu_backward_prune(dY, None, 0, act, n, m, scheme, seed, dtype, grad, dense, values, meta, mask),
+           "sdgp_relu_backward_prune")
 
 
 def sdgp_residual_relu_backward_prune(dY, dSkip, act, n, m, scheme, seed=0, dtype=BF16, grad=None, dense=None, values=None,
                                       meta=None, mask=None):
     """``sdgp_residual_relu_backward_prune``: dL/dO = dY + dSkip (rounded to the 16-bit type) where ``act`` > 0, pruned in
     the same pass. The three inputs are 2-byte-element tensors of the same shape whose last dimension is K."""
-    for t, name in ((dY, "dY"), (dSkip, "dSkip"), (act, "act"), (grad, "grad"), (dense, "dense"), (values, "values"),
-                    (meta, "meta"), (mask, "mask")):
-        _dev(t, name)
-    if dY.shape != act.shape or (dSkip is not None and dY.shape != dSkip.shape):   # (a missing dSkip is the library's to reject)
-        raise ValueError("dY, dSkip and act must have the same shape")
-    K = dY.shape[-1] if dY.dim() else 0
-    rows = dY.numel() // K if K else 0
-    _check(lib().sdgp_residual_relu_backward_prune(_ptr(dY), _ptr(dSkip), _ptr(act), rows, K, n, m, scheme, seed, dtype,
-                                                   _ptr(grad), _ptr(dense), _ptr(values), _ptr(meta), _ptr(mask), _stream()),
+    # (a missing dSkip is the library's to reject)
+    _check((_torch or _load()).relu_backward_prune(dY, dSkip, 1, act, n, m, scheme, seed, dtype, grad, dense, values, meta, mask),
            "sdgp_residual_relu_backward_prune")
 
 
@@ -236,75 +199,39 @@ def sdgp_maxpool_relu_backward_prune(dYp, act, n, m, scheme, seed=0, dtype=BF16,
     """``sdgp_maxpool_relu_backward_prune``: ``dYp`` [B, H/2, W/2, K] is the gradient above a 2 x 2 max pooling, ``act``
     [B, H, W, K] the activation of the ReLU below it; dL/dO [B, H, W, K] is formed and pruned in one pass. ``skip``
     (optional, the shape of ``dYp``) is a second gradient added to ``dYp`` first."""
-    for t, name in ((dYp, "dYp"), (act, "act"), (grad, "grad"), (dense, "dense"), (values, "values"), (meta, "meta"),
-                    (mask, "mask"), (skip, "skip")):
-        _dev(t, name)
-    if skip is not None and skip.shape != dYp.shape:
-        raise ValueError("skip must have the shape of dYp")
-    if act.dim() != 4 or dYp.dim() != 4:
-        raise ValueError("dYp and act must be NHWC tensors")
-    B, H, W, K = act.shape
-    if tuple(dYp.shape) != (B, H // 2, W // 2, K):
-        raise ValueError("dYp must be [B, H/2, W/2, K]")
-    _check(lib().sdgp_maxpool_relu_backward_prune(_ptr(dYp), _ptr(skip), _ptr(act), B, H, W, K, n, m, scheme, seed, dtype, _ptr(grad),
-                                                  _ptr(dense), _ptr(values), _ptr(meta), _ptr(mask), _stream()),
+    _check((_torch or _load()).maxpool_relu_backward_prune(dYp, skip, act, n, m, scheme, seed, dtype, grad, dense, values, meta, mask),
            "sdgp_maxpool_relu_backward_prune")
 
 
 def sdgp_dgrad_linear_typed(dO, W, dD, n, m, scheme, seed, dtype, workspace=None, flags=FLAG_TWO_PASS):
-    for t, name in ((dO, "dO"), (W, "W"), (dD, "dD"), (workspace, "workspace")):
-        _dev(t, name)
-    rows, K = dO.shape
-    N = W.shape[1]
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(lib().sdgp_dgrad_linear_typed(_ptr(dO), _ptr(W), _ptr(dD), rows, K, N, n, m, scheme, seed, dtype,
-                                         _ptr(workspace), ws_bytes, flags, _stream()), "sdgp_dgrad_linear_typed")
+    _check((_torch or _load()).dgrad_linear(dO, W, dD, n, m, scheme, seed, dtype, workspace, flags), "sdgp_dgrad_linear_typed")
 
 
 def sdgp_dgrad_conv2d_typed(dO, W, dD, stride, pad, n, m, scheme, seed, dtype, workspace=None, flags=FLAG_TWO_PASS):
-    for t, name in ((dO, "dO"), (W, "W"), (dD, "dD"), (workspace, "workspace")):
-        _dev(t, name)
-    B, H, Wd, Cin = dD.shape
-    Cout, R, S, _ = W.shape
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(lib().sdgp_dgrad_conv2d_typed(_ptr(dO), _ptr(W), _ptr(dD), B, H, Wd, Cin, Cout, R, S, stride, pad, n, m,
-                                         scheme, seed, dtype, _ptr(workspace), ws_bytes, flags, _stream()),
+    _check((_torch or _load()).dgrad_conv2d(dO, W, dD, stride, pad, 0, n, m, scheme, seed, dtype, workspace, flags),
            "sdgp_dgrad_conv2d_typed")
 
 
 def sdgp_workspace_size_conv2d_grouped(B, H, Wd, Cin, Cout, R, S, stride, pad, groups, flags=FLAG_TWO_PASS) -> int:
-    return int(lib().sdgp_workspace_size_conv2d_grouped(B, H, Wd, Cin, Cout, R, S, stride, pad, groups, flags))
+    if groups < 1:
+        return 0
+    return (_torch or _load()).workspace_size_conv2d(B, H, Wd, Cin, Cout, R, S, stride, pad, groups, flags)
 
 
 def sdgp_dgrad_conv2d_grouped(dO, W, dD, stride, pad, groups, n, m, scheme, seed=0, dtype=BF16, workspace=None,
                               flags=FLAG_TWO_PASS):
     """``sdgp_dgrad_conv2d_grouped``: dO NHWC [B,P,Q,Cout], W [Cout,R,S,Cin/groups], dD NHWC [B,H,W,Cin]."""
-    for t, name in ((dO, "dO"), (W, "W"), (dD, "dD"), (workspace, "workspace")):
-        _dev(t, name)
-    B, H, Wd, Cin = dD.shape
-    Cout, R, S, _ = W.shape
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(lib().sdgp_dgrad_conv2d_grouped(_ptr(dO), _ptr(W), _ptr(dD), B, H, Wd, Cin, Cout, R, S, stride, pad, groups,
-                                           n, m, scheme, seed, dtype, _ptr(workspace), ws_bytes, flags, _stream()),
+    # (groups == 0 would name the ungrouped entry point; the library rejects -1 just the same)
+    _check((_torch or _load()).dgrad_conv2d(dO, W, dD, stride, pad, groups or -1, n, m, scheme, seed, dtype, workspace, flags),
            "sdgp_dgrad_conv2d_grouped")
 
 
 def sdgp_spmm_linear_typed(values, meta, W, dD, dtype):
-    for t, name in ((values, "values"), (meta, "meta"), (W, "W"), (dD, "dD")):
-        _dev(t, name)
-    rows, N = dD.shape
-    K = W.shape[0]
-    _check(lib().sdgp_spmm_linear_typed(_ptr(values), _ptr(meta), _ptr(W), _ptr(dD), rows, K, N, dtype, _stream()),
-           "sdgp_spmm_linear_typed")
+    _check((_torch or _load()).spmm_linear(values, meta, W, dD, dtype), "sdgp_spmm_linear_typed")
 
 
 def sdgp_spmm_conv2d_typed(values, meta, W, dD, stride, pad, dtype):
-    for t, name in ((values, "values"), (meta, "meta"), (W, "W"), (dD, "dD")):
-        _dev(t, name)
-    B, H, Wd, Cin = dD.shape
-    Cout, R, S, _ = W.shape
-    _check(lib().sdgp_spmm_conv2d_typed(_ptr(values), _ptr(meta), _ptr(W), _ptr(dD), B, H, Wd, Cin, Cout, R, S,
-                                        stride, pad, dtype, _stream()), "sdgp_spmm_conv2d_typed")
+    _check((_torch or _load()).spmm_conv2d(values, meta, W, dD, stride, pad, dtype), "sdgp_spmm_conv2d_typed")
 
 
 def sdgp_channel_scales(dO, n, m, dtype, out):

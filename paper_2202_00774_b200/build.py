@@ -1,14 +1,18 @@
-"""Builds ``libsdgp.so`` (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds ``libsdgp.so`` (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and ``_sdgp_torch.so``, the module
+that calls it with torch tensors (plain C++ against torch's headers, no device code)."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsdgp.so")
 SOURCES = ["prune.cu", "dgrad.cu", "api.cu", "static_scratch.cu", "channel.cu", "grouped.cu"]
+BINDING = os.path.join(HERE, "_sdgp_torch.so")
+BINDING_SOURCE = os.path.join(CSRC, "torch_binding.cpp")
 HEADERS = ["ptx.cuh", "sdgp_internal.cuh", "prune_core.cuh", os.path.join("..", "..", "include", "sdgp.h")]
 
 
@@ -17,12 +21,31 @@ def _nvcc() -> str:
     return cand if os.path.exists(cand) else "nvcc"
 
 
-def needs_build() -> bool:
-    if not os.path.exists(LIB):
+def _stale(target, deps) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS] + [os.path.abspath(__file__)]
+    t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def needs_build() -> bool:
+    return _stale(LIB, [os.path.join(CSRC, f) for f in SOURCES + HEADERS] + [os.path.abspath(__file__)])
+
+
+def build_binding(force: bool = False) -> str:
+    """The torch module; needs ``libsdgp.so`` beside it (it finds it through its run path)."""
+    if not force and not _stale(BINDING, [BINDING_SOURCE, os.path.join(HERE, "..", "include", "sdgp.h"), os.path.abspath(__file__)]):
+        return BINDING
+    from torch.utils import cpp_extension
+    tmp = BINDING + ".%d.tmp" % os.getpid()
+    include = [sysconfig.get_paths()["include"]] + cpp_extension.include_paths("cuda")
+    libs = cpp_extension.library_paths("cuda")
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-o", tmp, BINDING_SOURCE]
+    cmd += ["-I" + d for d in include] + ["-L" + HERE, "-lsdgp"] + ["-L" + d for d in libs]
+    cmd += ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
+    subprocess.check_call(cmd)
+    os.replace(tmp, BINDING)
+    return BINDING
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -41,3 +64,4 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv))
+    print(build_binding(force="--force" in sys.argv))

@@ -6,11 +6,12 @@ import os
 import subprocess
 import sys
 import sysconfig
+from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsdgp.so")
-SOURCES = ["prune.cu", "dgrad.cu", "api.cu", "static_scratch.cu", "channel.cu", "grouped.cu"]
+SOURCES = ["prune.cu", "rank.cu", "dgrad.cu", "api.cu", "static_scratch.cu", "channel.cu", "grouped.cu"]
 BINDING = os.path.join(HERE, "_sdgp_torch.so")
 BINDING_SOURCE = os.path.join(CSRC, "torch_binding.cpp")
 HEADERS = ["ptx.cuh", "sdgp_internal.cuh", "prune_core.cuh", os.path.join("..", "..", "include", "sdgp.h")]
@@ -48,16 +49,26 @@ def build_binding(force: bool = False) -> str:
     return BINDING
 
 
+def _compile(src: str, force: bool, verbose: bool) -> str:
+    """One translation unit to an object file under ``_build/`` (skipped while it is newer than everything it reads)."""
+    obj = os.path.join(HERE, "_build", os.path.splitext(src)[0] + ".o")
+    deps = [os.path.join(CSRC, f) for f in [src] + HEADERS] + [os.path.abspath(__file__)]
+    if force or _stale(obj, deps):
+        tmp = "%s.%d.tmp.o" % (obj, os.getpid())
+        cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC"]
+        subprocess.check_call(cmd + (["-Xptxas", "-v"] if verbose else []) + ["-c", "-o", tmp, os.path.join(CSRC, src)])
+        os.replace(tmp, obj)
+    return obj
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not needs_build():
         return LIB
+    os.makedirs(os.path.join(HERE, "_build"), exist_ok=True)
+    with ThreadPoolExecutor() as pool:
+        objects = list(pool.map(lambda src: _compile(src, force, verbose), SOURCES))
     tmp = LIB + ".%d.tmp" % os.getpid()
-    cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-           "-shared", "-Xcompiler", "-fPIC", "-o", tmp] + [os.path.join(CSRC, f) for f in SOURCES]
-    if verbose:
-        cmd.insert(1, "-Xptxas")
-        cmd.insert(2, "-v")
-    subprocess.check_call(cmd)
+    subprocess.check_call([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-Xcompiler", "-fPIC", "-o", tmp] + objects)
     os.replace(tmp, LIB)
     return LIB
 

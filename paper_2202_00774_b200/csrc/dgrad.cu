@@ -195,40 +195,17 @@ template <int M, int N, int SCHEME>
 __device__ __forceinline__ void fused_prune_eighth(const uint8_t* raw, int a_bytes, uint8_t* a_tile, uint8_t* meta_rows,
                                                    int i, int e, int64_t vbase, uint32_t seed_lo, uint32_t seed_hi) {
   const int sw = i & 7;
-  uint32_t nibs = 0u;
-  uint2 out[2];
-  uint4 w[2];
+  uint4 w[2], out;
 #pragma unroll
   for (int jj = 0; jj < 2; ++jj) {
     const int j = 2 * e + jj;
     w[jj] = *(const uint4*)(raw + (j >> 3) * a_bytes + i * 128 + (((j & 7) ^ sw) << 4));
   }
-  uint32_t y[2][4], km[2][4];
-  if (M == 16) {  // the thread's two vectors are one group
-    top2_prune_group16<SCHEME>(w[0], w[1], vbase + 2 * e, seed_lo, seed_hi, N, y[0], km[0], y[1], km[1]);
-  } else {
-#pragma unroll
-    for (int jj = 0; jj < 2; ++jj) {
-      if (M == 4)
-        m4_prune_vector<N, SCHEME>(w[jj], vbase + 2 * e + jj, seed_lo, seed_hi, y[jj][0], y[jj][1], y[jj][2], y[jj][3], km[jj][0],
-                                   km[jj][1], km[jj][2], km[jj][3]);
-      else
-        top2_prune_vector<8, SCHEME>(w[jj], vbase + 2 * e + jj, seed_lo, seed_hi, N, 0, 0u, y[jj][0], y[jj][1], y[jj][2], y[jj][3],
-                                     km[jj][0], km[jj][1], km[jj][2], km[jj][3]);
-    }
-  }
-#pragma unroll
-  for (int jj = 0; jj < 2; ++jj) {
-    uint32_t slot0, slot1, nib2;
-    if (M == 4 && SCHEME == SDGP_RESCALED_MAGNITUDE)  // (the lanes above are dead code then: the slots are rescaled, not the lanes)
-      m4_rescaled_compressed<N, false>(w[jj], slot0, slot1, nib2, km[jj][0], km[jj][1], km[jj][2], km[jj][3]);
-    else
-      compressed_slots(y[jj][0], y[jj][1], y[jj][2], y[jj][3], km[jj][0], km[jj][1], km[jj][2], km[jj][3], slot0, slot1, nib2);
-    out[jj] = make_uint2(prmt(slot0, slot1, 0x5410), prmt(slot0, slot1, 0x7632));
-    nibs |= nib2 << (8 * jj);
-  }
-  *(uint4*)(a_tile + i * 128 + ((e ^ sw) << 4)) = make_uint4(out[0].x, out[0].y, out[1].x, out[1].y);
-  *(uint16_t*)(meta_rows + i * 16 + 2 * e) = (uint16_t)nibs;
+  uint32_t pos[2];
+  KeepFlags ka, kb;
+  compress_pair<M, N, SCHEME, false>(w[0], w[1], vbase + 2 * e, seed_lo, seed_hi, 0, 0u, out, pos[0], pos[1], ka, kb);
+  *(uint4*)(a_tile + i * 128 + ((e ^ sw) << 4)) = out;
+  *(uint16_t*)(meta_rows + i * 16 + 2 * e) = (uint16_t)prmt(pos[0], pos[1], 0x0073);
 }
 
 // The four epilogue warps move one 128-row x BN accumulator to global memory in 64-column
@@ -758,25 +735,13 @@ struct HaloParams {
 template <int M, int N, int SCHEME>
 __device__ __forceinline__ void fused_prune_vectors(const uint4 (&w)[4], int64_t vbase, int vstep, uint32_t seed_lo,
                                                     uint32_t seed_hi, int part, uint2 (&out)[4], uint32_t& metaw) {
-  metaw = 0u;
+  uint32_t pos[4];
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
-    uint32_t y0, y1, y2, y3, km0, km1, km2, km3, slot0, slot1, nib2;
-    if (M == 4 && SCHEME == SDGP_RESCALED_MAGNITUDE) {
-      m4_rescaled_compressed<N, false>(w[v], slot0, slot1, nib2, km0, km1, km2, km3);  // the slots are rescaled, not the lanes
-    } else if (SCHEME == SDGP_RESCALED_MAGNITUDE) {
-      top2_rescaled_compressed<(M == 4 ? 8 : M), false>(w[v], N, part, 0xFFFFFFFFu, slot0, slot1, nib2, km0, km1, km2, km3);
-    } else {
-      if (M == 4)
-        m4_prune_vector<N, SCHEME>(w[v], vbase + vstep * v, seed_lo, seed_hi, y0, y1, y2, y3, km0, km1, km2, km3);
-      else
-        top2_prune_vector<(M == 4 ? 8 : M), SCHEME>(w[v], vbase + vstep * v, seed_lo, seed_hi, N, part, 0xFFFFFFFFu, y0, y1, y2,
-                                                    y3, km0, km1, km2, km3);
-      compressed_slots(y0, y1, y2, y3, km0, km1, km2, km3, slot0, slot1, nib2);
-    }
-    out[v] = make_uint2(prmt(slot0, slot1, 0x5410), prmt(slot0, slot1, 0x7632));
-    metaw |= nib2 << (8 * v);
+    KeepFlags k;
+    compress_vector<M, N, SCHEME, false>(w[v], vbase + vstep * v, seed_lo, seed_hi, part, 0xFFFFFFFFu, out[v], pos[v], k);
   }
+  metaw = prmt(prmt(pos[0], pos[1], 0x0073), prmt(pos[2], pos[3], 0x0073), 0x5410);
 }
 
 // 16 bytes from global memory, read-only path, kept out of L1 (each byte is used once by this SM).
@@ -1468,6 +1433,8 @@ int current_device() {
   return dev;
 }
 
+}  // namespace
+
 int sm_count() {
   static int n[kMaxDevices] = {};
   const int dev = current_device();
@@ -1479,6 +1446,8 @@ int sm_count() {
   }
   return n[dev];
 }
+
+namespace {
 
 // Opts `kernel` in to the large dynamic shared-memory carve, once per device and instantiation.
 template <typename K>

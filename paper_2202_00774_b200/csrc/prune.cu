@@ -17,19 +17,11 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kVecPerThread = 4;
-// Resident blocks per SM the compiler is asked to make room for. Six (at most 40 registers per thread instead of the 42-46
-// it takes unasked, which round up to five blocks) measured 7 % more bytes per second for the magnitude function, 6 % for
-// groups of 8 and 3 % for the random function; the rescaled function and the producers below a ReLU spill at 40 registers
-// and measured slower, so they keep the compiler's own choice. Eight blocks (32 registers, 64-72 bytes spilled per thread)
-// measured 9 % fewer bytes per second than six.
-template <int SCHEME, bool RELU>
-constexpr int kBlocksPerSm = (!RELU && SCHEME != SDGP_RESCALED_MAGNITUDE) ? 6 : 0;
-
-// Survivor positions of a 4-chunk from its 4-bit keep mask: pad with the lowest unused
-// positions up to two, ascending; entry = p0 | p1 << 2 (16 nibbles packed in 64 bits).
-__device__ __forceinline__ uint32_t chunk_nibble(uint32_t keep4) {
-  return (uint32_t)(0x444E4DCC49884444ull >> (4 * keep4)) & 0xFu;
-}
+// Resident blocks per SM the compiler is asked to make room for. Pruning dL/dO itself under the magnitude function: six
+// (40 registers; five measured the same for groups of 4 and 3 % slower for groups of 8). The random and rescaled functions:
+// five (48 registers; six spill and measured 1-5 % slower). The producers below a ReLU keep the compiler's own choice.
+template <int SCHEME, int SRC>
+constexpr int kBlocksPerSm = SRC != 0 ? 0 : SCHEME == SDGP_MAGNITUDE ? 6 : 5;
 
 // Launch with programmatic stream serialisation: the kernel may be scheduled while the previous
 // kernel of the stream is still draining; it waits for that kernel before its first load.
@@ -48,6 +40,9 @@ cudaError_t launch_after_previous(void (*kernel)(Params...), dim3 grid, dim3 blo
   return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
 }
 
+// Where the vectors come from: dL/dO itself; the gradient above a ReLU; the gradient above a 2 x 2 max pooling and a ReLU.
+enum Source { kPlain, kRelu, kPool };
+
 // The producer of dL/dO below a ReLU (Section 2.1, Fig. 2): the 8 gradients g above the ReLU pass where the
 // ReLU's activation a is positive (a number greater than zero: sign clear, magnitude between 1 and the
 // pattern of infinity) and become +0.0 elsewhere. nan_add = 0x7FFF - (pattern of infinity) in both half-words:
@@ -62,6 +57,7 @@ struct ReluSource {
   // 2 x 2 max pooling of stride 2 above the ReLU (pool_k8 != 0): the input gradient has the pooled shape
   // [B, H/2, W/2, K] and `act` the full one [B, H, W, K]; pool_k8 = K / 8, pool_hp = H / 2, pool_wp = W / 2.
   int pool_k8, pool_hp, pool_wp;
+  bool aligned32;     // every vector tensor that is read (and `grad`) starts on a 32-byte boundary
 };
 
 // Two 16-bit elements of each gradient, added in fp32 (one rounding) and rounded to the 16-bit type to nearest-even;
@@ -79,22 +75,33 @@ __device__ __forceinline__ uint32_t relu_pass2(uint32_t g, uint32_t a, uint32_t 
   return g & prmt(ok, 0u, 0xBB99);  // top bits replicated over their half-words
 }
 
-template <bool RELU>
-__device__ __forceinline__ uint4 load_gradient(const uint4* __restrict__ dO, int64_t v, const ReluSource& src) {
-  uint4 g = __ldg(dO + v);
-  if (RELU) {
-    const uint4 a = __ldg(src.act + v);
-    if (src.skip) {
-      const uint4 k = __ldg(src.skip + v);
-      g = src.f16 ? make_uint4(add_pair<true>(g.x, k.x), add_pair<true>(g.y, k.y), add_pair<true>(g.z, k.z), add_pair<true>(g.w, k.w))
-                  : make_uint4(add_pair<false>(g.x, k.x), add_pair<false>(g.y, k.y), add_pair<false>(g.z, k.z),
-                               add_pair<false>(g.w, k.w));
-    }
-    g = make_uint4(relu_pass2(g.x, a.x, src.nan_add), relu_pass2(g.y, a.y, src.nan_add), relu_pass2(g.z, a.z, src.nan_add),
-                   relu_pass2(g.w, a.w, src.nan_add));
-    if (src.grad) src.grad[v] = g;
+__device__ __forceinline__ uint4 add_vectors(const uint4& g, const uint4& k, int f16) {
+  return f16 ? make_uint4(add_pair<true>(g.x, k.x), add_pair<true>(g.y, k.y), add_pair<true>(g.z, k.z), add_pair<true>(g.w, k.w))
+             : make_uint4(add_pair<false>(g.x, k.x), add_pair<false>(g.y, k.y), add_pair<false>(g.z, k.z), add_pair<false>(g.w, k.w));
+}
+
+__device__ __forceinline__ uint4 relu_vector(const uint4& g, const uint4& a, uint32_t nan_add) {
+  return make_uint4(relu_pass2(g.x, a.x, nan_add), relu_pass2(g.y, a.y, nan_add), relu_pass2(g.z, a.z, nan_add),
+                    relu_pass2(g.w, a.w, nan_add));
+}
+
+// Vectors v and v + 1 of dL/dO below a ReLU: the gradients above it, wa and wb, plus the second gradient where there is one,
+// gated by the activation; written out as well if the caller keeps the unpruned tensor.
+__device__ __forceinline__ void relu_pair(int64_t v, bool aligned32, const ReluSource& src, uint4& wa, uint4& wb) {
+  uint4 aa, ab;
+  load_pair(src.act + v, aligned32, aa, ab);
+  if (src.skip) {
+    uint4 ka, kb;
+    load_pair(src.skip + v, aligned32, ka, kb);
+    wa = add_vectors(wa, ka, src.f16);
+    wb = add_vectors(wb, kb, src.f16);
   }
-  return g;
+  wa = relu_vector(wa, aa, src.nan_add);
+  wb = relu_vector(wb, ab, src.nan_add);
+  if (src.grad) {
+    src.grad[v] = wa;
+    src.grad[v + 1] = wb;
+  }
 }
 
 // Pooling backward for one 32-bit word (two channels) of a window: a[0..3] are the activation words at the window's
@@ -125,10 +132,10 @@ __device__ __forceinline__ void pool_select2(const uint32_t (&a)[4], uint32_t g,
 // slots of four consecutive 256-vector stripes (every load of a warp is one contiguous 512 bytes). With pooling a
 // thread owns the four pixels of one window for one 8-channel vector: it reads the pooled gradient once and the four
 // activation vectors, and its lanes still hold neighbouring channel vectors of the same pixel.
-template <bool RELU>
+template <int SRC>
 __device__ __forceinline__ void load_unit(const uint4* __restrict__ dO, int64_t nvec, const ReluSource& src,
                                           int64_t (&vi)[kVecPerThread], uint4 (&in)[kVecPerThread]) {
-  if (RELU && src.pool_k8 != 0) {
+  if (SRC == kPool) {
     const int64_t u = (int64_t)blockIdx.x * kThreads + threadIdx.x;  // number of the pooled gradient's vector
     const bool live = u < (nvec >> 2);
     int64_t pix00 = 0;
@@ -150,10 +157,7 @@ __device__ __forceinline__ void load_unit(const uint4* __restrict__ dO, int64_t 
     }
     uint4 g = live ? __ldg(dO + u) : make_uint4(0u, 0u, 0u, 0u);
     if (live && src.skip) {  // a second gradient of the pooled shape (a residual connection joins below the pooling)
-      const uint4 k = __ldg(src.skip + u);
-      g = src.f16 ? make_uint4(add_pair<true>(g.x, k.x), add_pair<true>(g.y, k.y), add_pair<true>(g.z, k.z), add_pair<true>(g.w, k.w))
-                  : make_uint4(add_pair<false>(g.x, k.x), add_pair<false>(g.y, k.y), add_pair<false>(g.z, k.z),
-                               add_pair<false>(g.w, k.w));
+      g = add_vectors(g, __ldg(src.skip + u), src.f16);
     }
     uint32_t ox[4], oy[4], oz[4], ow[4];
     const uint32_t ax[4] = {a[0].x, a[1].x, a[2].x, a[3].x}, ay[4] = {a[0].y, a[1].y, a[2].y, a[3].y},
@@ -173,146 +177,14 @@ __device__ __forceinline__ void load_unit(const uint4* __restrict__ dO, int64_t 
 #pragma unroll
   for (int it = 0; it < kVecPerThread; ++it) {
     vi[it] = base + (int64_t)it * kThreads;
-    in[it] = (vi[it] < nvec) ? load_gradient<RELU>(dO, vi[it], src) : make_uint4(0, 0, 0, 0);
-  }
-}
-
-// M: group size; LANES = lanes that share a group (1, 2 or 4).
-template <int M, int SCHEME, bool F16>
-__global__ void __launch_bounds__(kThreads)
-prune_kernel(const uint4* __restrict__ dO, int64_t nvec, int n, uint32_t seed_lo, uint32_t seed_hi,
-             uint4* __restrict__ dense, uint2* __restrict__ values, uint8_t* __restrict__ meta,
-             uint8_t* __restrict__ mask) {
-  ptx::wait_for_previous_grid();
-  ptx::launch_dependents();  // only once this grid's own predecessor is done: at most one grid ever waits behind a running one
-  constexpr int LANES = (M <= 8) ? 1 : M / 8;
-  constexpr int SUB = (M == 4) ? 4 : 8;  // elements of this thread that share a group
-  const int64_t base = (int64_t)blockIdx.x * (kThreads * kVecPerThread) + threadIdx.x;
-
-  uint4 in[kVecPerThread];
-#pragma unroll
-  for (int it = 0; it < kVecPerThread; ++it) {
-    const int64_t v = base + (int64_t)it * kThreads;
-    in[it] = (v < nvec) ? __ldg(dO + v) : make_uint4(0, 0, 0, 0);
-  }
-
-#pragma unroll
-  for (int it = 0; it < kVecPerThread; ++it) {
-    const int64_t v = base + (int64_t)it * kThreads;
-    const uint32_t w[4] = {in[it].x, in[it].y, in[it].z, in[it].w};
-    uint32_t x[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] = (i & 1) ? (w[i >> 1] >> 16) : (w[i >> 1] & 0xFFFFu);
-
-    // ---- ranking key: larger composite = better; unique inside a group ----
-    uint32_t key16[8];
-    if (SCHEME == SDGP_RANDOM) {
-      const uint4 o = philox4x32_10((uint32_t)v, (uint32_t)((uint64_t)v >> 32), 0u, 0u, seed_lo, seed_hi);
-      const uint32_t r[4] = {o.x, o.y, o.z, o.w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const uint32_t r16 = (i & 1) ? (r[i >> 1] >> 16) : (r[i >> 1] & 0xFFFFu);
-        key16[i] = 0xFFFFu - r16;  // smallest random key ranks first
+    in[it] = make_uint4(0, 0, 0, 0);
+    if (vi[it] < nvec) {
+      in[it] = __ldg(dO + vi[it]);
+      if (SRC == kRelu) {
+        if (src.skip) in[it] = add_vectors(in[it], __ldg(src.skip + vi[it]), src.f16);
+        in[it] = relu_vector(in[it], __ldg(src.act + vi[it]), src.nan_add);
+        if (src.grad) src.grad[vi[it]] = in[it];
       }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) key16[i] = x[i] & 0x7FFFu;  // |x| as an integer
-    }
-    const int lane_in_group = (LANES == 1) ? 0 : (threadIdx.x & (LANES - 1));
-    uint32_t c[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int j = (M == 4) ? (i & 3) : (lane_in_group * 8 + i);  // position inside the group
-      c[i] = (key16[i] << 5) | (uint32_t)(31 - j);                 // ties: lower position wins
-    }
-
-    // ---- keep <=> fewer than n elements of the group rank above ----
-    int above[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      int cnt = 0;
-#pragma unroll
-      for (int o = 0; o < 8; ++o)
-        if (o != i && (o / SUB) == (i / SUB)) cnt += (c[o] > c[i]) ? 1 : 0;
-      above[i] = cnt;
-    }
-    if (LANES > 1) {
-#pragma unroll
-      for (int d = 1; d < LANES; ++d) {
-#pragma unroll
-        for (int o = 0; o < 8; ++o) {
-          const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, c[o], d);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) above[i] += (other > c[i]) ? 1 : 0;
-        }
-      }
-    }
-    uint32_t keep8 = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) keep8 |= (above[i] < n ? 1u : 0u) << i;
-
-    // ---- survivor values ----
-    uint32_t y[8];
-    if (SCHEME == SDGP_RESCALED_MAGNITUDE && n < M) {  // n == m: nothing pruned, nothing rescaled
-      float a[8], t[8], s[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        a[i] = lane_lo<F16>(x[i] & 0x7FFFu);
-        t[i] = a[i];
-        s[i] = ((keep8 >> i) & 1u) ? a[i] : 0.0f;
-      }
-      // balanced pairwise sums in index order; every add rounds once
-#pragma unroll
-      for (int width = 8; width > (8 / SUB); width >>= 1) {
-#pragma unroll
-        for (int i = 0; i < width / 2; ++i) {
-          t[i] = __fadd_rn(t[2 * i], t[2 * i + 1]);
-          s[i] = __fadd_rn(s[2 * i], s[2 * i + 1]);
-        }
-      }
-      // M == 4: t[0], t[1] are the two groups' sums; otherwise t[0] is this lane's partial
-      if (LANES > 1) {
-#pragma unroll
-        for (int d = 1; d < LANES; d <<= 1) {
-          t[0] = __fadd_rn(t[0], __shfl_xor_sync(0xFFFFFFFFu, t[0], d));
-          s[0] = __fadd_rn(s[0], __shfl_xor_sync(0xFFFFFFFFu, s[0], d));
-        }
-      }
-      float scale[2];
-#pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        const int src = (M == 4) ? g : 0;
-        scale[g] = (s[src] == 0.0f) ? 1.0f : __fdiv_rn(t[src], s[src]);
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float xf = lane_lo<F16>(x[i]);
-        y[i] = ((keep8 >> i) & 1u) ? f32_to_elem_bits<F16>(__fmul_rn(xf, scale[i >> 2])) : 0u;
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) y[i] = ((keep8 >> i) & 1u) ? x[i] : 0u;
-    }
-
-    if (v >= nvec) continue;
-
-    // ---- emit ----
-    if (dense) dense[v] = make_uint4(y[0] | (y[1] << 16), y[2] | (y[3] << 16), y[4] | (y[5] << 16), y[6] | (y[7] << 16));
-    if (mask) mask[v] = (uint8_t)keep8;
-    if (values || meta) {
-      uint32_t slots[4];
-      uint32_t nib2 = 0;
-#pragma unroll
-      for (int ch = 0; ch < 2; ++ch) {
-        const uint32_t nib = chunk_nibble((keep8 >> (4 * ch)) & 0xFu);
-        const uint64_t quad = (uint64_t)(y[4 * ch] | (y[4 * ch + 1] << 16)) |
-                              ((uint64_t)(y[4 * ch + 2] | (y[4 * ch + 3] << 16)) << 32);
-        slots[2 * ch] = (uint32_t)(quad >> (16 * (nib & 3u))) & 0xFFFFu;
-        slots[2 * ch + 1] = (uint32_t)(quad >> (16 * (nib >> 2))) & 0xFFFFu;
-        nib2 |= nib << (4 * ch);
-      }
-      if (values) values[v] = make_uint2(slots[0] | (slots[1] << 16), slots[2] | (slots[3] << 16));
-      if (meta) meta[v] = (uint8_t)nib2;
     }
   }
 }
@@ -349,10 +221,14 @@ __device__ __forceinline__ int64_t compressed_index(int64_t v, uint2* __restrict
   return vo;
 }
 
-__device__ __forceinline__ void emit_mask(int64_t v, uint32_t km0, uint32_t km1, uint32_t km2, uint32_t km3,
-                                          uint8_t* __restrict__ mask) {
-  const uint32_t t = (km0 & 0x00010001u) | (km1 & 0x00020002u) | (km2 & 0x00040004u) | (km3 & 0x00080008u);
-  mask[v] = (uint8_t)((t & 0xFu) | (t >> 12));
+// Keep flags (bit 15 of each lane) as the vector's mask byte, in the TOP byte of the result.
+__device__ __forceinline__ uint32_t mask_top_byte(const KeepFlags& k) {
+  constexpr uint32_t H = 0x80008000u;
+  uint32_t x = k.k0 & H;
+  x = (x >> 1) | (k.k1 & H);
+  x = (x >> 1) | (k.k2 & H);
+  x = (x >> 1) | (k.k3 & H);       // bits 12..15 and 28..31: elements 0..3 of chunk A and of chunk B
+  return x * 0x00001001u;          // ... side by side in bits 24..31
 }
 
 // Writes one vector's outputs from the lane-paired form (see m4_prune_vector). COMPRESS: every
@@ -363,173 +239,125 @@ __device__ __forceinline__ void emit_packed(int64_t v, uint32_t y0, uint32_t y1,
                                             uint4* __restrict__ dense, uint2* __restrict__ values,
                                             uint8_t* __restrict__ meta, uint8_t* __restrict__ mask,
                                             OutPitch pitch) {
-  const int64_t vo = COMPRESS ? compressed_index(v, values, meta, pitch) : v;
-  if (dense)
-    dense[v] = make_uint4(prmt(y0, y1, 0x5410), prmt(y2, y3, 0x5410), prmt(y0, y1, 0x7632), prmt(y2, y3, 0x7632));
-  if (mask) emit_mask(v, km0, km1, km2, km3, mask);
+  const uint4 pruned = make_uint4(prmt(y0, y1, 0x5410), prmt(y2, y3, 0x5410), prmt(y0, y1, 0x7632), prmt(y2, y3, 0x7632));
+  const KeepFlags k = {km0, km1, km2, km3};
+  if (dense) dense[v] = pruned;
+  if (mask) mask[v] = (uint8_t)(mask_top_byte(k) >> 24);
   if (COMPRESS && (values || meta)) {
-    uint32_t slot0, slot1, nib2;
-    compressed_slots(y0, y1, y2, y3, km0, km1, km2, km3, slot0, slot1, nib2);
-    if (values) values[vo] = make_uint2(prmt(slot0, slot1, 0x5410), prmt(slot0, slot1, 0x7632));
-    if (meta) meta[vo] = (uint8_t)nib2;
+    const int64_t vo = compressed_index(v, values, meta, pitch);
+    uint2 out, slot_mask;
+    uint32_t pos_top;
+    gather_slots<false>(pruned, k, out, slot_mask, pos_top);
+    if (values) values[vo] = out;
+    if (meta) meta[vo] = (uint8_t)(pos_top >> 24);
   }
 }
 
-template <int N, int SCHEME, bool F16, bool RELU>
-__global__ void __launch_bounds__(kThreads, kBlocksPerSm<SCHEME, RELU>)
-prune_m4_kernel(const uint4* __restrict__ dO, int64_t nvec, uint32_t seed_lo, uint32_t seed_hi,
-                uint4* __restrict__ dense, uint2* __restrict__ values, uint8_t* __restrict__ meta,
-                uint8_t* __restrict__ mask, OutPitch pitch, ReluSource src) {
+// Algorithm 1 for m = 4 (any n) and for groups of 8, 16 and 32 with n <= 2. Bound: HBM for the magnitude function of m = 4,
+// the integer pipe for the others. Without a dense copy a thread owns PAIRS of vectors: 32-byte loads, 16 bytes of values, two
+// of metadata and two of mask per store - half the memory instructions and address arithmetic per element of the
+// one-vector form, and a group of 16 needs no shuffles. DENSE (a dense pruned copy is asked for, or n > 2) and the pooling
+// source, whose threads own the four pixels of a window, keep single vectors.
+template <int M, int N, int SCHEME, bool F16, int SRC, bool DENSE>
+__global__ void __launch_bounds__(kThreads, kBlocksPerSm<SCHEME, SRC>)
+prune_kernel(const uint4* __restrict__ dO, int64_t nvec, uint32_t seed_lo, uint32_t seed_hi,
+             uint4* __restrict__ dense, uint2* __restrict__ values, uint8_t* __restrict__ meta,
+             uint8_t* __restrict__ mask, OutPitch pitch, ReluSource src) {
   ptx::wait_for_previous_grid();
   ptx::launch_dependents();  // only once this grid's own predecessor is done: at most one grid ever waits behind a running one
-  uint4 in[kVecPerThread];
-  int64_t vi[kVecPerThread];
-  load_unit<RELU>(dO, nvec, src, vi, in);
+  if constexpr (!DENSE && SRC != kPool) {
+    constexpr int kPairs = kVecPerThread / 2;
+    const int64_t npair = nvec >> 1;  // (nvec is even)
+    const int64_t base = (int64_t)blockIdx.x * kThreads + threadIdx.x, stride = (int64_t)gridDim.x * kThreads;
+    const bool al = src.aligned32;
+    uint4 wa[kPairs], wb[kPairs];
 #pragma unroll
-  for (int it = 0; it < kVecPerThread; ++it) {
-    const int64_t v = vi[it];
-    if (v >= nvec) continue;
-    const uint4 w = in[it];
-    uint32_t y0, y1, y2, y3, km0, km1, km2, km3;
-    if constexpr (SCHEME == SDGP_RESCALED_MAGNITUDE && N <= 2) {
-      if (!dense) {  // only the compressed form is wanted: rescale the two slots instead of the eight lanes
-        uint32_t slot0, slot1, nib2;
-        m4_rescaled_compressed<N, F16>(w, slot0, slot1, nib2, km0, km1, km2, km3);
-        const int64_t vo = compressed_index(v, values, meta, pitch);
-        if (mask) emit_mask(v, km0, km1, km2, km3, mask);
-        if (values) values[vo] = make_uint2(prmt(slot0, slot1, 0x5410), prmt(slot0, slot1, 0x7632));
-        if (meta) meta[vo] = (uint8_t)nib2;
-        continue;
+    for (int it = 0; it < kPairs; ++it) {
+      const int64_t p = base + it * stride;
+      wa[it] = wb[it] = make_uint4(0u, 0u, 0u, 0u);
+      if (p < npair) {
+        load_pair(dO + 2 * p, al, wa[it], wb[it]);
+        if (SRC == kRelu) relu_pair(2 * p, al, src, wa[it], wb[it]);
       }
     }
-    m4_prune_vector<N, SCHEME, F16>(w, v, seed_lo, seed_hi, y0, y1, y2, y3, km0, km1, km2, km3);
-    emit_packed<(N <= 2)>(v, y0, y1, y2, y3, km0, km1, km2, km3, dense, values, meta, mask, pitch);
+#pragma unroll
+    for (int it = 0; it < kPairs; ++it) {
+      const int64_t p = base + it * stride;
+      if (M < 32 && p >= npair) continue;  // (the lanes of a group of 32 meet in shuffles)
+      uint4 out;
+      uint32_t pa, pb;
+      KeepFlags ka, kb;
+      compress_pair<M, N, SCHEME, F16>(wa[it], wb[it], 2 * p, seed_lo, seed_hi, M == 32 ? (int)(threadIdx.x & 1) : 0, 0xFFFFFFFFu,
+                                       out, pa, pb, ka, kb);
+      if (M == 32 && p >= npair) continue;
+      const int64_t po = pitch.kpad8 == 0 ? p : compressed_index(2 * p + 1, values, meta, pitch) >> 1;
+      if (values) ((uint4*)values)[po] = out;
+      if (meta) ((uint16_t*)meta)[po] = (uint16_t)prmt(pa, pb, 0x0073);
+      if (mask) ((uint16_t*)mask)[p] = (uint16_t)prmt(mask_top_byte(ka), mask_top_byte(kb), 0x0073);
+    }
+  } else {
+    constexpr int LANES = M <= 8 ? 1 : M / 8;
+    const int part = (int)(threadIdx.x & (LANES - 1));
+    uint4 in[kVecPerThread];
+    int64_t vi[kVecPerThread];
+    load_unit<SRC>(dO, nvec, src, vi, in);
+#pragma unroll
+    for (int it = 0; it < kVecPerThread; ++it) {
+      const int64_t v = vi[it];
+      if (LANES == 1 && v >= nvec) continue;
+      if constexpr (!DENSE) {
+        uint2 out;
+        uint32_t pos_top;
+        KeepFlags k;
+        compress_vector<M, N, SCHEME, F16>(in[it], v, seed_lo, seed_hi, part, 0xFFFFFFFFu, out, pos_top, k);
+        if (LANES > 1 && v >= nvec) continue;
+        const int64_t vo = compressed_index(v, values, meta, pitch);
+        if (values) values[vo] = out;
+        if (meta) meta[vo] = (uint8_t)(pos_top >> 24);
+        if (mask) mask[v] = (uint8_t)(mask_top_byte(k) >> 24);
+      } else {
+        uint32_t y0, y1, y2, y3, km0, km1, km2, km3;
+        if constexpr (M == 4)
+          m4_prune_vector<N, SCHEME, F16>(in[it], v, seed_lo, seed_hi, y0, y1, y2, y3, km0, km1, km2, km3);
+        else
+          top2_prune_vector<M, SCHEME, F16>(in[it], v, seed_lo, seed_hi, N, part, 0xFFFFFFFFu, y0, y1, y2, y3, km0, km1, km2, km3);
+        if (LANES > 1 && v >= nvec) continue;
+        emit_packed<(N <= 2)>(v, y0, y1, y2, y3, km0, km1, km2, km3, dense, values, meta, mask, pitch);
+      }
+    }
   }
 }
 
 // Only the rescaled scheme reads values as numbers: the other two run the same (bf16-named)
 // instantiation for both element types.
-template <int N, bool RELU>
-cudaError_t launch_m4_n(int scheme, bool f16, const void* dO, int64_t nvec, uint64_t seed, void* dense, void* values,
-                        void* meta, void* mask, OutPitch pitch, cudaStream_t stream, ReluSource src) {
-  const int64_t per_block = (int64_t)kThreads * kVecPerThread;
-  const int64_t blocks = (nvec + per_block - 1) / per_block;
-  if (blocks == 0) return cudaSuccess;
-  if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)blocks), block(kThreads);
+template <int M, int N, int SRC>
+cudaError_t launch_select(int scheme, bool f16, const void* dO, int64_t nvec, uint64_t seed, void* dense, void* values,
+                          void* meta, void* mask, OutPitch pitch, cudaStream_t stream, ReluSource src) {
+  if (nvec == 0) return cudaSuccess;
   const uint32_t lo = (uint32_t)seed, hi = (uint32_t)(seed >> 32);
-#define SDGP_LAUNCH4(S, F)                                                                      \
-  launch_after_previous(prune_m4_kernel<N, S, F, RELU>, grid, block, stream, (const uint4*)dO, nvec, lo, hi, (uint4*)dense, \
-                                                    (uint2*)values, (uint8_t*)meta, (uint8_t*)mask, pitch, src)
-  switch (scheme) {
-    case SDGP_RANDOM: SDGP_LAUNCH4(SDGP_RANDOM, false); break;
-    case SDGP_MAGNITUDE: SDGP_LAUNCH4(SDGP_MAGNITUDE, false); break;
-    default:
-      if (f16) SDGP_LAUNCH4(SDGP_RESCALED_MAGNITUDE, true);
-      else SDGP_LAUNCH4(SDGP_RESCALED_MAGNITUDE, false);
-      break;
-  }
-#undef SDGP_LAUNCH4
-  return cudaGetLastError();
+  auto launch = [&](auto kernel, bool pairs) {
+    // Pairs: two per thread, or one where all blocks of that split are resident at once anyway (a small tensor is a matter of
+    // latency: 256 x 512 elements take 32 blocks instead of 16). A persistent grid that prefetches a thread's next pair
+    // measured 3-15 % slower than blocks that come and go.
+    const int64_t singles = (nvec + 2 * kThreads - 1) / (2 * kThreads);
+    const int64_t per_block = pairs && singles <= 4 * (int64_t)sm_count() ? 2 * kThreads : kThreads * kVecPerThread;
+    const int64_t blocks = (nvec + per_block - 1) / per_block;
+    if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
+    const dim3 grid((unsigned)blocks), block(kThreads);
+    return launch_after_previous(kernel, grid, block, stream, (const uint4*)dO, nvec, lo, hi, (uint4*)dense, (uint2*)values,
+                                 (uint8_t*)meta, (uint8_t*)mask, pitch, src);
+  };
+#define SDGP_SELECT(S, F)                                                                                          \
+  if (N > 2 || dense) return launch(prune_kernel<M, N, S, F, SRC, true>, false);                                \
+  else if constexpr (N <= 2) return launch(prune_kernel<M, N, S, F, SRC, false>, SRC != kPool)
+  if (scheme == SDGP_RANDOM) { SDGP_SELECT(SDGP_RANDOM, false); }
+  else if (scheme == SDGP_MAGNITUDE) { SDGP_SELECT(SDGP_MAGNITUDE, false); }
+  else if (f16) { SDGP_SELECT(SDGP_RESCALED_MAGNITUDE, true); }
+  else { SDGP_SELECT(SDGP_RESCALED_MAGNITUDE, false); }
+#undef SDGP_SELECT
 }
 
-// ------------------------------------------------------------------------------------------
-// Groups of 8, 16 or 32 with n <= 2: the survivors are the elements whose composite key
-// (rank key << 5 | 31 - position, unique inside a group) reaches the group's n-th largest key.
-// Each thread finds the two largest keys of its 8 elements with a max/min network, groups that
-// span 2 or 4 lanes merge their pairs through xor-shuffles, and the outputs are written from the
-// same lane-paired form as the m = 4 path.
-
-template <int M, int N, int SCHEME, bool F16, bool RELU>
-__global__ void __launch_bounds__(kThreads, kBlocksPerSm<SCHEME, RELU>)
-prune_top2_kernel(const uint4* __restrict__ dO, int64_t nvec, uint32_t seed_lo, uint32_t seed_hi,
-                  uint4* __restrict__ dense, uint2* __restrict__ values, uint8_t* __restrict__ meta,
-                  uint8_t* __restrict__ mask, OutPitch pitch, ReluSource src) {
-  ptx::wait_for_previous_grid();
-  ptx::launch_dependents();  // only once this grid's own predecessor is done: at most one grid ever waits behind a running one
-  constexpr int LANES = M / 8;
-  static_assert(N == 1 || N == 2, "threshold selection keeps one or two elements");
-  uint4 in[kVecPerThread];
-  int64_t vi[kVecPerThread];
-  load_unit<RELU>(dO, nvec, src, vi, in);
-#pragma unroll
-  for (int it = 0; it < kVecPerThread; ++it) {
-    const int64_t v = vi[it];
-    uint32_t y0, y1, y2, y3, km0, km1, km2, km3;
-    if constexpr (SCHEME == SDGP_RESCALED_MAGNITUDE) {
-      if (!dense) {  // (uniform over the grid: every lane of a group takes the same branch and meets in the shuffles)
-        uint32_t slot0, slot1, nib2;
-        top2_rescaled_compressed<M, F16>(in[it], N, (int)(threadIdx.x & (LANES - 1)), 0xFFFFFFFFu, slot0, slot1, nib2, km0, km1,
-                                         km2, km3);
-        if (v < nvec) {
-          const int64_t vo = compressed_index(v, values, meta, pitch);
-          if (mask) emit_mask(v, km0, km1, km2, km3, mask);
-          if (values) values[vo] = make_uint2(prmt(slot0, slot1, 0x5410), prmt(slot0, slot1, 0x7632));
-          if (meta) meta[vo] = (uint8_t)nib2;
-        }
-        continue;
-      }
-    }
-    top2_prune_vector<M, SCHEME, F16>(in[it], v, seed_lo, seed_hi, N, (int)(threadIdx.x & (LANES - 1)), 0xFFFFFFFFu, y0, y1, y2,
-                                      y3, km0, km1, km2, km3);
-    if (v < nvec) emit_packed<true>(v, y0, y1, y2, y3, km0, km1, km2, km3, dense, values, meta, mask, pitch);
-  }
-}
-
-template <int M, int N, bool RELU>
-cudaError_t launch_top2(int scheme, bool f16, const void* dO, int64_t nvec, uint64_t seed, void* dense, void* values,
-                        void* meta, void* mask, OutPitch pitch, cudaStream_t stream, ReluSource src) {
-  const int64_t per_block = (int64_t)kThreads * kVecPerThread;
-  const int64_t blocks = (nvec + per_block - 1) / per_block;
-  if (blocks == 0) return cudaSuccess;
-  if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)blocks), block(kThreads);
-  const uint32_t lo = (uint32_t)seed, hi = (uint32_t)(seed >> 32);
-#define SDGP_LAUNCH_T2(S, F)                                                                         \
-  launch_after_previous(prune_top2_kernel<M, N, S, F, RELU>, grid, block, stream, (const uint4*)dO, nvec, lo, hi, (uint4*)dense, \
-                                                         (uint2*)values, (uint8_t*)meta, (uint8_t*)mask, pitch, src)
-  switch (scheme) {
-    case SDGP_RANDOM: SDGP_LAUNCH_T2(SDGP_RANDOM, false); break;
-    case SDGP_MAGNITUDE: SDGP_LAUNCH_T2(SDGP_MAGNITUDE, false); break;
-    default:
-      if (f16) SDGP_LAUNCH_T2(SDGP_RESCALED_MAGNITUDE, true);
-      else SDGP_LAUNCH_T2(SDGP_RESCALED_MAGNITUDE, false);
-      break;
-  }
-#undef SDGP_LAUNCH_T2
-  return cudaGetLastError();
-}
-
-template <int M>
-cudaError_t launch_m(int scheme, bool f16, const void* dO, int64_t nvec, int n, uint64_t seed, void* dense,
-                     void* values, void* meta, void* mask, cudaStream_t stream) {
-  const int64_t per_block = (int64_t)kThreads * kVecPerThread;
-  const int64_t blocks = (nvec + per_block - 1) / per_block;
-  if (blocks == 0) return cudaSuccess;
-  if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)blocks), block(kThreads);
-  const uint32_t lo = (uint32_t)seed, hi = (uint32_t)(seed >> 32);
-  // Plain launch, without programmatic stream serialisation (the kernel's griddepcontrol
-  // instructions then do nothing). With the attribute, a stream of back-to-back masked-mode steps
-  // (this kernel, dense data-gradient kernel, this kernel, ...) stopped making progress on B200 after
-  // a few steps, at 4:8, 8:16 and 4:32 alike; the m = 4 and top-2 kernels run thousands of such steps
-  // with it. The cause was not found; the overlap it would buy on this slower path is small.
-#define SDGP_LAUNCH(S, F)                                                                           \
-  prune_kernel<M, S, F><<<grid, block, 0, stream>>>((const uint4*)dO, nvec, n, lo, hi, (uint4*)dense,       \
-                                                    (uint2*)values, (uint8_t*)meta, (uint8_t*)mask)
-  switch (scheme) {
-    case SDGP_RANDOM: SDGP_LAUNCH(SDGP_RANDOM, false); break;
-    case SDGP_MAGNITUDE: SDGP_LAUNCH(SDGP_MAGNITUDE, false); break;
-    default:
-      if (f16) SDGP_LAUNCH(SDGP_RESCALED_MAGNITUDE, true);
-      else SDGP_LAUNCH(SDGP_RESCALED_MAGNITUDE, false);
-      break;
-  }
-#undef SDGP_LAUNCH
-  return cudaGetLastError();
-}
-
-template <bool RELU>
+template <int SRC>
 cudaError_t launch_prune_src(const void* dO, int64_t rows, int64_t K, int n, int m, int scheme, uint64_t seed, void* dense,
                              void* values, void* meta, void* mask, cudaStream_t stream, int64_t k_pad, int dtype,
                              ReluSource src) {
@@ -543,17 +371,17 @@ cudaError_t launch_prune_src(const void* dO, int64_t rows, int64_t K, int n, int
   switch (m) {
     case 4:
       switch (n) {
-        case 1: return launch_m4_n<1, RELU>(scheme, f16, dO, nvec, seed, dense, values, meta, mask, pitch, stream, src);
-        case 2: return launch_m4_n<2, RELU>(scheme, f16, dO, nvec, seed, dense, values, meta, mask, pitch, stream, src);
-        case 3: return launch_m4_n<3, RELU>(scheme, f16, dO, nvec, seed, dense, values, meta, mask, pitch, stream, src);
-        default: return launch_m4_n<4, RELU>(scheme, f16, dO, nvec, seed, dense, values, meta, mask, pitch, stream, src);
+        case 1: return launch_select<4, 1, SRC>(scheme, f16, dO, nvec, seed, dense, values, meta, mask, pitch, stream, src);
+        case 2: return launch_select<4, 2, SRC>(scheme, f16, dO, nvec, seed, dense, values, meta, mask, pitch, stream, src);
+        case 3: return launch_select<4, 3, SRC>(scheme, f16, dO, nvec, seed, dense, values, meta, mask, pitch, stream, src);
+        default: return launch_select<4, 4, SRC>(scheme, f16, dO, nvec, seed, dense, values, meta, mask, pitch, stream, src);
       }
 #define SDGP_M_CASE(M)                                                                                     \
   case M:                                                                                                  \
-    if (n == 1) return launch_top2<M, 1, RELU>(scheme, f16, dO, nvec, seed, dense, values, meta, mask, pitch, stream, src); \
-    if (n == 2) return launch_top2<M, 2, RELU>(scheme, f16, dO, nvec, seed, dense, values, meta, mask, pitch, stream, src); \
-    if (RELU) return cudaErrorInvalidValue; /* the generic kernel reads dL/dO itself */                      \
-    return launch_m<M>(scheme, f16, dO, nvec, n, seed, dense, values, meta, mask, stream);
+    if (n == 1) return launch_select<M, 1, SRC>(scheme, f16, dO, nvec, seed, dense, values, meta, mask, pitch, stream, src); \
+    if (n == 2) return launch_select<M, 2, SRC>(scheme, f16, dO, nvec, seed, dense, values, meta, mask, pitch, stream, src); \
+    if (SRC != kPlain || values || meta) return cudaErrorInvalidValue;                                        \
+    return launch_rank(dO, nvec, n, m, scheme, seed, dense, mask, stream, dtype); /* reads dL/dO itself */
     SDGP_M_CASE(8)
     SDGP_M_CASE(16)
     SDGP_M_CASE(32)
@@ -562,29 +390,32 @@ cudaError_t launch_prune_src(const void* dO, int64_t rows, int64_t K, int n, int
   }
 }
 
+bool aligned32(const void* p) { return ((uintptr_t)p & 31u) == 0; }
+
 }  // namespace
 
 cudaError_t launch_prune(const void* dO, int64_t rows, int64_t K, int n, int m, int scheme,
                          uint64_t seed, void* dense, void* values, void* meta, void* mask,
                          cudaStream_t stream, int64_t k_pad, int dtype) {
-  return launch_prune_src<false>(dO, rows, K, n, m, scheme, seed, dense, values, meta, mask, stream, k_pad, dtype,
-                                 ReluSource{nullptr, nullptr, 0u, nullptr, 0, 0, 0, 0});
+  return launch_prune_src<kPlain>(dO, rows, K, n, m, scheme, seed, dense, values, meta, mask, stream, k_pad, dtype,
+                                  ReluSource{nullptr, nullptr, 0u, nullptr, 0, 0, 0, 0, aligned32(dO)});
 }
 
 cudaError_t launch_relu_backward_prune(const void* dY, const void* act, int64_t rows, int64_t K, int n, int m, int scheme,
                                        uint64_t seed, void* grad, void* dense, void* values, void* meta, void* mask,
                                        cudaStream_t stream, int dtype, const void* skip) {
   const ReluSource src = {(const uint4*)act, (uint4*)grad, dtype == SDGP_FP16 ? 0x03FF03FFu : 0x007F007Fu,
-                          (const uint4*)skip, dtype == SDGP_FP16 ? 1 : 0, 0, 0, 0};
-  return launch_prune_src<true>(dY, rows, K, n, m, scheme, seed, dense, values, meta, mask, stream, 0, dtype, src);
+                          (const uint4*)skip, dtype == SDGP_FP16 ? 1 : 0, 0, 0, 0,
+                          aligned32(dY) && aligned32(act) && aligned32(skip)};
+  return launch_prune_src<kRelu>(dY, rows, K, n, m, scheme, seed, dense, values, meta, mask, stream, 0, dtype, src);
 }
 
 cudaError_t launch_maxpool_relu_backward_prune(const void* dYp, const void* act, int B, int H, int W, int64_t K, int n, int m,
                                                int scheme, uint64_t seed, void* grad, void* dense, void* values, void* meta,
                                                void* mask, cudaStream_t stream, int dtype, const void* skip_pooled) {
   const ReluSource src = {(const uint4*)act, (uint4*)grad, dtype == SDGP_FP16 ? 0x03FF03FFu : 0x007F007Fu,
-                          (const uint4*)skip_pooled, dtype == SDGP_FP16 ? 1 : 0, (int)(K / 8), H / 2, W / 2};
-  return launch_prune_src<true>(dYp, (int64_t)B * H * W, K, n, m, scheme, seed, dense, values, meta, mask, stream, 0, dtype, src);
+                          (const uint4*)skip_pooled, dtype == SDGP_FP16 ? 1 : 0, (int)(K / 8), H / 2, W / 2, false};
+  return launch_prune_src<kPool>(dYp, (int64_t)B * H * W, K, n, m, scheme, seed, dense, values, meta, mask, stream, 0, dtype, src);
 }
 
 }  // namespace sdgp

@@ -62,6 +62,18 @@ __host__ __device__ constexpr int threshold_lut(bool na, bool nb, bool nc) {
 }
 
 
+// 32 bytes of a read-once stream: one 256-bit load where the tensor is 32-byte aligned, else two of 128 bits.
+__device__ __forceinline__ void load_pair(const uint4* ptr, bool aligned32, uint4& a, uint4& b) {
+  if (aligned32) {
+    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                 : "l"(ptr));
+  } else {
+    a = __ldg(ptr);
+    b = __ldg(ptr + 1);
+  }
+}
+
 // Element type of the 16-bit tensors. Ranking and selection only read bit patterns (the pattern
 // with the sign cleared orders bf16 and IEEE binary16 alike); the type matters where the rescale
 // of Section 3.2 reads values as numbers and rounds the survivors. F16 = false: bf16, true: binary16.
@@ -205,83 +217,160 @@ __device__ __forceinline__ void m4_prune_vector(const uint4& w, int64_t v, uint3
 
 }
 
-// Compressed form of both 4-chunks of a vector (at most two survivors per chunk): slot0 / slot1 =
-// lane-paired values at the chunk's survivor positions p0 < p1 (p1 = last survivor, at least 1;
-// p0 = first survivor if there are two, else 0: the pad takes the lowest free position), and
-// nib2 = the two position nibbles p0 | p1 << 2 (chunk A in bits 0-3, chunk B in bits 4-7).
-__device__ __forceinline__ void compressed_slots(uint32_t y0, uint32_t y1, uint32_t y2, uint32_t y3, uint32_t km0,
-                                                 uint32_t km1, uint32_t km2, uint32_t km3, uint32_t& slot0,
-                                                 uint32_t& slot1, uint32_t& nib2) {
-  const uint32_t k23 = km2 | km3;
-  slot0 = y0 | (y1 & k23) | (y2 & km3);
-  slot1 = y3 | (~km3 & (y2 | (~km2 & y1)));
-  const uint32_t pos0 = (km1 & k23 & 0x00010001u) | (km2 & km3 & 0x00020002u);
-  const uint32_t pos1 = 0x00010001u + (k23 & 0x00010001u) + (km3 & 0x00010001u);
-  const uint32_t nib = pos0 + 4u * pos1;
-  nib2 = (nib & 0xFu) | ((nib >> 12) & 0xF0u);
+// ---- Compressed form of a vector (n <= 2: every 4-chunk keeps at most two elements) ----
+//
+// A chunk's two slots are two of the four half-words of two registers, so ONE byte permute per chunk gathers them once its
+// selector is known, and the position nibbles can be read off that selector. Keep flags live in bit 15 of the two 16-bit
+// lanes of a register (low lane: chunk A, elements 0..3; high lane: chunk B, elements 4..7). In flags k0..k3 of a chunk
+//   p1 = last survivor, at least 1                  = 1 + [k2 | k3] + [k3]
+//   p0 = first survivor if there are two, else 0    = [maj(k1, k2, k3)] + [k2 & k3]
+// and a lane of the selector is 0x3210 (p0 = 0, p1 = 1) plus 0x0022 per unit of p0 and 0x2200 per unit of p1 - 1. A byte
+// permute in sign-replicating mode turns the flags of both terms into those bytes at once. Against gathering the survivors
+// with lane masks (four masks, four ANDs, nine logic operations for slots and positions) this is about half the integer
+// instructions of the m = 4 magnitude function (50 -> 30 per vector), which is what bounds the kernels that prune from
+// shared memory or registers and the functions with more arithmetic.
+struct KeepFlags {
+  uint32_t k0, k1, k2, k3;  // bit 15 of each lane: element kept (other bits: anything)
+};
+
+__device__ __forceinline__ uint32_t chunk_selectors(uint32_t p0_is_not_0, const KeepFlags& k) {
+  const uint32_t two = lop3<0xC0>(k.k2, k.k3, 0u), any = lop3<0xFC>(k.k2, k.k3, 0u);  // k2 & k3, k2 | k3
+  // bytes of the result: sign of lane A of the first operand, of lane A of the second, then the same for lane B
+  const uint32_t first = prmt(p0_is_not_0, k.k3, 0xFBD9) & 0x22222222u, second = prmt(two, any, 0xFBD9) & 0x22222222u;
+  return 0x32103210u + first + second;
 }
 
-// Magnitude function with the L1 rescale of Section 3.2 for callers that want only the compressed form (n <= 2):
-// the same survivors, sums, divisions and roundings as m4_prune_vector, but the survivors are gathered into their two
-// slots first, so that the sum over the kept elements is one addition of the slots' magnitudes (the other terms of
-// the tree are +0, which changes nothing) and only the slots are multiplied and rounded: half the conversions,
-// products and roundings of the lane-by-lane form. A slot that holds the pad of a chunk with one survivor is +0 and
-// stays +0 (its product with a finite positive scale is +0; where the scale is not finite it is masked out: with one
-// survivor the pad is slot 1 if the survivor is element 0 and slot 0 otherwise).
-// km_i: keep masks as m4_prune_vector returns them (for the bit mask output).
-template <int N, bool F16>
-__device__ __forceinline__ void m4_rescaled_compressed(const uint4& w, uint32_t& slot0, uint32_t& slot1, uint32_t& nib2,
-                                                       uint32_t& km0, uint32_t& km1, uint32_t& km2, uint32_t& km3) {
-  static_assert(N == 1 || N == 2, "a compressed form exists for one or two survivors");
-  uint32_t y0, y1, y2, y3;
-  m4_prune_vector<N, SDGP_MAGNITUDE, F16>(w, 0, 0u, 0u, y0, y1, y2, y3, km0, km1, km2, km3);  // survivors, not yet rescaled
-  const uint32_t p0 = prmt(w.x, w.z, 0x5410), p1 = prmt(w.x, w.z, 0x7632);
-  const uint32_t p2 = prmt(w.y, w.w, 0x5410), p3 = prmt(w.y, w.w, 0x7632);
-  const float tA = sum4_lo_abs<F16>(p0, p1, p2, p3), tB = sum4_hi_abs<F16>(p0, p1, p2, p3);
-  compressed_slots(y0, y1, y2, y3, km0, km1, km2, km3, slot0, slot1, nib2);
-  const float a0 = lane_lo<F16>(slot0), b0 = lane_hi<F16>(slot0), a1 = lane_lo<F16>(slot1), b1 = lane_hi<F16>(slot1);
-  const float sA = __fadd_rn(fabsf(a0), fabsf(a1)), sB = __fadd_rn(fabsf(b0), fabsf(b1));
-  const float scA = (sA == 0.0f) ? 1.0f : __fdiv_rn(tA, sA);
-  const float scB = (sB == 0.0f) ? 1.0f : __fdiv_rn(tB, sB);
-  const bool finite = (__float_as_uint(tA) & 0x7F800000u) != 0x7F800000u &&
-                      (__float_as_uint(tB) & 0x7F800000u) != 0x7F800000u;
-  if (finite) {  // every product is finite: the hardware's packed rounding applies (see rescale_packed)
-    slot0 = pack_pair_rn<F16>(__fmul_rn(a0, scA), __fmul_rn(b0, scB));
-    slot1 = pack_pair_rn<F16>(__fmul_rn(a1, scA), __fmul_rn(b1, scB));
+// Positions p0 | p1 << 2 of chunk A and << 4 of chunk B, in the TOP byte of the result: the four two-bit fields of the
+// selectors (bits 1, 9, 17, 25) are brought together by one multiplication (no two partial products share a bit).
+__device__ __forceinline__ uint32_t positions_top_byte(uint32_t sel) { return (sel & 0x06060606u) * 0x00820820u; }
+
+__device__ __forceinline__ uint32_t majority(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | (c & (a | b)); }
+
+// Keep flags of the two m = 4 groups of a vector under the magnitude or random function (v: number of the vector).
+template <int N, int SCHEME>
+__device__ __forceinline__ KeepFlags m4_flags(const uint4& w, int64_t v, uint32_t seed_lo, uint32_t seed_hi) {
+  constexpr int NEED = 4 - N;  // an element is kept iff it beats at least 4 - n of the other three
+  KeepFlags k;
+  if (SCHEME == SDGP_RANDOM) {
+    const uint4 o = philox4x32_10((uint32_t)v, (uint32_t)((uint64_t)v >> 32), 0u, 0u, seed_lo, seed_hi);
+    // 16-bit keys; smaller ranks first, equal keys: lower index. e(i,j) = r_j - r_i has its
+    // sign bit set iff j ranks before i (j < i in key), i.e. iff i loses against j (for i < j).
+    const uint32_t rA0 = o.x & 0xFFFFu, rA1 = o.x >> 16, rA2 = o.y & 0xFFFFu, rA3 = o.y >> 16;
+    const uint32_t rB0 = o.z & 0xFFFFu, rB1 = o.z >> 16, rB2 = o.w & 0xFFFFu, rB3 = o.w >> 16;
+    uint32_t a0, a1, a2, a3, b0, b1, b2, b3;  // keep flags in bit 31
+#define SDGP_KEEP4(r0, r1, r2, r3, k0, k1, k2, k3)                                                \
+{                                                                                                \
+  const uint32_t e01 = r1 - r0, e02 = r2 - r0, e03 = r3 - r0,             \
+                 e12 = r2 - r1, e13 = r3 - r1, e23 = r3 - r2;            \
+  k0 = lop3<threshold_lut<NEED>(true, true, true)>(e01, e02, e03);                               \
+  k1 = lop3<threshold_lut<NEED>(false, true, true)>(e01, e12, e13);                              \
+  k2 = lop3<threshold_lut<NEED>(false, false, true)>(e02, e12, e23);                             \
+  k3 = lop3<threshold_lut<NEED>(false, false, false)>(e03, e13, e23);                            \
+}
+    SDGP_KEEP4(rA0, rA1, rA2, rA3, a0, a1, a2, a3)
+    SDGP_KEEP4(rB0, rB1, rB2, rB3, b0, b1, b2, b3)
+#undef SDGP_KEEP4
+    k.k0 = prmt(a0, b0, 0x7733); k.k1 = prmt(a1, b1, 0x7733);
+    k.k2 = prmt(a2, b2, 0x7733); k.k3 = prmt(a3, b3, 0x7733);
   } else {
-    const uint32_t keep0 = N == 2 ? 0xFFFFFFFFu : km0, keep1 = N == 2 ? 0xFFFFFFFFu : ~km0;
-    slot0 = (f32_to_elem_bits<F16>(__fmul_rn(a0, scA)) | (f32_to_elem_bits<F16>(__fmul_rn(b0, scB)) << 16)) & keep0;
-    slot1 = (f32_to_elem_bits<F16>(__fmul_rn(a1, scA)) | (f32_to_elem_bits<F16>(__fmul_rn(b1, scB)) << 16)) & keep1;
+    // |x| as 15-bit integers, lanes (element i, element i + 4). d(i,j) = (a_i | 0x8000) - a_j per lane never borrows across
+    // lanes and has bit 15 of the lane set iff a_i >= a_j, i.e. iff i beats j (i < j: ties to i).
+    constexpr uint32_t H = 0x80008000u;
+    const uint32_t l0 = prmt(w.x, w.z, 0x5410) & ~H, l1 = prmt(w.x, w.z, 0x7632) & ~H;
+    const uint32_t l2 = prmt(w.y, w.w, 0x5410) & ~H, l3 = prmt(w.y, w.w, 0x7632) & ~H;
+    const uint32_t h0 = l0 + H, h1 = l1 + H, h2 = l2 + H;
+    const uint32_t d01 = h0 - l1, d02 = h0 - l2, d03 = h0 - l3, d12 = h1 - l2, d13 = h1 - l3,
+                   d23 = h2 - l3;
+    k.k0 = lop3<threshold_lut<NEED>(false, false, false)>(d01, d02, d03);
+    k.k1 = lop3<threshold_lut<NEED>(true, false, false)>(d01, d12, d13);
+    k.k2 = lop3<threshold_lut<NEED>(true, true, false)>(d02, d12, d23);
+    k.k3 = lop3<threshold_lut<NEED>(true, true, true)>(d03, d13, d23);
+  }
+  return k;
+}
+
+// Gathers the slots of a vector: out.x / out.y = slots 0 and 1 (low and high half-word) of chunk A / B, pads +0.
+// EXACT2: every chunk keeps exactly two elements (2:4), so there are no pads.
+template <bool EXACT2>
+__device__ __forceinline__ void gather_slots(const uint4& w, const KeepFlags& k, uint2& out, uint2& slot_mask, uint32_t& pos_top) {
+  const uint32_t not0 = EXACT2 ? ~k.k0 : majority(k.k1, k.k2, k.k3);
+  const uint32_t sel = chunk_selectors(not0, k);
+  pos_top = positions_top_byte(sel);
+  out = make_uint2(prmt(w.x, w.y, sel), prmt(w.z, w.w, sel >> 16));
+  if (EXACT2) {
+    slot_mask = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
+  } else {
+    // slot 0 holds a survivor if element 0 is kept or two are, slot 1 if anything but element 0 is
+    const uint32_t keep0 = k.k0 | not0, keep1 = lop3<0xFE>(k.k1, k.k2, k.k3);
+    slot_mask = make_uint2(prmt(keep0, keep1, 0xDD99), prmt(keep0, keep1, 0xFFBB));
+    out.x &= slot_mask.x;
+    out.y &= slot_mask.y;
+  }
+}
+
+// The L1 rescale of Section 3.2 on gathered slots: `lo`, `hi` of a chunk's word times its group's scale, rounded to the
+// element type. finite: both sums of the group are finite, so every product is (the hardware's packed rounding applies, and a
+// +0 pad stays +0); otherwise each value goes through the explicit rounding (NaN stored as the canonical quiet NaN) and pads
+// are masked (their product with a scale that is not finite is not +0).
+template <bool F16>
+__device__ __forceinline__ uint32_t rescale_slots(uint32_t word, float scale, bool finite, uint32_t mask) {
+  const float lo = __fmul_rn(lane_lo<F16>(word), scale), hi = __fmul_rn(lane_hi<F16>(word), scale);
+  if (finite) return pack_pair_rn<F16>(lo, hi);
+  return (f32_to_elem_bits<F16>(lo) | (f32_to_elem_bits<F16>(hi) << 16)) & mask;
+}
+
+__device__ __forceinline__ bool is_finite(float x) { return (__float_as_uint(x) & 0x7F800000u) != 0x7F800000u; }
+
+// Sum of the magnitudes of a word's two elements.
+template <bool F16>
+__device__ __forceinline__ float pair_abs(uint32_t word) { return __fadd_rn(lane_lo_abs<F16>(word), lane_hi_abs<F16>(word)); }
+
+// m = 4: both groups of vector w (number v in the tensor) in compressed form. The rescaled function's sums are the oracle's
+// (balanced pairwise in index order; over the survivors only the slots' terms are not +0, so that sum is one addition).
+template <int N, int SCHEME, bool F16>
+__device__ __forceinline__ void m4_compress(const uint4& w, int64_t v, uint32_t seed_lo, uint32_t seed_hi, uint2& out,
+                                            uint32_t& pos_top, KeepFlags& k) {
+  static_assert(N == 1 || N == 2, "a compressed form exists for one or two survivors");
+  k = m4_flags<N, SCHEME == SDGP_RANDOM ? SDGP_RANDOM : SDGP_MAGNITUDE>(w, v, seed_lo, seed_hi);
+  uint2 mask;
+  gather_slots<N == 2>(w, k, out, mask, pos_top);
+  if (SCHEME == SDGP_RESCALED_MAGNITUDE) {
+    const float tA = __fadd_rn(pair_abs<F16>(w.x), pair_abs<F16>(w.y)), tB = __fadd_rn(pair_abs<F16>(w.z), pair_abs<F16>(w.w));
+    const float sA = pair_abs<F16>(out.x), sB = pair_abs<F16>(out.y);
+    const float scA = (sA == 0.0f) ? 1.0f : __fdiv_rn(tA, sA), scB = (sB == 0.0f) ? 1.0f : __fdiv_rn(tB, sB);
+    const bool finite = is_finite(tA) && is_finite(tB);
+    out.x = rescale_slots<F16>(out.x, scA, finite, mask.x);
+    out.y = rescale_slots<F16>(out.y, scB, finite, mask.y);
   }
 }
 
 // Groups of 8, 16 or 32 with n <= 2 (Algorithm 1 with the same three pruning functions): the survivors are the
-// elements whose composite key (rank key << 5 | 31 - position, unique inside a group) reaches the group's n-th
+// elements whose composite key (rank key, then 31 - position: unique inside a group) reaches the group's n-th
 // largest. The M / 8 vectors of a group are held by M / 8 neighbouring lanes (lane bits 0 and up; `part` = this
 // lane's number among them, i.e. which eighth of the group the vector is); each lane finds the two largest keys
 // of its 8 elements with a max/min network and the lanes merge their pairs through xor-shuffles, which every
 // lane named in `lanes` must execute together. Output in the lane-paired form of m4_prune_vector.
 __device__ __forceinline__ void merge_top2(uint32_t& hi, uint32_t& lo, uint32_t hi2, uint32_t lo2) {
   const uint32_t h = max(hi, hi2);
-  lo = max(min(hi, hi2), max(lo, lo2));
+  lo = __vimax3_u32(min(hi, hi2), lo, lo2);
   hi = h;
 }
 
-// Composite keys of the 8 elements of vector w (number v in the tensor); pos0 = tie-break bits of element 0.
+// Composite keys (31 bits) of the 8 elements of vector w (number v in the tensor); pos0 = tie-break bits of element 0 (below
+// 2^15). Magnitude: |x| in bits 16..30, so that an element in a word's upper half costs one logic operation and one in the
+// lower half a shift more. Random: the complement of the 16-bit key in bits 15..30 (the smallest key ranks first).
 template <int SCHEME>
 __device__ __forceinline__ void top2_keys(const uint4& w, int64_t v, uint32_t seed_lo, uint32_t seed_hi, uint32_t pos0,
                                           uint32_t (&c)[8]) {
   const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
   if (SCHEME == SDGP_RANDOM) {
     const uint4 o = philox4x32_10((uint32_t)v, (uint32_t)((uint64_t)v >> 32), 0u, 0u, seed_lo, seed_hi);
-    const uint32_t r[4] = {~o.x, ~o.y, ~o.z, ~o.w};  // smallest random key ranks first
+    const uint32_t r[4] = {o.x, o.y, o.z, o.w};
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      c[i] = (((i & 1) ? (r[i >> 1] >> 11) : (r[i >> 1] << 5)) & 0x1FFFE0u) | (pos0 - i);
+    for (int i = 0; i < 8; ++i) c[i] = (~((i & 1) ? (r[i >> 1] >> 1) : (r[i >> 1] << 15)) & 0x7FFF8000u) | (pos0 - i);
   } else {
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      c[i] = (((i & 1) ? (ww[i >> 1] >> 11) : (ww[i >> 1] << 5)) & 0xFFFE0u) | (pos0 - i);  // |x| << 5 | tie-break
+    for (int i = 0; i < 8; ++i) c[i] = (((i & 1) ? ww[i >> 1] : (ww[i >> 1] << 16)) & 0x7FFF0000u) | (pos0 - i);
   }
 }
 
@@ -337,66 +426,96 @@ __device__ __forceinline__ void top2_prune_vector(const uint4& w, int64_t v, uin
   }
 }
 
-// top2_prune_vector for the magnitude function with the L1 rescale, for callers that want only the compressed form:
-// as m4_rescaled_compressed, the survivors of the vector's two chunks are gathered into the slots first; a chunk's share of
-// the sum over the kept elements is then one addition of its slots' magnitudes (a group keeps at most two elements, so
-// every other term of the oracle's tree is +0) and only the slots are scaled and rounded.
-template <int M, bool F16>
-__device__ __forceinline__ void top2_rescaled_compressed(const uint4& w, int n, int part, unsigned lanes, uint32_t& slot0,
-                                                         uint32_t& slot1, uint32_t& nib2, uint32_t& km0, uint32_t& km1,
-                                                         uint32_t& km2, uint32_t& km3) {
+// Keep flags in lane form of a vector whose elements with key > t1 survive.
+__device__ __forceinline__ KeepFlags top2_flags(const uint32_t (&c)[8], uint32_t t1) {
+  KeepFlags k;  // (t1 - key) negative <=> kept; the sign bits of elements i and i + 4 side by side
+  k.k0 = prmt(t1 - c[0], t1 - c[4], 0x7733); k.k1 = prmt(t1 - c[1], t1 - c[5], 0x7733);
+  k.k2 = prmt(t1 - c[2], t1 - c[6], 0x7733); k.k3 = prmt(t1 - c[3], t1 - c[7], 0x7733);
+  return k;
+}
+
+// Groups of M = 8, 16 or 32 in compressed form (arguments as top2_prune_vector). A group keeps at most two elements, so in
+// the rescaled function's sum over the survivors every term but the slots' is +0.
+template <int M, int SCHEME, bool F16>
+__device__ __forceinline__ void top2_compress(const uint4& w, int64_t v, uint32_t seed_lo, uint32_t seed_hi, int n, int part,
+                                              unsigned lanes, uint2& out, uint32_t& pos_top, KeepFlags& k) {
   constexpr int LANES = M / 8;
-  uint32_t y0, y1, y2, y3;
-  top2_prune_vector<M, SDGP_MAGNITUDE, F16>(w, 0, 0u, 0u, n, part, lanes, y0, y1, y2, y3, km0, km1, km2, km3);  // not yet rescaled
-  const uint32_t p0 = prmt(w.x, w.z, 0x5410), p1 = prmt(w.x, w.z, 0x7632);
-  const uint32_t p2 = prmt(w.y, w.w, 0x5410), p3 = prmt(w.y, w.w, 0x7632);
-  float tsum = __fadd_rn(sum4_lo_abs<F16>(p0, p1, p2, p3), sum4_hi_abs<F16>(p0, p1, p2, p3));
-  compressed_slots(y0, y1, y2, y3, km0, km1, km2, km3, slot0, slot1, nib2);
-  const float a0 = lane_lo<F16>(slot0), b0 = lane_hi<F16>(slot0), a1 = lane_lo<F16>(slot1), b1 = lane_hi<F16>(slot1);
-  float ssum = __fadd_rn(__fadd_rn(fabsf(a0), fabsf(a1)), __fadd_rn(fabsf(b0), fabsf(b1)));
+  uint32_t c[8], hi, lo;
+  top2_keys<SCHEME>(w, v, seed_lo, seed_hi, 31u - 8u * (uint32_t)part, c);
+  top2_of_8(c, hi, lo);
 #pragma unroll
   for (int d = 1; d < LANES; d <<= 1) {
-    tsum = __fadd_rn(tsum, __shfl_xor_sync(lanes, tsum, d));
-    ssum = __fadd_rn(ssum, __shfl_xor_sync(lanes, ssum, d));
+    const uint32_t oh = __shfl_xor_sync(lanes, hi, d), ol = __shfl_xor_sync(lanes, lo, d);
+    merge_top2(hi, lo, oh, ol);
   }
-  const float sc = (ssum == 0.0f) ? 1.0f : __fdiv_rn(tsum, ssum);
-  if ((__float_as_uint(tsum) & 0x7F800000u) != 0x7F800000u) {  // finite sums: finite scale, a +0 pad stays +0
-    slot0 = pack_pair_rn<F16>(__fmul_rn(a0, sc), __fmul_rn(b0, sc));
-    slot1 = pack_pair_rn<F16>(__fmul_rn(a1, sc), __fmul_rn(b1, sc));
-  } else {
-    // which slots hold survivors: slot 1 if anything but element 0 of the chunk is kept, slot 0 if element 0 is kept or two are
-    const uint32_t keep1 = km1 | km2 | km3, keep0 = km0 | (km1 & km2) | (km3 & (km1 | km2));
-    slot0 = (f32_to_elem_bits<F16>(__fmul_rn(a0, sc)) | (f32_to_elem_bits<F16>(__fmul_rn(b0, sc)) << 16)) & keep0;
-    slot1 = (f32_to_elem_bits<F16>(__fmul_rn(a1, sc)) | (f32_to_elem_bits<F16>(__fmul_rn(b1, sc)) << 16)) & keep1;
+  k = top2_flags(c, ((n == 1) ? hi : lo) - 1u);
+  uint2 mask;
+  gather_slots<false>(w, k, out, mask, pos_top);
+  if (SCHEME == SDGP_RESCALED_MAGNITUDE) {
+    float tsum = __fadd_rn(__fadd_rn(pair_abs<F16>(w.x), pair_abs<F16>(w.y)), __fadd_rn(pair_abs<F16>(w.z), pair_abs<F16>(w.w)));
+    float ssum = __fadd_rn(pair_abs<F16>(out.x), pair_abs<F16>(out.y));
+#pragma unroll
+    for (int d = 1; d < LANES; d <<= 1) {
+      tsum = __fadd_rn(tsum, __shfl_xor_sync(lanes, tsum, d));
+      ssum = __fadd_rn(ssum, __shfl_xor_sync(lanes, ssum, d));
+    }
+    const float sc = (ssum == 0.0f) ? 1.0f : __fdiv_rn(tsum, ssum);
+    const bool finite = is_finite(tsum);
+    out.x = rescale_slots<F16>(out.x, sc, finite, mask.x);
+    out.y = rescale_slots<F16>(out.y, sc, finite, mask.y);
   }
 }
 
-// One group of 16 whose two vectors (numbers v and v + 1) are held by the same thread.
-template <int SCHEME, bool F16 = false>
-__device__ __forceinline__ void top2_prune_group16(const uint4& wa, const uint4& wb, int64_t v, uint32_t seed_lo,
-                                                   uint32_t seed_hi, int n, uint32_t (&ya)[4], uint32_t (&kma)[4],
-                                                   uint32_t (&yb)[4], uint32_t (&kmb)[4]) {
-  uint32_t ca[8], cb[8], hi, lo, hb, lb;
-  top2_keys<SCHEME>(wa, v, seed_lo, seed_hi, 31u, ca);
-  top2_keys<SCHEME>(wb, v + 1, seed_lo, seed_hi, 23u, cb);
-  top2_of_8(ca, hi, lo);
-  top2_of_8(cb, hb, lb);
-  merge_top2(hi, lo, hb, lb);
-  const uint32_t t1 = ((n == 1) ? hi : lo) - 1u;
-  uint32_t pa[4], pb[4];
-  top2_apply(wa, ca, t1, pa[0], pa[1], pa[2], pa[3], ya[0], ya[1], ya[2], ya[3], kma[0], kma[1], kma[2], kma[3]);
-  top2_apply(wb, cb, t1, pb[0], pb[1], pb[2], pb[3], yb[0], yb[1], yb[2], yb[3], kmb[0], kmb[1], kmb[2], kmb[3]);
-  if (SCHEME == SDGP_RESCALED_MAGNITUDE) {
-    // the same tree as across two lanes: (sum of elements 0..7) + (sum of elements 8..15)
-    const float ta = __fadd_rn(sum4_lo_abs<F16>(pa[0], pa[1], pa[2], pa[3]), sum4_hi_abs<F16>(pa[0], pa[1], pa[2], pa[3]));
-    const float tb = __fadd_rn(sum4_lo_abs<F16>(pb[0], pb[1], pb[2], pb[3]), sum4_hi_abs<F16>(pb[0], pb[1], pb[2], pb[3]));
-    const float sa = __fadd_rn(sum4_lo_abs<F16>(ya[0], ya[1], ya[2], ya[3]), sum4_hi_abs<F16>(ya[0], ya[1], ya[2], ya[3]));
-    const float sb = __fadd_rn(sum4_lo_abs<F16>(yb[0], yb[1], yb[2], yb[3]), sum4_hi_abs<F16>(yb[0], yb[1], yb[2], yb[3]));
-    const float tsum = __fadd_rn(ta, tb), ssum = __fadd_rn(sa, sb);
-    const float sc = (ssum == 0.0f) ? 1.0f : __fdiv_rn(tsum, ssum);
-    rescale_packed<F16>(ya[0], ya[1], ya[2], ya[3], kma[0], kma[1], kma[2], kma[3], sc, sc, tsum, tsum);
-    rescale_packed<F16>(yb[0], yb[1], yb[2], yb[3], kmb[0], kmb[1], kmb[2], kmb[3], sc, sc, tsum, tsum);
+// One vector of a group of M (4, 8, 16, 32) in compressed form: out and pos_top as gather_slots.
+template <int M, int N, int SCHEME, bool F16>
+__device__ __forceinline__ void compress_vector(const uint4& w, int64_t v, uint32_t seed_lo, uint32_t seed_hi, int part,
+                                                unsigned lanes, uint2& out, uint32_t& pos_top, KeepFlags& k) {
+  if constexpr (M == 4) m4_compress<N, SCHEME, F16>(w, v, seed_lo, seed_hi, out, pos_top, k);
+  else top2_compress<M, SCHEME, F16>(w, v, seed_lo, seed_hi, N, part, lanes, out, pos_top, k);
+}
+
+// Two neighbouring vectors (numbers v and v + 1, v even) held by the same thread, in compressed form: both groups of an M = 8
+// pair, the group of 16 they form, or half a group of 32 whose other half the lane with bit 0 flipped holds (`part` =
+// which half this lane has; every lane named in `lanes` must call together).
+template <int M, int N, int SCHEME, bool F16>
+__device__ __forceinline__ void compress_pair(const uint4& wa, const uint4& wb, int64_t v, uint32_t seed_lo, uint32_t seed_hi,
+                                              int part, unsigned lanes, uint4& out, uint32_t& posa, uint32_t& posb,
+                                              KeepFlags& ka, KeepFlags& kb) {
+  uint2 oa, ob;
+  if constexpr (M <= 8) {
+    compress_vector<M, N, SCHEME, F16>(wa, v, seed_lo, seed_hi, 0, lanes, oa, posa, ka);
+    compress_vector<M, N, SCHEME, F16>(wb, v + 1, seed_lo, seed_hi, 0, lanes, ob, posb, kb);
+  } else {
+    uint32_t ca[8], cb[8], hi, lo, hb, lb;
+    const uint32_t pos0 = 31u - 16u * (uint32_t)part;
+    top2_keys<SCHEME>(wa, v, seed_lo, seed_hi, pos0, ca);
+    top2_keys<SCHEME>(wb, v + 1, seed_lo, seed_hi, pos0 - 8u, cb);
+    top2_of_8(ca, hi, lo);
+    top2_of_8(cb, hb, lb);
+    merge_top2(hi, lo, hb, lb);
+    if (M == 32) merge_top2(hi, lo, __shfl_xor_sync(lanes, hi, 1), __shfl_xor_sync(lanes, lo, 1));
+    const uint32_t t1 = ((N == 1) ? hi : lo) - 1u;
+    ka = top2_flags(ca, t1);
+    kb = top2_flags(cb, t1);
+    uint2 ma, mb;
+    gather_slots<false>(wa, ka, oa, ma, posa);
+    gather_slots<false>(wb, kb, ob, mb, posb);
+    if (SCHEME == SDGP_RESCALED_MAGNITUDE) {
+      // the oracle's tree: (elements 0..7) + (elements 8..15), then the other sixteen
+      float tsum = __fadd_rn(__fadd_rn(__fadd_rn(pair_abs<F16>(wa.x), pair_abs<F16>(wa.y)), __fadd_rn(pair_abs<F16>(wa.z), pair_abs<F16>(wa.w))),
+                             __fadd_rn(__fadd_rn(pair_abs<F16>(wb.x), pair_abs<F16>(wb.y)), __fadd_rn(pair_abs<F16>(wb.z), pair_abs<F16>(wb.w))));
+      float ssum = __fadd_rn(__fadd_rn(pair_abs<F16>(oa.x), pair_abs<F16>(oa.y)), __fadd_rn(pair_abs<F16>(ob.x), pair_abs<F16>(ob.y)));
+      if (M == 32) {
+        tsum = __fadd_rn(tsum, __shfl_xor_sync(lanes, tsum, 1));
+        ssum = __fadd_rn(ssum, __shfl_xor_sync(lanes, ssum, 1));
+      }
+      const float sc = (ssum == 0.0f) ? 1.0f : __fdiv_rn(tsum, ssum);
+      const bool finite = is_finite(tsum);
+      oa = make_uint2(rescale_slots<F16>(oa.x, sc, finite, ma.x), rescale_slots<F16>(oa.y, sc, finite, ma.y));
+      ob = make_uint2(rescale_slots<F16>(ob.x, sc, finite, mb.x), rescale_slots<F16>(ob.y, sc, finite, mb.y));
+    }
   }
+  out = make_uint4(oa.x, oa.y, ob.x, ob.y);
 }
 
 }  // namespace

@@ -7,12 +7,19 @@
 
 namespace sdgp {
 
+// Multiprocessors of the current device (148 if it cannot be asked).
+int sm_count();
+
 // k_pad (0 = none): row pitch, in elements, of the compressed outputs. When k_pad > K the extra
 // chunks of every row are written as zero values with the position pair (0,1), so a consumer can
 // treat the row as k_pad channels (used to bring a channel count up to a whole 128-channel block).
 cudaError_t launch_prune(const void* dO, int64_t rows, int64_t K, int n, int m, int scheme,
                          uint64_t seed, void* dense, void* values, void* meta, void* mask,
                          cudaStream_t stream, int64_t k_pad = 0, int dtype = SDGP_BF16);
+
+// n > 2 of groups of 8, 16 or 32 (rank.cu): dense pruned copy and / or mask; nvec 8-element vectors, an even number.
+cudaError_t launch_rank(const void* dO, int64_t nvec, int n, int m, int scheme, uint64_t seed, void* dense, void* mask,
+                        cudaStream_t stream, int dtype);
 
 // The producer of dL/dO below a ReLU fused with its pruning: the gradient above the ReLU (dY) passes where the
 // activation `act` is positive; `grad` (optional) receives that unpruned dL/dO, the other outputs are

@@ -118,3 +118,32 @@ def test_prune_full_size_fc_and_sampled_large():
 def test_prune_compressed_outputs_alone(n, m, scheme):
     compare_compressed_only(inputs.relu_masked_laplace_bf16((1237, 160), seed=n * 10 + m), n, m, scheme, seed=3)
     compare_compressed_only(inputs.adversarial_groups_bf16(513, 96, seed=m + 1), n, m, scheme, seed=4)
+
+
+@pytest.mark.parametrize("scheme", SCHEMES)
+@pytest.mark.parametrize("n,m", [(1, 4), (2, 4), (2, 8), (2, 16), (1, 32), (2, 32), (3, 8), (7, 8), (8, 8), (3, 16), (9, 16), (16, 16), (3, 32), (31, 32)])
+@pytest.mark.parametrize("rows,offset", [(77, 8), (9600, 0)])
+def test_prune_pairs_and_ranking_at_their_edges(rows, offset, n, m, scheme):
+    """Tensors that start 16 bytes past a 32-byte boundary (128-bit instead of 256-bit accesses), an odd number of pairs of
+    vectors (K = 176 = 22 vectors a row), and more pairs than one per thread covers (9600 rows x 272)."""
+    import paper_2202_00774_b200 as sdgp
+    K = (176 if rows == 77 else 272) if m < 32 else (160 if rows == 77 else 288)
+    x = inputs.relu_masked_laplace_bf16((rows, K), seed=n + m)
+    x[::3] = inputs.adversarial_groups_bf16(rows, K, seed=m)[::3]
+    comp, want_mask = oracle.compressible(n, m), K % 32 == 0
+    want = (("values", "meta") if comp else ("dense",)) + (("mask",) if want_mask else ())
+    ref = oracle.prune(x, n, m, scheme, 11, want=want)
+    flat = torch.empty(rows * K + offset, dtype=torch.int16, device="cuda")
+    d = flat[offset:].view(rows, K)
+    d.copy_(dev(x))
+    out = {}
+    for key, cols, dtype in (("dense", K, torch.int16), ("values", K // 2, torch.int16), ("meta", K // 16, torch.int16), ("mask", K // 32, torch.int32)):
+        if key in want:
+            out[key] = torch.full((rows * cols + offset,), -1, dtype=dtype, device="cuda")[offset:].view(rows, cols)
+    sdgp.sdgp_prune(d, n, m, scheme, 11, **out)
+    for key in want:
+        assert np.array_equal(out[key].cpu().numpy().view(ref[key].dtype), ref[key]), key
+    if want_mask:   # the mask alone
+        mask = torch.full((rows, K // 32), -1, dtype=torch.int32, device="cuda")
+        sdgp.sdgp_prune(d, n, m, scheme, 11, mask=mask)
+        assert np.array_equal(mask.cpu().numpy().view(np.uint32), ref["mask"])

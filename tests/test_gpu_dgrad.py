@@ -664,3 +664,27 @@ def test_bounded_wait_reports_timeout_and_context_survives():
     sdgp.sdgp_dgrad_linear(dev16(dO), dev16(W), dD, 4, 4, sdgp.MAGNITUDE, flags=sdgp.FLAG_DENSE)
     check_no_device_error()
     assert_close(to_f64(dD), *linear_ref(dO, W))
+
+
+# ------------------------------------------------- tile widths and epilogues
+
+
+@pytest.mark.parametrize("offset", [0, 8])
+@pytest.mark.parametrize("rows,K,N", [(1, 128, 64), (129, 128, 192), (300, 192, 320), (2000, 128, 448), (40000, 128, 192), (77000, 64, 64)])
+def test_linear_tile_widths_and_row_tails(rows, K, N, offset):
+    """Tiles of 64 .. 256 columns with a partly empty last one, few and many tiles per CTA pair (rows written straight from
+    registers, or boxes by TMA), a row count that ends inside a warp's 32 rows, a dD that starts 16 bytes past a 32-byte
+    boundary; the values beside dD stay untouched."""
+    import paper_2202_00774_b200 as sdgp
+    dO, W = inputs.fc_tensors(rows, K, N, seed=rows + N)
+    ws = torch.empty(max(16, sdgp.sdgp_workspace_size_linear(rows, K, N)), dtype=torch.uint8, device="cuda")
+    pruned = oracle.prune(dO, 2, 4, oracle.MAGNITUDE, want=("dense",))["dense"]
+    pick = np.unique(np.concatenate([np.arange(min(rows, 40)), np.arange(max(0, rows - 300), rows)]))   # whole rows
+    for flags, A in ((sdgp.FLAG_TWO_PASS, pruned), (sdgp.FLAG_DENSE, dO)):
+        flat = torch.full((rows * N + 16,), 0x5A5A, dtype=torch.int16, device="cuda")
+        dD = flat[offset:offset + rows * N].view(rows, N)
+        sdgp.sdgp_dgrad_linear(dev16(dO), dev16(W), dD, 2, 4, sdgp.MAGNITUDE, workspace=ws, flags=flags)
+        check_no_device_error()
+        assert_close(to_f64(dD)[pick], *linear_ref(A[pick], W))
+        edge = flat.cpu().numpy()
+        assert np.all(edge[:offset] == 0x5A5A) and np.all(edge[offset + rows * N:] == 0x5A5A)

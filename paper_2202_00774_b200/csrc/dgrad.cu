@@ -4,6 +4,7 @@
 
 #include "dgrad_general.cuh"
 #include "dgrad_halo_params.cuh"
+#include "dgrad_rows.cuh"
 
 namespace sdgp {
 
@@ -196,6 +197,10 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
   if (Cin % 64 != 0 || Cout % 64 != 0) return SDGP_ERR_UNSUPPORTED;
   if ((int64_t)R * S * Cin > 0x7FFFFFFF) return SDGP_ERR_UNSUPPORTED;
 
+  if (fused && B == 1 && H == 1 && R == 1 && S == 1 && stride == 1 && pad == 0 && fused->m <= 16) {
+    const RowsPlan plan = plan_rows(W, Cout, Cin);
+    if (plan.ok) return launch_rows_fused(plan, A, Wt, Cout, Cin, dD, *fused, dtype, stream);
+  }
   const int kb_channels = sparse ? 128 : 64;
 
   DgradView view;
@@ -306,7 +311,7 @@ sdgp_status read_device_error() {
   if (cudaDeviceSynchronize() != cudaSuccess) return SDGP_ERR_CUDA;
   bool timed_out = false;
   cudaError_t (*const words[])(unsigned int*) = {take_error_word, take_error_general, take_error_halo_sparse, take_error_halo_dense,
-                                                 take_error_halo_fused};
+                                                 take_error_halo_fused, take_error_rows};
   for (auto take : words) {
     unsigned int word = 0;
     if (take(&word) != cudaSuccess) return SDGP_ERR_CUDA;

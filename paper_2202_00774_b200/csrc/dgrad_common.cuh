@@ -53,7 +53,9 @@ constexpr int kBM = 128;             // output pixels (rows) per CTA tile = TMEM
 constexpr int kThreadsGemm = 320;    // 10 warps
 constexpr unsigned kIdleWaitNs = 200;  // sleep between polls of the waits that are off the critical path
 constexpr int kEHwBytes = kBM * 16;  // rearranged metadata of one (tap, channel block): 128 lanes x 16 B
-constexpr int kStageBytes = 4 * 32 * 128;  // epilogue staging (store_box): 32 rows of 64 columns for each of the four warps
+constexpr int kStageBufs = 2;
+constexpr int kWarpStage = kStageBufs * 32 * 128;  // epilogue staging of a warp (store_box): 32 rows of 64 columns, twice
+constexpr int kStageBytes = 4 * kWarpStage;
 constexpr uint32_t kTmemCols = 512;
 constexpr int kMaxImgRows = 192;     // pixel rows of one A stage (filter-row reuse: TW * (TH + R - 1))
 constexpr int kSmemLimit = 232448;   // opt-in dynamic shared memory per CTA
@@ -100,17 +102,21 @@ constexpr uint32_t kIdescBf16Operands = (1u << 7) | (1u << 10);
 // into the well-formed position pair (0,1) in every chunk.
 __device__ __forceinline__ uint32_t well_formed(uint32_t x) { return __vmaxu2(x, 0x44444444u); }
 
-// 64 columns of the 32 accumulator rows of a warp: TMEM -> registers -> 16-bit pairs. first_slab_read: signalled as soon as the
-// columns are in registers - they may then hold the next tile's metadata, and the MMA thread is waiting.
-__device__ __forceinline__ void read_slab(uint32_t taddr, uint32_t (&packed)[32], uint64_t* first_slab_read, bool f16) {
+// 64 columns of the 32 accumulator rows of a warp: TMEM -> registers -> 16-bit pairs. The barriers (null: none) of the MMA thread
+// are signalled as soon as the columns are in registers: first_read - they may then hold the next tile's metadata -, released - the
+// accumulator has been read to its end.
+__device__ __forceinline__ void read_slab(uint32_t taddr, uint32_t (&packed)[32], uint64_t* first_read, uint64_t* released, bool f16) {
   uint32_t v0[32], v1[32];
   ptx::tmem_ld_32x32(taddr, v0);
   ptx::tmem_ld_32x32(taddr + 32u, v1);
   ptx::tmem_ld_wait();
-  if (first_slab_read != nullptr) {
+  if (first_read != nullptr || released != nullptr) {
     ptx::tc_fence_before_sync();
     __syncwarp();
-    if ((threadIdx.x & 31) == 0) ptx::mbar_arrive_cluster(first_slab_read, 0);
+    if ((threadIdx.x & 31) == 0) {
+      if (first_read != nullptr) ptx::mbar_arrive_cluster(first_read, 0);
+      if (released != nullptr) ptx::mbar_arrive_cluster(released, 0);
+    }
   }
   if (f16) {
 #pragma unroll
@@ -134,17 +140,18 @@ __device__ __forceinline__ void read_slab(uint32_t taddr, uint32_t (&packed)[32]
 // store_rows: straight from registers. Each thread writes whole 32-byte sectors of its own row and L2 puts the lines together; the
 // shortest way from an accumulator to memory (702 x 256 . 256 x 192: 7.1 us against 8.5 us through store_box).
 // dst: the row's address at the tile's first channel, nullptr if the row lies outside dD; columns: channels of dD left from
-// there (warp-uniform).
+// there (warp-uniform). released: the MMA thread's barrier for the accumulator.
 template <int BN>
-__device__ __forceinline__ void store_rows(uint32_t taddr, uint8_t* dst, int columns, bool aligned32, uint64_t* first_slab_read, bool f16) {
+__device__ __forceinline__ void store_rows(uint32_t taddr, uint8_t* dst, int columns, bool aligned32, uint64_t* first_slab_read,
+                                           uint64_t* released, bool f16) {
 #pragma unroll 1
   for (int c0 = 0; c0 < BN; c0 += 64) {
-    if (c0 > 0 && c0 >= columns) break;
+    const bool last = c0 + 64 >= BN || c0 + 64 >= columns;
     uint32_t packed[32];
-    read_slab(taddr + (uint32_t)c0, packed, c0 == 0 ? first_slab_read : nullptr, f16);
-    if (dst == nullptr) continue;
+    read_slab(taddr + (uint32_t)c0, packed, c0 == 0 ? first_slab_read : nullptr, last ? released : nullptr, f16);
     uint8_t* out = dst + 2 * c0;
-    if (aligned32 && columns - c0 >= 64) {
+    if (dst == nullptr) {
+    } else if (aligned32 && columns - c0 >= 64) {
 #pragma unroll
       for (int c = 0; c < 4; ++c) ptx::st_global_256(out + 32 * c, &packed[8 * c]);
     } else {
@@ -152,35 +159,41 @@ __device__ __forceinline__ void store_rows(uint32_t taddr, uint8_t* dst, int col
       for (int c = 0; c < 8; ++c)
         if (c0 + 8 * c < columns) *(uint4*)(out + 16 * c) = make_uint4(packed[4 * c], packed[4 * c + 1], packed[4 * c + 2], packed[4 * c + 3]);
     }
+    if (last) break;
   }
 }
 
-// store_box: through 4 KB of the warp's own swizzled shared memory and its own TMA store (a box of 32 pixels, clipped at the
+// store_box: through 2 x 4 KB of the warp's own swizzled shared memory and its own TMA store (a box of 32 pixels, clipped at the
 // edges of dD): one line per request instead of 32 per instruction. For launches whose epilogues run beside other tiles' work:
 // the pruning warps of a fused kernel need the load/store unit (128 -> 128 channels at 28 x 28, batch 256: 47 us against 53 us).
 // (c1, c2, c3, c4): coordinates 1.. of the box in dD's map; five: the map has five dimensions.
 template <int BN>
 __device__ __forceinline__ void store_box(uint32_t taddr, uint8_t* stage, const CUtensorMap* tmD, bool five, int n0, int c1, int c2,
-                                          int c3, int c4, bool in_range, int columns, uint64_t* first_slab_read, bool f16) {
+                                          int c3, int c4, bool in_range, int columns, uint64_t* first_slab_read, uint64_t* released,
+                                          bool f16, uint32_t& chunk) {
   const int lane = threadIdx.x & 31;
 #pragma unroll 1
   for (int c0 = 0; c0 < BN; c0 += 64) {
-    if (c0 > 0 && c0 >= columns) break;
+    const bool last = c0 + 64 >= BN || c0 + 64 >= columns;
     uint32_t packed[32];
-    read_slab(taddr + (uint32_t)c0, packed, c0 == 0 ? first_slab_read : nullptr, f16);
-    if (lane == 0) ptx::bulk_wait_group_read<0>();  // the previous store has read the staging rows
+    read_slab(taddr + (uint32_t)c0, packed, c0 == 0 ? first_slab_read : nullptr, last ? released : nullptr, f16);
+    uint8_t* buf = stage + (chunk % kStageBufs) * (32 * 128);
+    if (lane == 0) ptx::bulk_wait_group_read<kStageBufs - 1>();  // the store that last used this buffer has read it
     __syncwarp();
 #pragma unroll
     for (int c = 0; c < 8; ++c)
-      *(uint4*)(stage + lane * 128 + ((c ^ (lane & 7)) << 4)) =
+      *(uint4*)(buf + lane * 128 + ((c ^ (lane & 7)) << 4)) =
           make_uint4(packed[4 * c], packed[4 * c + 1], packed[4 * c + 2], packed[4 * c + 3]);
     ptx::fence_proxy_async_smem();
     __syncwarp();
-    if (lane == 0 && in_range) {
-      if (five) ptx::tma_store_5d(tmD, stage, n0 + c0, c1, c2, c3, c4);
-      else ptx::tma_store_4d(tmD, stage, n0 + c0, c1, c2, c3);
-      ptx::bulk_commit_group();
+    if (lane == 0) {
+      if (!in_range) {
+      } else if (five) ptx::tma_store_5d(tmD, buf, n0 + c0, c1, c2, c3, c4);
+      else ptx::tma_store_4d(tmD, buf, n0 + c0, c1, c2, c3);
+      ptx::bulk_commit_group();  // (an empty group where nothing is stored: the waits count groups)
     }
+    ++chunk;
+    if (last) break;
   }
 }
 

@@ -436,7 +436,7 @@ dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     const int q = warp & 3;  // a warp may only touch TMEM lanes [32*(warp%4), +32)
     const int row = q * 32 + lane;
     const int iw = row % p.TW, ih = (row / p.TW) % p.TH, ib = row / (p.TW * p.TH);  // this thread's pixel of a patch
-    uint32_t aph = 0;
+    uint32_t aph = 0, chunk = 0;
     int acc = 0;
     for (int pt = first_pair; pt < p.pair_tiles; pt += pair_stride) {
       const int n0 = (pt % p.tiles_n) * BN;
@@ -450,16 +450,13 @@ dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
       uint64_t* first_slab_read = p.meta_shared ? &meta_free[acc] : nullptr;
       if (p.box_store) {
-        store_box<BN>(taddr, sOut + q * (kStageBytes / 4), &tmD, false, n0, w - lane, h, b, 0, mt < p.m_tiles, p.d.channels - n0,
-                      first_slab_read, p.f16 != 0);
+        store_box<BN>(taddr, sOut + q * kWarpStage, &tmD, false, n0, w - lane, h, b, 0, mt < p.m_tiles, p.d.channels - n0,
+                      first_slab_read, &acc_empty[acc], p.f16 != 0, chunk);
       } else {
         const bool inside = row < rows_used && mt < p.m_tiles && w < p.W && h < p.H && b < p.B;
         uint8_t* dst = inside ? p.d.base + b * p.d.sb + h * p.d.sh + w * p.d.sw + 2 * n0 : nullptr;
-        store_rows<BN>(taddr, dst, p.d.channels - n0, p.d.aligned32 != 0, first_slab_read, p.f16 != 0);
+        store_rows<BN>(taddr, dst, p.d.channels - n0, p.d.aligned32 != 0, first_slab_read, &acc_empty[acc], p.f16 != 0);
       }
-      ptx::tc_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive_cluster(&acc_empty[acc], 0);
       if (++acc == NACC) { acc = 0; aph ^= 1u; }
     }
     // the staging rows have been read; the writes themselves complete with the grid (whoever depends on dD waits for that)

@@ -22,6 +22,7 @@
 
 #pragma once
 #include "dgrad_halo_params.cuh"
+#include "dgrad_prune.cuh"
 
 namespace sdgp {
 namespace {
@@ -34,32 +35,6 @@ constexpr int kHaloAStages = 4;  // at most: A stages in use are p.a_stages = 2,
 // slots they take from it (14 -> 16 -> 18 pruning warps: 1062 -> 1107 -> 1111 TFLOP/s on the ResNet-9 chain).
 constexpr int kPruneWarps = 18;
 constexpr int kThreadsHaloFused = 24 * 32;
-
-// Fused pruning of four vectors (8 channels each, already in registers) of one pixel row: out[v] = the 8
-// compressed bytes of vector v, metaw = their four bytes of position metadata (byte v = the two nibbles of
-// vector v). Number of vector v in the whole dL/dO tensor (random keys): vbase + vstep * v. Groups of M = 8, 16
-// or 32 channels span 1, 2 or 4 vectors held by neighbouring lanes (lane bits 0 and up; `part` = which of
-// them this lane's vectors are); all 32 lanes must call together.
-template <int M, int N, int SCHEME>
-__device__ __forceinline__ void fused_prune_vectors(const uint4 (&w)[4], int64_t vbase, int vstep, uint32_t seed_lo,
-                                                    uint32_t seed_hi, int part, uint2 (&out)[4], uint32_t& metaw) {
-  uint32_t pos[4];
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    KeepFlags k;
-    compress_vector<M, N, SCHEME, false>(w[v], vbase + vstep * v, seed_lo, seed_hi, part, 0xFFFFFFFFu, out[v], pos[v], k);
-  }
-  metaw = prmt(prmt(pos[0], pos[1], 0x0073), prmt(pos[2], pos[3], 0x0073), 0x5410);
-}
-
-// 16 bytes from global memory, read-only path, kept out of L1 (each byte is used once by this SM).
-__device__ __forceinline__ uint4 ldg_stream(const uint8_t* ptr) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(ptr));
-  return v;
-}
 
 template <bool SPARSE, int BN, int NT, bool FUSED>
 __global__ void __launch_bounds__(FUSED ? kThreadsHaloFused : kThreadsGemm, 1)
@@ -525,7 +500,7 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           uint32_t metaw;
           // (a group of M channels = vectors c + 4v of M / 8 neighbouring lanes c, same v)
           if (live) {
-            fused_prune_vectors<M, N, SCHEME>(w, u_pix * (p.Cout >> 3) + u_kb * 16 + c, 4, p.seed_lo, p.seed_hi, c & (M / 8 - 1), out, metaw);
+            fused_prune_vectors<M, N, SCHEME, false>(w, u_pix * (p.Cout >> 3) + u_kb * 16 + c, 4, p.seed_lo, p.seed_hi, c & (M / 8 - 1), out, metaw);
           } else {
             // a unit of padding only: zeros, whatever positions the metadata names (it names the pair (0, 1))
 #pragma unroll
@@ -607,7 +582,7 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     // of two neighbouring images)
     const int srow = row >> 3, dh = srow / p.tb, px = row & 7;
     const int db = (srow % p.tb) * p.img_per_row + (p.split ? px >> 2 : 0), dw = p.split ? px & 3 : px;
-    uint32_t cph = 0;
+    uint32_t cph = 0, chunk = 0;
     int acc = 0;
     for (int lt = 0; lt < my_tiles; ++lt) {
       int n0, w0, h0, b0;
@@ -619,24 +594,22 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       for (int j = 0; j < NT; ++j) {
         const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * set_cols + j * BN);
         uint64_t* first_slab_read = (p.meta_shared && j == 0) ? &meta_free[acc] : nullptr;
+        uint64_t* released = j == NT - 1 ? &acc_empty[acc] : nullptr;
         const bool strip_live = in_range && (strips & (1u << j));
         if constexpr (FUSED) {
           // this warp's 4 strip rows: 4 / tb pixel rows of tb images
           const int hq = h0 + q * (4 / p.tb);
-          if (p.split) store_box<BN>(taddr, sOut + q * (kStageBytes / 4), &tmD, true, n0, 0, 2 * j, b0 / p.img_per_row, hq, strip_live,
-                                     p.d.channels - n0, first_slab_read, p.f16 != 0);
-          else store_box<BN>(taddr, sOut + q * (kStageBytes / 4), &tmD, false, n0, w0 + 8 * j, b0, hq, 0, strip_live && w0 + 8 * j < p.W,
-                             p.d.channels - n0, first_slab_read, p.f16 != 0);
+          if (p.split) store_box<BN>(taddr, sOut + q * kWarpStage, &tmD, true, n0, 0, 2 * j, b0 / p.img_per_row, hq, strip_live,
+                                     p.d.channels - n0, first_slab_read, released, p.f16 != 0, chunk);
+          else store_box<BN>(taddr, sOut + q * kWarpStage, &tmD, false, n0, w0 + 8 * j, b0, hq, 0, strip_live && w0 + 8 * j < p.W,
+                             p.d.channels - n0, first_slab_read, released, p.f16 != 0, chunk);
         } else {
           const int w = w0 + dw + (p.split ? 0 : 8 * j), h = h0 + dh, b = b0 + db + (p.split ? 2 * j : 0);
           const bool inside = strip_live && w < p.W && h < p.H && b < p.B;
           uint8_t* dst = inside ? p.d.base + b * p.d.sb + h * p.d.sh + w * p.d.sw + 2 * n0 : nullptr;
-          store_rows<BN>(taddr, dst, p.d.channels - n0, p.d.aligned32 != 0, first_slab_read, p.f16 != 0);
+          store_rows<BN>(taddr, dst, p.d.channels - n0, p.d.aligned32 != 0, first_slab_read, released, p.f16 != 0);
         }
       }
-      ptx::tc_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive_cluster(&acc_empty[acc], 0);
       if (++acc == 2) { acc = 0; cph ^= 1u; }
     }
     // the staging rows have been read; the writes themselves complete with the grid (whoever depends on dD waits for that)

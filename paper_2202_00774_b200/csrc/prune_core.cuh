@@ -359,19 +359,23 @@ __device__ __forceinline__ void merge_top2(uint32_t& hi, uint32_t& lo, uint32_t 
 // Composite keys (31 bits) of the 8 elements of vector w (number v in the tensor); pos0 = tie-break bits of element 0 (below
 // 2^15). Magnitude: |x| in bits 16..30, so that an element in a word's upper half costs one logic operation and one in the
 // lower half a shift more. Random: the complement of the 16-bit key in bits 15..30 (the smallest key ranks first).
+// src: the vector itself, or (random function) its four words of random bits.
+template <int SCHEME>
+__device__ __forceinline__ void top2_keys_of(const uint4& src, uint32_t pos0, uint32_t (&c)[8]) {
+  const uint32_t ww[4] = {src.x, src.y, src.z, src.w};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    if (SCHEME == SDGP_RANDOM) c[i] = (~((i & 1) ? (ww[i >> 1] >> 1) : (ww[i >> 1] << 15)) & 0x7FFF8000u) | (pos0 - i);
+    else c[i] = (((i & 1) ? ww[i >> 1] : (ww[i >> 1] << 16)) & 0x7FFF0000u) | (pos0 - i);
+  }
+}
 template <int SCHEME>
 __device__ __forceinline__ void top2_keys(const uint4& w, int64_t v, uint32_t seed_lo, uint32_t seed_hi, uint32_t pos0,
                                           uint32_t (&c)[8]) {
-  const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-  if (SCHEME == SDGP_RANDOM) {
-    const uint4 o = philox4x32_10((uint32_t)v, (uint32_t)((uint64_t)v >> 32), 0u, 0u, seed_lo, seed_hi);
-    const uint32_t r[4] = {o.x, o.y, o.z, o.w};
-#pragma unroll
-    for (int i = 0; i < 8; ++i) c[i] = (~((i & 1) ? (r[i >> 1] >> 1) : (r[i >> 1] << 15)) & 0x7FFF8000u) | (pos0 - i);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) c[i] = (((i & 1) ? ww[i >> 1] : (ww[i >> 1] << 16)) & 0x7FFF0000u) | (pos0 - i);
-  }
+  if (SCHEME == SDGP_RANDOM)
+    top2_keys_of<SCHEME>(philox4x32_10((uint32_t)v, (uint32_t)((uint64_t)v >> 32), 0u, 0u, seed_lo, seed_hi), pos0, c);
+  else
+    top2_keys_of<SCHEME>(w, pos0, c);
 }
 
 // The two largest of eight keys.
@@ -516,6 +520,47 @@ __device__ __forceinline__ void compress_pair(const uint4& wa, const uint4& wb, 
     }
   }
   out = make_uint4(oa.x, oa.y, ob.x, ob.y);
+}
+
+// One group of 32 whose four vectors (numbers v .. v + 3) are held by the same thread, in compressed form. The keys are made
+// twice, once for the two largest and once for the decision: 32 of them at a time do not fit the registers.
+template <int N, int SCHEME, bool F16>
+__device__ __forceinline__ void compress_quad32(const uint4 (&w)[4], int64_t v, uint32_t seed_lo, uint32_t seed_hi, uint2 (&out)[4],
+                                                uint32_t (&pos)[4]) {
+  uint4 r[4];  // random function: the keys' source, generated once
+  uint32_t hi = 0u, lo = 0u;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    if (SCHEME == SDGP_RANDOM) r[t] = philox4x32_10((uint32_t)(v + t), (uint32_t)((uint64_t)(v + t) >> 32), 0u, 0u, seed_lo, seed_hi);
+    uint32_t c[8], h, l;
+    top2_keys_of<SCHEME>(SCHEME == SDGP_RANDOM ? r[t] : w[t], 31u - 8u * t, c);
+    top2_of_8(c, h, l);
+    if (t == 0) { hi = h; lo = l; }
+    else merge_top2(hi, lo, h, l);
+  }
+  const uint32_t t1 = ((N == 1) ? hi : lo) - 1u;
+  uint2 mask[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    uint32_t c[8];
+    top2_keys_of<SCHEME>(SCHEME == SDGP_RANDOM ? r[t] : w[t], 31u - 8u * t, c);
+    gather_slots<false>(w[t], top2_flags(c, t1), out[t], mask[t], pos[t]);
+  }
+  if (SCHEME == SDGP_RESCALED_MAGNITUDE) {
+    float ts[4], ss[4];  // the oracle's tree, eight elements at a time
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      ts[t] = __fadd_rn(__fadd_rn(pair_abs<F16>(w[t].x), pair_abs<F16>(w[t].y)), __fadd_rn(pair_abs<F16>(w[t].z), pair_abs<F16>(w[t].w)));
+      ss[t] = __fadd_rn(pair_abs<F16>(out[t].x), pair_abs<F16>(out[t].y));
+    }
+    const float tsum = __fadd_rn(__fadd_rn(ts[0], ts[1]), __fadd_rn(ts[2], ts[3]));
+    const float ssum = __fadd_rn(__fadd_rn(ss[0], ss[1]), __fadd_rn(ss[2], ss[3]));
+    const float sc = (ssum == 0.0f) ? 1.0f : __fdiv_rn(tsum, ssum);
+    const bool finite = is_finite(tsum);
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      out[t] = make_uint2(rescale_slots<F16>(out[t].x, sc, finite, mask[t].x), rescale_slots<F16>(out[t].y, sc, finite, mask[t].y));
+  }
 }
 
 }  // namespace

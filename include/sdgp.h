@@ -74,7 +74,8 @@ typedef enum {
 
 /* `flags` of the dgrad entry points. */
 enum {
-  SDGP_FLAG_TWO_PASS = 0, /* prune kernel writes compressed dL/dO into the workspace, sparse GEMM reads it */
+  SDGP_FLAG_TWO_PASS = 0, /* prune kernel writes compressed dL/dO into the workspace, sparse GEMM reads it (or, where that is
+                             faster, one kernel prunes on the way to the tensor cores and leaves the workspace alone) */
   SDGP_FLAG_FUSED = 1,    /* pruning happens inside the dgrad kernel (n <= 2; m = 4, 8 or 16, also 32 for convolutions
                              that run on the whole-filter-reuse kernel); no workspace, no compressed tensor in
                              global memory */

@@ -258,6 +258,11 @@ sdgp_status sdgp_dgrad_conv2d_typed(const void* dO, const void* W, void* dD, int
   }
   if (!workspace || workspace_bytes < c.bytes) return SDGP_ERR_WORKSPACE;
   if (((uintptr_t)workspace & 255u) != 0) return SDGP_ERR_ALIGNMENT;
+  if (R == 1 && S == 1 && stride == 1 && pad == 0) {
+    bool taken = false;
+    const sdgp_status st = sdgp::try_rows_fused(dO, W, dD, (int64_t)B * H * Wd, Cout, Cin, {n, m, (int)scheme, seed}, dt, s, &taken);
+    if (taken) return st;
+  }
   cudaError_t e = sdgp::launch_prune(dO, (int64_t)B * P * Q, Cout, n, m, (int)scheme, seed, nullptr, c.values,
                                      c.meta, nullptr, s, Cpad, dt);
   if (e != cudaSuccess) return SDGP_ERR_CUDA;
@@ -313,6 +318,11 @@ sdgp_status sdgp_dgrad_conv2d_grouped(const void* dO, const void* W, void* dD, i
   if (((uintptr_t)workspace & 255u) != 0) return SDGP_ERR_ALIGNMENT;
   cudaStream_t s = (cudaStream_t)stream;
   const int dt = (int)dtype;
+  if (prunes && flags == SDGP_FLAG_TWO_PASS && groups == 1 && R == 1 && S == 1 && stride == 1 && pad == 0) {
+    bool taken = false;  // (TMA pads the filters' channels with zeros itself)
+    const sdgp_status st = sdgp::try_rows_fused(dO, W, dD, (int64_t)B * H * Wd, Cout, Cin, {n, m, (int)scheme, seed}, dt, s, &taken);
+    if (taken) return st;
+  }
   const void* w_full = W;  // one group and whole 64-channel blocks: the filters are already in the kernels' form
   void* rest = (uint8_t*)workspace + w_bytes;
   if (groups > 1 || Cin != cin_k || Cout != cout_k) {

@@ -58,10 +58,16 @@ bool encode(CUtensorMap* tm, CUtensorMapDataType dt, int rank, const void* base,
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   cuuint32_t ones[5] = {1, 1, 1, 1, 1};
-  if (fn(tm, dt, (cuuint32_t)rank, const_cast<void*>(base), (const cuuint64_t*)dims, (const cuuint64_t*)strides_bytes,
-         (const cuuint32_t*)box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return false;
+  auto make = [&]() {
+    return fn(tm, dt, (cuuint32_t)rank, const_cast<void*>(base), (const cuuint64_t*)dims, (const cuuint64_t*)strides_bytes,
+              (const cuuint32_t*)box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  if (!make()) {
+    // a thread whose first CUDA call this is has no context yet (the encoder is a driver function): cudaSetDevice binds it
+    const int dev = current_device();
+    if (dev < 0 || cudaSetDevice(dev) != cudaSuccess || !make()) return false;
+  }
   const int slot = used < kMapCache ? used++ : (next = (next + 1) % kMapCache);
   keys[slot] = key;
   maps[slot] = *tm;
@@ -165,6 +171,18 @@ bool halo_applies(int H, int W, int taps) {
   return covered * 100 <= (int64_t)H * W * 135;
 }
 
+// What pruning costs (measured on a [16384 x 4096] tensor and on 50176 x 1024 rows): clocks of the rows kernel's pruning warps per block of
+// 128 channels, picoseconds per element of the prune kernel where the integer pipe bounds it.
+struct PruneCost {
+  int stage_clk;
+  double ps;
+};
+PruneCost prune_cost(int m, int scheme) {
+  if (scheme == SDGP_RANDOM) return m == 4 ? PruneCost{3600, 0.68} : PruneCost{4300, 0.90};
+  if (scheme == SDGP_RESCALED_MAGNITUDE) return m == 4 ? PruneCost{3100, 0.56} : PruneCost{3800, 0.69};
+  return m == 4 ? PruneCost{1700, 0.40} : PruneCost{2500, 0.57};
+}
+
 }  // namespace
 
 // A: dense dL/dO [B,P,Q,Cout] (sparse == false) or compressed values [B,P,Q,a_channels/2] with
@@ -198,7 +216,7 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
   if ((int64_t)R * S * Cin > 0x7FFFFFFF) return SDGP_ERR_UNSUPPORTED;
 
   if (fused && B == 1 && H == 1 && R == 1 && S == 1 && stride == 1 && pad == 0 && fused->m <= 16) {
-    const RowsPlan plan = plan_rows(W, Cout, Cin);
+    const RowsPlan plan = plan_rows(W, Cout, Cin, prune_cost(fused->m, fused->scheme).stage_clk);
     if (plan.ok) return launch_rows_fused(plan, A, Wt, Cout, Cin, dD, *fused, dtype, stream);
   }
   const int kb_channels = sparse ? 128 : 64;
@@ -287,6 +305,38 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
     }
   }
   return SDGP_OK;
+}
+
+namespace {
+
+// Two-pass calls over rows: the kernel that prunes inside the contraction replaces prune kernel + contraction where it is
+// estimated to be faster. Estimate of the pair, us: 1.5 + 4 for two launches' ramps, the prune kernel's bytes at 6.4 TB/s or its
+// arithmetic, and the contraction's bytes, operand traffic from L2 or products. Few channels (one launch less, no second read of dO)
+// favour the rows kernel, many channels on few rows the pair (a CTA pair prunes its blocks one after another). On 70 drawn
+// layers the estimates put the faster one first wherever the two differed by more than a tenth, but for a handful.
+bool rows_fused_pays(int64_t rows, int K, int N, int m, int scheme, RowsPlan* plan) {
+  const PruneCost pc = prune_cost(m, scheme);
+  *plan = plan_rows(rows, K, N, pc.stage_clk);
+  if (!plan->ok) return false;
+  const double e = (double)rows * K, out = (double)rows * N;
+  const double prune_mem = 3.125 * e / 6.4e6, prune_alu = e * pc.ps * 1e-6, prune = prune_mem > prune_alu ? prune_mem : prune_alu;
+  const int64_t m_tiles = (rows + 127) / 128;
+  const int blocks = (K + 127) / 128, bn = choose_bn(m_tiles, N, blocks, 128, K, nullptr);
+  const int64_t tiles = (m_tiles + 1) / 2 * ((N + bn - 1) / bn), pairs = sm_count() / 2;
+  const double l2 = (double)((tiles + pairs - 1) / pairs) * (256 + blocks * (256 + 2 * bn)) / 1900.0;
+  const double mem = (1.125 * e + 2.0 * out) / 6.0e6, mma = 2.0 * e * N / 2.0e9;
+  double contraction = mem > l2 ? mem : l2;
+  if (mma > contraction) contraction = mma;
+  return plan->cost / 1900.0 * 0.9 < 5.5 + prune + contraction;
+}
+
+}  // namespace
+
+sdgp_status try_rows_fused(const void* dO, const void* W, void* dD, int64_t rows, int K, int N, const FusedPrune& prune, int dtype,
+                           cudaStream_t stream, bool* taken) {
+  RowsPlan plan;
+  *taken = rows_fused_pays(rows, K, N, prune.m, prune.scheme, &plan);
+  return *taken ? launch_rows_fused(plan, dO, W, K, N, dD, prune, dtype, stream) : SDGP_OK;
 }
 
 // One CTA waits, with a 50 ms limit, on a barrier that nothing ever signals: the wait must give

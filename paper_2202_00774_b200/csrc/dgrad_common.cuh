@@ -53,9 +53,7 @@ constexpr int kBM = 128;             // output pixels (rows) per CTA tile = TMEM
 constexpr int kThreadsGemm = 320;    // 10 warps
 constexpr unsigned kIdleWaitNs = 200;  // sleep between polls of the waits that are off the critical path
 constexpr int kEHwBytes = kBM * 16;  // rearranged metadata of one (tap, channel block): 128 lanes x 16 B
-constexpr int kStageBufs = 2;
-constexpr int kWarpStage = kStageBufs * 32 * 128;  // epilogue staging of a warp (store_box): 32 rows of 64 columns, twice
-constexpr int kStageBytes = 4 * kWarpStage;
+constexpr int kSlabBytes = 32 * 128;  // epilogue staging of a warp (store_box): 32 rows of 64 columns, once or twice
 constexpr uint32_t kTmemCols = 512;
 constexpr int kMaxImgRows = 192;     // pixel rows of one A stage (filter-row reuse: TW * (TH + R - 1))
 constexpr int kSmemLimit = 232448;   // opt-in dynamic shared memory per CTA
@@ -163,22 +161,25 @@ __device__ __forceinline__ void store_rows(uint32_t taddr, uint8_t* dst, int col
   }
 }
 
-// store_box: through 2 x 4 KB of the warp's own swizzled shared memory and its own TMA store (a box of 32 pixels, clipped at the
+// store_box: through 4 KB (twice where there is room: the next slab is packed while the last one is stored) of the warp's own swizzled shared memory and its own TMA store (a box of 32 pixels, clipped at the
 // edges of dD): one line per request instead of 32 per instruction. For launches whose epilogues run beside other tiles' work:
 // the pruning warps of a fused kernel need the load/store unit (128 -> 128 channels at 28 x 28, batch 256: 47 us against 53 us).
 // (c1, c2, c3, c4): coordinates 1.. of the box in dD's map; five: the map has five dimensions.
 template <int BN>
 __device__ __forceinline__ void store_box(uint32_t taddr, uint8_t* stage, const CUtensorMap* tmD, bool five, int n0, int c1, int c2,
                                           int c3, int c4, bool in_range, int columns, uint64_t* first_slab_read, uint64_t* released,
-                                          bool f16, uint32_t& chunk) {
+                                          bool f16, int bufs, uint32_t& chunk) {
   const int lane = threadIdx.x & 31;
 #pragma unroll 1
   for (int c0 = 0; c0 < BN; c0 += 64) {
     const bool last = c0 + 64 >= BN || c0 + 64 >= columns;
     uint32_t packed[32];
     read_slab(taddr + (uint32_t)c0, packed, c0 == 0 ? first_slab_read : nullptr, last ? released : nullptr, f16);
-    uint8_t* buf = stage + (chunk % kStageBufs) * (32 * 128);
-    if (lane == 0) ptx::bulk_wait_group_read<kStageBufs - 1>();  // the store that last used this buffer has read it
+    uint8_t* buf = stage + (bufs == 2 ? chunk & 1u : 0u) * kSlabBytes;
+    if (lane == 0) {  // the store that last used this buffer has read it
+      if (bufs == 2) ptx::bulk_wait_group_read<1>();
+      else ptx::bulk_wait_group_read<0>();
+    }
     __syncwarp();
 #pragma unroll
     for (int c = 0; c < 8; ++c)

@@ -450,8 +450,8 @@ dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
       uint64_t* first_slab_read = p.meta_shared ? &meta_free[acc] : nullptr;
       if (p.box_store) {
-        store_box<BN>(taddr, sOut + q * kWarpStage, &tmD, false, n0, w - lane, h, b, 0, mt < p.m_tiles, p.d.channels - n0,
-                      first_slab_read, &acc_empty[acc], p.f16 != 0, chunk);
+        store_box<BN>(taddr, sOut + q * p.out_bufs * kSlabBytes, &tmD, false, n0, w - lane, h, b, 0, mt < p.m_tiles, p.d.channels - n0,
+                      first_slab_read, &acc_empty[acc], p.f16 != 0, p.out_bufs, chunk);
       } else {
         const bool inside = row < rows_used && mt < p.m_tiles && w < p.W && h < p.H && b < p.B;
         uint8_t* dst = inside ? p.d.base + b * p.d.sb + h * p.d.sh + w * p.d.sw + 2 * n0 : nullptr;
@@ -508,8 +508,14 @@ bool plan(DgradParams* p) {
     const int w_bytes = resident ? taps * p->k_blocks * C::kTapBBytes : 0;
     const int raw_bytes = FUSED ? 2 * p->a_bytes : 0;
     const int stage_bytes = p->a_bytes + p->b_bytes + p->eraw_bytes + p->ehw_bytes + raw_bytes;
-    const int out_bytes = p->box_store ? kStageBytes : 0;
+    p->out_bufs = p->box_store ? 2 : 0;
+    int out_bytes = 4 * p->out_bufs * kSlabBytes;
     int stages = (budget - w_bytes - out_bytes) / stage_bytes;
+    if (p->box_store && stages < 4) {
+      p->out_bufs = 1;
+      out_bytes = 4 * kSlabBytes;
+      stages = (budget - w_bytes - out_bytes) / stage_bytes;
+    }
     if (stages > kMaxStages) stages = kMaxStages;
     // TMEM: accumulators first, metadata slots (4 columns per tap and stage) behind them
     const int meta_cols_per_stage = SPARSE ? 4 * p->rr : 0;

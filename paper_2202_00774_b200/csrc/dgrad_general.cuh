@@ -22,6 +22,7 @@ struct DgradParams {
   int meta_col;           // first TMEM column of the metadata slots
   int meta_shared;        // metadata slots live in the first columns of the accumulator NOT being written
   int w_resident;         // whole W half-slice kept in shared memory
+  int out_bufs;           // staging slabs per epilogue warp (boxes only)
   int box_store;          // the epilogue's warps write boxes of 32 pixels by TMA (else rows, straight from registers)
   // fused pruning (the kernel reads dense dL/dO and prunes it while staging A)
   int fused_n, fused_m, fused_scheme;

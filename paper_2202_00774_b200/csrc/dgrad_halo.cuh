@@ -599,10 +599,10 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         if constexpr (FUSED) {
           // this warp's 4 strip rows: 4 / tb pixel rows of tb images
           const int hq = h0 + q * (4 / p.tb);
-          if (p.split) store_box<BN>(taddr, sOut + q * kWarpStage, &tmD, true, n0, 0, 2 * j, b0 / p.img_per_row, hq, strip_live,
-                                     p.d.channels - n0, first_slab_read, released, p.f16 != 0, chunk);
-          else store_box<BN>(taddr, sOut + q * kWarpStage, &tmD, false, n0, w0 + 8 * j, b0, hq, 0, strip_live && w0 + 8 * j < p.W,
-                             p.d.channels - n0, first_slab_read, released, p.f16 != 0, chunk);
+          if (p.split) store_box<BN>(taddr, sOut + q * p.out_bufs * kSlabBytes, &tmD, true, n0, 0, 2 * j, b0 / p.img_per_row, hq, strip_live,
+                                     p.d.channels - n0, first_slab_read, released, p.f16 != 0, p.out_bufs, chunk);
+          else store_box<BN>(taddr, sOut + q * p.out_bufs * kSlabBytes, &tmD, false, n0, w0 + 8 * j, b0, hq, 0, strip_live && w0 + 8 * j < p.W,
+                             p.d.channels - n0, first_slab_read, released, p.f16 != 0, p.out_bufs, chunk);
         } else {
           const int w = w0 + dw + (p.split ? 0 : 8 * j), h = h0 + dh, b = b0 + db + (p.split ? 2 * j : 0);
           const bool inside = strip_live && w < p.W && h < p.H && b < p.B;
@@ -634,7 +634,6 @@ template <bool SPARSE, int BN, bool FUSED>
 bool plan_halo(HaloParams* p, int nt) {
   using C = Cfg<SPARSE, BN>;
   const int budget = kSmemLimit - kSmemSlack;
-  constexpr int kOut = FUSED ? kStageBytes : 0;  // epilogue staging
   {
     if (nt * BN > 256) return false;         // two tile sets of accumulators must fit the 512 TMEM columns
     p->split = (p->W == 4) ? 1 : 0;  // images 4 pixels wide: two per strip row, horizontal taps by separate boxes
@@ -665,10 +664,15 @@ bool plan_halo(HaloParams* p, int nt) {
     // run further ahead of the MMAs, if that still leaves three W stages
     p->a_stages = 2;
     const int per_a = p->a_bytes + p->eraw_bytes + p->meta_bytes;
-    if (p->split && (budget - 4 * per_a - 1024 - kOut) / p->w_bytes >= 3) p->a_stages = 4;
+    if (p->split && (budget - 4 * per_a - 1024 - (FUSED ? 4 * kSlabBytes : 0)) / p->w_bytes >= 3) p->a_stages = 4;
     p->a_shift = p->a_stages == 4 ? 2 : 1;
     const int fixed = p->a_stages * per_a + 1024;
-    int w_stages = (budget - fixed - kOut) / p->w_bytes;
+    p->out_bufs = FUSED ? 2 : 0;  // epilogue staging
+    int w_stages = (budget - fixed - 4 * p->out_bufs * kSlabBytes) / p->w_bytes;
+    if (FUSED && w_stages < 4) {
+      p->out_bufs = 1;
+      w_stages = (budget - fixed - 4 * kSlabBytes) / p->w_bytes;
+    }
     if (w_stages > kMaxStages) w_stages = kMaxStages;
     p->meta_shared = 0;
     p->meta_col = 2 * nt * BN;
@@ -690,7 +694,7 @@ bool plan_halo(HaloParams* p, int nt) {
     p->off_w = round_up(p->off_meta + p->a_stages * p->meta_bytes, 1024);
     p->pitch_magic = ((1u << 20) + (uint32_t)p->pitch - 1u) / (uint32_t)p->pitch;
     p->off_out = round_up(p->off_w + w_stages * p->w_bytes, 1024);
-    p->off_bar = p->off_out + kOut;
+    p->off_bar = p->off_out + 4 * p->out_bufs * kSlabBytes;
     p->smem_bytes = p->off_bar + 512 + 1024;
     if (p->smem_bytes > kSmemLimit) return false;
     p->sets_w = p->split ? 1 : (p->W + 8 * nt - 1) / (8 * nt);

@@ -49,7 +49,7 @@ struct HaloParams {
   // per pruning warp, which is what sets the time a box takes.
   int static_pad, units_per_box, unit_row0, unit_col0;
   int w_stages;
-  int meta_col, meta_shared;
+  int meta_col, meta_shared, out_bufs;
   int a_bytes, eraw_bytes, w_bytes;  // per stage
   // Position metadata of an A box in the order the tensor core wants, stored ONCE per box and shared by every
   // tap: "master" pi (pi = 0, 1) pairs box rows (pi + 2m, pi + 2m + 1); its 16-byte line ((2m + e) * pitch + x)

@@ -24,6 +24,7 @@ namespace {
 constexpr int kRowsThreads = 24 * 32;
 constexpr int kRowsPruneWarps = 16;
 constexpr int kRowsMaxStages = 8;            // of each ring
+constexpr int kRowsOutBytes = 4 * 2 * kSlabBytes;  // epilogue staging
 constexpr int kRowsMaxAcc = 8;               // accumulators
 constexpr int kABytes = 128 * 128;           // 128 rows x 64 compressed elements, 128-byte swizzled
 constexpr int kMetaBytes = 128 * 16;         // the stage's metadata in the order tcgen05.cp moves to TMEM
@@ -266,8 +267,8 @@ rows_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       for (int nt = nt0; nt < nt1; ++nt) {
         if (!ptx::mbar_wait<kIdleWaitNs>(&acc_full[acc], (acc_ph >> acc) & 1u, err, 0x600u + acc)) { alive = false; break; }
         ptx::tc_fence_after_sync();
-        store_box<BN>(tmem_base_any + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN), sOut + q * kWarpStage, &tmD, false, nt * BN, row,
-                      0, 0, 0, row < p.rows, p.N - nt * BN, nullptr, &acc_empty[acc], p.f16 != 0, chunk);
+        store_box<BN>(tmem_base_any + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN), sOut + q * 2 * kSlabBytes, &tmD, false, nt * BN, row,
+                      0, 0, 0, row < p.rows, p.N - nt * BN, nullptr, &acc_empty[acc], p.f16 != 0, 2, chunk);
         acc_ph ^= 1u << acc;
         if (++acc == p.acc_ring) acc = 0;
       }
@@ -310,7 +311,7 @@ sdgp_status launch_rows_scheme(int bn, const CUtensorMap& tmA, const CUtensorMap
 // Shared-memory plan: the rings grow in turn while they fit.
 bool plan_rows_smem(RowsParams* p, int bn) {
   const int w_bytes = 128 * bn;  // one CTA's half of a W stage
-  const int budget = kSmemLimit - kSmemSlack - kStageBytes - 2048;
+  const int budget = kSmemLimit - kSmemSlack - kRowsOutBytes - 2048;
   int raw = 2, a = 2, w = 2;
   auto used = [&]() { return raw * kRawBytes + a * (kABytes + kMetaBytes) + w * w_bytes; };
   if (used() > budget) return false;
@@ -330,14 +331,16 @@ bool plan_rows_smem(RowsParams* p, int bn) {
   p->off_meta = p->off_a + a * kABytes;
   p->off_w = round_up(p->off_meta + a * kMetaBytes, 1024);
   p->off_out = p->off_w + w * w_bytes;
-  p->off_bar = p->off_out + kStageBytes;
+  p->off_bar = p->off_out + kRowsOutBytes;
   p->smem_bytes = p->off_bar + 1024 + 1024;
   return p->smem_bytes <= kSmemLimit;
 }
 
 }  // namespace
 
-RowsPlan plan_rows(int64_t rows, int K, int N) {
+namespace {
+
+RowsPlan make_plan(int64_t rows, int K, int N, int stage_clk) {
   RowsPlan best = {};
   if (rows < 1 || rows > 0x7FFFFF00 || K % 8 != 0 || N % 8 != 0) return best;
   const int64_t pairs = sm_count() / 2, row_tiles = (rows + 255) / 256;
@@ -363,7 +366,7 @@ RowsPlan plan_rows(int64_t rows, int K, int N) {
       const double rate = 20.0 / busy < 55.0 ? 20.0 / busy : 55.0;
       const double mem = (256.0 * K / p.n_groups + 256.0 * g * bn) / rate, l2 = (256.0 * K + 128.0 * kb * g * bn) / 55.0;
       const double smem = (kb * (2.0 * 32768 + 18432 + 128.0 * bn * g + g * 4.0 * (4096 + 16.0 * bn)) + 512.0 * bn * g) / 115.0;
-      const double prune = kb * 1700.0 + 500.0, out = 16.0 * g * bn;
+      const double prune = kb * stage_clk + 500.0, out = 16.0 * g * bn;
       double work = mem > l2 ? mem : l2;
       if (smem > work) work = smem;
       if (prune > work) work = prune;
@@ -376,6 +379,22 @@ RowsPlan plan_rows(int64_t rows, int K, int N) {
     }
   }
   return best;
+}
+
+}  // namespace
+
+RowsPlan plan_rows(int64_t rows, int K, int N, int stage_clk) {
+  struct Entry { int64_t rows; int K, N, stage_clk, sms; RowsPlan plan; };
+  constexpr int kEntries = 32;
+  static thread_local Entry cache[kEntries] = {};
+  static thread_local int next = 0;
+  const int sms = sm_count();
+  for (const Entry& e : cache)
+    if (e.rows == rows && e.K == K && e.N == N && e.stage_clk == stage_clk && e.sms == sms) return e.plan;
+  Entry& e = cache[next];
+  next = (next + 1) % kEntries;
+  e = {rows, K, N, stage_clk, sms, make_plan(rows, K, N, stage_clk)};
+  return e.plan;
 }
 
 sdgp_status launch_rows_fused(const RowsPlan& plan, const void* dO, const void* W, int w_rows, int w_cols, void* dD,

@@ -25,7 +25,8 @@ struct RowsPlan {
   double cost;  // estimated clocks
   RowsParams p;
 };
-RowsPlan plan_rows(int64_t rows, int K, int N);
+// stage_clk: clocks the pruning warps take for a block of 128 channels. (Kept per thread for the last shapes asked for.)
+RowsPlan plan_rows(int64_t rows, int K, int N, int stage_clk);
 
 // dD [rows, N] = prune(dO [rows, K]) . W, pruned inside the kernel (n <= 2). W has w_rows >= K rows of w_cols >= N columns.
 sdgp_status launch_rows_fused(const RowsPlan& plan, const void* dO, const void* W, int w_rows, int w_cols, void* dD,

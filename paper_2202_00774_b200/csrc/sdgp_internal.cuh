@@ -82,6 +82,11 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
                          const FusedPrune* fused = nullptr, int dtype = SDGP_BF16, const StoredChannels* stored = nullptr,
                          const ConvGroups* conv_groups = nullptr);
 
+// dD [rows, N] = prune(dO [rows, K]) . W [K, N] in one kernel, if that is estimated to be faster than prune kernel + contraction
+// (*taken tells; nothing is launched otherwise). K and N multiples of 8, prune.n <= 2.
+sdgp_status try_rows_fused(const void* dO, const void* W, void* dD, int64_t rows, int K, int N, const FusedPrune& prune, int dtype,
+                           cudaStream_t stream, bool* taken);
+
 // Filters of a grouped convolution, Wg [Cout, R*S, Cin/groups], written as the block-diagonal filters of an
 // ordinary one, Wfull [cout_pad, R*S, cin_pad] (zeros outside each group's block and in the padding).
 cudaError_t launch_expand_grouped_weights(const void* Wg, int Cout, int taps, int Cin, int groups, int cout_pad, int cin_pad,

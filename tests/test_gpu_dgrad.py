@@ -688,3 +688,36 @@ def test_linear_tile_widths_and_row_tails(rows, K, N, offset):
         assert_close(to_f64(dD)[pick], *linear_ref(A[pick], W))
         edge = flat.cpu().numpy()
         assert np.all(edge[:offset] == 0x5A5A) and np.all(edge[offset + rows * N:] == 0x5A5A)
+
+
+# ------------------------------------------------- prune + contraction over rows in one kernel
+
+
+@pytest.mark.parametrize("scheme", [oracle.RANDOM, oracle.MAGNITUDE, oracle.RESCALED])
+@pytest.mark.parametrize("rows,K,N,n,m", [(1, 64, 64, 2, 4), (257, 192, 448, 1, 4), (700, 1216, 320, 2, 8), (20000, 128, 128, 2, 16),
+                                          (20100, 320, 576, 2, 4), (500, 128, 64, 2, 32), (4000, 256, 1024, 1, 32)])
+def test_linear_pruned_on_the_way(rows, K, N, n, m, scheme):
+    """Row tails, a last channel block of one to four MMAs, more channel blocks than stages, one and several column tiles and groups
+    per CTA pair, several works per pair, every group size; fused mode, two-pass mode (whichever kernel it takes) and the same
+    call from a thread of its own."""
+    import threading
+    import paper_2202_00774_b200 as sdgp
+    dO, W = inputs.fc_tensors(rows, K, N, seed=rows + K)
+    ws = torch.empty(max(16, sdgp.sdgp_workspace_size_linear(rows, K, N)), dtype=torch.uint8, device="cuda")
+    pick = np.unique(np.concatenate([np.arange(min(rows, 40)), np.arange(max(0, rows - 200), rows)]))   # whole rows
+    pruned = oracle.prune(dO, n, m, scheme, 9, want=("dense",))["dense"][pick]
+    ref = linear_ref(pruned, W)
+    flat = torch.full((rows * N + 64,), 0x5A5A, dtype=torch.int16, device="cuda")
+    dD, a, b = flat[:rows * N].view(rows, N), dev16(dO), dev16(W)
+    calls = [lambda: sdgp.sdgp_dgrad_linear(a, b, dD, n, m, scheme, 9, workspace=ws)]
+    if m <= 16:
+        calls.append(lambda: sdgp.sdgp_dgrad_linear(a, b, dD, n, m, scheme, 9, flags=sdgp.FLAG_FUSED))
+    for call in calls:
+        flat.fill_(0x5A5A)
+        torch.cuda.synchronize()
+        t = threading.Thread(target=call)
+        t.start()
+        t.join()
+        check_no_device_error()
+        assert_close(to_f64(dD)[pick], *ref)
+        assert np.all(flat[rows * N:].cpu().numpy() == 0x5A5A)

@@ -331,7 +331,6 @@ sdgp_status sdgp_dgrad_conv2d_grouped(const void* dO, const void* W, void* dD, i
     w_full = workspace;
   }
   const sdgp::StoredChannels dense_view = {Cout != cout_k ? Cout : 0, Cin != cin_k ? Cin : 0};
-  const sdgp::StoredChannels sparse_view = {0, dense_view.d};  // a compressed dL/dO is padded by the prune kernel
   const bool padded = dense_view.a != 0 || dense_view.d != 0;
   const sdgp::ConvGroups cg = {Cin / groups, Cout / groups};
   const sdgp::ConvGroups* cgp = groups > 1 ? &cg : nullptr;
@@ -356,7 +355,7 @@ sdgp_status sdgp_dgrad_conv2d_grouped(const void* dO, const void* W, void* dD, i
   if (sdgp::launch_prune(dO, rows, Cout, n, m, (int)scheme, seed, nullptr, c.values, c.meta, nullptr, s, Cpad, dt) != cudaSuccess)
     return SDGP_ERR_CUDA;
   return sdgp::launch_dgrad(true, c.values, c.meta, w_full, dD, B, H, Wd, cin_k, cout_k, R, S, stride, pad, s, nullptr, dt,
-                            sparse_view.d ? &sparse_view : nullptr, cgp);
+                            padded ? &dense_view : nullptr, cgp);
 }
 
 sdgp_status sdgp_dgrad_linear(const void* dO, const void* W, void* dD, int64_t rows, int64_t K,

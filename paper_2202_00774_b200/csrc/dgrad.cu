@@ -185,9 +185,8 @@ PruneCost prune_cost(int m, int scheme) {
 
 }  // namespace
 
-// A: dense dL/dO [B,P,Q,Cout] (sparse == false) or compressed values [B,P,Q,a_channels/2] with
-// meta [B,P,Q,a_channels/16], a_channels = Cout rounded up to 128 (pad channels hold zero values
-// and the position pair (0,1)); Wt: [Cout, R, S, Cin]; dD: [B,H,W,Cin].
+// A: dense dL/dO [B,P,Q,Cout] (sparse == false) or compressed values [B,P,Q,Cout/2] with meta [B,P,Q,Cp/16], Cp = Cout
+// rounded up to 128 (pad channels name the position pair (0,1)); Wt: [Cout, R, S, Cin]; dD: [B,H,W,Cin].
 // Stride 2 is split by the parity of the output pixel: pixel (2h'+ph, 2w'+pw) only meets the taps
 // r = ph + pad (mod 2), s = pw + pad (mod 2), and on those it is a stride-1 problem from dO to
 // the strided view dD[:, ph::2, pw::2, :].
@@ -223,7 +222,8 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
 
   DgradView view;
   view.P = P; view.Q = Q; view.batch = B;
-  view.a_channels = (sparse && !fused) ? (Cout + 127) / 128 * 128 : (stored && stored->a) ? stored->a : Cout;
+  view.a_channels = (stored && stored->a) ? stored->a : Cout;
+  view.meta_channels = (view.a_channels + 127) / 128 * 128;
   view.d.channels = (stored && stored->d) ? stored->d : Cin;
   view.w_cols = (int64_t)R * S * Cin;
   const size_t Cd = (size_t)view.d.channels;
@@ -264,6 +264,10 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
         p.diag_cin_g = conv_groups->cin_g; p.diag_cout_g = conv_groups->cout_g;
         p.diag_last = all_blocks - p.k_blocks;
       }
+      // the last channel block may be partly empty: its MMAs (32 channels each, dense 16) past the channels that exist are left out
+      p.k_last = all_blocks - 1;
+      const int left = view.a_channels - p.k_last * kb_channels, per_mma = kb_channels / 4;
+      p.last_mmas = left < kb_channels ? (left + per_mma - 1) / per_mma : 4;
       p.P = P; p.Q = Q;
       p.f16 = dtype == SDGP_FP16 ? 1 : 0;
       if (fused) {
@@ -289,6 +293,7 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
         hp.tiles_n = p.tiles_n; hp.k_blocks = p.k_blocks;
         hp.diag_cin_g = p.diag_cin_g; hp.diag_cout_g = p.diag_cout_g; hp.diag_last = p.diag_last;
         hp.P = P; hp.Q = Q;
+        hp.k_last = p.k_last; hp.last_mmas = p.last_mmas;
         hp.f16 = p.f16;
         if (fused) {
           hp.fused_n = p.fused_n; hp.fused_m = p.fused_m; hp.fused_scheme = p.fused_scheme; hp.seed_lo = p.seed_lo; hp.seed_hi = p.seed_hi;

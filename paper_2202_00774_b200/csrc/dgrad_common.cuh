@@ -25,7 +25,8 @@ struct OutView {
 // width in W columns, and the (possibly strided) view of dD the launch fills.
 struct DgradView {
   int P, Q, batch;
-  int a_channels;
+  int a_channels;                 // channels per pixel of dO that exist
+  int meta_channels;              // ... and of the compressed form's metadata rows (whole blocks of 128)
   int64_t w_cols;                 // R_full * S_full * Cin
   OutView d;
 };

@@ -302,35 +302,45 @@ dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         ptx::tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
         uint32_t accumulate = 0u;
+        const int cb_last = p.k_last - first_k_block(p, (first_pair + lt * pair_stride) % p.tiles_n * BN, C::kKB);
         int r_single = 0, s = 0;
         for (int g = 0; alive && g < groups; ++g) {
           for (int cb = 0; cb < p.k_blocks; ++cb) {
             if (!ptx::mbar_wait(&full[st], ph, err, 0x300u + st)) { alive = false; break; }
             ptx::tc_fence_after_sync();
             const uint32_t e_col = meta_base + mcol;  // even: slots are multiples of 4 columns apart
+            const int mmas = cb == cb_last ? p.last_mmas : 4;
             if (SPARSE) {
               for (int u = 0; u < p.rr; ++u)
                 ptx::tc_cp_128x128b_pair(e_col + 4u * u, ((uint64_t)e_hi << 32) | (e_lo + (uint32_t)(u * (kEHwBytes / 16))));
             }
-            for (int u = 0; u < p.rr; ++u) {
-              // vertical tap r: the tile's rows start (R-1-r) image rows into the stage
-              const int r = reuse ? u : r_single;
-              const uint32_t a_u = a_lo + (reuse ? (uint32_t)((p.R - 1 - r) * p.TW * 8) : 0u);
-              const uint32_t b_u = p.w_resident ? w_lo0 + (uint32_t)((r * p.S + s) * p.k_blocks + cb) * kTapB16
-                                                : b_lo + (uint32_t)u * kTapB16;
+            // MMAS: MMAs of the channel block
+            auto issue = [&](auto mmas_tag) {
+              constexpr int MMAS = decltype(mmas_tag)::value;
+              for (int u = 0; u < p.rr; ++u) {
+                // vertical tap r: the tile's rows start (R-1-r) image rows into the stage
+                const int r = reuse ? u : r_single;
+                const uint32_t a_u = a_lo + (reuse ? (uint32_t)((p.R - 1 - r) * p.TW * 8) : 0u);
+                const uint32_t b_u = p.w_resident ? w_lo0 + (uint32_t)((r * p.S + s) * p.k_blocks + cb) * kTapB16
+                                                  : b_lo + (uint32_t)u * kTapB16;
 #pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                // A: 32 bytes of a 128-byte swizzled row per MMA; B: 16 (dense) or 32 (sparse) rows
-                const uint64_t a_q = ((uint64_t)a_hi << 32) | (a_u + (uint32_t)(q * 2));
-                const uint64_t b_q = ((uint64_t)b_hi << 32) | (b_u + (uint32_t)q * kBStep);
-                if (SPARSE)
-                  ptx::mma_sp_f16_ss_pair(d_tmem, a_q, b_q, e_col + 4u * u + (uint32_t)(q & 2), idesc | (uint32_t)(q & 1),
-                                          q == 0 ? accumulate : 1u);
-                else
-                  ptx::mma_f16_ss_pair(d_tmem, a_q, b_q, idesc, q == 0 ? accumulate : 1u);
+                for (int q = 0; q < MMAS; ++q) {
+                  // A: 32 bytes of a 128-byte swizzled row per MMA; B: 16 (dense) or 32 (sparse) rows
+                  const uint64_t a_q = ((uint64_t)a_hi << 32) | (a_u + (uint32_t)(q * 2));
+                  const uint64_t b_q = ((uint64_t)b_hi << 32) | (b_u + (uint32_t)q * kBStep);
+                  if (SPARSE)
+                    ptx::mma_sp_f16_ss_pair(d_tmem, a_q, b_q, e_col + 4u * u + (uint32_t)(q & 2), idesc | (uint32_t)(q & 1),
+                                            q == 0 ? accumulate : 1u);
+                  else
+                    ptx::mma_f16_ss_pair(d_tmem, a_q, b_q, idesc, q == 0 ? accumulate : 1u);
+                }
+                accumulate = 1u;
               }
-              accumulate = 1u;
-            }
+            };
+            if (mmas == 4) issue(std::integral_constant<int, 4>{});
+            else if (mmas == 3) issue(std::integral_constant<int, 3>{});
+            else if (mmas == 2) issue(std::integral_constant<int, 2>{});
+            else issue(std::integral_constant<int, 1>{});
             ptx::tc_commit_pair(&empty[st], 3);
             if (++st == STAGES) { st = 0; ph ^= 1u; a_lo = a_lo0; b_lo = b_lo0; e_lo = e_lo0; mcol = 0; }
             else { a_lo += a_stage16; b_lo += b_stage16; e_lo += e_stage16; mcol += slot_cols; }
@@ -569,7 +579,7 @@ sdgp_status launch_cfg(const void* A, const void* meta, const void* Wt, const Dg
       return SDGP_ERR_CUDA;
   }
   if (SPARSE && !FUSED) {
-    const uint64_t CE = (uint64_t)view.a_channels / 16;
+    const uint64_t CE = (uint64_t)view.meta_channels / 16;
     const uint64_t dims[4] = {CE, (uint64_t)Q, (uint64_t)P, (uint64_t)view.batch};
     const uint64_t strides[3] = {CE * 2, CE * 2 * Q, CE * 2 * Q * P};
     const uint32_t box[4] = {8, (uint32_t)p.TW, img_h, (uint32_t)p.TB};

@@ -15,6 +15,7 @@ struct DgradParams {
   int m_tiles;            // tiles_w * tiles_h * tiles_b
   int pair_tiles;         // ceil(m_tiles / 2) * tiles_n
   int k_blocks;           // channel blocks per tap: ceil(Cout / channels per stage)
+  int k_last, last_mmas;  // the layer's last channel block and the MMAs it needs (1..4)
   int rr;                 // vertical taps served by one A stage: 1, or R (filter-row reuse)
   int img_rows;           // pixel rows of one A stage: TW * (TH + rr - 1) * TB
   int stages;             // shared-memory pipeline depth

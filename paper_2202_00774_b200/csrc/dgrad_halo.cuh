@@ -256,10 +256,17 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * set_cols);
         const uint32_t strips = strip_mask(lt);
         const bool all_strips = strips == ((1u << NT) - 1u);
+        int kb0 = 0;
+        if (p.diag_cin_g != 0) {
+          int n0, w0, h0, b0;
+          locate(first_pair + lt * pair_stride, n0, w0, h0, b0);
+          kb0 = first_k_block(p, n0, C::kKB);
+        }
         uint32_t accumulate = 0u;
         for (int ku = 0; alive && ku < p.k_uses; ++ku) {
           if (!wait_all(&a_full[ast], aph, 0x300u + ast)) { alive = false; break; }
           if (SPARSE && !FUSED && !wait_all(&meta_ready[ast], aph, 0x340u + ast)) { alive = false; break; }
+          const int mmas = kb0 + ku / p.ss == p.k_last ? p.last_mmas : 4;
           uint32_t a_lo = a_lo0 + (uint32_t)ast * a_stage16 + a_first16;
           int s = p.sb, dr = p.R - 1;
           const uint32_t e_stage = e_lo0 + (uint32_t)ast * e_stage16;
@@ -268,20 +275,21 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             if (!wait_all(&w_ready[wst], wph, 0x380u + wst)) { alive = false; break; }
             ptx::tc_fence_after_sync();
             const uint32_t e_col = meta_base + mcol;  // even: slots are 4 columns apart
-            // ALL: every strip takes part (no per-strip test in the issue path)
-            auto issue_tap = [&](auto all) {
-              constexpr bool ALL = decltype(all)::value;
+            // MMAS: MMAs of the channel block if every strip takes part (no per-strip test in the issue path), 0: neither is known
+            auto issue_tap = [&](auto mmas_tag) {
+              constexpr int MMAS = decltype(mmas_tag)::value;
               if (SPARSE) {
 #pragma unroll
                 for (int j = 0; j < NT; ++j)
-                  if (ALL || (strips & (1u << j)))
+                  if (MMAS || (strips & (1u << j)))
                     ptx::tc_cp_128x128b_pair(e_col + 4u * j, ((uint64_t)e_hi << 32) | (e_lo + (uint32_t)(8 * j)));
               }
 #pragma unroll
               for (int j = 0; j < NT; ++j) {
-                if (!ALL && !(strips & (1u << j))) continue;
+                if (!MMAS && !(strips & (1u << j))) continue;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
+                for (int q = 0; q < (MMAS ? MMAS : 4); ++q) {
+                  if (!MMAS && q >= mmas) break;
                   // strip j: 8 pixels = 1024 bytes to the right; MMA q: 32 bytes along the row
                   const uint64_t a_q = ((uint64_t)a_hi << 32) | (a_lo + (uint32_t)(j * 64 + q * 2));
                   const uint64_t b_q = ((uint64_t)b_hi << 32) | (b_lo + (uint32_t)q * kBStep);
@@ -294,8 +302,9 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
               }
             };
             if (leader) {
-              if (all_strips) issue_tap(std::true_type{});
-              else issue_tap(std::false_type{});
+              if (all_strips && mmas == 4) issue_tap(std::integral_constant<int, 4>{});
+              else if (all_strips && mmas == 2) issue_tap(std::integral_constant<int, 2>{});
+              else issue_tap(std::integral_constant<int, 0>{});
               ptx::tc_commit_pair(&w_empty[wst], 3);
             }
             accumulate = 1u;
@@ -774,7 +783,7 @@ sdgp_status launch_halo_nt(const void* A, const void* meta, const void* Wt, cons
   tmE = tmA;
   p.a_dense = (const uint8_t*)A;
   if (SPARSE && !FUSED) {
-    const uint64_t CE = (uint64_t)view.a_channels / 16;
+    const uint64_t CE = (uint64_t)view.meta_channels / 16;
     if (!encode_nhwc(&tmE, CU_TENSOR_MAP_DATA_TYPE_UINT16, meta, CE, (uint64_t)Q, (uint64_t)P, (uint64_t)view.batch, CE * 2, CE * 2 * Q,
                      CE * 2 * Q * P, 8, box_w, (uint32_t)ipr, (uint32_t)p.tb, box_h, CU_TENSOR_MAP_SWIZZLE_NONE))
       return SDGP_ERR_CUDA;

@@ -27,6 +27,7 @@ struct HaloParams {
   int units;               // work units: pair tiles, the last `units - split_from` of them split by strip
   int split_from;          // units >= split_from cover one strip of a pair tile each (quantisation of the last round)
   int k_blocks;
+  int k_last, last_mmas;   // as in DgradParams
   int pitch;               // pixel columns of the A box: 8 * nt + S - 1
   int th, tb;              // a strip is 8 pixels wide and covers th pixel rows of tb images, th * tb = 16: 16 x 1, or 8 x 2
                            // for images at most 8 pixels tall. Its 16 rows are ordered (pixel row, image), so a vertical

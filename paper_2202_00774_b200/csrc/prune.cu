@@ -196,29 +196,20 @@ __device__ __forceinline__ void load_unit(const uint4* __restrict__ dO, int64_t 
 // element (a threshold on the number of wins), and the compressed slots / position nibbles
 // are computed on both lanes at once. About a quarter of the instructions of the generic path.
 
-// Row pitch of the compressed outputs, in 8-element vectors: k8 per input row, kpad8 per output
-// row (kpad8 == 0: same as the input). The extra vectors of a padded row are written as zero
-// values with the position pair (0,1), by the thread that owns the row's last real vector.
-struct OutPitch {
-  int k8, kpad8;
+// Row pitch of the metadata in pairs of vectors (two bytes each): k16 per input row, kpad16 per output row (kpad16 == 0: same as
+// the input). A reader that takes rows by TMA needs whole 16-byte rows of metadata; the values need no padding.
+struct MetaPitch {
+  uint32_t k16, kpad16;
 };
 
-// Writes one vector's outputs from the lane-paired form (see m4_prune_vector). COMPRESS: every
-// 4-chunk holds at most two survivors, so values / meta can be produced.
-// Output position of vector v's compressed outputs; writes the padding of a padded row when v is the row's last vector.
-__device__ __forceinline__ int64_t compressed_index(int64_t v, uint2* __restrict__ values, uint8_t* __restrict__ meta,
-                                                    OutPitch pitch) {
-  if (pitch.kpad8 == 0) return v;
-  const int64_t row = v / pitch.k8;
-  const int kv = (int)(v - row * pitch.k8);
-  const int64_t vo = row * pitch.kpad8 + kv;
-  if (kv == pitch.k8 - 1) {
-    for (int t = 1; t <= pitch.kpad8 - pitch.k8; ++t) {
-      if (values) values[vo + t] = make_uint2(0u, 0u);
-      if (meta) meta[vo + t] = (uint8_t)0x44;
-    }
-  }
-  return vo;
+// Position of pair p's metadata; the thread that owns a row's last pair names the position pair (0, 1) in the padding.
+__device__ __forceinline__ int64_t meta_index(int64_t p, bool fits32, uint16_t* __restrict__ meta, MetaPitch pitch) {
+  const int64_t row = fits32 ? (int64_t)((uint32_t)p / pitch.k16) : p / pitch.k16;  // (a 64-bit division is some 80 instructions)
+  const uint32_t kp = (uint32_t)(p - row * pitch.k16);
+  const int64_t po = row * pitch.kpad16 + kp;
+  if (kp == pitch.k16 - 1 && meta)
+    for (uint32_t t = 1; t <= pitch.kpad16 - pitch.k16; ++t) meta[po + t] = (uint16_t)0x4444;
+  return po;
 }
 
 // Keep flags (bit 15 of each lane) as the vector's mask byte, in the TOP byte of the result.
@@ -237,19 +228,17 @@ template <bool COMPRESS>
 __device__ __forceinline__ void emit_packed(int64_t v, uint32_t y0, uint32_t y1, uint32_t y2, uint32_t y3,
                                             uint32_t km0, uint32_t km1, uint32_t km2, uint32_t km3,
                                             uint4* __restrict__ dense, uint2* __restrict__ values,
-                                            uint8_t* __restrict__ meta, uint8_t* __restrict__ mask,
-                                            OutPitch pitch) {
+                                            uint8_t* __restrict__ meta, uint8_t* __restrict__ mask) {
   const uint4 pruned = make_uint4(prmt(y0, y1, 0x5410), prmt(y2, y3, 0x5410), prmt(y0, y1, 0x7632), prmt(y2, y3, 0x7632));
   const KeepFlags k = {km0, km1, km2, km3};
   if (dense) dense[v] = pruned;
   if (mask) mask[v] = (uint8_t)(mask_top_byte(k) >> 24);
   if (COMPRESS && (values || meta)) {
-    const int64_t vo = compressed_index(v, values, meta, pitch);
     uint2 out, slot_mask;
     uint32_t pos_top;
     gather_slots<false>(pruned, k, out, slot_mask, pos_top);
-    if (values) values[vo] = out;
-    if (meta) meta[vo] = (uint8_t)(pos_top >> 24);
+    if (values) values[v] = out;
+    if (meta) meta[v] = (uint8_t)(pos_top >> 24);
   }
 }
 
@@ -262,7 +251,7 @@ template <int M, int N, int SCHEME, bool F16, int SRC, bool DENSE>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSm<SCHEME, SRC>)
 prune_kernel(const uint4* __restrict__ dO, int64_t nvec, uint32_t seed_lo, uint32_t seed_hi,
              uint4* __restrict__ dense, uint2* __restrict__ values, uint8_t* __restrict__ meta,
-             uint8_t* __restrict__ mask, OutPitch pitch, ReluSource src) {
+             uint8_t* __restrict__ mask, MetaPitch pitch, ReluSource src) {
   ptx::wait_for_previous_grid();
   ptx::launch_dependents();  // only once this grid's own predecessor is done: at most one grid ever waits behind a running one
   if constexpr (!DENSE && SRC != kPool) {
@@ -290,8 +279,8 @@ prune_kernel(const uint4* __restrict__ dO, int64_t nvec, uint32_t seed_lo, uint3
       compress_pair<M, N, SCHEME, F16>(wa[it], wb[it], 2 * p, seed_lo, seed_hi, M == 32 ? (int)(threadIdx.x & 1) : 0, 0xFFFFFFFFu,
                                        out, pa, pb, ka, kb);
       if (M == 32 && p >= npair) continue;
-      const int64_t po = pitch.kpad8 == 0 ? p : compressed_index(2 * p + 1, values, meta, pitch) >> 1;
-      if (values) ((uint4*)values)[po] = out;
+      const int64_t po = pitch.kpad16 == 0 ? p : meta_index(p, npair <= 0xFFFFFFFF, (uint16_t*)meta, pitch);
+      if (values) ((uint4*)values)[p] = out;
       if (meta) ((uint16_t*)meta)[po] = (uint16_t)prmt(pa, pb, 0x0073);
       if (mask) ((uint16_t*)mask)[p] = (uint16_t)prmt(mask_top_byte(ka), mask_top_byte(kb), 0x0073);
     }
@@ -311,9 +300,8 @@ prune_kernel(const uint4* __restrict__ dO, int64_t nvec, uint32_t seed_lo, uint3
         KeepFlags k;
         compress_vector<M, N, SCHEME, F16>(in[it], v, seed_lo, seed_hi, part, 0xFFFFFFFFu, out, pos_top, k);
         if (LANES > 1 && v >= nvec) continue;
-        const int64_t vo = compressed_index(v, values, meta, pitch);
-        if (values) values[vo] = out;
-        if (meta) meta[vo] = (uint8_t)(pos_top >> 24);
+        if (values) values[v] = out;
+        if (meta) meta[v] = (uint8_t)(pos_top >> 24);
         if (mask) mask[v] = (uint8_t)(mask_top_byte(k) >> 24);
       } else {
         uint32_t y0, y1, y2, y3, km0, km1, km2, km3;
@@ -322,7 +310,7 @@ prune_kernel(const uint4* __restrict__ dO, int64_t nvec, uint32_t seed_lo, uint3
         else
           top2_prune_vector<M, SCHEME, F16>(in[it], v, seed_lo, seed_hi, N, part, 0xFFFFFFFFu, y0, y1, y2, y3, km0, km1, km2, km3);
         if (LANES > 1 && v >= nvec) continue;
-        emit_packed<(N <= 2)>(v, y0, y1, y2, y3, km0, km1, km2, km3, dense, values, meta, mask, pitch);
+        emit_packed<(N <= 2)>(v, y0, y1, y2, y3, km0, km1, km2, km3, dense, values, meta, mask);
       }
     }
   }
@@ -332,7 +320,7 @@ prune_kernel(const uint4* __restrict__ dO, int64_t nvec, uint32_t seed_lo, uint3
 // instantiation for both element types.
 template <int M, int N, int SRC>
 cudaError_t launch_select(int scheme, bool f16, const void* dO, int64_t nvec, uint64_t seed, void* dense, void* values,
-                          void* meta, void* mask, OutPitch pitch, cudaStream_t stream, ReluSource src) {
+                          void* meta, void* mask, MetaPitch pitch, cudaStream_t stream, ReluSource src) {
   if (nvec == 0) return cudaSuccess;
   const uint32_t lo = (uint32_t)seed, hi = (uint32_t)(seed >> 32);
   auto launch = [&](auto kernel, bool pairs) {
@@ -363,10 +351,11 @@ cudaError_t launch_prune_src(const void* dO, int64_t rows, int64_t K, int n, int
                              ReluSource src) {
   const bool f16 = dtype == SDGP_FP16;
   const int64_t nvec = rows * (K / 8);
-  OutPitch pitch = {(int)(K / 8), 0};
+  MetaPitch pitch = {(uint32_t)(K / 16), 0};
   if (k_pad != 0 && k_pad != K) {
-    if (k_pad < K || k_pad % 8 != 0 || n > 2) return cudaErrorInvalidValue;  // padded rows exist only for compressed outputs
-    pitch.kpad8 = (int)(k_pad / 8);
+    // padded metadata rows exist only for compressed outputs
+    if (k_pad < K || k_pad % 16 != 0 || K % 16 != 0 || n > 2 || dense || SRC != kPlain) return cudaErrorInvalidValue;
+    pitch.kpad16 = (uint32_t)(k_pad / 16);
   }
   switch (m) {
     case 4:

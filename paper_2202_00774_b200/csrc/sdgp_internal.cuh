@@ -10,9 +10,9 @@ namespace sdgp {
 // Multiprocessors of the current device (148 if it cannot be asked).
 int sm_count();
 
-// k_pad (0 = none): row pitch, in elements, of the compressed outputs. When k_pad > K the extra
-// chunks of every row are written as zero values with the position pair (0,1), so a consumer can
-// treat the row as k_pad channels (used to bring a channel count up to a whole 128-channel block).
+// k_pad (0 = none): row pitch, in elements, of the metadata (compressed outputs only, no dense copy): the extra chunks of every
+// row name the position pair (0,1), so that a reader can take a row as k_pad channels - those past K of zero value, which it supplies
+// itself (TMA reads them as zeros).
 cudaError_t launch_prune(const void* dO, int64_t rows, int64_t K, int n, int m, int scheme,
                          uint64_t seed, void* dense, void* values, void* meta, void* mask,
                          cudaStream_t stream, int64_t k_pad = 0, int dtype = SDGP_BF16);
@@ -50,8 +50,8 @@ cudaError_t launch_scale_weights(const void* W, const float* sums, int64_t K, in
                                  float* scales, cudaStream_t stream);
 
 // Data gradient on the tensor cores (stride 1 or 2). sparse == false: A is dense dL/dO
-// [B,P,Q,Cout]; sparse == true: A is the compressed values [B,P,Q,Cp/2] and meta [B,P,Q,Cp/16]
-// with Cp = Cout rounded up to a multiple of 128 (see launch_prune's k_pad).
+// [B,P,Q,Cout]; sparse == true: A is the compressed values [B,P,Q,Cout/2] and meta [B,P,Q,Cp/16]
+// with Cp = Cout rounded up to a multiple of 128 (see launch_prune's k_pad); values rows are not padded.
 // Wt [Cout,R,S,Cin], dD [B,H,W,Cin]. A fully connected layer is B = H = 1, W = rows, R = S = 1.
 // fused != nullptr: A is the dense dL/dO and the kernel prunes it on the fly (n <= 2).
 struct FusedPrune {
@@ -64,7 +64,7 @@ struct FusedPrune {
 // Fused pruning with the rescaled scheme exists for bf16 only.
 // stored != nullptr: Cin and Cout are the channel counts the kernels tile by (multiples of 64; Wt has that
 // many rows and columns, the extra ones zero) while the tensors in global memory hold fewer channels per
-// pixel: `a` for a dense A (0 = Cout; a compressed A is always padded to whole 128-channel blocks), `d` for dD
+// pixel: `a` for dL/dO, dense or compressed (0 = Cout), `d` for dD
 // (0 = Cin), both multiples of 8. TMA reads the missing channels of A as zeros and clips the stores of dD.
 struct StoredChannels {
   int a;

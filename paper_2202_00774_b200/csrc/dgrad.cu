@@ -160,15 +160,29 @@ int choose_bn(int64_t m_tiles, int channels, int all, int kbc, int Cout, const C
   return best;
 }
 
-// Whole-filter reuse pays when there is more than one tap and strips of 8 x 16 pixels cover the
-// image without much padding.
-bool halo_applies(int H, int W, int taps) {
+// Whole-filter reuse pays when there is more than one tap and strips of 8 x 16 pixels (images at most 8 pixels tall: 8 rows of two
+// images) cover the image without too much padding. How much is too much was measured (two-pass, us, general kernel -> this one): nine
+// taps, 27 x 27 (140 % covered) 34.5 -> 16.8, 13 x 13 (151 %) 49 -> 27.5, 10 x 10 (256 %) 18.6 -> 15.8, 9 x 9 (316 %) 15.6 -> 19.3;
+// two to four taps, 7 x 7 (131 %) 31 -> 37. Pruning inside the general kernel costs so much more that the fused mode takes
+// any image of at least 5 x 5 (9 x 9: 36.7 -> 24.5).
+bool halo_applies(int H, int W, int taps, bool sparse, bool fused) {
   if (taps < 2) return false;
-  if (W == 4 && H >= 3 && H <= 4) return true;  // two images per strip row, four pixel rows of eight images per strip
-  if (W < 8 || (H < 12 && H > 8) || H < 6) return false;
-  const int th = H <= 8 ? 8 : kHaloRows;  // images at most 8 pixels tall: strips of 8 rows of two images
+  // two images per strip row, four pixel rows of eight images per strip. With a sparse A only: fused, it prunes each box S times instead
+  // of R * S times; two-pass it measured the same as the general kernel; the dense twin measured slower there (one tile per CTA
+  // pair: set-up and the single epilogue dominate either way).
+  if (W == 4 && H >= 3 && H <= 4) return sparse;
+  if (W < 5 || H < 5) return false;
+  if (fused) return true;
+  if (taps < 6 && (W < 8 || (H < 12 && H > 8) || H < 6)) return false;
+  const int th = H <= 8 ? 8 : kHaloRows;
   const int64_t covered = (int64_t)((W + 7) / 8 * 8) * ((H + th - 1) / th * th);
-  return covered * 100 <= (int64_t)H * W * 135;
+  return covered * 100 <= (int64_t)H * W * (taps < 6 ? 135 : 260);
+}
+
+// Accumulators (128 rows) that kernel's strips need.
+int64_t halo_strips(int B, int H, int W) {
+  const int th = H <= 4 ? 4 : H <= 8 ? 8 : kHaloRows, tb = kHaloRows / th, per_row = W == 4 ? 2 : 1;
+  return (int64_t)((W + 7) / 8) * ((H + th - 1) / th) * ((B + tb * per_row - 1) / (tb * per_row));
 }
 
 // What pruning costs (measured on a [16384 x 4096] tensor and on 50176 x 1024 rows): clocks of the rows kernel's pruning warps per block of
@@ -254,7 +268,8 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
       p.tiles_b = (B + p.TB - 1) / p.TB;
       const int64_t m_tiles = (int64_t)p.tiles_w * p.tiles_h * p.tiles_b;
       const int all_blocks = (Cout + kb_channels - 1) / kb_channels;
-      const int BN = choose_bn(m_tiles, view.d.channels, all_blocks, kb_channels, Cout, conv_groups);
+      const bool halo = halo_applies(Hs, Ws, p.R * p.S, sparse, fused != nullptr);
+      const int BN = choose_bn(halo ? halo_strips(B, Hs, Ws) : m_tiles, view.d.channels, all_blocks, kb_channels, Cout, conv_groups);
       p.tiles_n = (view.d.channels + BN - 1) / BN;
       if (m_tiles * p.tiles_n > 0x3FFFFFFF) return SDGP_ERR_UNSUPPORTED;
       p.m_tiles = (int)m_tiles;
@@ -280,11 +295,7 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
       view.d.sb = (int64_t)H * W * Cd * 2;
       view.d.aligned32 = ((uintptr_t)dD & 31u) == 0 && Cd % 16 == 0;
       sdgp_status st = SDGP_ERR_UNSUPPORTED;
-      // Images 4 pixels wide take the whole-filter-reuse kernel (column-split mode) with a sparse A: fused, it prunes
-      // each box S times instead of R * S times; two-pass it measured the same as the general kernel; the dense twin
-      // measured slower there (one tile per CTA pair: set-up and the single epilogue dominate either way) and stays
-      // on the general kernel.
-      if (halo_applies(Hs, Ws, p.R * p.S) && (Ws != 4 || sparse)) {
+      if (halo) {
         HaloParams hp = {};
         hp.B = B; hp.H = Hs; hp.W = Ws; hp.Cin = Cin; hp.Cout = Cout;
         hp.R = p.R; hp.S = p.S; hp.pad_h = p.pad_h; hp.pad_w = p.pad_w;

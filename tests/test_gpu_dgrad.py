@@ -721,3 +721,21 @@ def test_linear_pruned_on_the_way(rows, K, N, n, m, scheme):
         check_no_device_error()
         assert_close(to_f64(dD)[pick], *ref)
         assert np.all(flat[rows * N:].cpu().numpy() == 0x5A5A)
+
+
+@pytest.mark.parametrize("B,H,Wd,Cin,Cout,R,pad", [(3, 5, 5, 64, 64, 3, 1), (5, 7, 7, 192, 192, 3, 1), (2, 7, 6, 128, 64, 3, 0), (3, 9, 11, 64, 128, 3, 1),
+                                                   (2, 10, 10, 320, 128, 3, 1), (4, 13, 13, 128, 192, 3, 1), (2, 27, 27, 64, 64, 3, 1), (2, 13, 9, 64, 128, 5, 2)])
+@pytest.mark.parametrize("mode", ["two_pass", "dense", "fused", "fused_random"])
+def test_conv_image_sizes_that_leave_strips_partly_empty(B, H, Wd, Cin, Cout, R, pad, mode):
+    """Odd image sizes and batches on strips of 8 x 16 pixels, last channel blocks of 64, tiles wider than the channels left."""
+    import paper_2202_00774_b200 as sdgp
+    layer = inputs.ConvLayer("t", B, H, Wd, Cin, Cout, R, R, 1, pad)
+    dO, W = inputs.conv_layer_tensors(layer, seed=H + Wd)
+    scheme = oracle.RANDOM if mode == "fused_random" else oracle.MAGNITUDE
+    flags = {"two_pass": sdgp.FLAG_TWO_PASS, "dense": sdgp.FLAG_DENSE}.get(mode, sdgp.FLAG_FUSED)
+    ws = torch.empty(max(16, sdgp.sdgp_workspace_size_conv2d(B, H, Wd, Cin, Cout, R, R, 1, pad)), dtype=torch.uint8, device="cuda")
+    dD = torch.full(layer.dD_shape(), -1, dtype=torch.int16, device="cuda")
+    sdgp.sdgp_dgrad_conv2d(dev16(dO), dev16(W), dD, 1, pad, 2, 4, scheme, 6, workspace=ws, flags=flags)
+    check_no_device_error()
+    src = dO if mode == "dense" else oracle.prune(dO.reshape(-1, Cout), 2, 4, scheme, 6, want=("dense",))["dense"].reshape(dO.shape)
+    assert_close(to_f64(dD), *conv_ref(src, W, H, Wd, 1, pad))

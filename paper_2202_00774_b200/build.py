@@ -14,7 +14,7 @@ LIB = os.path.join(HERE, "libsdgp.so")
 SOURCES = ["prune.cu", "rank.cu", "dgrad.cu", "dgrad_general.cu", "dgrad_halo_sparse.cu", "dgrad_halo_dense.cu",
            "dgrad_halo_fused.cu", "dgrad_rows.cu", "api.cu", "static_scratch.cu", "channel.cu", "grouped.cu"]
 BINDING = os.path.join(HERE, "_sdgp_torch.so")
-BINDING_SOURCE = os.path.join(CSRC, "torch_binding.cpp")
+BINDING_SOURCES = [os.path.join(CSRC, f) for f in ("torch_binding.cpp", "torch_autograd.cpp")]
 HEADERS = ["ptx.cuh", "sdgp_internal.cuh", "prune_core.cuh", "dgrad_common.cuh", "dgrad_general.cuh", "dgrad_halo.cuh",
            "dgrad_halo_params.cuh", "dgrad_prune.cuh", "dgrad_rows.cuh", os.path.join("..", "..", "include", "sdgp.h")]
 
@@ -37,15 +37,16 @@ def needs_build() -> bool:
 
 def build_binding(force: bool = False) -> str:
     """The torch module; needs ``libsdgp.so`` beside it (it finds it through its run path)."""
-    if not force and not _stale(BINDING, [BINDING_SOURCE, os.path.join(HERE, "..", "include", "sdgp.h"), os.path.abspath(__file__)]):
+    if not force and not _stale(BINDING, BINDING_SOURCES + [os.path.join(CSRC, "torch_autograd.h"), os.path.join(CSRC, "sdgp_internal.cuh"),
+                                                            os.path.join(HERE, "..", "include", "sdgp.h"), os.path.abspath(__file__)]):
         return BINDING
     from torch.utils import cpp_extension
     tmp = BINDING + ".%d.tmp" % os.getpid()
     include = [sysconfig.get_paths()["include"]] + cpp_extension.include_paths("cuda")
     libs = cpp_extension.library_paths("cuda")
-    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-o", tmp, BINDING_SOURCE]
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-o", tmp] + BINDING_SOURCES
     cmd += ["-I" + d for d in include] + ["-L" + HERE, "-lsdgp"] + ["-L" + d for d in libs]
-    cmd += ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
+    cmd += ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
     subprocess.check_call(cmd)
     os.replace(tmp, BINDING)
     return BINDING

@@ -38,6 +38,10 @@ cudaError_t launch_maxpool_relu_backward_prune(const void* dYp, const void* act,
                                                void* mask, cudaStream_t stream, int dtype = SDGP_BF16,
                                                const void* skip_pooled = nullptr);
 
+// y [B, H/2, W/2, K] = 2 x 2 max pooling of relu(x), x [B, H, W, K] NHWC (prune.cu); H and W even, K a multiple of 8. A NaN in a window
+// gives NaN.
+cudaError_t launch_relu_maxpool(const void* x, int64_t B, int64_t H, int64_t W, int64_t K, int dtype, void* y, cudaStream_t stream);
+
 // Per-channel reading of the L1 rescale (channel.cu). sums: 2 * K floats (cleared by the call): the
 // column sums of |x| over all rows, then the same over the survivors of the magnitude function.
 cudaError_t launch_channel_sums(const void* dO, int64_t rows, int64_t K, int n, int m, int dtype, float* sums,

@@ -5,9 +5,11 @@
 // tensors are contiguous CUDA tensors, and returns the sdgp_status as an int.
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "../../include/sdgp.h"
+#include "torch_autograd.h"
 
 namespace {
 
@@ -262,6 +264,40 @@ ENTRY(spmm_conv2d) {  // values, meta, W, dD, stride, pad, dtype
   });
 }
 
+// Differentiable layers: x, weight, then `integers` numbers, the last of them a seed.
+template <class F>
+PyObject* layer(PyObject* const* args, Py_ssize_t nargs, int integers, F call) {
+  HANDLE_TH_ERRORS
+  Args in(args, nargs, 2 + integers);
+  at::Tensor t[2];
+  for (int k = 0; in.ok && k < 2; ++k, ++in.a) {
+    if (!THPVariable_Check(*in.a)) {
+      PyErr_SetString(PyExc_TypeError, "input and weight must be torch tensors");
+      return nullptr;
+    }
+    t[k] = THPVariable_Unpack(*in.a);
+  }
+  std::vector<int64_t> numbers;
+  for (int k = 0; k < integers; ++k) numbers.push_back(k + 1 < integers ? (int64_t)in.i32() : (int64_t)in.u64());
+  if (!in.ok) return nullptr;
+  at::Tensor y;
+  {
+    struct NoGil {
+      PyThreadState* state = PyEval_SaveThread();
+      ~NoGil() { PyEval_RestoreThread(state); }
+    } no_gil;
+    y = call(t[0], t[1], std::move(numbers));
+  }
+  return THPVariable_Wrap(std::move(y));
+  END_HANDLE_TH_ERRORS
+}
+ENTRY(linear_layer) {  // x, weight, n, m, scheme, seed
+  return layer(args, nargs, 4, sdgp_torch::linear);
+}
+ENTRY(conv2d_layer) {  // x, weight, stride, padding, kind, n, m, scheme, seed
+  return layer(args, nargs, 7, sdgp_torch::conv2d);
+}
+
 ENTRY(workspace_size_linear) {  // rows, K, N, flags
   Args in(args, nargs, 4);
   const int64_t rows = in.i64(), K = in.i64(), N = in.i64();
@@ -295,7 +331,8 @@ PyObject* guarded(PyObject* self, PyObject* const* args, Py_ssize_t nargs) {
 #define METHOD(name) {#name, (PyCFunction)(void (*)(void))guarded<name>, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {METHOD(prune), METHOD(relu_backward_prune), METHOD(maxpool_relu_backward_prune), METHOD(dgrad_linear),
                          METHOD(dgrad_linear_static), METHOD(dgrad_conv2d), METHOD(spmm_linear), METHOD(spmm_conv2d),
-                         METHOD(workspace_size_linear), METHOD(workspace_size_conv2d), {nullptr, nullptr, 0, nullptr}};
+                         METHOD(workspace_size_linear), METHOD(workspace_size_conv2d), METHOD(linear_layer),
+                         METHOD(conv2d_layer), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_sdgp_torch", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

@@ -99,3 +99,42 @@ def test_conv_relu_layer_backward_uses_the_producer(pool, Cout, n, m):
     dO = torch.from_numpy(inputs.bf16_bits_to_f32(ref["grad"].reshape(B, H, H, Cout))).cuda().permute(0, 3, 1, 2)
     ref_w = torch.nn.grad.conv2d_weight(x.detach().float(), w.shape, dO.contiguous(), 1, 1).cpu().numpy()
     assert rel_fro(w.grad.float().cpu().numpy(), ref_w) <= 1e-2
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("pool,shape", [(True, (2, 64, 128, 6, 10)), (True, (3, 64, 64, 8, 8)), (False, (2, 128, 64, 7, 9))])
+def test_conv_relu_pool_matches_the_separate_operators(dtype, pool, shape):
+    """Forward values (ReLU and pooling in one pass, a NaN in the input included) and both gradients with n = m, against torch's
+    own operators chained under autograd; the operands are 16-bit, sums fp32, so one rounding (2^-8 / 2^-11) with room for the order."""
+    from paper_2202_00774_b200 import autograd as sa
+    B, Cin, Cout, H, W = shape
+    g = torch.Generator(device="cuda").manual_seed(H * W)
+    make = lambda *s: torch.randn(s, generator=g, device="cuda").to(dtype)   # noqa: E731
+    x = make(B, Cin, H, W).contiguous(memory_format=torch.channels_last)
+    w = (make(Cout, Cin, 3, 3) / 24).contiguous(memory_format=torch.channels_last)
+    if pool:
+        x[0, 0, 1, 1] = float("nan")
+    x.requires_grad_(), w.requires_grad_()
+    y = sa.sdgp_conv2d_relu(x, w, 1, 1, pool=pool, n=4, m=4)
+    ref = torch.relu(torch.nn.functional.conv2d(x, w, None, 1, 1))
+    ref = torch.nn.functional.max_pool2d(ref, 2) if pool else ref
+    assert torch.equal(torch.isnan(y), torch.isnan(ref)) and torch.equal(torch.nan_to_num(y, 0.0), torch.nan_to_num(ref, 0.0))
+    if pool:
+        return   # (where a NaN wins a window the gradients differ: a NaN passes nothing here)
+    dY = make(*y.shape)
+    got, want = torch.autograd.grad(y, (x, w), dY), torch.autograd.grad(ref, (x, w), dY)
+    for a, b in zip(got, want):
+        assert rel_fro(a.double().cpu().numpy(), b.double().cpu().numpy()) <= 5e-3
+
+
+def test_layers_raise_what_the_binding_raises():
+    from paper_2202_00774_b200 import autograd as sa
+    import paper_2202_00774_b200 as sdgp
+    x = torch.randn(64, 96, device="cuda", dtype=torch.bfloat16, requires_grad=True)   # 96: not a multiple of 64
+    w = torch.randn(64, 96, device="cuda", dtype=torch.bfloat16, requires_grad=True)
+    with pytest.raises(sdgp.SdgpError) as e:
+        sa.sdgp_linear(x, w).sum().backward()
+    assert e.value.status == 2
+    with pytest.raises(TypeError):
+        a = torch.randn(64, 64, device="cuda", requires_grad=True)
+        sa.sdgp_linear(a, a.detach()).sum().backward()

@@ -249,11 +249,8 @@ sdgp_status sdgp_dgrad_conv2d_typed(const void* dO, const void* W, void* dD, int
     if (((uintptr_t)workspace & 255u) != 0) return SDGP_ERR_ALIGNMENT;
     float* floats = (float*)((uint8_t*)workspace + c.bytes);       // [0,K) factors, [K,3K) the two sums
     void* w_scaled = (uint8_t*)floats + channel_floats_bytes(Cout);
-    if (sdgp::launch_channel_sums(dO, rows, Cout, n, m, dt, floats + Cout, s) != cudaSuccess) return SDGP_ERR_CUDA;
+    if (sdgp::launch_prune_sums(dO, rows, Cout, n, m, dt, floats + Cout, c.values, c.meta, Cpad, s) != cudaSuccess) return SDGP_ERR_CUDA;
     if (sdgp::launch_scale_weights(W, floats + Cout, Cout, w_row, dt, w_scaled, floats, s) != cudaSuccess) return SDGP_ERR_CUDA;
-    if (sdgp::launch_prune(dO, rows, Cout, n, m, SDGP_MAGNITUDE, seed, nullptr, c.values, c.meta, nullptr, s, Cpad, dt) !=
-        cudaSuccess)
-      return SDGP_ERR_CUDA;
     return sdgp::launch_dgrad(true, c.values, c.meta, w_scaled, dD, B, H, Wd, Cin, Cout, R, S, stride, pad, s, nullptr, dt);
   }
   if (!workspace || workspace_bytes < c.bytes) return SDGP_ERR_WORKSPACE;

@@ -6,8 +6,8 @@
 // (dD = (A diag(s)) W = A (diag(s) W)): the pruned tensor itself is never rescaled, and the sparse
 // contraction runs unchanged on the scaled copy of W.
 //
-// Cost: one more read of dL/dO (column sums cannot be known before the whole tensor has been seen)
-// and one pass over W.
+// The sums come out of the pass that prunes (prune_sums_kernel), so the mode costs one pass over W more than plain pruning; the sums
+// alone, for any n, are channel_sums_kernel's.
 #include "prune_core.cuh"
 #include "sdgp_internal.cuh"
 
@@ -110,6 +110,112 @@ channel_sums_kernel(const uint4* __restrict__ dO, int64_t rows, int K, int n, fl
   }
 }
 
+// Algorithm 1 (magnitude function, n <= 2) in compressed form and the column sums in one read of dO. A thread owns 16 channels (a pair
+// of vectors) and walks down the rows, its 32 partial sums in registers; a block adds up its threads' and adds to each global sum once. Bound: HBM on large tensors (3.1 B per element). Against a pass
+// for the sums and a pass that prunes: 16384 x 4096 at 2:4 75 -> 43 us for the two.
+constexpr int kSumRows = 2;  // rows whose loads are in flight together
+template <int M, int N, bool F16>
+__global__ void __launch_bounds__(kChThreads, 2)
+prune_sums_kernel(const uint4* __restrict__ dO, int64_t rows, int pairs, uint4* __restrict__ values, uint16_t* __restrict__ meta,
+                  int meta_pitch, float* __restrict__ sums, int64_t rows_per_block, bool aligned32) {
+  __shared__ float sh[2][kChThreads * 16];
+  const int cols = pairs < kChThreads ? pairs : kChThreads;  // columns side by side; a multiple of two where groups span two threads
+  const int lanes = kChThreads / cols;                       // rows side by side
+  const int lane = threadIdx.x / cols, cc = threadIdx.x - lane * cols;
+  const int col = blockIdx.y * cols + cc;
+  const bool mine = lane < lanes && col < pairs;
+  float t[16], s[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) t[i] = s[i] = 0.0f;
+  const int64_t row_end = (blockIdx.x + 1) * rows_per_block < rows ? (blockIdx.x + 1) * rows_per_block : rows;
+  for (int64_t r0 = blockIdx.x * rows_per_block; r0 < row_end; r0 += kSumRows * lanes) {  // (the same trips for all threads)
+    uint4 wa[kSumRows], wb[kSumRows];
+#pragma unroll
+    for (int u = 0; u < kSumRows; ++u) {
+      const int64_t r = r0 + u * lanes + lane;
+      wa[u] = wb[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (mine && r < row_end) load_pair(dO + 2 * (r * pairs + col), aligned32, wa[u], wb[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kSumRows; ++u) {
+      const int64_t r = r0 + u * lanes + lane;
+      uint4 out;
+      uint32_t pa, pb;
+      KeepFlags ka, kb;
+      compress_pair<M, N, SDGP_MAGNITUDE, F16>(wa[u], wb[u], 0, 0u, 0u, M == 32 ? (int)(threadIdx.x & 1) : 0, 0xFFFFFFFFu, out, pa, pb, ka, kb);
+      if (mine && r < row_end) {
+        values[r * pairs + col] = out;
+        uint16_t* m = meta + r * meta_pitch + col;
+        *m = (uint16_t)prmt(pa, pb, 0x0073);
+        if (col == pairs - 1)
+          for (int pad = 1; pad <= meta_pitch - pairs; ++pad) m[pad] = (uint16_t)0x4444;  // rows of whole 16 bytes, position pair (0, 1)
+      }
+      auto add = [&](const uint4& w, const KeepFlags& k, int base) {
+        // keep masks of the words (elements 2q, 2q + 1) from the lane-paired flags (elements i, i + 4)
+        const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+        const uint32_t km[4] = {prmt(k.k0, k.k1, 0xDD99), prmt(k.k2, k.k3, 0xDD99), prmt(k.k0, k.k1, 0xFFBB), prmt(k.k2, k.k3, 0xFFBB)};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          t[base + 2 * q] += lane_lo_abs<F16>(x[q]);
+          t[base + 2 * q + 1] += lane_hi_abs<F16>(x[q]);
+          s[base + 2 * q] += lane_lo_abs<F16>(x[q] & km[q]);
+          s[base + 2 * q + 1] += lane_hi_abs<F16>(x[q] & km[q]);
+        }
+      };
+      add(wa[u], ka, 0);
+      add(wb[u], kb, 8);
+    }
+  }
+  // the rows side by side: every thread's sums in shared memory, one thread per channel adds them up (shared-memory float atomics
+  // are compare-and-swap loops)
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    sh[0][i * kChThreads + threadIdx.x] = t[i];
+    sh[1][i * kChThreads + threadIdx.x] = s[i];
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; lanes > 1 && j < cols * 16; j += kChThreads) {
+    const int i = j / cols, at = i * kChThreads + (j - i * cols);
+    float st = sh[0][at], ss = sh[1][at];
+    for (int l = 1; l < lanes; ++l) {
+      st += sh[0][at + l * cols];
+      ss += sh[1][at + l * cols];
+    }
+    sh[0][at] = st;
+    sh[1][at] = ss;
+  }
+  __syncthreads();
+  const int64_t K = (int64_t)pairs * 16;
+  for (int j = threadIdx.x; j < cols * 16; j += kChThreads) {
+    const int64_t k = (int64_t)blockIdx.y * cols * 16 + j;
+    if (k < K) {
+      atomicAdd(sums + k, sh[0][(j & 15) * kChThreads + (j >> 4)]);
+      atomicAdd(sums + K + k, sh[1][(j & 15) * kChThreads + (j >> 4)]);
+    }
+  }
+}
+
+template <int M, int N>
+cudaError_t launch_prune_sums_n(bool f16, const void* dO, int64_t rows, int K, float* sums, void* values, void* meta, int k_pad,
+                                cudaStream_t stream) {
+  const int pairs = K / 16, cols = pairs < kChThreads ? pairs : kChThreads, lanes = kChThreads / cols;
+  const unsigned by = (unsigned)((pairs + cols - 1) / cols);
+  const int64_t step = (int64_t)lanes * kSumRows, sms = sm_count();
+  // blocks: two per SM at most (all resident), so that the closing adds stay few; at least two steps of rows each
+  int64_t blocks = (rows + 2 * step - 1) / (2 * step);
+  const int64_t most = (2 * sms + by - 1) / by;
+  if (blocks > most) blocks = most;
+  const int64_t rows_per_block = ((rows + blocks - 1) / blocks + step - 1) / step * step;
+  blocks = (rows + rows_per_block - 1) / rows_per_block;
+  auto launch = [&](auto kernel) {
+    kernel<<<dim3((unsigned)blocks, by), kChThreads, 0, stream>>>((const uint4*)dO, rows, pairs, (uint4*)values, (uint16_t*)meta, k_pad / 16,
+                                                                  sums, rows_per_block, ((uintptr_t)dO & 31u) == 0);
+  };
+  if (f16) launch(prune_sums_kernel<M, N, true>);
+  else launch(prune_sums_kernel<M, N, false>);
+  return cudaGetLastError();
+}
+
 __device__ __forceinline__ float channel_scale(const float* sums, int K, int k) {
   const float t = sums[k], s = sums[K + k];
   return s == 0.0f ? 1.0f : __fdiv_rn(t, s);
@@ -171,6 +277,26 @@ cudaError_t launch_channel_sums(const void* dO, int64_t rows, int64_t K, int n, 
     case 32: return launch_sums_m<32>(f16, dO, rows, (int)K, n, sums, stream);
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t launch_prune_sums(const void* dO, int64_t rows, int64_t K, int n, int m, int dtype, float* sums, void* values, void* meta,
+                              int64_t k_pad, cudaStream_t stream) {
+  if (K > 0x7FFFFFFF || K % 16 != 0 || K % m != 0 || k_pad < K || k_pad % 16 != 0 || n < 1 || n > 2) return cudaErrorInvalidValue;
+  if (cudaMemsetAsync(sums, 0, (size_t)K * 2 * sizeof(float), stream) != cudaSuccess) return cudaErrorUnknown;
+  if (rows == 0) return cudaSuccess;
+  const bool f16 = dtype == SDGP_FP16;
+#define SDGP_CASE(M)                                                                                                \
+  case M:                                                                                                           \
+    return n == 1 ? launch_prune_sums_n<M, 1>(f16, dO, rows, (int)K, sums, values, meta, (int)k_pad, stream)        \
+                  : launch_prune_sums_n<M, 2>(f16, dO, rows, (int)K, sums, values, meta, (int)k_pad, stream);
+  switch (m) {
+    SDGP_CASE(4)
+    SDGP_CASE(8)
+    SDGP_CASE(16)
+    SDGP_CASE(32)
+    default: return cudaErrorInvalidValue;
+  }
+#undef SDGP_CASE
 }
 
 cudaError_t launch_channel_scales(const float* sums, int64_t K, float* scales, cudaStream_t stream) {

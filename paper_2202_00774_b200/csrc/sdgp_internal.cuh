@@ -46,6 +46,9 @@ cudaError_t launch_relu_maxpool(const void* x, int64_t B, int64_t H, int64_t W, 
 // column sums of |x| over all rows, then the same over the survivors of the magnitude function.
 cudaError_t launch_channel_sums(const void* dO, int64_t rows, int64_t K, int n, int m, int dtype, float* sums,
                                 cudaStream_t stream);
+// Both at once for n <= 2: launch_channel_sums' sums and launch_prune's compressed form under the magnitude function, in one read of dO.
+cudaError_t launch_prune_sums(const void* dO, int64_t rows, int64_t K, int n, int m, int dtype, float* sums, void* values, void* meta,
+                              int64_t k_pad, cudaStream_t stream);
 // scales[k] = sums[k] / sums[K + k] (1 where the denominator is 0)
 cudaError_t launch_channel_scales(const float* sums, int64_t K, float* scales, cudaStream_t stream);
 // Wout[k, :] = W[k, :] * scale[k] rounded to the element type (row_elems elements per row, a multiple of 8); also

@@ -133,7 +133,7 @@ __device__ __forceinline__ void read_slab(uint32_t taddr, uint32_t (&packed)[32]
 }
 
 // A warp's 32 rows (pixels) of a 128-row x BN accumulator to global memory. The four epilogue warps share nothing: no barrier
-// between them and no shared tile. Against one staging tile for all four, two barriers per slab and one TMA store of the whole
+// between them and no shared tile (but in store_patch). Against one staging tile for all four, two barriers per slab and one TMA store of the whole
 // patch, a small layer ends 1-2 us earlier (256 x 512 . 512 x 256, dense: 7.6 -> 5.8 us per call).
 //
 // store_rows: straight from registers. Each thread writes whole 32-byte sectors of its own row and L2 puts the lines together; the
@@ -196,6 +196,39 @@ __device__ __forceinline__ void store_box(uint32_t taddr, uint8_t* stage, const 
     }
     ++chunk;
     if (last) break;
+  }
+}
+
+// store_patch: the four warps together, a 128-row slab of 64 columns through one 16 KB tile (twice where there is room) and one TMA box of
+// the whole patch, clipped at the edges of dD. Two barriers of the four warps a slab, but a quarter of store_box's requests and of the
+// write requests that rows make at L2: for launches whose stores set the pace (plan_halo()).
+template <int BN, bool FIVE>
+__device__ __forceinline__ void store_patch(uint32_t taddr, uint8_t* staging, int bufs, const CUtensorMap* tmD, int n0, int c1, int c2, int c3,
+                                            int c4, bool in_range, uint32_t& chunk, uint64_t* first_slab_read, bool f16) {
+  const int row = ((threadIdx.x >> 5) & 3) * 32 + (threadIdx.x & 31);
+  const bool issuer = row == 0;
+#pragma unroll 1
+  for (int c0 = 0; c0 < BN; c0 += 64, ++chunk) {
+    uint32_t packed[32];
+    read_slab(taddr + (uint32_t)c0, packed, c0 == 0 ? first_slab_read : nullptr, nullptr, f16);
+    uint8_t* buf = staging + (bufs == 2 ? chunk & 1u : 0u) * 4 * kSlabBytes;
+    if (issuer) {  // the store that last used this buffer has read it
+      if (bufs == 2) ptx::bulk_wait_group_read<1>();
+      else ptx::bulk_wait_group_read<0>();
+    }
+    ptx::named_bar_sync(1, 128);
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      *(uint4*)(buf + row * 128 + ((c ^ (row & 7)) << 4)) =
+          make_uint4(packed[4 * c], packed[4 * c + 1], packed[4 * c + 2], packed[4 * c + 3]);
+    ptx::fence_proxy_async_smem();
+    ptx::named_bar_sync(1, 128);
+    if (issuer) {
+      if (!in_range) {
+      } else if (FIVE) ptx::tma_store_5d(tmD, buf, n0 + c0, c1, c2, c3, c4);
+      else ptx::tma_store_4d(tmD, buf, n0 + c0, c1, c2, c3);
+      ptx::bulk_commit_group();  // (an empty group where nothing is stored: the waits count groups)
+    }
   }
 }
 

@@ -302,7 +302,9 @@ dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         ptx::tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
         uint32_t accumulate = 0u;
-        const int cb_last = p.k_last - first_k_block(p, (first_pair + lt * pair_stride) % p.tiles_n * BN, C::kKB);
+        // (this thread's instructions are the MMAs' issue rate: no division where every block is whole or every tile sees all blocks)
+        int cb_last = p.last_mmas == 4 ? -1 : p.k_last;
+        if (p.last_mmas != 4 && p.diag_cin_g != 0) cb_last -= first_k_block(p, (first_pair + lt * pair_stride) % p.tiles_n * BN, C::kKB);
         int r_single = 0, s = 0;
         for (int g = 0; alive && g < groups; ++g) {
           for (int cb = 0; cb < p.k_blocks; ++cb) {
@@ -314,7 +316,7 @@ dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
               for (int u = 0; u < p.rr; ++u)
                 ptx::tc_cp_128x128b_pair(e_col + 4u * u, ((uint64_t)e_hi << 32) | (e_lo + (uint32_t)(u * (kEHwBytes / 16))));
             }
-            // MMAS: MMAs of the channel block
+            // MMAS: MMAs of the channel block, 0: `mmas` of them (one form for every partial block keeps the loop's code small)
             auto issue = [&](auto mmas_tag) {
               constexpr int MMAS = decltype(mmas_tag)::value;
               for (int u = 0; u < p.rr; ++u) {
@@ -324,7 +326,8 @@ dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                 const uint32_t b_u = p.w_resident ? w_lo0 + (uint32_t)((r * p.S + s) * p.k_blocks + cb) * kTapB16
                                                   : b_lo + (uint32_t)u * kTapB16;
 #pragma unroll
-                for (int q = 0; q < MMAS; ++q) {
+                for (int q = 0; q < (MMAS ? MMAS : 4); ++q) {
+                  if (!MMAS && q >= mmas) break;
                   // A: 32 bytes of a 128-byte swizzled row per MMA; B: 16 (dense) or 32 (sparse) rows
                   const uint64_t a_q = ((uint64_t)a_hi << 32) | (a_u + (uint32_t)(q * 2));
                   const uint64_t b_q = ((uint64_t)b_hi << 32) | (b_u + (uint32_t)q * kBStep);
@@ -338,9 +341,7 @@ dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
               }
             };
             if (mmas == 4) issue(std::integral_constant<int, 4>{});
-            else if (mmas == 3) issue(std::integral_constant<int, 3>{});
-            else if (mmas == 2) issue(std::integral_constant<int, 2>{});
-            else issue(std::integral_constant<int, 1>{});
+            else issue(std::integral_constant<int, 0>{});
             ptx::tc_commit_pair(&empty[st], 3);
             if (++st == STAGES) { st = 0; ph ^= 1u; a_lo = a_lo0; b_lo = b_lo0; e_lo = e_lo0; mcol = 0; }
             else { a_lo += a_stage16; b_lo += b_stage16; e_lo += e_stage16; mcol += slot_cols; }

@@ -36,7 +36,9 @@ constexpr int kHaloAStages = 4;  // at most: A stages in use are p.a_stages = 2,
 constexpr int kPruneWarps = 18;
 constexpr int kThreadsHaloFused = 24 * 32;
 
-template <bool SPARSE, int BN, int NT, bool FUSED>
+// PATCH (not fused): strips leave as one TMA box each (store_patch), else as rows; plan_halo() has the rule. Two kernels, so that
+// neither carries the other's code.
+template <bool SPARSE, int BN, int NT, bool FUSED, bool PATCH>
 __global__ void __launch_bounds__(FUSED ? kThreadsHaloFused : kThreadsGemm, 1)
 dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmE,
                   const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmD,
@@ -90,6 +92,7 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   if (warp == 0 && lane == 0) {
     ptx::prefetch_tensormap(&tmA);
     ptx::prefetch_tensormap(&tmB);
+    if (PATCH) ptx::prefetch_tensormap(&tmD);
     if (SPARSE) ptx::prefetch_tensormap(&tmE);
   }
   if (warp == 1) {
@@ -256,8 +259,10 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * set_cols);
         const uint32_t strips = strip_mask(lt);
         const bool all_strips = strips == ((1u << NT) - 1u);
+        // (this warp's instructions are the MMAs' issue rate: one form for whole blocks, one for the rest, no division for whole ones)
+        const bool partial = p.last_mmas != 4;
         int kb0 = 0;
-        if (p.diag_cin_g != 0) {
+        if (partial && p.diag_cin_g != 0) {
           int n0, w0, h0, b0;
           locate(first_pair + lt * pair_stride, n0, w0, h0, b0);
           kb0 = first_k_block(p, n0, C::kKB);
@@ -266,7 +271,7 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         for (int ku = 0; alive && ku < p.k_uses; ++ku) {
           if (!wait_all(&a_full[ast], aph, 0x300u + ast)) { alive = false; break; }
           if (SPARSE && !FUSED && !wait_all(&meta_ready[ast], aph, 0x340u + ast)) { alive = false; break; }
-          const int mmas = kb0 + ku / p.ss == p.k_last ? p.last_mmas : 4;
+          const int mmas = (partial && kb0 + ku / p.ss == p.k_last) ? p.last_mmas : 4;
           uint32_t a_lo = a_lo0 + (uint32_t)ast * a_stage16 + a_first16;
           int s = p.sb, dr = p.R - 1;
           const uint32_t e_stage = e_lo0 + (uint32_t)ast * e_stage16;
@@ -303,7 +308,6 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             };
             if (leader) {
               if (all_strips && mmas == 4) issue_tap(std::integral_constant<int, 4>{});
-              else if (all_strips && mmas == 2) issue_tap(std::integral_constant<int, 2>{});
               else issue_tap(std::integral_constant<int, 0>{});
               ptx::tc_commit_pair(&w_empty[wst], 3);
             }
@@ -597,7 +601,9 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       int n0, w0, h0, b0;
       const bool in_range = locate(first_pair + lt * pair_stride, n0, w0, h0, b0);
       const uint32_t strips = strip_mask(lt);
-      if (!ptx::mbar_wait<kIdleWaitNs>(&acc_full[acc], cph, err, 0x600u + acc)) break;
+      // (patches: the four warps stay or leave together, they meet at a named barrier in every slab)
+      const bool ready = ptx::mbar_wait<kIdleWaitNs>(&acc_full[acc], cph, err, 0x600u + acc);
+      if (PATCH ? !ptx::named_bar_all(1, 128, ready) : !ready) break;
       ptx::tc_fence_after_sync();
 #pragma unroll
       for (int j = 0; j < NT; ++j) {
@@ -612,6 +618,16 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                                      p.d.channels - n0, first_slab_read, released, p.f16 != 0, p.out_bufs, chunk);
           else store_box<BN>(taddr, sOut + q * p.out_bufs * kSlabBytes, &tmD, false, n0, w0 + 8 * j, b0, hq, 0, strip_live && w0 + 8 * j < p.W,
                              p.d.channels - n0, first_slab_read, released, p.f16 != 0, p.out_bufs, chunk);
+        } else if constexpr (PATCH) {
+          if (p.split) store_patch<BN, true>(taddr, sOut, p.out_bufs, &tmD, n0, 0, 2 * j, b0 / p.img_per_row, h0, strip_live, chunk,
+                                             first_slab_read, p.f16 != 0);
+          else store_patch<BN, false>(taddr, sOut, p.out_bufs, &tmD, n0, w0 + 8 * j, b0, h0, 0, strip_live && w0 + 8 * j < p.W, chunk,
+                                      first_slab_read, p.f16 != 0);
+          if (released != nullptr) {
+            ptx::tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive_cluster(released, 0);
+          }
         } else {
           const int w = w0 + dw + (p.split ? 0 : 8 * j), h = h0 + dh, b = b0 + db + (p.split ? 2 * j : 0);
           const bool inside = strip_live && w < p.W && h < p.H && b < p.B;
@@ -622,7 +638,7 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       if (++acc == 2) { acc = 0; cph ^= 1u; }
     }
     // the staging rows have been read; the writes themselves complete with the grid (whoever depends on dD waits for that)
-    if (FUSED && lane == 0) ptx::bulk_wait_group_read<0>();
+    if ((FUSED || PATCH) && lane == 0) ptx::bulk_wait_group_read<0>();
   }
 
   __syncwarp();
@@ -669,18 +685,33 @@ bool plan_halo(HaloParams* p, int nt) {
     p->pairs1 = (p->tb == 1 && p->R > 1) ? 8 + ((p->R - 2) >> 1) : 0;
     p->m0_bytes = SPARSE ? p->pairs0 * 2 * p->pitch * 16 : 0;
     p->meta_bytes = SPARSE ? round_up((p->pairs0 + p->pairs1) * 2 * p->pitch * 16, 128) : 0;
+    p->sets_w = p->split ? 1 : (p->W + 8 * nt - 1) / (8 * nt);
+    p->tiles_h = (p->H + p->th - 1) / p->th;
+    const int tile_imgs = p->tb * p->img_per_row;  // images of one tile set
+    const int64_t m_sets = (int64_t)p->sets_w * p->tiles_h * ((p->B + tile_imgs - 1) / tile_imgs);
+    if (m_sets * p->tiles_n > 0x3FFFFFFF) return false;
+    p->m_sets = (int)m_sets;
+    p->pair_tiles = (int)((m_sets + 1) / 2) * p->tiles_n;
+    // Stride 2 stores boxes: its classes have few taps, so that the stores set the pace, and dD's pixels are not neighbours. 128 -> 128
+    // channels, 3 x 3 stride 2 at 56 x 56, batch 256: 2.29 M write requests at L2 a class as rows, 0.60 M as boxes; the four classes 89 us
+    // -> 83. Stride 1 keeps the rows (128 -> 64 channels at 32 x 32, batch 512, prune kernel included: 82 us, as boxes 88).
+    p->patch_store = (!FUSED && p->r_step == 2) ? 1 : 0;
     // A ring: two stages; four where a box feeds few taps (column-split mode: R taps per box), so that the loads
     // run further ahead of the MMAs, if that still leaves three W stages
     p->a_stages = 2;
     const int per_a = p->a_bytes + p->eraw_bytes + p->meta_bytes;
-    if (p->split && (budget - 4 * per_a - 1024 - (FUSED ? 4 * kSlabBytes : 0)) / p->w_bytes >= 3) p->a_stages = 4;
+    if (p->split && (budget - 4 * per_a - 1024 - ((FUSED || p->patch_store) ? 4 * kSlabBytes : 0)) / p->w_bytes >= 3) p->a_stages = 4;
     p->a_shift = p->a_stages == 4 ? 2 : 1;
     const int fixed = p->a_stages * per_a + 1024;
-    p->out_bufs = FUSED ? 2 : 0;  // epilogue staging
+    p->out_bufs = (FUSED || p->patch_store) ? 2 : 0;  // epilogue staging
     int w_stages = (budget - fixed - 4 * p->out_bufs * kSlabBytes) / p->w_bytes;
-    if (FUSED && w_stages < 4) {
+    if (p->out_bufs == 2 && w_stages < 4) {
       p->out_bufs = 1;
       w_stages = (budget - fixed - 4 * kSlabBytes) / p->w_bytes;
+    }
+    if (p->patch_store && w_stages < 3) {
+      p->patch_store = p->out_bufs = 0;
+      w_stages = (budget - fixed) / p->w_bytes;
     }
     if (w_stages > kMaxStages) w_stages = kMaxStages;
     p->meta_shared = 0;
@@ -706,8 +737,6 @@ bool plan_halo(HaloParams* p, int nt) {
     p->off_bar = p->off_out + 4 * p->out_bufs * kSlabBytes;
     p->smem_bytes = p->off_bar + 512 + 1024;
     if (p->smem_bytes > kSmemLimit) return false;
-    p->sets_w = p->split ? 1 : (p->W + 8 * nt - 1) / (8 * nt);
-    p->tiles_h = (p->H + p->th - 1) / p->th;
     if (FUSED && p->sets_w == 1 && p->tiles_h == 1 && p->a_bytes % 16 == 0 && p->meta_bytes % 16 == 0) {
       // Box pixel row 0 is dL/dO row p0 and box column 0 is dL/dO column q0 (every tile set starts at h0 = w0 = 0); the
       // rows and columns of the box that lie inside dL/dO's P x Q pixels are the same for every box.
@@ -723,11 +752,6 @@ bool plan_halo(HaloParams* p, int nt) {
         p->units_per_box = (row_hi - row_lo) * p->tb * nt;
       }
     }
-    const int tile_imgs = p->tb * p->img_per_row;  // images of one tile set
-    const int64_t m_sets = (int64_t)p->sets_w * p->tiles_h * ((p->B + tile_imgs - 1) / tile_imgs);
-    if (m_sets * p->tiles_n > 0x3FFFFFFF) return false;
-    p->m_sets = (int)m_sets;
-    p->pair_tiles = (int)((m_sets + 1) / 2) * p->tiles_n;
     p->mg_tiles_n = div_magic((uint32_t)p->tiles_n);
     p->mg_sets_w = div_magic((uint32_t)p->sets_w);
     p->mg_tiles_h = div_magic((uint32_t)p->tiles_h);
@@ -797,17 +821,22 @@ sdgp_status launch_halo_nt(const void* A, const void* meta, const void* Wt, cons
       return SDGP_ERR_CUDA;
   }
   tmD = tmA;
-  if (FUSED) {
-    // dD, one warp's part of a strip per store: 8 pixel columns (column-split mode: the 4 columns of two neighbouring images)
+  if (FUSED || p.patch_store) {
+    // dD, a strip (fused: one warp's quarter of it) per store: 8 pixel columns (column-split mode: the 4 columns of two neighbouring images)
     if (!encode_nhwc(&tmD, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, view.d.base, (uint64_t)view.d.channels, (uint64_t)p.W, (uint64_t)p.H,
                      (uint64_t)p.B, (uint64_t)view.d.sw, (uint64_t)view.d.sh, (uint64_t)view.d.sb, 64, (uint32_t)(p.split ? 4 : 8), 2,
-                     (uint32_t)p.tb, (uint32_t)(4 / p.tb), CU_TENSOR_MAP_SWIZZLE_128B))
+                     (uint32_t)p.tb, (uint32_t)(FUSED ? 4 / p.tb : p.th), CU_TENSOR_MAP_SWIZZLE_128B))
       return SDGP_ERR_CUDA;
   }
-  static bool configured[kMaxDevices] = {};
-  auto kernel = dgrad_halo_kernel<SPARSE, BN, NT, FUSED>;
-  if (!configure_once(kernel, configured)) return SDGP_ERR_CUDA;
-  return launch_pairs(kernel, pairs_for(p.units), FUSED ? kThreadsHaloFused : kThreadsGemm, p.smem_bytes, stream, tmA, tmE, tmB, tmD, p);
+  auto launch = [&](auto patch_tag) -> sdgp_status {
+    static bool configured[kMaxDevices] = {};
+    auto kernel = dgrad_halo_kernel<SPARSE, BN, NT, FUSED, decltype(patch_tag)::value>;
+    if (!configure_once(kernel, configured)) return SDGP_ERR_CUDA;
+    return launch_pairs(kernel, pairs_for(p.units), FUSED ? kThreadsHaloFused : kThreadsGemm, p.smem_bytes, stream, tmA, tmE, tmB, tmD, p);
+  };
+  if constexpr (!FUSED)
+    if (p.patch_store) return launch(std::true_type{});
+  return launch(std::false_type{});
 }
 
 // Two strips per CTA where the accumulators of two tile sets fit TMEM, else one.

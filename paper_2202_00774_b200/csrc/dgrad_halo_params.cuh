@@ -51,6 +51,7 @@ struct HaloParams {
   int static_pad, units_per_box, unit_row0, unit_col0;
   int w_stages;
   int meta_col, meta_shared, out_bufs;
+  int patch_store;         // not fused: strips are stored as TMA boxes by the four epilogue warps together (else rows)
   int a_bytes, eraw_bytes, w_bytes;  // per stage
   // Position metadata of an A box in the order the tensor core wants, stored ONCE per box and shared by every
   // tap: "master" pi (pi = 0, 1) pairs box rows (pi + 2m, pi + 2m + 1); its 16-byte line ((2m + e) * pitch + x)

@@ -73,7 +73,7 @@ def layer_inputs(l, workload, seed, dtype="bf16"):
 # resnet9 two-pass step, from the ncu capture summarised in profiles/traffic_dgrad_sparse_resnet9.md,
 # and the hash of the kernel sources it was taken with (the figure is dropped once they change).
 NCU_TRAFFIC = {"workload": "resnet9", "mode": "two_pass", "bytes_per_step": 213.0e6, "sources_sha": "9e2b4e39f6d4dd4c"}
-KERNEL_SOURCES = ["dgrad.cu", "ptx.cuh"]   # all the code of the non-fused data-gradient kernels
+KERNEL_SOURCES = ["dgrad.cu", "dgrad_common.cuh", "dgrad_general.cu", "dgrad_general.cuh", "dgrad_halo.cuh", "dgrad_halo_params.cuh", "ptx.cuh"]   # all the code of the non-fused data-gradient kernels
 
 
 def kernel_sources_sha():

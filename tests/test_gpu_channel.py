@@ -98,6 +98,30 @@ def test_conv_channel_mode(case):
     assert rel_fro(got, want) <= TOL
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "fp16"])
+@pytest.mark.parametrize("rows,K,n,m", [(1, 64, 2, 4), (3, 192, 2, 32), (255, 320, 1, 8), (515, 4096, 2, 16), (257, 4160, 1, 32),
+                                        (5000, 64, 2, 8), (2049, 8256, 2, 4)])
+def test_pruned_with_its_column_sums(rows, K, n, m, dtype):
+    """Prune and column sums in one read at the edges of its blocks: a single row, rows that fill no block, one column block
+    and several with a partly empty last one, channels that end inside a block of 128. Tolerance as above."""
+    import paper_2202_00774_b200 as sdgp
+    N = 64
+    dO, W = inputs.fc_tensors(rows, K, N, seed=rows + K + m)
+    odt, gdt, to_f = oracle.BF16, sdgp.BF16, inputs.bf16_bits_to_f32
+    if dtype == "fp16":
+        dO, W = inputs.bf16_bits_as_f16_bits(dO), inputs.bf16_bits_as_f16_bits(W)
+        odt, gdt, to_f = oracle.FP16, sdgp.FP16, inputs.f16_bits_to_f32
+    ws = torch.empty(sdgp.sdgp_workspace_size_linear(rows, K, N, sdgp.FLAG_CHANNEL), dtype=torch.uint8, device="cuda")
+    dD = torch.full((rows, N), -1, dtype=torch.int16, device="cuda")
+    sdgp.sdgp_dgrad_linear_typed(dev16(dO), dev16(W), dD, n, m, sdgp.RESCALED_MAGNITUDE, 0, gdt, workspace=ws,
+                                 flags=sdgp.FLAG_CHANNEL)
+    assert sdgp.sdgp_last_device_error() == 0
+    pruned = oracle.prune(dO, n, m, oracle.MAGNITUDE, want=("dense",), dtype=odt)["dense"]
+    want = oracle.dgrad_linear(pruned, W, dtype=odt, k_scale=oracle.channel_scales(dO, n, m, dtype=odt))
+    got = to_f(dD.cpu().numpy().view(np.uint16)).astype(np.float64)
+    assert rel_fro(got, want) <= TOL
+
+
 def test_channel_mode_wants_the_rescaled_scheme():
     import paper_2202_00774_b200 as sdgp
     dO = torch.zeros((64, 128), dtype=torch.int16, device="cuda")

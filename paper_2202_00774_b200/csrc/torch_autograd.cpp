@@ -8,6 +8,7 @@
 
 #include <ATen/ATen.h>
 #include <Python.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/custom_function.h>
@@ -71,6 +72,7 @@ struct Linear : torch::autograd::Function<Linear> {
       const Tensor W = weight.contiguous();
       on_gpu(dO, "dO");
       on_gpu(W, "W");
+      const c10::cuda::CUDAGuard guard(dO.device());
       const int64_t rows = dO.size(0), K = dO.size(1), N = W.size(1);
       const Tensor dD = at::empty({rows, N}, dO.options());
       const Tensor ws = bytes_like(dO, sdgp_workspace_size_linear(rows, K, N, SDGP_FLAG_TWO_PASS));
@@ -107,6 +109,7 @@ struct Conv2d : torch::autograd::Function<Conv2d> {
     if (kind == kConvReluPool && out.is_cuda() && (f16 || out.scalar_type() == at::kBFloat16) && H % 2 == 0 && W % 2 == 0 && C % 8 == 0 &&
         out.numel() > 0 && ((uintptr_t)out.data_ptr() & 15u) == 0) {
       // ReLU and pooling in one pass; what the backward pass needs of the activation is the convolution's output itself
+      const c10::cuda::CUDAGuard guard(out.device());  // (the tensors' device need not be the current one)
       const Tensor y = at::empty({B, C, H / 2, W / 2}, out.options(), MemoryFormat::ChannelsLast);
       TORCH_CHECK(sdgp::launch_relu_maxpool(out.data_ptr(), B, H, W, C, f16 ? SDGP_FP16 : SDGP_BF16, y.data_ptr(), (cudaStream_t)stream()) ==
                       cudaSuccess,
@@ -138,6 +141,7 @@ struct Conv2d : torch::autograd::Function<Conv2d> {
       const int P = (int)act.size(2), Q = (int)act.size(3);
       const Tensor dY = grads[0].contiguous(MemoryFormat::ChannelsLast);
       on_gpu(dY, "dY");
+      const c10::cuda::CUDAGuard guard(dY.device());
       const bool pool = kind == kConvReluPool;
       if (pool) {
         TORCH_CHECK_VALUE(dY.size(0) == B && dY.size(1) == Cout && dY.size(2) == P / 2 && dY.size(3) == Q / 2, "dYp must be [B, H/2, W/2, K]");
@@ -167,6 +171,7 @@ struct Conv2d : torch::autograd::Function<Conv2d> {
       const sdgp_dtype dt = dtype_of(g);
       on_gpu(g, "dO");
       on_gpu(W, "W");
+      const c10::cuda::CUDAGuard guard(g.device());
       grad_x = at::empty(x.sizes(), g.options(), MemoryFormat::ChannelsLast);
       if (vals.defined()) {
         check(sdgp_spmm_conv2d_typed(vals.data_ptr(), meta.data_ptr(), W.data_ptr(), grad_x.data_ptr(), B, H, Wd, Cin, Cout, R, S, stride,

@@ -3,10 +3,13 @@
 // per pointer, torch.cuda.current_stream()) a call took 13-18 us of host time, so the host set the pace of every layer
 // below some 15 us. Each function takes exactly the positional arguments its wrapper in binding.py passes, checks that
 // tensors are contiguous CUDA tensors, and returns the sdgp_status as an int.
+#include <ATen/PythonTorchFunctionTLS.h>
+#include <ATen/TensorSubclassLikeUtils.h>
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/jit/frontend/tracer.h>
 
 #include "../../include/sdgp.h"
 #include "torch_autograd.h"
@@ -264,19 +267,35 @@ ENTRY(spmm_conv2d) {  // values, meta, W, dD, stride, pad, dtype
   });
 }
 
-// Differentiable layers: x, weight, then `integers` numbers, the last of them a seed.
+// Whether the C++ layers take a tensor: what Python hands over is an ordinary tensor (no subclass) in GPU memory of a 16-bit type, and
+// nothing watches or transforms the operators that run on it.
+bool plain_tensor(PyObject* o, int64_t dims) {
+  if (!THPVariable_CheckExact(o)) return false;
+  const at::Tensor& t = THPVariable_Unpack(o);
+  return t.defined() && t.is_cuda() && t.layout() == at::kStrided && (dims < 0 ? t.dim() >= -dims : t.dim() == dims) &&
+         (t.scalar_type() == at::kBFloat16 || t.scalar_type() == at::kHalf) && !at::isTensorSubclassLike(t) && !t._fw_grad(0).defined();
+}
+
+bool plain_int(PyObject* o) {  // (no bool, no object with __index__: the operators' own argument parser has its rules for those)
+  if (!PyLong_CheckExact(o)) return false;
+  int overflow = 0;
+  const long long v = PyLong_AsLongLongAndOverflow(o, &overflow);
+  return overflow == 0 && v >= INT32_MIN && v <= INT32_MAX;
+}
+
+// Differentiable layers: x, weight, then `integers` numbers, the last of them a seed. NotImplemented: not a plain call, the caller takes
+// the Python form (which also gives the errors of arguments that are none).
 template <class F>
-PyObject* layer(PyObject* const* args, Py_ssize_t nargs, int integers, F call) {
+PyObject* layer(PyObject* const* args, Py_ssize_t nargs, int integers, int64_t x_dims, int64_t weight_dims, F call) {
   HANDLE_TH_ERRORS
   Args in(args, nargs, 2 + integers);
+  if (!in.ok) return nullptr;
+  bool plain = !torch::jit::tracer::isTracing() && !at::impl::torch_function_mode_enabled() && plain_tensor(args[0], x_dims) &&
+               plain_tensor(args[1], weight_dims) && PyLong_CheckExact(args[1 + integers]);
+  for (int k = 2; plain && k < 1 + integers; ++k) plain = plain_int(args[k]);
   at::Tensor t[2];
-  for (int k = 0; in.ok && k < 2; ++k, ++in.a) {
-    if (!THPVariable_Check(*in.a)) {
-      PyErr_SetString(PyExc_TypeError, "input and weight must be torch tensors");
-      return nullptr;
-    }
-    t[k] = THPVariable_Unpack(*in.a);
-  }
+  for (int k = 0; plain && k < 2; ++k, ++in.a) t[k] = THPVariable_Unpack(*in.a);
+  if (!plain || t[0].scalar_type() != t[1].scalar_type() || t[0].device() != t[1].device()) Py_RETURN_NOTIMPLEMENTED;
   std::vector<int64_t> numbers;
   for (int k = 0; k < integers; ++k) numbers.push_back(k + 1 < integers ? (int64_t)in.i32() : (int64_t)in.u64());
   if (!in.ok) return nullptr;
@@ -292,10 +311,10 @@ PyObject* layer(PyObject* const* args, Py_ssize_t nargs, int integers, F call) {
   END_HANDLE_TH_ERRORS
 }
 ENTRY(linear_layer) {  // x, weight, n, m, scheme, seed
-  return layer(args, nargs, 4, sdgp_torch::linear);
+  return layer(args, nargs, 4, -1, 2, sdgp_torch::linear);
 }
 ENTRY(conv2d_layer) {  // x, weight, stride, padding, kind, n, m, scheme, seed
-  return layer(args, nargs, 7, sdgp_torch::conv2d);
+  return layer(args, nargs, 7, 4, 4, sdgp_torch::conv2d);
 }
 
 ENTRY(workspace_size_linear) {  // rows, K, N, flags

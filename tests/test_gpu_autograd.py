@@ -127,6 +127,44 @@ def test_conv_relu_pool_matches_the_separate_operators(dtype, pool, shape):
         assert rel_fro(a.double().cpu().numpy(), b.double().cpu().numpy()) <= 5e-3
 
 
+@pytest.mark.parametrize("kind", ["conv", "relu", "pool", "linear"])
+@pytest.mark.parametrize("dtype,n,m,scheme", [(torch.bfloat16, 2, 4, 1), (torch.float16, 2, 8, 2), (torch.bfloat16, 2, 16, 0)])
+def test_plain_calls_and_the_python_form_agree(kind, dtype, n, m, scheme):
+    """The same kernels on the same operands: values and input gradients to the bit; the weight gradient is the framework's, whose sums
+    may run in another order (fp32 sums, one rounding to 16 bits)."""
+    from paper_2202_00774_b200 import autograd as sa
+    g = torch.Generator(device="cuda").manual_seed(5)
+    make = lambda *s: torch.randn(s, generator=g, device="cuda").to(dtype)   # noqa: E731
+    if kind == "linear":
+        x, w = make(3, 70, 128).requires_grad_(), (make(192, 128) / 16).requires_grad_()
+        plain, general = sa.sdgp_linear(x, w, n, m, scheme, 9), sa._SDGPLinearFn.apply(x, w, n, m, scheme, 9)
+    else:
+        x = make(3, 64, 8, 10).contiguous(memory_format=torch.channels_last).requires_grad_()
+        w = (make(128, 64, 3, 3) / 24).contiguous(memory_format=torch.channels_last).requires_grad_()
+        if kind == "conv":
+            plain, general = sa.sdgp_conv2d(x, w, 1, 1, n, m, scheme, 9), sa._SDGPConv2dFn.apply(x, w, 1, 1, n, m, scheme, 9)
+        else:
+            plain = sa.sdgp_conv2d_relu(x, w, 1, 1, kind == "pool", n, m, scheme, 9)
+            general = sa._SDGPConv2dReLUFn.apply(x, w, 1, 1, kind == "pool", n, m, scheme, 9)
+    assert type(plain.grad_fn) is not type(general.grad_fn) and plain.stride() == general.stride() and torch.equal(plain, general)
+    dY = make(*plain.shape)
+    a, b = torch.autograd.grad(plain, (x, w), dY), torch.autograd.grad(general, (x, w), dY)
+    assert torch.equal(a[0], b[0]) and a[0].stride() == b[0].stride()
+    assert rel_fro(a[1].double().cpu().numpy(), b[1].double().cpu().numpy()) <= 2.0 ** -8
+
+
+def test_traced_layers_compute():
+    """A trace of a layer holds operators only: it works on other inputs."""
+    from torch.fx.experimental.proxy_tensor import make_fx
+    from paper_2202_00774_b200 import autograd as sa
+    x, other = (torch.randn(2, 64, 8, 8, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    w = torch.randn(64, 64, 3, 3, device="cuda", dtype=torch.bfloat16) / 24
+    layer = lambda a, b: sa.sdgp_conv2d_relu(a, b, 1, 1, pool=True)   # noqa: E731
+    want = layer(other, w)
+    assert torch.equal(torch.jit.trace(layer, (x, w))(other, w), want)
+    assert torch.equal(make_fx(layer)(x, w)(other, w), want)
+
+
 def test_layers_raise_what_the_binding_raises():
     from paper_2202_00774_b200 import autograd as sa
     import paper_2202_00774_b200 as sdgp

@@ -244,9 +244,12 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
 
   // Output parities that no tap reaches are zero: clear dD first if there is any such class.
   bool any_empty = false;
+  int last_class = 0;  // of those that launch a kernel
   for (int ph = 0; ph < stride; ++ph)
-    for (int pw = 0; pw < stride; ++pw)
+    for (int pw = 0; pw < stride; ++pw) {
       if ((ph + pad) % stride >= R || (pw + pad) % stride >= S) any_empty = true;
+      else if (ph < H && pw < W) last_class = ph * stride + pw;
+    }
   if (any_empty && cudaMemsetAsync(dD, 0, (size_t)B * H * W * Cd * 2, stream) != cudaSuccess) return SDGP_ERR_CUDA;
   for (int ph = 0; ph < stride; ++ph) {
     for (int pw = 0; pw < stride; ++pw) {
@@ -285,6 +288,7 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
       p.last_mmas = left < kb_channels ? (left + per_mma - 1) / per_mma : 4;
       p.P = P; p.Q = Q;
       p.f16 = dtype == SDGP_FP16 ? 1 : 0;
+      p.last_launch = ph * stride + pw == last_class;
       if (fused) {
         p.fused_n = fused->n; p.fused_m = fused->m; p.fused_scheme = fused->scheme;
         p.seed_lo = (uint32_t)fused->seed; p.seed_hi = (uint32_t)(fused->seed >> 32);
@@ -306,6 +310,7 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
         hp.P = P; hp.Q = Q;
         hp.k_last = p.k_last; hp.last_mmas = p.last_mmas;
         hp.f16 = p.f16;
+        hp.last_launch = p.last_launch;
         if (fused) {
           hp.fused_n = p.fused_n; hp.fused_m = p.fused_m; hp.fused_scheme = p.fused_scheme; hp.seed_lo = p.seed_lo; hp.seed_hi = p.seed_hi;
           st = launch_halo_fused(BN, A, Wt, view, hp, stream);

@@ -188,7 +188,7 @@ dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   // never sit between this grid and a resource it still needs, and at most one grid is resident
   // behind a running one. The younger grid's own TMEM allocation then simply waits for this grid
   // to free its columns, which it does without anyone's help.
-  ptx::launch_dependents();
+  if (p.early) ptx::launch_dependents();
 
   const int rows_used = p.TW * p.TH * p.TB;
   const int taps = p.R * p.S;
@@ -568,6 +568,7 @@ sdgp_status launch_cfg(const void* A, const void* meta, const void* Wt, const Dg
   using C = Cfg<SPARSE, BN>;
   if (!plan<SPARSE, BN, FUSED>(&p)) return SDGP_ERR_UNSUPPORTED;
   p.d = view.d;
+  p.early = early_for(SPARSE && !FUSED && p.last_launch, pairs_for(p.pair_tiles));
 
   CUtensorMap tmA, tmE, tmB, tmD;
   const uint32_t img_h = (uint32_t)(p.TH + p.rr - 1);

@@ -22,6 +22,8 @@ struct DgradParams {
   int nacc;               // TMEM accumulators (2 = epilogue overlaps the next tile)
   int meta_col;           // first TMEM column of the metadata slots
   int meta_shared;        // metadata slots live in the first columns of the accumulator NOT being written
+  int last_launch;        // no further launch of the same call follows
+  int early;              // the next kernel may be scheduled while this one runs (early_for())
   int w_resident;         // whole W half-slice kept in shared memory
   int out_bufs;           // staging slabs per epilogue warp (boxes only)
   int box_store;          // the epilogue's warps write boxes of 32 pixels by TMA (else rows, straight from registers)

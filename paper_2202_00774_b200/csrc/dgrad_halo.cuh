@@ -111,7 +111,7 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   // never sit between this grid and a resource it still needs, and at most one grid is resident
   // behind a running one. The younger grid's own TMEM allocation then simply waits for this grid
   // to free its columns, which it does without anyone's help.
-  ptx::launch_dependents();
+  if (p.early) ptx::launch_dependents();
 
   const int taps = p.R * p.sb;  // filter taps served by one A box
   const int pair_stride = gridDim.x >> 1;
@@ -778,6 +778,7 @@ sdgp_status launch_halo_nt(const void* A, const void* meta, const void* Wt, cons
 
   CUtensorMap tmA, tmE, tmB, tmD;
   p.d = view.d;
+  p.early = early_for(SPARSE && !FUSED && p.last_launch, pairs_for(p.units));
   const int P = view.P, Q = view.Q;
   const uint64_t CA = (SPARSE && !FUSED) ? (uint64_t)view.a_channels / 2 : (uint64_t)view.a_channels;
   // Dimensions: channel, pixel column, [column-split mode only: image within a box row (img_per_row images lie side by

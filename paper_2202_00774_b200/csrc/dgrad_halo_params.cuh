@@ -72,6 +72,7 @@ struct HaloParams {
   uint32_t seed_lo, seed_hi;
   int P, Q;                // dO pixel grid (linear element index of the random scheme)
   OutView d;
+  int last_launch, early;  // as in DgradParams
   int f16;                 // element type of A, W and dD: 0 = bf16, 1 = IEEE binary16
 };
 

@@ -739,3 +739,39 @@ def test_conv_image_sizes_that_leave_strips_partly_empty(B, H, Wd, Cin, Cout, R,
     check_no_device_error()
     src = dO if mode == "dense" else oracle.prune(dO.reshape(-1, Cout), 2, 4, scheme, 6, want=("dense",))["dense"].reshape(dO.shape)
     assert_close(to_f64(dD), *conv_ref(src, W, H, Wd, 1, pad))
+
+
+@pytest.mark.parametrize("rows,K,N", [(2412, 128, 448), (512, 128, 1152), (300, 128, 64)])
+def test_back_to_back_steps_see_each_others_results(rows, K, N):
+    """Pruning and contraction in turn on one stream, each step's gradient read from the last one's result, over contractions that
+    hold most of the chip and ones that leave room: no kernel may start on data that its predecessor has not written yet."""
+    import paper_2202_00774_b200 as sdgp
+    dO, W = inputs.fc_tensors(rows, K, N, seed=rows)
+    back = torch.randn((N, K), device="cuda", dtype=torch.float32).div_(N ** 0.5).to(torch.bfloat16)
+    ws = torch.empty(max(16, sdgp.sdgp_workspace_size_linear(rows, K, N)), dtype=torch.uint8, device="cuda")
+    values = torch.empty((rows, K // 2), dtype=torch.int16, device="cuda")
+    meta = torch.empty((rows, K // 16), dtype=torch.int16, device="cuda")
+    w, act = dev16(W), dev16(np.full((rows, K), 0x3F80, np.uint16))   # (an activation of ones: the gate passes everything)
+
+    def steps(wait):
+        x = dev16(dO)
+        for step in range(6):
+            dD = torch.full((rows, N), -1, dtype=torch.int16, device="cuda")
+            if step % 2:
+                sdgp.sdgp_relu_backward_prune(x, act, 2, 4, sdgp.MAGNITUDE, values=values, meta=meta)
+            else:
+                sdgp.sdgp_prune(x, 2, 4, sdgp.MAGNITUDE, values=values, meta=meta)
+            wait()
+            sdgp.sdgp_spmm_linear(values, meta, w, dD)
+            wait()
+            y = torch.full((rows, K), -1, dtype=torch.int16, device="cuda")
+            sdgp.sdgp_dgrad_linear(dD, back.view(torch.int16), y, 4, 4, sdgp.MAGNITUDE, flags=sdgp.FLAG_DENSE)
+            wait()
+            x = y
+        return x
+
+    want = steps(torch.cuda.synchronize)
+    for _ in range(5):
+        got = steps(lambda: None)
+        check_no_device_error()
+        assert torch.equal(got, want)

@@ -302,23 +302,26 @@ dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         ptx::tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
         uint32_t accumulate = 0u;
-        // (this thread's instructions are the MMAs' issue rate: no division where every block is whole or every tile sees all blocks)
-        int cb_last = p.last_mmas == 4 ? -1 : p.k_last;
-        if (p.last_mmas != 4 && p.diag_cin_g != 0) cb_last -= first_k_block(p, (first_pair + lt * pair_stride) % p.tiles_n * BN, C::kKB);
-        int r_single = 0, s = 0;
-        for (int g = 0; alive && g < groups; ++g) {
-          for (int cb = 0; cb < p.k_blocks; ++cb) {
-            if (!ptx::mbar_wait(&full[st], ph, err, 0x300u + st)) { alive = false; break; }
-            ptx::tc_fence_after_sync();
-            const uint32_t e_col = meta_base + mcol;  // even: slots are multiples of 4 columns apart
-            const int mmas = cb == cb_last ? p.last_mmas : 4;
-            if (SPARSE) {
-              for (int u = 0; u < p.rr; ++u)
-                ptx::tc_cp_128x128b_pair(e_col + 4u * u, ((uint64_t)e_hi << 32) | (e_lo + (uint32_t)(u * (kEHwBytes / 16))));
-            }
-            // MMAS: MMAs of the channel block, 0: `mmas` of them (one form for every partial block keeps the loop's code small)
-            auto issue = [&](auto mmas_tag) {
-              constexpr int MMAS = decltype(mmas_tag)::value;
+        // This thread's instructions set the pace of narrow tiles (65 x 2688 . 2688 x 576: 20 ns more per block with a test for partial
+        // blocks in it). WHOLE: every channel block is, and the loop holds no such test; else the layer's last block may be partial.
+        auto tile = [&](auto whole_tag) {
+          constexpr bool WHOLE = decltype(whole_tag)::value;
+          int cb_last = 0;  // the partial block's place in the tile's window
+          if (!WHOLE) {
+            cb_last = p.k_last;
+            if (p.diag_cin_g != 0) cb_last -= first_k_block(p, (first_pair + lt * pair_stride) % p.tiles_n * BN, C::kKB);
+          }
+          int r_single = 0, s = 0;
+          for (int g = 0; alive && g < groups; ++g) {
+            for (int cb = 0; cb < p.k_blocks; ++cb) {
+              if (!ptx::mbar_wait(&full[st], ph, err, 0x300u + st)) { alive = false; break; }
+              ptx::tc_fence_after_sync();
+              const uint32_t e_col = meta_base + mcol;  // even: slots are multiples of 4 columns apart
+              const int mmas = !WHOLE && cb == cb_last ? p.last_mmas : 4;
+              if (SPARSE) {
+                for (int u = 0; u < p.rr; ++u)
+                  ptx::tc_cp_128x128b_pair(e_col + 4u * u, ((uint64_t)e_hi << 32) | (e_lo + (uint32_t)(u * (kEHwBytes / 16))));
+              }
               for (int u = 0; u < p.rr; ++u) {
                 // vertical tap r: the tile's rows start (R-1-r) image rows into the stage
                 const int r = reuse ? u : r_single;
@@ -326,8 +329,8 @@ dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                 const uint32_t b_u = p.w_resident ? w_lo0 + (uint32_t)((r * p.S + s) * p.k_blocks + cb) * kTapB16
                                                   : b_lo + (uint32_t)u * kTapB16;
 #pragma unroll
-                for (int q = 0; q < (MMAS ? MMAS : 4); ++q) {
-                  if (!MMAS && q >= mmas) break;
+                for (int q = 0; q < 4; ++q) {
+                  if (!WHOLE && q >= mmas) break;
                   // A: 32 bytes of a 128-byte swizzled row per MMA; B: 16 (dense) or 32 (sparse) rows
                   const uint64_t a_q = ((uint64_t)a_hi << 32) | (a_u + (uint32_t)(q * 2));
                   const uint64_t b_q = ((uint64_t)b_hi << 32) | (b_u + (uint32_t)q * kBStep);
@@ -339,15 +342,15 @@ dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                 }
                 accumulate = 1u;
               }
-            };
-            if (mmas == 4) issue(std::integral_constant<int, 4>{});
-            else issue(std::integral_constant<int, 0>{});
-            ptx::tc_commit_pair(&empty[st], 3);
-            if (++st == STAGES) { st = 0; ph ^= 1u; a_lo = a_lo0; b_lo = b_lo0; e_lo = e_lo0; mcol = 0; }
-            else { a_lo += a_stage16; b_lo += b_stage16; e_lo += e_stage16; mcol += slot_cols; }
+              ptx::tc_commit_pair(&empty[st], 3);
+              if (++st == STAGES) { st = 0; ph ^= 1u; a_lo = a_lo0; b_lo = b_lo0; e_lo = e_lo0; mcol = 0; }
+              else { a_lo += a_stage16; b_lo += b_stage16; e_lo += e_stage16; mcol += slot_cols; }
+            }
+            if (++s == p.S) { s = 0; ++r_single; }
           }
-          if (++s == p.S) { s = 0; ++r_single; }
-        }
+        };
+        if (p.last_mmas == 4) tile(std::true_type{});
+        else tile(std::false_type{});
         if (alive) ptx::tc_commit_pair(&acc_full[acc], 3);
         if (++acc == NACC) { acc = 0; aph ^= 1u; }
       }

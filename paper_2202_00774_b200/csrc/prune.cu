@@ -272,7 +272,7 @@ prune_kernel(const uint4* __restrict__ dO, int64_t nvec, uint32_t seed_lo, uint3
 #pragma unroll
     for (int it = 0; it < kPairs; ++it) {
       const int64_t p = base + it * stride;
-      if (M < 32 && p >= npair) continue;  // (the lanes of a group of 32 meet in shuffles)
+      if (M == 32 ? !__any_sync(0xFFFFFFFFu, p < npair) : p >= npair) continue;  // (the lanes of a group of 32 meet in shuffles)
       uint4 out;
       uint32_t pa, pb;
       KeepFlags ka, kb;
@@ -325,10 +325,12 @@ cudaError_t launch_select(int scheme, bool f16, const void* dO, int64_t nvec, ui
   const uint32_t lo = (uint32_t)seed, hi = (uint32_t)(seed >> 32);
   auto launch = [&](auto kernel, bool pairs) {
     // Pairs: two per thread, or one where all blocks of that split are resident at once anyway (a small tensor is a matter of
-    // latency: 256 x 512 elements take 32 blocks instead of 16). A persistent grid that prefetches a thread's next pair
-    // measured 3-15 % slower than blocks that come and go.
+    // latency: 256 x 512 elements take 32 blocks instead of 16; groups of 32, whose lanes wait for each other's keys, gain by it up to a
+    // block per multiprocessor only). A warp whose second pairs all lie past the end leaves them out: 1067 x 2112, 2:32 with a mask, 4.8 us
+    // when it went through their ranking, 3.0 without. A persistent grid that prefetches a thread's next pair measured 3-15 % slower
+    // than blocks that come and go.
     const int64_t singles = (nvec + 2 * kThreads - 1) / (2 * kThreads);
-    const int64_t per_block = pairs && singles <= 4 * (int64_t)sm_count() ? 2 * kThreads : kThreads * kVecPerThread;
+    const int64_t per_block = pairs && singles <= (M == 32 ? 1 : 4) * (int64_t)sm_count() ? 2 * kThreads : kThreads * kVecPerThread;
     const int64_t blocks = (nvec + per_block - 1) / per_block;
     if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)blocks), block(kThreads);

@@ -230,7 +230,11 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
 
   if (fused && B == 1 && H == 1 && R == 1 && S == 1 && stride == 1 && pad == 0 && fused->m <= 16) {
     const RowsPlan plan = plan_rows(W, Cout, Cin, prune_cost(fused->m, fused->scheme).stage_clk);
-    if (plan.ok) return launch_rows_fused(plan, A, Wt, Cout, Cin, dD, *fused, dtype, stream);
+    // The rows kernel's warps prune 8 rows each of all 128, whatever exists; the general kernel's 384 pruning threads an eighth of a row each,
+    // 48 rows in one pass. Where pruning sets the pace (random and rescaled functions) few rows are faster there: 35 x 3264 . 3264 x 192,
+    // random 2:16, 48.4 us against 68.7; 36 x 896 . 896 x 576, rescaled 1:4, 14.2 against 15.3; magnitude 47 x 2944 . 2944 x 64 35.4 against 33.9.
+    const bool few_rows = W <= 48 && fused->scheme != SDGP_MAGNITUDE;
+    if (plan.ok && !few_rows) return launch_rows_fused(plan, A, Wt, Cout, Cin, dD, *fused, dtype, stream);
   }
   const int kb_channels = sparse ? 128 : 64;
 

@@ -775,3 +775,17 @@ def test_back_to_back_steps_see_each_others_results(rows, K, N):
         got = steps(lambda: None)
         check_no_device_error()
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("scheme", [oracle.RANDOM, oracle.RESCALED])
+@pytest.mark.parametrize("rows,K,N,n,m", [(1, 64, 64, 2, 4), (47, 320, 192, 2, 16), (48, 1024, 64, 1, 4), (49, 256, 320, 2, 8)])
+def test_linear_fused_of_few_rows(rows, K, N, n, m, scheme):
+    """Up to 48 rows with the functions that take longest go to the general kernel's pruning threads, 49 to the rows kernel."""
+    import paper_2202_00774_b200 as sdgp
+    dO, W = inputs.fc_tensors(rows, K, N, seed=rows + m)
+    flat = torch.full((rows * N + 64,), 0x5A5A, dtype=torch.int16, device="cuda")
+    dD = flat[:rows * N].view(rows, N)
+    sdgp.sdgp_dgrad_linear(dev16(dO), dev16(W), dD, n, m, scheme, 9, flags=sdgp.FLAG_FUSED)
+    check_no_device_error()
+    assert_close(to_f64(dD), *linear_ref(oracle.prune(dO, n, m, scheme, 9, want=("dense",))["dense"], W))
+    assert np.all(flat[rows * N:].cpu().numpy() == 0x5A5A)

@@ -59,6 +59,10 @@ constexpr uint32_t kTmemCols = 512;
 constexpr int kMaxImgRows = 192;     // pixel rows of one A stage (filter-row reuse: TW * (TH + R - 1))
 constexpr int kSmemLimit = 232448;   // opt-in dynamic shared memory per CTA
 constexpr int kSmemSlack = 1536;     // 1024-byte alignment of the carve + barrier block
+// A CTA asks for at least this much, so that no two share a multiprocessor: the second sits in its TMEM allocation until the first is done,
+// and the multiprocessor it could have had stays empty (29 x 16 x 16 images, 128 -> 128, dense, tiles of one strip of 64 columns: 19.1 us
+// with its pruning pass, 12.3 alone).
+constexpr int kSmemAlone = 116 * 1024;
 constexpr int kMaxStages = 8;
 
 
@@ -267,7 +271,7 @@ sdgp_status launch_pairs(void (*kernel)(Params...), int pairs, int threads, int 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(2 * pairs));
   cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = (size_t)smem_bytes;
+  cfg.dynamicSmemBytes = (size_t)(smem_bytes > kSmemAlone ? smem_bytes : kSmemAlone);
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;

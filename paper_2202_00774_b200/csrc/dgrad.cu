@@ -2,6 +2,9 @@
 // dgrad_halo.cuh for the kernels).
 #include <string.h>
 
+#include <algorithm>
+#include <iterator>
+
 #include "dgrad_general.cuh"
 #include "dgrad_halo_params.cuh"
 #include "dgrad_rows.cuh"
@@ -179,10 +182,32 @@ bool halo_applies(int H, int W, int taps, bool sparse, bool fused) {
   return covered * 100 <= (int64_t)H * W * (taps < 6 ? 135 : 260);
 }
 
-// Accumulators (128 rows) that kernel's strips need.
-int64_t halo_strips(int B, int H, int W) {
-  const int th = H <= 4 ? 4 : H <= 8 ? 8 : kHaloRows, tb = kHaloRows / th, per_row = W == 4 ? 2 : 1;
-  return (int64_t)((W + 7) / 8) * ((H + th - 1) / th) * ((B + tb * per_row - 1) / (tb * per_row));
+// Estimated time of one launch of that kernel over bn input channels and nt strips per tile, in units of the fixed part of a tap (some
+// 0.3 us: barriers and the MMA issue, whatever the width). A round of tiles takes, per channel block, its taps at 1 + 1/8 per 64
+// accumulator columns (dense A: 1/16) and the box's bytes or - fused - the pruning of the box, whichever is longer; then an epilogue. Two
+// strips side by side share every W stage and the fixed part; where there are too few strips for every CTA pair, or a box's pruning
+// sets the pace, one is better. Constants fitted to 790 layers timed in all six shapes, dense, two-pass and fused: 0.3 % behind the best
+// shape in the mean, more than 5 % behind in 20 of them. A rule that looked at the width alone was 2.4 % behind. Us, that rule and this one:
+// 20 x 4 x 4 images, 256 -> 256, fused, random 2:16, 49.6, 30.5; 110 x 32 x 32, 256 -> 384, dense after pruning, 169.8, 139.3; 339 x 14 x 14,
+// 12 groups of 16, 53.7, 39.7; 32 x 28 x 28, 128 -> 320, 11 x 11, fused (192 columns do not fit), 1034, 265. 0: no such shape for this layer.
+double halo_cost(int B, int H, int W, int R, int S, int bn, int nt, bool sparse, int tiles_n, int k_blocks, const FusedPrune* fused) {
+  const bool split = W == 4;
+  if (nt * bn > 256 || (!split && nt == 2 && W <= 8)) return 0.0;
+  const int per_row = split ? 2 * nt : 1, th = H <= 4 ? 4 : H <= 8 ? 8 : kHaloRows, tb = kHaloRows / th;
+  if (B % per_row != 0) return 0.0;
+  const int sb = split ? 1 : S, boxes = split ? S : 1;
+  const int sets_w = split ? 1 : (W + 8 * nt - 1) / (8 * nt), tiles_h = (H + th - 1) / th;
+  const int64_t sets = (int64_t)sets_w * tiles_h * ((B + tb * per_row - 1) / (tb * per_row));
+  const int64_t pairs = sm_count() / 2, rounds = ((sets + 1) / 2 * tiles_n + pairs - 1) / pairs;
+  const double columns = nt * bn / 64.0, img_rows = (8 * nt + sb - 1) * (th + R - 1) * tb;
+  double box = R * sb * (1.0 + columns * (sparse ? 0.125 : 0.0625)) + 0.003 * img_rows;
+  if (fused) {
+    const bool whole_images = sets_w == 1 && tiles_h == 1;  // only the units inside the images are pruned (plan_halo())
+    const double units = whole_images ? (H < th ? H : th) * tb * nt : img_rows / 8;
+    const double unit = fused->scheme == SDGP_MAGNITUDE ? 0.37 : fused->scheme == SDGP_RANDOM ? 0.92 : 1.1;
+    if (5.0 + units * unit > box) box = 5.0 + units * unit;
+  }
+  return (double)rounds * (k_blocks * boxes * box + 4.3 + 0.5 * columns);
 }
 
 // What pruning costs (measured on a [16384 x 4096] tensor and on 50176 x 1024 rows): clocks of the rows kernel's pruning warps per block of
@@ -249,11 +274,26 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
   // Output parities that no tap reaches are zero: clear dD first if there is any such class.
   bool any_empty = false;
   int last_class = 0;  // of those that launch a kernel
+  const int all_blocks = (Cout + kb_channels - 1) / kb_channels;
+  // Tile shapes of the strip kernel, one for all classes of the call (kernels that alternate between shapes measured up to 10 % slower).
+  struct Shape { int bn, nt; double cost; } shapes[] = {{64, 1, 0}, {64, 2, 0}, {128, 1, 0}, {128, 2, 0}, {192, 1, 0}, {256, 1, 0}};
   for (int ph = 0; ph < stride; ++ph)
     for (int pw = 0; pw < stride; ++pw) {
-      if ((ph + pad) % stride >= R || (pw + pad) % stride >= S) any_empty = true;
-      else if (ph < H && pw < W) last_class = ph * stride + pw;
+      const int r0 = (ph + pad) % stride, s0 = (pw + pad) % stride;
+      if (r0 >= R || s0 >= S) { any_empty = true; continue; }
+      if (ph >= H || pw >= W) continue;
+      last_class = ph * stride + pw;
+      const int Hs = (H - ph + stride - 1) / stride, Ws = (W - pw + stride - 1) / stride;
+      const int Rs = (R - r0 + stride - 1) / stride, Ss = (S - s0 + stride - 1) / stride;
+      if (!halo_applies(Hs, Ws, Rs * Ss, sparse, fused != nullptr)) continue;
+      for (Shape& s : shapes) {
+        const int tiles_n = (view.d.channels + s.bn - 1) / s.bn;
+        const double cost = halo_cost(B, Hs, Ws, Rs, Ss, s.bn, s.nt, sparse, tiles_n,
+                                      k_window(s.bn, view.d.channels, all_blocks, kb_channels, Cout, conv_groups), fused);
+        s.cost += cost > 0.0 ? cost : 1e9;  // (does not exist for this class: tried last)
+      }
     }
+  std::sort(std::begin(shapes), std::end(shapes), [](const Shape& a, const Shape& b) { return a.cost < b.cost; });
   if (any_empty && cudaMemsetAsync(dD, 0, (size_t)B * H * W * Cd * 2, stream) != cudaSuccess) return SDGP_ERR_CUDA;
   for (int ph = 0; ph < stride; ++ph) {
     for (int pw = 0; pw < stride; ++pw) {
@@ -274,18 +314,17 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
       p.tiles_h = (Hs + p.TH - 1) / p.TH;
       p.tiles_b = (B + p.TB - 1) / p.TB;
       const int64_t m_tiles = (int64_t)p.tiles_w * p.tiles_h * p.tiles_b;
-      const int all_blocks = (Cout + kb_channels - 1) / kb_channels;
-      const bool halo = halo_applies(Hs, Ws, p.R * p.S, sparse, fused != nullptr);
-      const int BN = choose_bn(halo ? halo_strips(B, Hs, Ws) : m_tiles, view.d.channels, all_blocks, kb_channels, Cout, conv_groups);
-      p.tiles_n = (view.d.channels + BN - 1) / BN;
-      if (m_tiles * p.tiles_n > 0x3FFFFFFF) return SDGP_ERR_UNSUPPORTED;
       p.m_tiles = (int)m_tiles;
-      p.pair_tiles = (int)((m_tiles + 1) / 2) * p.tiles_n;
-      p.k_blocks = k_window(BN, view.d.channels, all_blocks, kb_channels, Cout, conv_groups);
-      if (p.k_blocks < all_blocks) {
-        p.diag_cin_g = conv_groups->cin_g; p.diag_cout_g = conv_groups->cout_g;
-        p.diag_last = all_blocks - p.k_blocks;
-      }
+      // what depends on the width of a tile
+      auto set_width = [&](int bn) {
+        p.tiles_n = (view.d.channels + bn - 1) / bn;
+        p.k_blocks = k_window(bn, view.d.channels, all_blocks, kb_channels, Cout, conv_groups);
+        p.diag_cin_g = p.diag_cout_g = p.diag_last = 0;
+        if (p.k_blocks < all_blocks) {
+          p.diag_cin_g = conv_groups->cin_g; p.diag_cout_g = conv_groups->cout_g;
+          p.diag_last = all_blocks - p.k_blocks;
+        }
+      };
       // the last channel block may be partly empty: its MMAs (32 channels each, dense 16) past the channels that exist are left out
       p.k_last = all_blocks - 1;
       const int left = view.a_channels - p.k_last * kb_channels, per_mma = kb_channels / 4;
@@ -303,28 +342,37 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
       view.d.sb = (int64_t)H * W * Cd * 2;
       view.d.aligned32 = ((uintptr_t)dD & 31u) == 0 && Cd % 16 == 0;
       sdgp_status st = SDGP_ERR_UNSUPPORTED;
-      if (halo) {
+      if (halo_applies(Hs, Ws, p.R * p.S, sparse, fused != nullptr)) {
         HaloParams hp = {};
         hp.B = B; hp.H = Hs; hp.W = Ws; hp.Cin = Cin; hp.Cout = Cout;
         hp.R = p.R; hp.S = p.S; hp.pad_h = p.pad_h; hp.pad_w = p.pad_w;
         hp.r_first = p.r_first; hp.r_step = p.r_step; hp.s_first = p.s_first; hp.s_step = p.s_step;
         hp.S_full = S;
-        hp.tiles_n = p.tiles_n; hp.k_blocks = p.k_blocks;
-        hp.diag_cin_g = p.diag_cin_g; hp.diag_cout_g = p.diag_cout_g; hp.diag_last = p.diag_last;
         hp.P = P; hp.Q = Q;
         hp.k_last = p.k_last; hp.last_mmas = p.last_mmas;
         hp.f16 = p.f16;
         hp.last_launch = p.last_launch;
         if (fused) {
           hp.fused_n = p.fused_n; hp.fused_m = p.fused_m; hp.fused_scheme = p.fused_scheme; hp.seed_lo = p.seed_lo; hp.seed_hi = p.seed_hi;
-          st = launch_halo_fused(BN, A, Wt, view, hp, stream);
-        } else {
-          st = sparse ? launch_halo_sparse(BN, A, meta, Wt, view, hp, stream) : launch_halo_dense(BN, A, Wt, view, hp, stream);
+        }
+        // from the cheapest on, until one fits shared memory (a large filter's box and a wide tile may not)
+        for (const Shape& s : shapes) {
+          set_width(s.bn);
+          hp.tiles_n = p.tiles_n; hp.k_blocks = p.k_blocks;
+          hp.diag_cin_g = p.diag_cin_g; hp.diag_cout_g = p.diag_cout_g; hp.diag_last = p.diag_last;
+          st = fused    ? launch_halo_fused(s.bn, s.nt, A, Wt, view, hp, stream)
+               : sparse ? launch_halo_sparse(s.bn, s.nt, A, meta, Wt, view, hp, stream)
+                        : launch_halo_dense(s.bn, s.nt, A, Wt, view, hp, stream);
+          if (st != SDGP_ERR_UNSUPPORTED) break;
         }
         if (st == SDGP_OK) continue;
-        if (st != SDGP_ERR_UNSUPPORTED) return st;  // otherwise: does not fit, use the general kernel
+        if (st != SDGP_ERR_UNSUPPORTED) return st;  // otherwise: no shape fits, use the general kernel
       }
       if (fused && fused->m == 32) return SDGP_ERR_UNSUPPORTED;  // this kernel's threads hold 16 channels each: groups of up to 16
+      const int BN = choose_bn(m_tiles, view.d.channels, all_blocks, kb_channels, Cout, conv_groups);
+      set_width(BN);
+      if (m_tiles * p.tiles_n > 0x3FFFFFFF) return SDGP_ERR_UNSUPPORTED;
+      p.pair_tiles = (int)((m_tiles + 1) / 2) * p.tiles_n;
       st = launch_general(sparse, fused != nullptr, BN, A, meta, Wt, view, p, stream);
       if (st != SDGP_OK) return st;
     }

@@ -840,26 +840,17 @@ sdgp_status launch_halo_nt(const void* A, const void* meta, const void* Wt, cons
   return launch(std::false_type{});
 }
 
-// Two strips per CTA where the accumulators of two tile sets fit TMEM, else one.
-template <bool SPARSE, int BN, bool FUSED>
-sdgp_status launch_halo(const void* A, const void* meta, const void* Wt, const DgradView& view, const HaloParams& p,
-                        cudaStream_t stream) {
-  if (BN <= 128) {
-    const sdgp_status st = launch_halo_nt<SPARSE, (BN <= 128 ? BN : 64), 2, FUSED>(A, meta, Wt, view, p, stream);
-    if (st != SDGP_ERR_UNSUPPORTED) return st;
-  }
-  return launch_halo_nt<SPARSE, BN, 1, FUSED>(A, meta, Wt, view, p, stream);
-}
-
-
 template <bool SPARSE, bool FUSED>
-sdgp_status launch_halo_bn(int bn, const void* A, const void* meta, const void* Wt, const DgradView& view, const HaloParams& p,
-                           cudaStream_t stream) {
-  switch (bn) {
-    case 64: return launch_halo<SPARSE, 64, FUSED>(A, meta, Wt, view, p, stream);
-    case 128: return launch_halo<SPARSE, 128, FUSED>(A, meta, Wt, view, p, stream);
-    case 192: return launch_halo<SPARSE, 192, FUSED>(A, meta, Wt, view, p, stream);
-    default: return launch_halo<SPARSE, 256, FUSED>(A, meta, Wt, view, p, stream);
+sdgp_status launch_halo(int bn, int nt, const void* A, const void* meta, const void* Wt, const DgradView& view, const HaloParams& p,
+                        cudaStream_t stream) {
+  switch (bn * nt) {
+    case 64: return launch_halo_nt<SPARSE, 64, 1, FUSED>(A, meta, Wt, view, p, stream);
+    case 128: return nt == 2 ? launch_halo_nt<SPARSE, 64, 2, FUSED>(A, meta, Wt, view, p, stream)
+                             : launch_halo_nt<SPARSE, 128, 1, FUSED>(A, meta, Wt, view, p, stream);
+    case 192: return launch_halo_nt<SPARSE, 192, 1, FUSED>(A, meta, Wt, view, p, stream);
+    case 256: return nt == 2 ? launch_halo_nt<SPARSE, 128, 2, FUSED>(A, meta, Wt, view, p, stream)
+                             : launch_halo_nt<SPARSE, 256, 1, FUSED>(A, meta, Wt, view, p, stream);
+    default: return SDGP_ERR_UNSUPPORTED;
   }
 }
 

@@ -3,8 +3,8 @@
 
 namespace sdgp {
 
-sdgp_status launch_halo_dense(int bn, const void* A, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream) {
-  return launch_halo_bn<false, false>(bn, A, nullptr, Wt, view, p, stream);
+sdgp_status launch_halo_dense(int bn, int nt, const void* A, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream) {
+  return launch_halo<false, false>(bn, nt, A, nullptr, Wt, view, p, stream);
 }
 
 cudaError_t take_error_halo_dense(unsigned int* word) { return take_error_word(word); }

@@ -3,8 +3,8 @@
 
 namespace sdgp {
 
-sdgp_status launch_halo_fused(int bn, const void* dO, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream) {
-  return launch_halo_bn<true, true>(bn, dO, nullptr, Wt, view, p, stream);
+sdgp_status launch_halo_fused(int bn, int nt, const void* dO, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream) {
+  return launch_halo<true, true>(bn, nt, dO, nullptr, Wt, view, p, stream);
 }
 
 cudaError_t take_error_halo_fused(unsigned int* word) { return take_error_word(word); }

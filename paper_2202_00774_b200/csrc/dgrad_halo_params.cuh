@@ -76,10 +76,11 @@ struct HaloParams {
   int f16;                 // element type of A, W and dD: 0 = bf16, 1 = IEEE binary16
 };
 
-// Plans and launches the kernel over BN = bn input channels per tile; SDGP_ERR_UNSUPPORTED if no plan fits.
-sdgp_status launch_halo_sparse(int bn, const void* A, const void* meta, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream);
-sdgp_status launch_halo_dense(int bn, const void* A, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream);
-sdgp_status launch_halo_fused(int bn, const void* dO, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream);
+// Plans and launches the kernel over BN = bn input channels and nt strips (two at most, 256 columns together) per tile;
+// SDGP_ERR_UNSUPPORTED if no plan fits.
+sdgp_status launch_halo_sparse(int bn, int nt, const void* A, const void* meta, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream);
+sdgp_status launch_halo_dense(int bn, int nt, const void* A, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream);
+sdgp_status launch_halo_fused(int bn, int nt, const void* dO, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream);
 cudaError_t take_error_halo_sparse(unsigned int* word);
 cudaError_t take_error_halo_dense(unsigned int* word);
 cudaError_t take_error_halo_fused(unsigned int* word);

@@ -3,8 +3,8 @@
 
 namespace sdgp {
 
-sdgp_status launch_halo_sparse(int bn, const void* A, const void* meta, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream) {
-  return launch_halo_bn<true, false>(bn, A, meta, Wt, view, p, stream);
+sdgp_status launch_halo_sparse(int bn, int nt, const void* A, const void* meta, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream) {
+  return launch_halo<true, false>(bn, nt, A, meta, Wt, view, p, stream);
 }
 
 cudaError_t take_error_halo_sparse(unsigned int* word) { return take_error_word(word); }

@@ -789,3 +789,35 @@ def test_linear_fused_of_few_rows(rows, K, N, n, m, scheme):
     check_no_device_error()
     assert_close(to_f64(dD), *linear_ref(oracle.prune(dO, n, m, scheme, 9, want=("dense",))["dense"], W))
     assert np.all(flat[rows * N:].cpu().numpy() == 0x5A5A)
+
+
+@pytest.mark.parametrize("Cin,R,pad", [(320, 11, 5), (192, 11, 10)])
+def test_fused_groups_of_32_under_a_large_filter(Cin, R, pad):
+    """The widest tiles do not fit beside the box of an 11 x 11 filter: a narrower one is taken, the layer is not refused."""
+    import paper_2202_00774_b200 as sdgp
+    layer = inputs.ConvLayer("t", 2, 12, 12, Cin, 64, R, R, 1, pad)
+    dO, W = inputs.conv_layer_tensors(layer, seed=Cin)
+    dD = torch.full(layer.dD_shape(), -1, dtype=torch.int16, device="cuda")
+    sdgp.sdgp_dgrad_conv2d(dev16(dO), dev16(W), dD, 1, pad, 2, 32, oracle.MAGNITUDE, flags=sdgp.FLAG_FUSED)
+    check_no_device_error()
+    pruned = oracle.prune(dO.reshape(-1, 64), 2, 32, oracle.MAGNITUDE, want=("dense",))["dense"].reshape(dO.shape)
+    assert_close(to_f64(dD), *conv_ref(pruned, W, 12, 12, 1, pad))
+
+
+# batch, image, input and output channels: 64 and 128 columns with one strip (few strips) and with two (many), 192, 256
+@pytest.mark.parametrize("B,H,Cin,Cout", [(2, 16, 64, 128), (40, 16, 64, 64), (20, 4, 256, 128), (9, 14, 128, 192), (80, 16, 128, 64),
+                                          (60, 8, 192, 64), (100, 8, 256, 64)])
+@pytest.mark.parametrize("mode", ["two_pass", "dense", "fused", "fused_rescaled"])
+def test_conv_tile_shapes(B, H, Cin, Cout, mode):
+    """One and two strips side by side at every tile width, whole last rounds and partly filled ones."""
+    import paper_2202_00774_b200 as sdgp
+    layer = inputs.ConvLayer("t", B, H, H, Cin, Cout, 3, 3, 1, 1)
+    dO, W = inputs.conv_layer_tensors(layer, seed=B + Cin)
+    scheme = oracle.RESCALED if mode == "fused_rescaled" else oracle.MAGNITUDE
+    flags = {"two_pass": sdgp.FLAG_TWO_PASS, "dense": sdgp.FLAG_DENSE}.get(mode, sdgp.FLAG_FUSED)
+    ws = torch.empty(max(16, sdgp.sdgp_workspace_size_conv2d(B, H, H, Cin, Cout, 3, 3, 1, 1)), dtype=torch.uint8, device="cuda")
+    dD = torch.full(layer.dD_shape(), -1, dtype=torch.int16, device="cuda")
+    sdgp.sdgp_dgrad_conv2d(dev16(dO), dev16(W), dD, 1, 1, 2, 8, scheme, 6, workspace=ws, flags=flags)
+    check_no_device_error()
+    src = dO if mode == "dense" else oracle.prune(dO.reshape(-1, Cout), 2, 8, scheme, 6, want=("dense",))["dense"].reshape(dO.shape)
+    assert_close(to_f64(dD), *conv_ref(src, W, H, H, 1, 1))

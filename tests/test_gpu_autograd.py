@@ -104,23 +104,29 @@ def test_conv_relu_layer_backward_uses_the_producer(pool, Cout, n, m):
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
 @pytest.mark.parametrize("pool,shape", [(True, (2, 64, 128, 6, 10)), (True, (3, 64, 64, 8, 8)), (False, (2, 128, 64, 7, 9))])
 def test_conv_relu_pool_matches_the_separate_operators(dtype, pool, shape):
-    """Forward values (ReLU and pooling in one pass, a NaN in the input included) and both gradients with n = m, against torch's
-    own operators chained under autograd; the operands are 16-bit, sums fp32, so one rounding (2^-8 / 2^-11) with room for the order."""
+    """Forward values (ReLU and pooling in one pass, a NaN in the input included) and, without the NaN, both gradients with n = m, against
+    torch's own operators chained under autograd; the operands are 16-bit, sums fp32, so one rounding (2^-8 / 2^-11) with room for the
+    order. Equal maxima of a window: both give the gradient to the first."""
     from paper_2202_00774_b200 import autograd as sa
     B, Cin, Cout, H, W = shape
     g = torch.Generator(device="cuda").manual_seed(H * W)
     make = lambda *s: torch.randn(s, generator=g, device="cuda").to(dtype)   # noqa: E731
+
+    def both(x, w):
+        y = sa.sdgp_conv2d_relu(x, w, 1, 1, pool=pool, n=4, m=4)
+        ref = torch.relu(torch.nn.functional.conv2d(x, w, None, 1, 1))
+        ref = torch.nn.functional.max_pool2d(ref, 2) if pool else ref
+        assert torch.equal(torch.isnan(y), torch.isnan(ref)) and torch.equal(torch.nan_to_num(y, 0.0), torch.nan_to_num(ref, 0.0))
+        return y, ref
+
     x = make(B, Cin, H, W).contiguous(memory_format=torch.channels_last)
     w = (make(Cout, Cin, 3, 3) / 24).contiguous(memory_format=torch.channels_last)
-    if pool:
-        x[0, 0, 1, 1] = float("nan")
+    if pool:   # (where a NaN wins a window the gradients differ: a NaN passes nothing here)
+        with_nan = x.clone()
+        with_nan[0, 0, 1, 1] = float("nan")
+        assert torch.isnan(both(with_nan, w)[0]).any()
     x.requires_grad_(), w.requires_grad_()
-    y = sa.sdgp_conv2d_relu(x, w, 1, 1, pool=pool, n=4, m=4)
-    ref = torch.relu(torch.nn.functional.conv2d(x, w, None, 1, 1))
-    ref = torch.nn.functional.max_pool2d(ref, 2) if pool else ref
-    assert torch.equal(torch.isnan(y), torch.isnan(ref)) and torch.equal(torch.nan_to_num(y, 0.0), torch.nan_to_num(ref, 0.0))
-    if pool:
-        return   # (where a NaN wins a window the gradients differ: a NaN passes nothing here)
+    y, ref = both(x, w)
     dY = make(*y.shape)
     got, want = torch.autograd.grad(y, (x, w), dY), torch.autograd.grad(ref, (x, w), dY)
     for a, b in zip(got, want):

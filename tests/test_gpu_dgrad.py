@@ -54,6 +54,14 @@ def conv_ref(src, W, H, Wd, stride, pad, **kw):
             oracle.dgrad_conv2d(magnitudes(src), magnitudes(W), H, Wd, stride, pad, **kw))
 
 
+def assert_all_close_on_device(dD, src, W, dtype=torch.bfloat16, unit=2.0 ** -7):
+    """Every element of dD [rows, N] (bit patterns) against the product in fp64, computed on the device; bound as assert_close's."""
+    a, w = dev16(src).view(dtype).double(), dev16(W).view(dtype).double()
+    got, want = dD.view(dtype).double(), a @ w
+    off = ((got - want).abs() > unit * want.abs() + 2.0 ** -16 * (a.abs() @ w.abs())) | got.isnan()
+    assert not bool(off.any()), "%d elements off, first at %s" % (int(off.sum()), off.nonzero()[0].tolist())
+
+
 def check_no_device_error():
     import paper_2202_00774_b200 as sdgp
     assert sdgp.sdgp_last_device_error() == 0
@@ -686,6 +694,7 @@ def test_linear_tile_widths_and_row_tails(rows, K, N, offset):
         sdgp.sdgp_dgrad_linear(dev16(dO), dev16(W), dD, 2, 4, sdgp.MAGNITUDE, workspace=ws, flags=flags)
         check_no_device_error()
         assert_close(to_f64(dD)[pick], *linear_ref(A[pick], W))
+        assert_all_close_on_device(dD, A, W)
         edge = flat.cpu().numpy()
         assert np.all(edge[:offset] == 0x5A5A) and np.all(edge[offset + rows * N:] == 0x5A5A)
 
@@ -695,18 +704,19 @@ def test_linear_tile_widths_and_row_tails(rows, K, N, offset):
 
 @pytest.mark.parametrize("scheme", [oracle.RANDOM, oracle.MAGNITUDE, oracle.RESCALED])
 @pytest.mark.parametrize("rows,K,N,n,m", [(1, 64, 64, 2, 4), (257, 192, 448, 1, 4), (700, 1216, 320, 2, 8), (20000, 128, 128, 2, 16),
-                                          (20100, 320, 576, 2, 4), (500, 128, 64, 2, 32), (4000, 256, 1024, 1, 32)])
+                                          (20100, 320, 576, 2, 4), (500, 128, 64, 2, 32), (4000, 256, 1024, 1, 32), (60000, 384, 64, 2, 8)])
 def test_linear_pruned_on_the_way(rows, K, N, n, m, scheme):
     """Row tails, a last channel block of one to four MMAs, more channel blocks than stages, one and several column tiles and groups
     per CTA pair, several works per pair, every group size; fused mode, two-pass mode (whichever kernel it takes) and the same
-    call from a thread of its own."""
+    call from a thread of its own. Some rows against the oracle's contraction, every element against the device's fp64 product of the
+    oracle-pruned gradient."""
     import threading
     import paper_2202_00774_b200 as sdgp
     dO, W = inputs.fc_tensors(rows, K, N, seed=rows + K)
     ws = torch.empty(max(16, sdgp.sdgp_workspace_size_linear(rows, K, N)), dtype=torch.uint8, device="cuda")
     pick = np.unique(np.concatenate([np.arange(min(rows, 40)), np.arange(max(0, rows - 200), rows)]))   # whole rows
-    pruned = oracle.prune(dO, n, m, scheme, 9, want=("dense",))["dense"][pick]
-    ref = linear_ref(pruned, W)
+    pruned = oracle.prune(dO, n, m, scheme, 9, want=("dense",))["dense"]
+    ref = linear_ref(pruned[pick], W)
     flat = torch.full((rows * N + 64,), 0x5A5A, dtype=torch.int16, device="cuda")
     dD, a, b = flat[:rows * N].view(rows, N), dev16(dO), dev16(W)
     calls = [lambda: sdgp.sdgp_dgrad_linear(a, b, dD, n, m, scheme, 9, workspace=ws)]
@@ -720,7 +730,24 @@ def test_linear_pruned_on_the_way(rows, K, N, n, m, scheme):
         t.join()
         check_no_device_error()
         assert_close(to_f64(dD)[pick], *ref)
+        assert_all_close_on_device(dD, pruned, W)
         assert np.all(flat[rows * N:].cpu().numpy() == 0x5A5A)
+
+
+@pytest.mark.parametrize("rows,K,N,n,m", [(20000, 128, 128, 2, 16), (12000, 192, 256, 2, 4), (30000, 64, 320, 1, 8)])
+def test_linear_two_pass_binary16_rescaled_every_element(rows, K, N, n, m):
+    """Sizes at which two-pass calls prune on the way; binary16 with the rescaled function exists there only for them. (One rounding to
+    binary16 is 2^-11, a factor two to spare.)"""
+    import paper_2202_00774_b200 as sdgp
+    rng = np.random.default_rng(rows)
+    dO = rng.standard_normal((rows, K), dtype=np.float32).astype(np.float16).view(np.uint16)
+    W = (rng.standard_normal((K, N), dtype=np.float32) / np.float32(K ** 0.5)).astype(np.float16).view(np.uint16)
+    ws = torch.empty(max(16, sdgp.sdgp_workspace_size_linear(rows, K, N)), dtype=torch.uint8, device="cuda")
+    dD = torch.full((rows, N), 0x7E00, dtype=torch.int16, device="cuda")
+    sdgp.sdgp_dgrad_linear_typed(dev16(dO), dev16(W), dD, n, m, sdgp.RESCALED_MAGNITUDE, 9, sdgp.FP16, workspace=ws)
+    check_no_device_error()
+    pruned = oracle.prune(dO, n, m, oracle.RESCALED, 9, want=("dense",), dtype=oracle.FP16)["dense"]
+    assert_all_close_on_device(dD, pruned, W, torch.float16, 2.0 ** -10)
 
 
 @pytest.mark.parametrize("B,H,Wd,Cin,Cout,R,pad", [(3, 5, 5, 64, 64, 3, 1), (5, 7, 7, 192, 192, 3, 1), (2, 7, 6, 128, 64, 3, 0), (3, 9, 11, 64, 128, 3, 1),

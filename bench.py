@@ -73,18 +73,22 @@ def layer_inputs(l, workload, seed, dtype="bf16"):
 # resnet9 two-pass step, from the ncu capture summarised in profiles/traffic_dgrad_sparse_resnet9.md,
 # and the hash of the kernel sources it was taken with (the figure is dropped once they change).
 NCU_TRAFFIC = {"workload": "resnet9", "mode": "two_pass", "bytes_per_step": 213.0e6, "sources_sha": "9e2b4e39f6d4dd4c"}
-KERNEL_SOURCES = ["dgrad.cu", "dgrad_common.cuh", "dgrad_general.cu", "dgrad_general.cuh", "dgrad_halo.cuh", "dgrad_halo_params.cuh", "ptx.cuh"]   # all the code of the non-fused data-gradient kernels
+# everything that the kernels of a two-pass data gradient are compiled from
+KERNEL_SOURCES = ["dgrad.cu", "dgrad_common.cuh", "dgrad_general.cu", "dgrad_general.cuh", "dgrad_halo.cuh", "dgrad_halo_dense.cu",
+                  "dgrad_halo_params.cuh", "dgrad_halo_sparse.cu", "dgrad_prune.cuh", "dgrad_rows.cu", "dgrad_rows.cuh", "prune.cu",
+                  "prune_core.cuh", "ptx.cuh", "sdgp_internal.cuh"]
 
 
 def kernel_sources_sha():
     """Hash of the data-gradient kernels' code with comments and blank lines left out (a comment edit is not a
-    changed kernel)."""
+    changed kernel; a file that is gone or renamed is a changed one)."""
     import hashlib
     import re
     h = hashlib.sha256()
     for f in KERNEL_SOURCES:
         path = os.path.join(ROOT, "paper_2202_00774_b200", "csrc", f)
         if not os.path.exists(path):
+            h.update(b"no " + f.encode() + b"\n")
             continue
         with open(path) as fh:
             for line in fh:

@@ -89,6 +89,14 @@ def test_kernel_sources_hash_ignores_comments_but_not_code(monkeypatch, tmp_path
     assert write("int x = 1;\nint z;\n", ptx="int y = 0;\n") != base
 
 
+def test_kernel_sources_exist_and_a_missing_one_changes_the_hash(monkeypatch):
+    csrc = os.path.join(bench.ROOT, "paper_2202_00774_b200", "csrc")
+    assert all(os.path.exists(os.path.join(csrc, f)) for f in bench.KERNEL_SOURCES)
+    base = bench.kernel_sources_sha()
+    monkeypatch.setattr(bench, "KERNEL_SOURCES", bench.KERNEL_SOURCES + ["renamed.cu"])
+    assert bench.kernel_sources_sha() != base
+
+
 def test_traffic_is_reported_only_for_the_sources_it_was_measured_on(monkeypatch):
     assert bench.measured_traffic("gemm_large", "two_pass") is None
     assert bench.measured_traffic("resnet9", "fused") is None

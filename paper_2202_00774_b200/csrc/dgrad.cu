@@ -229,8 +229,8 @@ PruneCost prune_cost(int m, int scheme) {
 // Stride 2 is split by the parity of the output pixel: pixel (2h'+ph, 2w'+pw) only meets the taps
 // r = ph + pad (mod 2), s = pw + pad (mod 2), and on those it is a stride-1 problem from dO to
 // the strided view dD[:, ph::2, pw::2, :].
-// fused != nullptr (with sparse == true): A is the DENSE dL/dO and the kernel prunes it itself
-// (m = 4, n = fused->n in {1, 2}); no compressed tensor exists in global memory.
+// fused != nullptr (with sparse == true): A is the DENSE dL/dO and the kernel prunes it itself (n = 1 or 2; m = 4, 8 or 16, in the
+// strip kernel also 32); no compressed tensor exists in global memory.
 sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const void* Wt, void* dD, int B,
                          int H, int W, int Cin, int Cout, int R, int S, int stride, int pad, cudaStream_t stream,
                          const FusedPrune* fused, int dtype, const StoredChannels* stored, const ConvGroups* conv_groups) {

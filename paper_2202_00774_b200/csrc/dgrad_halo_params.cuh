@@ -64,7 +64,7 @@ struct HaloParams {
   int m0_bytes, meta_bytes;  // bytes of master 0; of both (one A stage)
   int off_eraw, off_meta, off_w, off_out, off_bar;
   int smem_bytes;
-  // fused pruning (A is the dense dL/dO; m = 4): the pruning warps read it straight from global memory
+  // fused pruning (A is the dense dL/dO): the pruning warps read it straight from global memory
   const uint8_t* a_dense;  // dL/dO [B, P, Q, Cout], 16-bit elements
   int diag_cin_g, diag_cout_g, diag_last;  // grouped convolution: see first_k_block()
   uint32_t pitch_magic;    // ceil(2^20 / pitch): i / pitch == (i * pitch_magic) >> 20 for every box pixel row i

@@ -1,11 +1,9 @@
 // N:M pruning of the output data gradient (Algorithm 1, Section 3.2), sm_100a.
 //
-// One thread owns one aligned run of 8 bf16 elements (a single 128-bit load). Groups of
-// m = 4 (two per thread) and m = 8 (one per thread) are ranked inside the thread; groups of
-// 16 and 32 span 2 and 4 neighbouring lanes, which trade their keys with warp shuffles.
-// The kernel is a pure stream: 2 B read per element, 1 B of compressed values, 1/8 B of
-// position metadata (+ 1/8 B mask, + 2 B dense copy when asked for), every output indexed by
-// the same 8-element vector number so all stores coalesce.
+// A thread owns pairs of aligned runs of 8 elements (a 256-bit load each); where a dense copy is asked for, and below a pooling, single
+// runs of 8. Groups of m = 4, 8 and 16 are ranked inside the thread (16: single runs span two lanes); groups of 32 span two lanes
+// (four), which trade their keys with warp shuffles. The kernel is a pure stream: 2 B read per element, 1 B of compressed values, 1/8 B of
+// position metadata (+ 1/8 B mask, + 2 B dense copy when asked for), every output indexed by the run's number so all stores coalesce.
 #include <cuda_bf16.h>
 
 #include "prune_core.cuh"
@@ -188,13 +186,6 @@ __device__ __forceinline__ void load_unit(const uint4* __restrict__ dO, int64_t 
     }
   }
 }
-
-// ------------------------------------------------------------------------------------------
-// m = 4 fast path. The two groups of a vector are processed as 16-bit SIMD lanes of one
-// register: p_i = (element i of group A, element i of group B). Pairwise "i beats j" flags
-// come from one packed subtraction each, the keep decision is one 3-input logic op per
-// element (a threshold on the number of wins), and the compressed slots / position nibbles
-// are computed on both lanes at once. About a quarter of the instructions of the generic path.
 
 // Row pitch of the metadata in pairs of vectors (two bytes each): k16 per input row, kpad16 per output row (kpad16 == 0: same as
 // the input). A reader that takes rows by TMA needs whole 16-byte rows of metadata; the values need no padding.

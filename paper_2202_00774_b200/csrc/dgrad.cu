@@ -383,10 +383,11 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
 namespace {
 
 // Two-pass calls over rows: the kernel that prunes inside the contraction replaces prune kernel + contraction where it is
-// estimated to be faster. Estimate of the pair, us: 1.5 + 4 for two launches' ramps, the prune kernel's bytes at 6.4 TB/s or its
-// arithmetic, and the contraction's bytes, operand traffic from L2 or products. Few channels (one launch less, no second read of dO)
-// favour the rows kernel, many channels on few rows the pair (a CTA pair prunes its blocks one after another). On 70 drawn
-// layers the estimates put the faster one first wherever the two differed by more than a tenth, but for a handful.
+// estimated to be faster. Estimate of the pair, us: 4 for two launches' ramps, the prune kernel's bytes at 6.4 TB/s or its
+// arithmetic, and the contraction's bytes, operand traffic from L2 or products; of the one kernel, 0.8 of plan_rows()'s clocks. Few channels
+// (one launch less, no second read of dO) favour the rows kernel, many channels on few rows the pair (a CTA pair prunes its blocks one after
+// another). Of 1540 drawn layers timed both ways the estimate picks a kernel more than 5 % behind the other on 76, more than 10 % on 31, 0.6 % in
+// the mean; with 5.5 and 0.9, from when the pair was slower, 140, 73 and 1.2 %.
 bool rows_fused_pays(int64_t rows, int K, int N, int m, int scheme, RowsPlan* plan) {
   const PruneCost pc = prune_cost(m, scheme);
   *plan = plan_rows(rows, K, N, pc.stage_clk);
@@ -400,7 +401,7 @@ bool rows_fused_pays(int64_t rows, int K, int N, int m, int scheme, RowsPlan* pl
   const double mem = (1.125 * e + 2.0 * out) / 6.0e6, mma = 2.0 * e * N / 2.0e9;
   double contraction = mem > l2 ? mem : l2;
   if (mma > contraction) contraction = mma;
-  return plan->cost / 1900.0 * 0.9 < 5.5 + prune + contraction;
+  return plan->cost / 1900.0 * 0.8 < 4.0 + prune + contraction;
 }
 
 }  // namespace

@@ -146,11 +146,11 @@ int k_window(int bn, int channels, int all, int kbc, int Cout, const ConvGroups*
   return widest > 0 && widest < all ? widest : all;
 }
 
-// Input channels per tile. A tile's main loop is bound by the bytes an SM pulls in from L2 per channel block (16 KB of A, and
+// Input channels per tile of the general kernel. A tile's main loop is bound by the bytes an SM pulls in from L2 per channel block (16 KB of A, and
 // W in proportion to BN) and it has a fixed part, so a round of tiles costs about k_blocks * (256 + 2 BN) + 256 units; the last tile
 // of a row may be partly empty (columns past the stored channels are computed and not stored). Narrow tiles win where there
 // are too few for every CTA pair (1777 x 1088 . 1088 x 832: 14.7 -> 10.9 us), 192 where 128 or 256 would leave a third of the columns
-// idle or double the tiles (192 -> 192 at 28 x 28: 50 -> 40 us; 10736 x 1152 . 1152 x 576: 31 -> 19 us, all prune included).
+// idle or double the tiles (10736 x 1152 . 1152 x 576: 31 -> 19 us, prune included).
 int choose_bn(int64_t m_tiles, int channels, int all, int kbc, int Cout, const ConvGroups* groups) {
   const int64_t pairs = sm_count() / 2, rows = (m_tiles + 1) / 2;
   int best = 64;

@@ -12,7 +12,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsdgp.so")
 SOURCES = ["prune.cu", "rank.cu", "dgrad.cu", "dgrad_general.cu", "dgrad_halo_sparse.cu", "dgrad_halo_dense.cu",
-           "dgrad_halo_fused.cu", "dgrad_rows.cu", "api.cu", "static_scratch.cu", "channel.cu", "grouped.cu"]
+           "dgrad_halo_fused.cu", "dgrad_rows.cu", "dgrad_grouped.cu", "api.cu", "static_scratch.cu", "channel.cu", "grouped.cu"]
 BINDING = os.path.join(HERE, "_sdgp_torch.so")
 BINDING_SOURCES = [os.path.join(CSRC, f) for f in ("torch_binding.cpp", "torch_autograd.cpp")]
 HEADERS = ["ptx.cuh", "sdgp_internal.cuh", "prune_core.cuh", "dgrad_common.cuh", "dgrad_general.cuh", "dgrad_halo.cuh",

@@ -320,6 +320,11 @@ sdgp_status sdgp_dgrad_conv2d_grouped(const void* dO, const void* W, void* dD, i
     const sdgp_status st = sdgp::try_rows_fused(dO, W, dD, (int64_t)B * H * Wd, Cout, Cin, {n, m, (int)scheme, seed}, dt, s, &taken);
     if (taken) return st;
   }
+  if (prunes && flags == SDGP_FLAG_TWO_PASS && groups > 1 && Cin == Cout) {
+    // narrow groups: pruned and multiplied in one kernel that reads the groups' filters as they are
+    const sdgp_status st = sdgp::launch_grouped_fused(dO, W, dD, B, H, Wd, Cin, groups, R, S, stride, pad, {n, m, (int)scheme, seed}, dt, s);
+    if (st != SDGP_ERR_UNSUPPORTED) return st;
+  }
   const void* w_full = W;  // one group and whole 64-channel blocks: the filters are already in the kernels' form
   void* rest = (uint8_t*)workspace + w_bytes;
   if (groups > 1 || Cin != cin_k || Cout != cout_k) {

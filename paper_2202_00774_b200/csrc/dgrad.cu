@@ -435,7 +435,7 @@ sdgp_status read_device_error() {
   if (cudaDeviceSynchronize() != cudaSuccess) return SDGP_ERR_CUDA;
   bool timed_out = false;
   cudaError_t (*const words[])(unsigned int*) = {take_error_word, take_error_general, take_error_halo_sparse, take_error_halo_dense,
-                                                 take_error_halo_fused, take_error_rows};
+                                                 take_error_halo_fused, take_error_rows, take_error_grouped};
   for (auto take : words) {
     unsigned int word = 0;
     if (take(&word) != cudaSuccess) return SDGP_ERR_CUDA;

@@ -99,6 +99,12 @@ sdgp_status try_rows_fused(const void* dO, const void* W, void* dD, int64_t rows
 cudaError_t launch_expand_grouped_weights(const void* Wg, int Cout, int taps, int Cin, int groups, int cout_pad, int cin_pad,
                                           void* Wfull, cudaStream_t stream);
 
+// Data gradient of a grouped convolution with C channels on both sides, pruned inside the kernel (n <= 2); Wg [C, R, S, C / groups].
+// SDGP_ERR_UNSUPPORTED (nothing launched): groups of other widths than 16 or 32 channels, filters or images that no plan fits.
+sdgp_status launch_grouped_fused(const void* dO, const void* Wg, void* dD, int B, int H, int W, int C, int groups, int R, int S, int stride,
+                                 int pad, const FusedPrune& prune, int dtype, cudaStream_t stream);
+cudaError_t take_error_grouped(unsigned int* word);
+
 // Launches a one-CTA kernel whose only wait can never be satisfied (50 ms limit).
 sdgp_status launch_bounded_wait_selftest(cudaStream_t stream);
 

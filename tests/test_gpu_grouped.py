@@ -119,3 +119,21 @@ def test_argument_errors():
     with pytest.raises(sdgp.SdgpError) as e:      # 4 input channels per group: below one 16-byte vector
         sdgp.sdgp_dgrad_conv2d_grouped(dev16(dO), dev16(W[..., :4].copy()), dD, 1, 1, 8, 2, 4, sdgp.MAGNITUDE, workspace=ws)
     assert e.value.status == 2
+
+
+# The kernel for narrow groups (16 or 32 channels on both sides): widths, partial blocks of 64 channels, lines shorter and longer than
+# a round of units, odd and uneven images, filters with fewer and more taps, every group size of the pruning functions
+@pytest.mark.parametrize("B,H,Wd,C,R,S,stride,pad,groups,n,m,scheme", [
+    (1, 4, 4, 32, 3, 3, 1, 1, 2, 2, 4, oracle.MAGNITUDE),       # one unit, one block that is half empty
+    (1, 5, 3, 48, 1, 3, 1, 0, 3, 1, 8, oracle.RESCALED),        # three slices of a block, one row of taps
+    (3, 13, 27, 112, 3, 3, 2, 1, 7, 2, 4, oracle.RANDOM),       # four classes of uneven size
+    (2, 9, 12, 96, 5, 5, 1, 2, 3, 2, 32, oracle.RESCALED),      # groups of 32 on both sides of the pruning, 25 taps
+    (2, 10, 7, 64, 3, 3, 1, 2, 4, 2, 16, oracle.RANDOM),        # padding of a whole filter: dL/dO is larger than dD
+    (2, 11, 11, 160, 3, 3, 1, 0, 5, 2, 32, oracle.MAGNITUDE),   # no padding: dL/dO is smaller; groups of 32, two blocks and a half
+    (1, 3, 260, 32, 3, 3, 1, 1, 2, 2, 4, oracle.MAGNITUDE),     # rows too long for a box: the other path
+    (170, 14, 14, 176, 3, 3, 1, 1, 11, 2, 4, oracle.RESCALED),  # several units of every multiprocessor, a last block of 48 channels
+])
+def test_narrow_groups(B, H, Wd, C, R, S, stride, pad, groups, n, m, scheme):
+    import paper_2202_00774_b200 as sdgp
+    layer = inputs.ConvLayer("narrow", B, H, Wd, C, C, R, S, stride, pad, groups)
+    run(layer, n, m, scheme, sdgp.FLAG_TWO_PASS)

@@ -210,6 +210,44 @@ double halo_cost(int B, int H, int W, int R, int S, int bn, int nt, bool sparse,
   return (double)rounds * (k_blocks * boxes * box + 4.3 + 0.5 * columns);
 }
 
+// The same for the four output parities of a stride-2 convolution in one launch, the mean over them per unit; H, W: their largest images,
+// R, S: the whole filter. A unit's stores take at least 2.2 per 64 columns (they are what bounds parities of one or two taps).
+double halo_cost_classes(int B, int H, int W, int R, int S, int pad, int bn, int nt, bool sparse, int tiles_n, int k_blocks) {
+  if (nt * bn > 256 || (nt == 2 && W <= 8)) return 0.0;
+  const int th = H <= 8 ? 8 : kHaloRows, tb = kHaloRows / th;
+  const int sets_w = (W + 8 * nt - 1) / (8 * nt), tiles_h = (H + th - 1) / th;
+  const int64_t sets = (int64_t)sets_w * tiles_h * ((B + tb - 1) / tb);
+  const int64_t pairs = sm_count() / 2, rounds = ((sets + 1) / 2 * tiles_n * 4 + pairs - 1) / pairs;
+  const double columns = nt * bn / 64.0, img_rows = (8 * nt + (S + 1) / 2 - 1) * (th + (R + 1) / 2 - 1) * tb;
+  double sum = 0.0;
+  for (int c = 0; c < 4; ++c) {
+    const int Rc = (R - ((c >> 1) + pad) % 2 + 1) / 2, Sc = (S - ((c & 1) + pad) % 2 + 1) / 2;
+    const double box = Rc * Sc * (1.0 + columns * (sparse ? 0.125 : 0.0625)) + 0.003 * img_rows;
+    const double main_loop = k_blocks * box, stores = 2.2 * columns;
+    sum += (main_loop > stores ? main_loop : stores) + 4.3 + 0.5 * columns;
+  }
+  return (double)rounds * sum / 4.0;
+}
+
+// Whether one launch for the four parities is faster than one each. It saves three launches and reads of dL/dO, some 25 us, but its strips
+// are laid out for the largest parity's images, where the general kernel's patches, which most classes of small images get otherwise, fit
+// each parity's (some 125 %); and with a dense A the general kernel is the faster one per product. The constants (us per 1e9 products, one
+// launch and four) follow 34 layers timed both ways. Us, four launches -> one, prune kernel included, sparse: 265 x 13 x 13 images, 896 -> 896
+// (160 % covered) 122 -> 156; 60 x 20 x 20, 512 -> 512 (256 %) 41 -> 48; 325 x 27 x 27, 128 -> 128 54 -> 34; 479 x 14 x 14, 448 -> 256 68 -> 49;
+// 18 x 32 x 32, 384 -> 128 25 -> 10. Dense after pruning: 64 x 27 x 27, 896 -> 896 212 -> 264; 256 x 16 x 16, 512 -> 512 (100 %) 100 -> 83.
+bool classes_pay(int B, int H, int W, int Cin, int Cout, int R, int S, int pad, bool sparse) {
+  const int H0 = (H + 1) / 2, W0 = (W + 1) / 2, th = H0 <= 8 ? 8 : kHaloRows;
+  const double covered = (double)((W0 + 7) / 8 * 8) * ((H0 + th - 1) / th * th);
+  double one = 0.0, four = 0.0;  // positions times taps
+  for (int c = 0; c < 4; ++c) {
+    const int ph = c >> 1, pw = c & 1, taps = ((R - (ph + pad) % 2 + 1) / 2) * ((S - (pw + pad) % 2 + 1) / 2);
+    one += taps * covered;
+    four += (double)taps * ((H - ph + 1) / 2) * ((W - pw + 1) / 2);
+  }
+  const double excess = sparse ? 0.87 * one - 1.09 * four : 1.05 * one - 0.96 * four;
+  return 2.0e-9 * excess * B * Cin * Cout < (sparse ? 25.0 : 20.0);
+}
+
 // What pruning costs (measured on a [16384 x 4096] tensor and on 50176 x 1024 rows): clocks of the rows kernel's pruning warps per block of
 // 128 channels, picoseconds per element of the prune kernel where the integer pipe bounds it.
 struct PruneCost {
@@ -270,6 +308,57 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
   view.d.channels = (stored && stored->d) ? stored->d : Cin;
   view.w_cols = (int64_t)R * S * Cin;
   const size_t Cd = (size_t)view.d.channels;
+
+  // All four output parities of a strided layer in one launch of the strip kernel, where its strips cover their images well enough (the
+  // same bounds as for a filter of its size at stride 1) and that is estimated to be faster.
+  if (stride == 2 && !fused && R >= 2 && S >= 2 && W > 8 && halo_applies((H + 1) / 2, (W + 1) / 2, R * S, sparse, false) &&
+      classes_pay(B, H, W, view.d.channels, view.a_channels, R, S, pad, sparse)) {
+    HaloParams hp = {};
+    hp.B = B; hp.H = (H + 1) / 2; hp.W = (W + 1) / 2; hp.Cin = Cin; hp.Cout = Cout;
+    hp.r_step = hp.s_step = 2;
+    hp.S_full = S;
+    hp.P = P; hp.Q = Q;
+    hp.f16 = dtype == SDGP_FP16 ? 1 : 0;
+    hp.last_launch = 1;
+    hp.classes = 4;
+    for (int c = 0; c < 4; ++c) {
+      HaloClass& k = hp.cls[c];
+      const int ph = c >> 1, pw = c & 1;
+      k.r_first = (ph + pad) % 2; k.s_first = (pw + pad) % 2;
+      k.R = (R - k.r_first + 1) / 2; k.S = (S - k.s_first + 1) / 2;
+      k.pad_h = (ph + pad - k.r_first) / 2; k.pad_w = (pw + pad - k.s_first) / 2;
+      k.H = (H - ph + 1) / 2; k.W = (W - pw + 1) / 2;
+      hp.R = k.R > hp.R ? k.R : hp.R;
+      hp.S = k.S > hp.S ? k.S : hp.S;
+    }
+    const int blocks = (Cout + kb_channels - 1) / kb_channels;
+    hp.k_last = blocks - 1;
+    const int left = view.a_channels - hp.k_last * kb_channels, per_mma = kb_channels / 4;
+    hp.last_mmas = left < kb_channels ? (left + per_mma - 1) / per_mma : 4;
+    view.d.base = (uint8_t*)dD;
+    view.d.sw = 2 * (int64_t)Cd * 2;
+    view.d.sh = 2 * (int64_t)W * Cd * 2;
+    view.d.sb = (int64_t)H * W * Cd * 2;
+    view.d.aligned32 = 0;
+    struct Shape { int bn, nt; double cost; } shapes[] = {{64, 1, 0}, {64, 2, 0}, {128, 1, 0}, {128, 2, 0}, {192, 1, 0}, {256, 1, 0}};
+    for (Shape& s : shapes) {
+      const double cost = halo_cost_classes(B, hp.H, hp.W, R, S, pad, s.bn, s.nt, sparse, (view.d.channels + s.bn - 1) / s.bn,
+                                            k_window(s.bn, view.d.channels, blocks, kb_channels, Cout, conv_groups));
+      s.cost = cost > 0.0 ? cost : 1e9;
+    }
+    std::sort(std::begin(shapes), std::end(shapes), [](const Shape& a, const Shape& b) { return a.cost < b.cost; });
+    for (const Shape& s : shapes) {
+      hp.tiles_n = (view.d.channels + s.bn - 1) / s.bn;
+      hp.k_blocks = k_window(s.bn, view.d.channels, blocks, kb_channels, Cout, conv_groups);
+      hp.diag_cin_g = hp.diag_cout_g = hp.diag_last = 0;
+      if (hp.k_blocks < blocks) {
+        hp.diag_cin_g = conv_groups->cin_g; hp.diag_cout_g = conv_groups->cout_g;
+        hp.diag_last = blocks - hp.k_blocks;
+      }
+      const sdgp_status st = sparse ? launch_halo_sparse(s.bn, s.nt, A, meta, Wt, view, hp, stream) : launch_halo_dense(s.bn, s.nt, A, Wt, view, hp, stream);
+      if (st != SDGP_ERR_UNSUPPORTED) return st;
+    }
+  }
 
   // Output parities that no tap reaches are zero: clear dD first if there is any such class.
   bool any_empty = false;
@@ -344,6 +433,7 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
       sdgp_status st = SDGP_ERR_UNSUPPORTED;
       if (halo_applies(Hs, Ws, p.R * p.S, sparse, fused != nullptr)) {
         HaloParams hp = {};
+        hp.classes = 1;
         hp.B = B; hp.H = Hs; hp.W = Ws; hp.Cin = Cin; hp.Cout = Cout;
         hp.R = p.R; hp.S = p.S; hp.pad_h = p.pad_h; hp.pad_w = p.pad_w;
         hp.r_first = p.r_first; hp.r_step = p.r_step; hp.s_first = p.s_first; hp.s_step = p.s_step;

@@ -36,13 +36,17 @@ constexpr int kHaloAStages = 4;  // at most: A stages in use are p.a_stages = 2,
 constexpr int kPruneWarps = 18;
 constexpr int kThreadsHaloFused = 24 * 32;
 
-// PATCH (not fused): strips leave as one TMA box each (store_patch), else as rows; plan_halo() has the rule. Two kernels, so that
-// neither carries the other's code.
+// PATCH (not fused): strips leave as one TMA box each (store_patch), else as rows; plan_halo() has the rule. Such a launch may also hold
+// the four output parities of a stride-2 convolution (p.classes == 4): a work unit is then a tile set of one parity. The four of a
+// tile are neighbouring units, so that its dL/dO comes from memory once and the pixels of dD that lie side by side are stored at
+// about the same time; which of them falls to which CTA pair turns from tile to tile, for they have one, two, two and four taps. Us, 128 -> 128
+// channels at 56 x 56, batch 256, random pruning included: four launches 104, this 92. Two kernels, so that neither carries the
+// other's code.
 template <bool SPARSE, int BN, int NT, bool FUSED, bool PATCH>
 __global__ void __launch_bounds__(FUSED ? kThreadsHaloFused : kThreadsGemm, 1)
 dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmE,
-                  const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmD,
-                  const HaloParams p) {
+                  const __grid_constant__ CUtensorMap tmB, const __grid_constant__ HaloOutMaps<PATCH> tmD,
+                  const __grid_constant__ HaloParams p) {
   using C = Cfg<SPARSE, BN>;
   constexpr int kEpilogueWarp0 = FUSED ? 4 : 6;  // first of the four epilogue warps
   extern __shared__ uint8_t smem_raw[];
@@ -92,7 +96,7 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   if (warp == 0 && lane == 0) {
     ptx::prefetch_tensormap(&tmA);
     ptx::prefetch_tensormap(&tmB);
-    if (PATCH) ptx::prefetch_tensormap(&tmD);
+    if (PATCH) ptx::prefetch_tensormap(&tmD.m[0]);
     if (SPARSE) ptx::prefetch_tensormap(&tmE);
   }
   if (warp == 1) {
@@ -113,9 +117,21 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   // to free its columns, which it does without anyone's help.
   if (p.early) ptx::launch_dependents();
 
-  const int taps = p.R * p.sb;  // filter taps served by one A box
   const int pair_stride = gridDim.x >> 1;
   const int first_pair = blockIdx.x >> 1;
+  // pair tile (p.classes == 4: and output parity) of unit number lt of this CTA
+  auto unit_of = [&p, first_pair, pair_stride](int lt, int& c) -> int {
+    c = 0;
+    const int u = first_pair + lt * pair_stride;
+    const int pt = u < p.split_from ? u : p.split_from + ((u - p.split_from) >> 1);
+    if (!PATCH || p.classes == 1) return pt;
+    c = (pt + (pt >> 2)) & 3;
+    return pt >> 2;
+  };
+  auto class_of = [&p](int c) -> HaloClass {
+    if (PATCH) return p.cls[c];
+    return HaloClass{p.R, p.S, p.sb, p.pad_h, p.pad_w, p.r_first, p.s_first, p.H, p.W};
+  };
   const int my_tiles = first_pair < p.units ? (p.units - first_pair + pair_stride - 1) / pair_stride : 0;
   const int n_half = (int)rank * C::kBCols;
   constexpr int set_cols = NT * BN;  // TMEM columns of one tile set's accumulators
@@ -126,9 +142,9 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     const int u = first_pair + lt * pair_stride;
     return u < p.split_from ? ((1u << NT) - 1u) : (1u << ((u - p.split_from) & 1));
   };
-  // tile set of unit `u` for this CTA: first input channel, first pixel column / row, image
-  auto locate = [&p, rank](int u, int& n0, int& w0, int& h0, int& b0) -> bool {
-    const int pt = u < p.split_from ? u : p.split_from + ((u - p.split_from) >> 1);
+  // tile set of unit number lt for this CTA: first input channel, first pixel column / row, image; its parity
+  auto locate = [&p, rank, &unit_of](int lt, int& n0, int& w0, int& h0, int& b0, int& c) -> bool {
+    const int pt = unit_of(lt, c);
     uint32_t q, r;
     divmod((uint32_t)pt, (uint32_t)p.tiles_n, p.mg_tiles_n, q, r);
     n0 = (int)r * BN;
@@ -161,10 +177,11 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
         const int lt = ia / p.k_uses, ku = ia - lt * p.k_uses;
         const int kl = ku / p.ss, si = ku - kl * p.ss;  // channel block of the tile's window, filter column of the box (column-split mode)
-        int n0, w0, h0, b0;
-        locate(first_pair + lt * pair_stride, n0, w0, h0, b0);
+        int n0, w0, h0, b0, c;
+        locate(lt, n0, w0, h0, b0, c);
         const int kb = first_k_block(p, n0, C::kKB) + kl;
-        const int q0 = w0 + p.pad_w - (p.sb - 1) - si, p0 = h0 + p.pad_h - (p.R - 1);
+        const HaloClass cl = class_of(c);
+        const int q0 = w0 + cl.pad_w - (cl.sb - 1) - si, p0 = h0 + cl.pad_h - (cl.R - 1);
         // coordinates: channel, pixel column, image within a box row, image group, pixel row
         const int bg = b0 / p.img_per_row;
         if (rank == 0) ptx::mbar_arrive_expect_tx(&a_full[ast], a_tx);
@@ -184,10 +201,12 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       int wst = 0, use = 0;
       uint32_t wph = 0;
       for (int lt = 0; alive && lt < my_tiles; ++lt) {
-        int n0, w0_unused, h0_unused, b0_unused;
-        locate(first_pair + lt * pair_stride, n0, w0_unused, h0_unused, b0_unused);
+        int n0, w0_unused, h0_unused, b0_unused, c;
+        locate(lt, n0, w0_unused, h0_unused, b0_unused, c);
         const int kb0 = first_k_block(p, n0, C::kKB);
         n0 += n_half;
+        const HaloClass cl = class_of(c);
+        const int taps = cl.R * cl.sb;  // filter taps served by one A box
         for (int ku = 0; alive && ku < p.k_uses; ++ku, ++use) {
           const int kl = ku / p.ss, si = ku - kl * p.ss, kb = kb0 + kl;
           // (fused: the pruning warps fetch dL/dO themselves; this thread streams W only)
@@ -198,8 +217,8 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             if (!FUSED && ia < a_uses && ia < use + p.a_stages && issue_a(false) < 0) { alive = false; break; }
             if (!ptx::mbar_wait<kIdleWaitNs>(&w_empty[wst], wph ^ 1u, err, 0x180u + wst)) { alive = false; break; }
             if (rank == 0) ptx::mbar_arrive_expect_tx(&w_ready[wst], w_tx);
-            const int r = t / p.sb, s = t - r * p.sb + si;
-            const int ft = (p.r_first + p.r_step * r) * p.S_full + p.s_first + p.s_step * s;
+            const int r = t / cl.sb, s = t - r * cl.sb + si;
+            const int ft = (cl.r_first + p.r_step * r) * p.S_full + cl.s_first + p.s_step * s;
 #pragma unroll
             for (int j = 0; j < C::kBoxes; ++j)
               ptx::tma_load_2d_pair(sW + wst * p.w_bytes + j * C::kBoxBytes, &tmB, &w_ready[wst],
@@ -236,8 +255,6 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const int off = dr * p.tb;  // box rows
         return ((off & 1) ? m1_off16 : 0u) + (uint32_t)((off >> 1) * 2 * p.pitch);
       };
-      const uint32_t a_first16 = (uint32_t)(((p.R - 1) * p.tb * p.pitch + (p.sb - 1)) * 8);  // tap (0,0), in 16-byte units
-      const uint32_t a_rowstep16 = (uint32_t)((p.tb * p.pitch - (p.sb - 1)) * 8);            // last tap of a filter row -> first of the next
       constexpr uint32_t kBStep = (uint32_t)((C::kKB / 4) * C::kRowB / 16);  // W rows of one MMA
       constexpr uint32_t kSlotCols = 4u * NT;                                // metadata columns of one W stage
       bool alive = true;
@@ -257,6 +274,12 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const uint32_t meta_base = tmem_base + (uint32_t)(p.meta_shared ? (acc ^ 1) * set_cols : p.meta_col);
         ptx::tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * set_cols);
+        int c;
+        unit_of(lt, c);
+        const HaloClass cl = class_of(c);
+        const int taps = cl.R * cl.sb;
+        const uint32_t a_first16 = (uint32_t)(((cl.R - 1) * p.tb * p.pitch + (cl.sb - 1)) * 8);  // tap (0,0), in 16-byte units
+        const uint32_t a_rowstep16 = (uint32_t)((p.tb * p.pitch - (cl.sb - 1)) * 8);             // last tap of a filter row -> first of the next
         const uint32_t strips = strip_mask(lt);
         const bool all_strips = strips == ((1u << NT) - 1u);
         // (this warp's instructions are the MMAs' issue rate: one form for whole blocks, one for the rest, no division for whole ones)
@@ -264,7 +287,7 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         int kb0 = 0;
         if (partial && p.diag_cin_g != 0) {
           int n0, w0, h0, b0;
-          locate(first_pair + lt * pair_stride, n0, w0, h0, b0);
+          locate(lt, n0, w0, h0, b0, c);
           kb0 = first_k_block(p, n0, C::kKB);
         }
         uint32_t accumulate = 0u;
@@ -273,9 +296,9 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           if (SPARSE && !FUSED && !wait_all(&meta_ready[ast], aph, 0x340u + ast)) { alive = false; break; }
           const int mmas = (partial && kb0 + ku / p.ss == p.k_last) ? p.last_mmas : 4;
           uint32_t a_lo = a_lo0 + (uint32_t)ast * a_stage16 + a_first16;
-          int s = p.sb, dr = p.R - 1;
+          int s = cl.sb, dr = cl.R - 1;
           const uint32_t e_stage = e_lo0 + (uint32_t)ast * e_stage16;
-          uint32_t e_lo = e_stage + meta_row16(dr) + (uint32_t)(p.sb - 1);
+          uint32_t e_lo = e_stage + meta_row16(dr) + (uint32_t)(cl.sb - 1);
           for (int t = 0; t < taps; ++t) {
             if (!wait_all(&w_ready[wst], wph, 0x380u + wst)) { alive = false; break; }
             ptx::tc_fence_after_sync();
@@ -313,7 +336,7 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             }
             accumulate = 1u;
             // next tap: one pixel to the left, or the end of the filter row above
-            if (--s == 0) { s = p.sb; a_lo -= a_rowstep16; --dr; e_lo = e_stage + meta_row16(dr) + (uint32_t)(p.sb - 1); }
+            if (--s == 0) { s = cl.sb; a_lo -= a_rowstep16; --dr; e_lo = e_stage + meta_row16(dr) + (uint32_t)(cl.sb - 1); }
             else { a_lo -= 8u; e_lo -= 1u; }
             if (++wst == WS) { wst = 0; wph ^= 1u; b_lo = b_lo0; mcol = 0; }
             else { b_lo += w_stage16; mcol += kSlotCols; }
@@ -416,8 +439,8 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         bool org_ok = false;
         int org_kb0 = 0;              // first channel block of its tile's window
         auto set_origin = [&](int box_lt, int box_ku, const uint8_t*& ptr, int& p0, int& q0, int& b0, int64_t& pix, bool& ok, int& kb0) {
-          int n0, w0, h0;
-          ok = locate(first_pair + box_lt * pair_stride, n0, w0, h0, b0);
+          int n0, w0, h0, parity;
+          ok = locate(box_lt, n0, w0, h0, b0, parity);
           const int box_kl = box_ku / p.ss, si = box_ku - box_kl * p.ss;
           kb0 = first_k_block(p, n0, 128);
           const int box_kb = kb0 + box_kl;
@@ -598,8 +621,8 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     uint32_t cph = 0, chunk = 0;
     int acc = 0;
     for (int lt = 0; lt < my_tiles; ++lt) {
-      int n0, w0, h0, b0;
-      const bool in_range = locate(first_pair + lt * pair_stride, n0, w0, h0, b0);
+      int n0, w0, h0, b0, c;
+      const bool in_range = locate(lt, n0, w0, h0, b0, c);
       const uint32_t strips = strip_mask(lt);
       // (patches: the four warps stay or leave together, they meet at a named barrier in every slab)
       const bool ready = ptx::mbar_wait<kIdleWaitNs>(&acc_full[acc], cph, err, 0x600u + acc);
@@ -614,15 +637,15 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         if constexpr (FUSED) {
           // this warp's 4 strip rows: 4 / tb pixel rows of tb images
           const int hq = h0 + q * (4 / p.tb);
-          if (p.split) store_box<BN>(taddr, sOut + q * p.out_bufs * kSlabBytes, &tmD, true, n0, 0, 2 * j, b0 / p.img_per_row, hq, strip_live,
+          if (p.split) store_box<BN>(taddr, sOut + q * p.out_bufs * kSlabBytes, &tmD.m[0], true, n0, 0, 2 * j, b0 / p.img_per_row, hq, strip_live,
                                      p.d.channels - n0, first_slab_read, released, p.f16 != 0, p.out_bufs, chunk);
-          else store_box<BN>(taddr, sOut + q * p.out_bufs * kSlabBytes, &tmD, false, n0, w0 + 8 * j, b0, hq, 0, strip_live && w0 + 8 * j < p.W,
+          else store_box<BN>(taddr, sOut + q * p.out_bufs * kSlabBytes, &tmD.m[0], false, n0, w0 + 8 * j, b0, hq, 0, strip_live && w0 + 8 * j < p.W,
                              p.d.channels - n0, first_slab_read, released, p.f16 != 0, p.out_bufs, chunk);
         } else if constexpr (PATCH) {
-          if (p.split) store_patch<BN, true>(taddr, sOut, p.out_bufs, &tmD, n0, 0, 2 * j, b0 / p.img_per_row, h0, strip_live, chunk,
+          if (p.split) store_patch<BN, true>(taddr, sOut, p.out_bufs, &tmD.m[0], n0, 0, 2 * j, b0 / p.img_per_row, h0, strip_live, chunk,
                                              first_slab_read, p.f16 != 0);
-          else store_patch<BN, false>(taddr, sOut, p.out_bufs, &tmD, n0, w0 + 8 * j, b0, h0, 0, strip_live && w0 + 8 * j < p.W, chunk,
-                                      first_slab_read, p.f16 != 0);
+          else store_patch<BN, false>(taddr, sOut, p.out_bufs, &tmD.m[c], n0, w0 + 8 * j, b0, h0, 0,
+                                      strip_live && w0 + 8 * j < p.cls[c].W && h0 < p.cls[c].H, chunk, first_slab_read, p.f16 != 0);
           if (released != nullptr) {
             ptx::tc_fence_before_sync();
             __syncwarp();
@@ -677,6 +700,7 @@ bool plan_halo(HaloParams* p, int nt) {
     p->static_pad = 0;
     p->units_per_box = (p->img_rows + 7) / 8;
     if (p->pitch > 256 || p->img_h > 256) return false;
+    if (p->classes == 4 && p->split) return false;
     p->a_bytes = round_up(p->img_rows * 128, 1024);
     p->eraw_bytes = (SPARSE && !FUSED) ? round_up(p->img_rows * 16, 128) : 0;
     p->w_bytes = C::kTapBBytes;
@@ -689,9 +713,9 @@ bool plan_halo(HaloParams* p, int nt) {
     p->tiles_h = (p->H + p->th - 1) / p->th;
     const int tile_imgs = p->tb * p->img_per_row;  // images of one tile set
     const int64_t m_sets = (int64_t)p->sets_w * p->tiles_h * ((p->B + tile_imgs - 1) / tile_imgs);
-    if (m_sets * p->tiles_n > 0x3FFFFFFF) return false;
+    if (m_sets * p->tiles_n * p->classes > 0x3FFFFFFF) return false;
     p->m_sets = (int)m_sets;
-    p->pair_tiles = (int)((m_sets + 1) / 2) * p->tiles_n;
+    p->pair_tiles = (int)((m_sets + 1) / 2) * p->tiles_n * p->classes;
     // Stride 2 stores boxes: its classes have few taps, so that the stores set the pace, and dD's pixels are not neighbours. 128 -> 128
     // channels, 3 x 3 stride 2 at 56 x 56, batch 256: 2.29 M write requests at L2 a class as rows, 0.60 M as boxes; the four classes 89 us
     // -> 83. Stride 1 keeps the rows (128 -> 64 channels at 32 x 32, batch 512, prune kernel included: 82 us, as boxes 88).
@@ -710,6 +734,7 @@ bool plan_halo(HaloParams* p, int nt) {
       w_stages = (budget - fixed - 4 * kSlabBytes) / p->w_bytes;
     }
     if (p->patch_store && w_stages < 3) {
+      if (p->classes == 4) return false;
       p->patch_store = p->out_bufs = 0;
       w_stages = (budget - fixed) / p->w_bytes;
     }
@@ -776,7 +801,11 @@ sdgp_status launch_halo_nt(const void* A, const void* meta, const void* Wt, cons
   using C = Cfg<SPARSE, BN>;
   if (!plan_halo<SPARSE, BN, FUSED>(&p, NT)) return SDGP_ERR_UNSUPPORTED;
 
-  CUtensorMap tmA, tmE, tmB, tmD;
+  if (p.classes == 1) p.cls[0] = HaloClass{p.R, p.S, p.sb, p.pad_h, p.pad_w, p.r_first, p.s_first, p.H, p.W};
+  else
+    for (HaloClass& c : p.cls) c.sb = c.S;
+  CUtensorMap tmA, tmE, tmB;
+  HaloOutMaps<true> tmD;
   p.d = view.d;
   p.early = early_for(SPARSE && !FUSED && p.last_launch, pairs_for(p.units));
   const int P = view.P, Q = view.Q;
@@ -821,19 +850,27 @@ sdgp_status launch_halo_nt(const void* A, const void* meta, const void* Wt, cons
                 C::kRowB == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
       return SDGP_ERR_CUDA;
   }
-  tmD = tmA;
+  tmD.m[0] = tmA;
   if (FUSED || p.patch_store) {
     // dD, a strip (fused: one warp's quarter of it) per store: 8 pixel columns (column-split mode: the 4 columns of two neighbouring images)
-    if (!encode_nhwc(&tmD, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, view.d.base, (uint64_t)view.d.channels, (uint64_t)p.W, (uint64_t)p.H,
-                     (uint64_t)p.B, (uint64_t)view.d.sw, (uint64_t)view.d.sh, (uint64_t)view.d.sb, 64, (uint32_t)(p.split ? 4 : 8), 2,
-                     (uint32_t)p.tb, (uint32_t)(FUSED ? 4 / p.tb : p.th), CU_TENSOR_MAP_SWIZZLE_128B))
-      return SDGP_ERR_CUDA;
+    for (int c = 0; c < p.classes; ++c) {
+      const uint8_t* base = view.d.base;  // of parity (0, 0); a pixel of dD is half a step of the parities' images
+      if (p.classes == 4) base += (c >> 1) * (view.d.sh / 2) + (c & 1) * (view.d.sw / 2);
+      if (!encode_nhwc(&tmD.m[c], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, base, (uint64_t)view.d.channels, (uint64_t)p.cls[c].W, (uint64_t)p.cls[c].H,
+                       (uint64_t)p.B, (uint64_t)view.d.sw, (uint64_t)view.d.sh, (uint64_t)view.d.sb, 64, (uint32_t)(p.split ? 4 : 8), 2,
+                       (uint32_t)p.tb, (uint32_t)(FUSED ? 4 / p.tb : p.th), CU_TENSOR_MAP_SWIZZLE_128B))
+        return SDGP_ERR_CUDA;
+    }
   }
+  for (int c = p.classes; c < 4; ++c) tmD.m[c] = tmD.m[0];
   auto launch = [&](auto patch_tag) -> sdgp_status {
+    constexpr bool PATCH = decltype(patch_tag)::value;
     static bool configured[kMaxDevices] = {};
-    auto kernel = dgrad_halo_kernel<SPARSE, BN, NT, FUSED, decltype(patch_tag)::value>;
+    auto kernel = dgrad_halo_kernel<SPARSE, BN, NT, FUSED, PATCH>;
     if (!configure_once(kernel, configured)) return SDGP_ERR_CUDA;
-    return launch_pairs(kernel, pairs_for(p.units), FUSED ? kThreadsHaloFused : kThreadsGemm, p.smem_bytes, stream, tmA, tmE, tmB, tmD, p);
+    HaloOutMaps<PATCH> maps;
+    for (int c = 0; c < (PATCH ? 4 : 1); ++c) maps.m[c] = tmD.m[c];
+    return launch_pairs(kernel, pairs_for(p.units), FUSED ? kThreadsHaloFused : kThreadsGemm, p.smem_bytes, stream, tmA, tmE, tmB, maps, p);
   };
   if constexpr (!FUSED)
     if (p.patch_store) return launch(std::true_type{});

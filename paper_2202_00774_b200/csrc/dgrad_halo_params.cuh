@@ -15,10 +15,19 @@ __device__ __forceinline__ void divmod(uint32_t x, uint32_t d, uint32_t m, uint3
   if (r >= d) { ++q; r -= d; }
 }
 
+// One output parity of a stride-2 convolution (or the whole of a stride-1 one): its filter taps, where they start, its pixels.
+struct HaloClass {
+  int R, S, sb;                          // sb: filter columns served by one box (see HaloParams)
+  int pad_h, pad_w, r_first, s_first;
+  int H, W;
+};
+
 struct HaloParams {
   int B, H, W, Cin, Cout;
   int R, S, pad_h, pad_w;
   int r_first, r_step, s_first, s_step, S_full;  // as in DgradParams
+  int classes;             // 1, or 4: all output parities of a stride-2 convolution in one launch; R, S, H, W are then the largest
+  HaloClass cls[4];        // parity 2 * (row) + (column); classes == 1: cls[0] repeats the fields of this struct
   int nt;                  // strips per CTA tile set (1 or 2), side by side, sharing every W stage
   int sets_w, tiles_h, tiles_n;
   int m_sets;              // sets_w * tiles_h * B
@@ -74,6 +83,12 @@ struct HaloParams {
   OutView d;
   int last_launch, early;  // as in DgradParams
   int f16;                 // element type of A, W and dD: 0 = bf16, 1 = IEEE binary16
+};
+
+// dD's tensor maps: one, or one per parity.
+template <bool CLASSES>
+struct HaloOutMaps {
+  CUtensorMap m[CLASSES ? 4 : 1];
 };
 
 // Plans and launches the kernel over BN = bn input channels and nt strips (two at most, 256 columns together) per tile;

@@ -485,6 +485,41 @@ def test_whole_filter_reuse_kernel(case, mode):
     assert_close(got, *conv_ref(src, W, H, Wd, stride, pad))
 
 
+# The four output parities of a strided layer in one launch: classes of unequal size whose last strips lie outside the smaller ones, filters
+# of two to five rows and columns, no padding, images of less than a strip, several column tiles and channel blocks (the last
+# one half full), several rounds of units with a split last one.
+STRIDE2_CLASS_CASES = [
+    # B, H, W, Cin, Cout, R, S, pad
+    (1, 33, 20, 64, 128, 3, 3, 1),
+    (2, 18, 49, 128, 192, 3, 3, 1),
+    (3, 12, 12, 192, 64, 3, 3, 0),
+    (1, 40, 24, 64, 64, 5, 5, 2),
+    (2, 22, 30, 128, 128, 2, 3, 1),
+    (5, 14, 14, 320, 256, 3, 3, 1),
+    (1, 9, 64, 64, 128, 3, 3, 1),
+    (24, 56, 56, 64, 128, 3, 3, 1),
+]
+
+
+@pytest.mark.parametrize("mode", ["dense", "two_pass"])
+@pytest.mark.parametrize("case", STRIDE2_CLASS_CASES)
+def test_stride2_classes_in_one_launch(case, mode):
+    import paper_2202_00774_b200 as sdgp
+    B, H, Wd, Cin, Cout, R, S, pad = case
+    layer = inputs.ConvLayer("t", B, H, Wd, Cin, Cout, R, S, 2, pad)
+    dO, W = inputs.conv_layer_tensors(layer, seed=41)
+    dD = torch.full((B, H, Wd, Cin), -1, dtype=torch.int16, device="cuda")
+    if mode == "dense":
+        sdgp.sdgp_dgrad_conv2d(dev16(dO), dev16(W), dD, 2, pad, 4, 4, sdgp.MAGNITUDE, flags=sdgp.FLAG_DENSE)
+        src = dO
+    else:
+        ws = torch.empty(sdgp.sdgp_workspace_size_conv2d(B, H, Wd, Cin, Cout, R, S, 2, pad), dtype=torch.uint8, device="cuda")
+        sdgp.sdgp_dgrad_conv2d(dev16(dO), dev16(W), dD, 2, pad, 2, 4, sdgp.MAGNITUDE, seed=3, workspace=ws)
+        src = oracle.prune(dO.reshape(-1, Cout), 2, 4, oracle.MAGNITUDE, 3, want=("dense",))["dense"].reshape(dO.shape)
+    check_no_device_error()
+    assert_close(to_f64(dD), *conv_ref(src, W, H, Wd, 2, pad))
+
+
 @pytest.mark.parametrize("n,m,scheme", [(2, 8, oracle.MAGNITUDE), (1, 8, oracle.RESCALED), (2, 16, oracle.MAGNITUDE),
                                         (2, 16, oracle.RANDOM), (2, 8, oracle.RANDOM), (1, 16, oracle.RESCALED)])
 @pytest.mark.parametrize("case", [(3, 16, 16, 64, 128, 3, 3, 1, 1),      # whole-filter-reuse kernel, two strips

@@ -35,6 +35,12 @@ constexpr int kHaloAStages = 4;  // at most: A stages in use are p.a_stages = 2,
 // slots they take from it (14 -> 16 -> 18 pruning warps: 1062 -> 1107 -> 1111 TFLOP/s on the ResNet-9 chain).
 constexpr int kPruneWarps = 18;
 constexpr int kThreadsHaloFused = 24 * 32;
+// Not fused: one warp more than the general kernel's ten. It fetches the A boxes: with both in one warp W's loads waited for A's stages and A's
+// for a place between W's (the MMA warp stood 100 to 130 clocks a tap for W, and a launch began with A before W). Us, prune
+// kernel included: 64 -> 128 channels at 32 x 32, batch 512, 82.0 -> 75.0; 512 -> 512 at 4 x 4 (four boxes ahead) 22.9 -> 18.0; 64 x 7 x 7, 512 -> 512
+// 17.2 -> 15.4; 256 -> 512 at 8 x 8 39.6 -> 37.6; 72 x 56 x 56, 192 -> 64, bound by stores, 69.4 -> 70.6.
+constexpr int kABoxWarp = 10;
+constexpr int kThreadsHalo = 11 * 32;
 
 // PATCH (not fused): strips leave as one TMA box each (store_patch), else as rows; plan_halo() has the rule. Such a launch may also hold
 // the four output parities of a stride-2 convolution (p.classes == 4): a work unit is then a tile set of one parity. The four of a
@@ -43,7 +49,7 @@ constexpr int kThreadsHaloFused = 24 * 32;
 // channels at 56 x 56, batch 256, random pruning included: four launches 104, this 92. Two kernels, so that neither carries the
 // other's code.
 template <bool SPARSE, int BN, int NT, bool FUSED, bool PATCH>
-__global__ void __launch_bounds__(FUSED ? kThreadsHaloFused : kThreadsGemm, 1)
+__global__ void __launch_bounds__(FUSED ? kThreadsHaloFused : kThreadsHalo, 1)
 dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmE,
                   const __grid_constant__ CUtensorMap tmB, const __grid_constant__ HaloOutMaps<PATCH> tmD,
                   const __grid_constant__ HaloParams p) {
@@ -158,47 +164,44 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     return in_range;
   };
 
-  if (warp == 0) {
-    // ------------------------------------------------------------ producer
+  if (!FUSED && warp == kABoxWarp) {
+    // ------------------------------------------------------------ A boxes and their raw metadata
     if (ptx::elect_one()) {
       const uint32_t a_tx = 2u * (uint32_t)(p.img_rows * 128);
       const uint32_t meta_tx = (uint32_t)(p.img_rows * 16);
-      const uint32_t w_tx = 2u * (uint32_t)C::kTapBBytes;
-      const int a_uses = my_tiles * p.k_uses;
-      int ia = 0, ast = 0;
+      bool alive = true;
+      int ast = 0;
       uint32_t aph = 0;
-      // Loads the A box (and raw metadata) of stage use `ia`. blocking == false: only if the
-      // stage is free right now. Returns 1 issued, 0 not free, -1 wait gave up.
-      auto issue_a = [&](bool blocking) -> int {
-        if (blocking) {
-          if (!ptx::mbar_wait(&a_empty[ast], aph ^ 1u, err, 0x100u + ast)) return -1;
-        } else if (!ptx::mbar_test(&a_empty[ast], aph ^ 1u)) {
-          return 0;
-        }
-        const int lt = ia / p.k_uses, ku = ia - lt * p.k_uses;
-        const int kl = ku / p.ss, si = ku - kl * p.ss;  // channel block of the tile's window, filter column of the box (column-split mode)
+      for (int lt = 0; alive && lt < my_tiles; ++lt) {
         int n0, w0, h0, b0, c;
         locate(lt, n0, w0, h0, b0, c);
-        const int kb = first_k_block(p, n0, C::kKB) + kl;
+        const int kb0 = first_k_block(p, n0, C::kKB);
         const HaloClass cl = class_of(c);
-        const int q0 = w0 + cl.pad_w - (cl.sb - 1) - si, p0 = h0 + cl.pad_h - (cl.R - 1);
-        // coordinates: channel, pixel column, image within a box row, image group, pixel row
-        const int bg = b0 / p.img_per_row;
-        if (rank == 0) ptx::mbar_arrive_expect_tx(&a_full[ast], a_tx);
-        // (the tensor maps have the image-within-row dimension only in column-split mode)
-        if (SPARSE) {
-          ptx::mbar_arrive_expect_tx(&meta_full[ast], meta_tx);
-          if (p.split) ptx::tma_load_5d(sEraw + ast * p.eraw_bytes, &tmE, &meta_full[ast], kb * 8, q0, 0, bg, p0);
-          else ptx::tma_load_4d(sEraw + ast * p.eraw_bytes, &tmE, &meta_full[ast], kb * 8, q0, b0, p0);
+        const int p0 = h0 + cl.pad_h - (cl.R - 1), bg = b0 / p.img_per_row;
+        for (int ku = 0; ku < p.k_uses; ++ku) {
+          const int kl = ku / p.ss, si = ku - kl * p.ss;  // channel block of the tile's window, filter column of the box (column-split mode)
+          const int kb = kb0 + kl, q0 = w0 + cl.pad_w - (cl.sb - 1) - si;
+          if (!ptx::mbar_wait<kIdleWaitNs>(&a_empty[ast], aph ^ 1u, err, 0x100u + ast)) { alive = false; break; }
+          // coordinates: channel, pixel column, image within a box row, image group, pixel row
+          // (the tensor maps have the image-within-row dimension only in column-split mode)
+          if (rank == 0) ptx::mbar_arrive_expect_tx(&a_full[ast], a_tx);
+          if (SPARSE) {
+            ptx::mbar_arrive_expect_tx(&meta_full[ast], meta_tx);
+            if (p.split) ptx::tma_load_5d(sEraw + ast * p.eraw_bytes, &tmE, &meta_full[ast], kb * 8, q0, 0, bg, p0);
+            else ptx::tma_load_4d(sEraw + ast * p.eraw_bytes, &tmE, &meta_full[ast], kb * 8, q0, b0, p0);
+          }
+          if (p.split) ptx::tma_load_5d_pair(sA + ast * p.a_bytes, &tmA, &a_full[ast], kb * 64, q0, 0, bg, p0);
+          else ptx::tma_load_4d_pair(sA + ast * p.a_bytes, &tmA, &a_full[ast], kb * 64, q0, b0, p0);
+          if (++ast == p.a_stages) { ast = 0; aph ^= 1u; }
         }
-        if (p.split) ptx::tma_load_5d_pair(sA + ast * p.a_bytes, &tmA, &a_full[ast], kb * 64, q0, 0, bg, p0);
-        else ptx::tma_load_4d_pair(sA + ast * p.a_bytes, &tmA, &a_full[ast], kb * 64, q0, b0, p0);
-        ++ia;
-        if (++ast == p.a_stages) { ast = 0; aph ^= 1u; }
-        return 1;
-      };
+      }
+    }
+  } else if (warp == 0) {
+    // ------------------------------------------------------------ W taps (fused: the pruning warps fetch dL/dO themselves)
+    if (ptx::elect_one()) {
+      const uint32_t w_tx = 2u * (uint32_t)C::kTapBBytes;
       bool alive = true;
-      int wst = 0, use = 0;
+      int wst = 0;
       uint32_t wph = 0;
       for (int lt = 0; alive && lt < my_tiles; ++lt) {
         int n0, w0_unused, h0_unused, b0_unused, c;
@@ -207,14 +210,9 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         n0 += n_half;
         const HaloClass cl = class_of(c);
         const int taps = cl.R * cl.sb;  // filter taps served by one A box
-        for (int ku = 0; alive && ku < p.k_uses; ++ku, ++use) {
+        for (int ku = 0; alive && ku < p.k_uses; ++ku) {
           const int kl = ku / p.ss, si = ku - kl * p.ss, kb = kb0 + kl;
-          // (fused: the pruning warps fetch dL/dO themselves; this thread streams W only)
-          while (!FUSED && alive && ia <= use)
-            if (issue_a(true) < 0) alive = false;
-          for (int t = 0; alive && t < taps; ++t) {
-            // the next A box goes out as soon as its stage is released, between W taps
-            if (!FUSED && ia < a_uses && ia < use + p.a_stages && issue_a(false) < 0) { alive = false; break; }
+          for (int t = 0; t < taps; ++t) {
             if (!ptx::mbar_wait<kIdleWaitNs>(&w_empty[wst], wph ^ 1u, err, 0x180u + wst)) { alive = false; break; }
             if (rank == 0) ptx::mbar_arrive_expect_tx(&w_ready[wst], w_tx);
             const int r = t / cl.sb, s = t - r * cl.sb + si;
@@ -870,7 +868,7 @@ sdgp_status launch_halo_nt(const void* A, const void* meta, const void* Wt, cons
     if (!configure_once(kernel, configured)) return SDGP_ERR_CUDA;
     HaloOutMaps<PATCH> maps;
     for (int c = 0; c < (PATCH ? 4 : 1); ++c) maps.m[c] = tmD.m[c];
-    return launch_pairs(kernel, pairs_for(p.units), FUSED ? kThreadsHaloFused : kThreadsGemm, p.smem_bytes, stream, tmA, tmE, tmB, maps, p);
+    return launch_pairs(kernel, pairs_for(p.units), FUSED ? kThreadsHaloFused : kThreadsHalo, p.smem_bytes, stream, tmA, tmE, tmB, maps, p);
   };
   if constexpr (!FUSED)
     if (p.patch_store) return launch(std::true_type{});

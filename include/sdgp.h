@@ -222,9 +222,10 @@ sdgp_status sdgp_maxpool_relu_backward_prune(const void* dYp, const void* dSkipP
  * are not multiples of 64 (RegNetX-400MF has 32 and 160): Cout % 16 == 0 when anything is pruned (% 8 otherwise),
  * (Cin/groups) % 8 == 0. flags: SDGP_FLAG_TWO_PASS, SDGP_FLAG_DENSE, SDGP_FLAG_MASKED, and SDGP_FLAG_FUSED where both
  * channel counts are multiples of 64 (SDGP_ERR_UNSUPPORTED otherwise). Other requirements as sdgp_dgrad_conv2d.
- * The call first writes the filters as the block-diagonal filters of an ordinary convolution, channel counts
- * rounded up to multiples of 64, into the workspace (read again by the contraction on `stream`), then runs the
- * ordinary kernels on them; dL/dO and dD are used as stored, without padded copies.
+ * Two-pass calls with Cin == Cout and 16 or 32 channels a group run as one kernel that prunes dL/dO on its way into shared memory and reads
+ * the filters as they are. All others first write the filters as the block-diagonal filters of an ordinary convolution,
+ * channel counts rounded up to multiples of 64, into the workspace (read again by the contraction on `stream`), then run the
+ * ordinary kernels on them. dL/dO and dD are used as stored, without padded copies, either way.
  * Workspace: sdgp_workspace_size_conv2d_grouped() bytes (every mode needs one), 256-byte aligned, owned by the caller. */
 size_t sdgp_workspace_size_conv2d_grouped(int B, int H, int Wd, int Cin, int Cout, int R, int S, int stride, int pad,
                                           int groups, uint32_t flags);

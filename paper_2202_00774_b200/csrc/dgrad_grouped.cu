@@ -16,8 +16,9 @@
 // and warp 2 the filters by TMA, warp 1 issues the MMAs (128 x width x 16, one group at a time), warps 4..7 are the epilogue, the other
 // seventeen prune: a thread takes two vectors of 8 channels out of the stage that TMA filled and puts them back pruned, dense, for the
 // tensor core. Dense, because the MMA's time is reading its 128 rows of A (4 KB: 41 clocks at best) for either kind and 16 columns leave the
-// tensor pipe idle anyway. (A version whose pruning warps loaded dL/dO into registers waited for memory: 256 images of 14 x 14, 10
-// groups of 16, 22 us.)
+// tensor pipe idle anyway. (Loading dL/dO into the pruning warps' registers instead
+// measured the same within 3 %.) 256 images of 14 x 14, 10 groups of 16, rescaled, us: three kernels 32.8, this 22.8; 124 x 4 x 4, 11 groups, 11.2 and
+// 5.2; 60 x 32 x 32, 15 groups, 31.7 and 26.5. What bounds it: the MMAs at 51 to 59 clocks each, the pruning close behind.
 #include "dgrad_prune.cuh"
 
 namespace sdgp {

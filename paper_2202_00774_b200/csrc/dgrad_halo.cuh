@@ -301,7 +301,11 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             if (!wait_all(&w_ready[wst], wph, 0x380u + wst)) { alive = false; break; }
             ptx::tc_fence_after_sync();
             const uint32_t e_col = meta_base + mcol;  // even: slots are 4 columns apart
-            // MMAS: MMAs of the channel block if every strip takes part (no per-strip test in the issue path), 0: neither is known
+            // MMAS: MMAs of the channel block if every strip takes part (no per-strip test in the issue path), 0: neither is known. Whole and half
+            // blocks have a form of their own: with 64 output channels, the tests of the last form are what a tap waits for. Us, prune kernel
+            // included, half blocks through the last form and their own: 8 x 6 x 6 images, 192 -> 64 channels, 5 x 5, 11.4 -> 10.4; 22 x 7 x 7, 384 -> 64,
+            // 8.0 -> 7.6; 64 x 28 x 28, 64 -> 64, fused, 16.9 -> 16.1. (Forms for one and three MMAs too made every form slower: 512 x 32 x 32, 64 -> 128,
+            // 75 -> 84.)
             auto issue_tap = [&](auto mmas_tag) {
               constexpr int MMAS = decltype(mmas_tag)::value;
               if (SPARSE) {
@@ -315,7 +319,7 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 if (!MMAS && !(strips & (1u << j))) continue;
 #pragma unroll
                 for (int q = 0; q < (MMAS ? MMAS : 4); ++q) {
-                  if (!MMAS && q >= mmas) break;
+                  if (!MMAS && q >= mmas) continue;  // (not break: 18 x 18, 224 channels in 7 groups, 5 x 5, 15.2 us, so 14.7)
                   // strip j: 8 pixels = 1024 bytes to the right; MMA q: 32 bytes along the row
                   const uint64_t a_q = ((uint64_t)a_hi << 32) | (a_lo + (uint32_t)(j * 64 + q * 2));
                   const uint64_t b_q = ((uint64_t)b_hi << 32) | (b_lo + (uint32_t)q * kBStep);
@@ -329,6 +333,7 @@ dgrad_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             };
             if (leader) {
               if (all_strips && mmas == 4) issue_tap(std::integral_constant<int, 4>{});
+              else if (all_strips && mmas == 2) issue_tap(std::integral_constant<int, 2>{});
               else issue_tap(std::integral_constant<int, 0>{});
               ptx::tc_commit_pair(&w_empty[wst], 3);
             }

@@ -27,7 +27,6 @@ struct HaloParams {
   int R, S, pad_h, pad_w;
   int r_first, r_step, s_first, s_step, S_full;  // as in DgradParams
   int classes;             // 1, or 4: all output parities of a stride-2 convolution in one launch; R, S, H, W are then the largest
-  HaloClass cls[4];        // parity 2 * (row) + (column); classes == 1: cls[0] repeats the fields of this struct
   int nt;                  // strips per CTA tile set (1 or 2), side by side, sharing every W stage
   int sets_w, tiles_h, tiles_n;
   int m_sets;              // sets_w * tiles_h * B
@@ -83,6 +82,8 @@ struct HaloParams {
   OutView d;
   int last_launch, early;  // as in DgradParams
   int f16;                 // element type of A, W and dD: 0 = bf16, 1 = IEEE binary16
+  // parity 2 * (row) + (column); classes == 1: cls[0] repeats the fields above (last: what every launch reads stays on fewer lines of parameters)
+  HaloClass cls[4];
 };
 
 // dD's tensor maps: one, or one per parity.

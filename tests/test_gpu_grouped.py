@@ -137,3 +137,14 @@ def test_narrow_groups(B, H, Wd, C, R, S, stride, pad, groups, n, m, scheme):
     import paper_2202_00774_b200 as sdgp
     layer = inputs.ConvLayer("narrow", B, H, Wd, C, C, R, S, stride, pad, groups)
     run(layer, n, m, scheme, sdgp.FLAG_TWO_PASS)
+
+
+# The last channel block of the strip kernel holds one to four MMAs' channels: every count, in tiles of one strip and of two, and in a last round
+# that is dealt out strip by strip (176 images: 88 pair tiles of two strips on 74 pairs)
+@pytest.mark.parametrize("B", [3, 176])
+@pytest.mark.parametrize("Cout,mode", [(32, "two_pass"), (64, "two_pass"), (96, "two_pass"), (160, "two_pass"), (192, "two_pass"), (64, "fused"), (192, "fused"),
+                                       (80, "dense"), (96, "dense"), (112, "dense"), (96, "masked")])
+def test_last_channel_block_of_the_strip_kernel(B, Cout, mode):
+    import paper_2202_00774_b200 as sdgp
+    layer = inputs.ConvLayer("last", B, 16, 16, 64, Cout, 3, 3, 1, 1, 1)
+    run(layer, 2, 4, oracle.MAGNITUDE, {"two_pass": sdgp.FLAG_TWO_PASS, "fused": sdgp.FLAG_FUSED, "dense": sdgp.FLAG_DENSE, "masked": sdgp.FLAG_MASKED}[mode])

@@ -222,8 +222,8 @@ sdgp_status sdgp_maxpool_relu_backward_prune(const void* dYp, const void* dSkipP
  * are not multiples of 64 (RegNetX-400MF has 32 and 160): Cout % 16 == 0 when anything is pruned (% 8 otherwise),
  * (Cin/groups) % 8 == 0. flags: SDGP_FLAG_TWO_PASS, SDGP_FLAG_DENSE, SDGP_FLAG_MASKED, and SDGP_FLAG_FUSED where both
  * channel counts are multiples of 64 (SDGP_ERR_UNSUPPORTED otherwise). Other requirements as sdgp_dgrad_conv2d.
- * Two-pass calls with Cin == Cout and 16 or 32 channels a group run as one kernel that prunes dL/dO on its way into shared memory and reads
- * the filters as they are. All others first write the filters as the block-diagonal filters of an ordinary convolution,
+ * Two-pass calls with Cin == Cout and 16 or 32 channels a group run, where that is estimated to be faster, as one kernel that prunes dL/dO on its
+ * way into shared memory and reads the filters as they are. All others first write the filters as the block-diagonal filters of an ordinary convolution,
  * channel counts rounded up to multiples of 64, into the workspace (read again by the contraction on `stream`), then run the
  * ordinary kernels on them. dL/dO and dD are used as stored, without padded copies, either way.
  * Workspace: sdgp_workspace_size_conv2d_grouped() bytes (every mode needs one), 256-byte aligned, owned by the caller. */
@@ -277,6 +277,16 @@ sdgp_status sdgp_last_device_error(void);
  * with a 50 ms limit, on a barrier nothing signals. The kernel must end by itself and leave
  * SDGP_ERR_TIMEOUT for the next sdgp_last_device_error() call; the context stays usable. */
 sdgp_status sdgp_selftest_bounded_wait(void* stream);
+
+/* Self-test of the choice of kernel (no counterpart in the paper; looks at sizes only, launches nothing, needs no GPU): the path that
+ * sdgp_dgrad_conv2d_grouped (groups == 1 and channel counts that are multiples of 64: also sdgp_dgrad_conv2d) takes for these arguments.
+ * `plan`: 8 ints on the host, unused ones 0.
+ *   plan[0] = 0  any other path
+ *   plan[0] = 1  the kernel for narrow groups; work units, accumulators of a unit and parity, output parities, operand stages, positions of a unit
+ *   plan[0] = 2  the four output parities of a stride-2 layer in one launch; work units, the first one of a last round that is dealt out strip
+ *                by strip (== work units: none), CTA pairs, input channels of a tile, its strips, images of a strip */
+sdgp_status sdgp_selftest_plan(int B, int H, int Wd, int Cin, int Cout, int R, int S, int stride, int pad, int groups, int n, int m,
+                               sdgp_scheme scheme, uint32_t flags, int* plan);
 
 /* Static, NUL-terminated description of a status code. */
 const char* sdgp_status_string(sdgp_status status);

@@ -20,7 +20,7 @@ FLAG_TWO_PASS, FLAG_FUSED, FLAG_DENSE, FLAG_MASKED, FLAG_CHANNEL = 0, 1, 2, 3, 4
 BF16, FP16 = 0, 1   # sdgp_dtype
 EXPORTS = ["sdgp_prune", "sdgp_dgrad_linear", "sdgp_dgrad_conv2d", "sdgp_spmm_linear", "sdgp_spmm_conv2d",
            "sdgp_prune_typed", "sdgp_dgrad_linear_typed", "sdgp_dgrad_conv2d_typed", "sdgp_spmm_linear_typed",
-           "sdgp_spmm_conv2d_typed", "sdgp_channel_scales", "sdgp_relu_backward_prune", "sdgp_residual_relu_backward_prune", "sdgp_maxpool_relu_backward_prune", "sdgp_dgrad_linear_static", "sdgp_selftest_bounded_wait",
+           "sdgp_spmm_conv2d_typed", "sdgp_channel_scales", "sdgp_relu_backward_prune", "sdgp_residual_relu_backward_prune", "sdgp_maxpool_relu_backward_prune", "sdgp_dgrad_linear_static", "sdgp_selftest_bounded_wait", "sdgp_selftest_plan",
            "sdgp_workspace_size_linear", "sdgp_workspace_size_conv2d", "sdgp_workspace_size_conv2d_grouped",
            "sdgp_dgrad_conv2d_grouped", "sdgp_last_device_error",
            "sdgp_status_string"]
@@ -89,6 +89,8 @@ def lib() -> ctypes.CDLL:
         L.sdgp_last_device_error.restype = i32
         L.sdgp_selftest_bounded_wait.argtypes = [vp]
         L.sdgp_selftest_bounded_wait.restype = i32
+        L.sdgp_selftest_plan.argtypes = [i32] * 13 + [u32, ctypes.POINTER(i32)]
+        L.sdgp_selftest_plan.restype = i32
         L.sdgp_status_string.argtypes = [i32]
         L.sdgp_status_string.restype = ctypes.c_char_p
         _lib = L

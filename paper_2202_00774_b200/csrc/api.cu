@@ -392,6 +392,24 @@ sdgp_status sdgp_channel_scales(const void* dO, int64_t rows, int64_t K, int n, 
 
 sdgp_status sdgp_last_device_error(void) { return sdgp::read_device_error(); }
 
+sdgp_status sdgp_selftest_plan(int B, int H, int Wd, int Cin, int Cout, int R, int S, int stride, int pad, int groups, int n, int m,
+                               sdgp_scheme scheme, uint32_t flags, int* plan) {
+  if (!plan || B < 1 || H < 1 || Wd < 1 || Cin < 1 || Cout < 1 || R < 1 || S < 1 || stride < 1 || stride > 2 || pad < 0 || groups < 1 ||
+      Cin % groups != 0 || Cout % groups != 0 || H + 2 * pad < R || Wd + 2 * pad < S || pad > R - 1 || pad > S - 1 || flags > SDGP_FLAG_MASKED)
+    return SDGP_ERR_INVALID_ARG;
+  for (int i = 0; i < 8; ++i) plan[i] = 0;
+  const bool prunes = flags != SDGP_FLAG_DENSE && n != m;
+  if (flags == SDGP_FLAG_FUSED) return SDGP_OK;
+  if (prunes && flags == SDGP_FLAG_TWO_PASS && groups > 1 && Cin == Cout &&
+      sdgp::query_grouped(B, H, Wd, Cin, groups, R, S, stride, pad, {n, m, (int)scheme, 0}, plan))
+    return SDGP_OK;
+  const int cin_k = round64(Cin), cout_k = round64(Cout);
+  const sdgp::StoredChannels stored = {Cout != cout_k ? Cout : 0, Cin != cin_k ? Cin : 0};
+  const sdgp::ConvGroups cg = {Cin / groups, Cout / groups};
+  sdgp::query_parities(prunes && flags == SDGP_FLAG_TWO_PASS, B, H, Wd, cin_k, cout_k, R, S, stride, pad, &stored, groups > 1 ? &cg : nullptr, plan);
+  return SDGP_OK;
+}
+
 sdgp_status sdgp_selftest_bounded_wait(void* stream) { return sdgp::launch_bounded_wait_selftest((cudaStream_t)stream); }
 
 }  // extern "C"

@@ -248,6 +248,76 @@ bool classes_pay(int B, int H, int W, int Cin, int Cout, int R, int S, int pad, 
   return 2.0e-9 * excess * B * Cin * Cout < (sparse ? 25.0 : 20.0);
 }
 
+// A tile of the strip kernel: input channels, strips side by side, estimated time.
+struct TileShape {
+  int bn, nt;
+  double cost;
+};
+
+// Channel blocks that a tile of bn input channels visits (grouped convolutions: a window of them).
+void set_width(HaloParams* p, int bn, int channels, int kb_channels, const ConvGroups* groups) {
+  const int blocks = (p->Cout + kb_channels - 1) / kb_channels;
+  p->tiles_n = (channels + bn - 1) / bn;
+  p->k_blocks = k_window(bn, channels, blocks, kb_channels, p->Cout, groups);
+  p->diag_cin_g = p->diag_cout_g = p->diag_last = 0;
+  if (p->k_blocks < blocks) {
+    p->diag_cin_g = groups->cin_g; p->diag_cout_g = groups->cout_g;
+    p->diag_last = blocks - p->k_blocks;
+  }
+}
+
+// All four output parities of a strided layer in one launch of the strip kernel, where its strips cover their images well enough (the
+// same bounds as for a filter of its size at stride 1) and that is estimated to be faster: its parameters and the tile shapes, cheapest first.
+bool plan_parities(bool sparse, const DgradView& view, int B, int H, int W, int Cin, int Cout, int R, int S, int stride, int pad,
+                   const ConvGroups* conv_groups, HaloParams* hp, TileShape (&shapes)[6]) {
+  if (stride != 2 || R < 2 || S < 2 || W <= 8 || !halo_applies((H + 1) / 2, (W + 1) / 2, R * S, sparse, false) ||
+      !classes_pay(B, H, W, view.d.channels, view.a_channels, R, S, pad, sparse))
+    return false;
+  *hp = HaloParams{};
+  hp->B = B; hp->H = (H + 1) / 2; hp->W = (W + 1) / 2; hp->Cin = Cin; hp->Cout = Cout;
+  hp->r_step = hp->s_step = 2;
+  hp->S_full = S;
+  hp->P = view.P; hp->Q = view.Q;
+  hp->last_launch = 1;
+  hp->classes = 4;
+  for (int c = 0; c < 4; ++c) {
+    HaloClass& k = hp->cls[c];
+    const int ph = c >> 1, pw = c & 1;
+    k.r_first = (ph + pad) % 2; k.s_first = (pw + pad) % 2;
+    k.R = (R - k.r_first + 1) / 2; k.S = (S - k.s_first + 1) / 2;
+    k.pad_h = (ph + pad - k.r_first) / 2; k.pad_w = (pw + pad - k.s_first) / 2;
+    k.H = (H - ph + 1) / 2; k.W = (W - pw + 1) / 2;
+    hp->R = k.R > hp->R ? k.R : hp->R;
+    hp->S = k.S > hp->S ? k.S : hp->S;
+  }
+  const int kb_channels = sparse ? 128 : 64, blocks = (Cout + kb_channels - 1) / kb_channels;
+  hp->k_last = blocks - 1;
+  const int left = view.a_channels - hp->k_last * kb_channels, per_mma = kb_channels / 4;
+  hp->last_mmas = left < kb_channels ? (left + per_mma - 1) / per_mma : 4;
+  const TileShape all[] = {{64, 1, 0}, {64, 2, 0}, {128, 1, 0}, {128, 2, 0}, {192, 1, 0}, {256, 1, 0}};
+  for (int i = 0; i < 6; ++i) {
+    shapes[i] = all[i];
+    set_width(hp, all[i].bn, view.d.channels, kb_channels, conv_groups);
+    const double cost = halo_cost_classes(B, hp->H, hp->W, R, S, pad, all[i].bn, all[i].nt, sparse, hp->tiles_n, hp->k_blocks);
+    shapes[i].cost = cost > 0.0 ? cost : 1e9;
+  }
+  std::sort(std::begin(shapes), std::end(shapes), [](const TileShape& a, const TileShape& b) { return a.cost < b.cost; });
+  return true;
+}
+
+// What a call reads and writes per pixel; base and strides of dD are the launch's.
+DgradView dgrad_view(int B, int H, int W, int Cin, int Cout, int R, int S, int stride, int pad, const StoredChannels* stored) {
+  DgradView view = {};
+  view.P = (H + 2 * pad - R) / stride + 1;
+  view.Q = (W + 2 * pad - S) / stride + 1;
+  view.batch = B;
+  view.a_channels = (stored && stored->a) ? stored->a : Cout;
+  view.meta_channels = (view.a_channels + 127) / 128 * 128;
+  view.d.channels = (stored && stored->d) ? stored->d : Cin;
+  view.w_cols = (int64_t)R * S * Cin;
+  return view;
+}
+
 // What pruning costs (measured on a [16384 x 4096] tensor and on 50176 x 1024 rows): clocks of the rows kernel's pruning warps per block of
 // 128 channels, picoseconds per element of the prune kernel where the integer pipe bounds it.
 struct PruneCost {
@@ -301,61 +371,21 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
   }
   const int kb_channels = sparse ? 128 : 64;
 
-  DgradView view;
-  view.P = P; view.Q = Q; view.batch = B;
-  view.a_channels = (stored && stored->a) ? stored->a : Cout;
-  view.meta_channels = (view.a_channels + 127) / 128 * 128;
-  view.d.channels = (stored && stored->d) ? stored->d : Cin;
-  view.w_cols = (int64_t)R * S * Cin;
+  DgradView view = dgrad_view(B, H, W, Cin, Cout, R, S, stride, pad, stored);
   const size_t Cd = (size_t)view.d.channels;
 
-  // All four output parities of a strided layer in one launch of the strip kernel, where its strips cover their images well enough (the
-  // same bounds as for a filter of its size at stride 1) and that is estimated to be faster.
-  if (stride == 2 && !fused && R >= 2 && S >= 2 && W > 8 && halo_applies((H + 1) / 2, (W + 1) / 2, R * S, sparse, false) &&
-      classes_pay(B, H, W, view.d.channels, view.a_channels, R, S, pad, sparse)) {
-    HaloParams hp = {};
-    hp.B = B; hp.H = (H + 1) / 2; hp.W = (W + 1) / 2; hp.Cin = Cin; hp.Cout = Cout;
-    hp.r_step = hp.s_step = 2;
-    hp.S_full = S;
-    hp.P = P; hp.Q = Q;
-    hp.f16 = dtype == SDGP_FP16 ? 1 : 0;
-    hp.last_launch = 1;
-    hp.classes = 4;
-    for (int c = 0; c < 4; ++c) {
-      HaloClass& k = hp.cls[c];
-      const int ph = c >> 1, pw = c & 1;
-      k.r_first = (ph + pad) % 2; k.s_first = (pw + pad) % 2;
-      k.R = (R - k.r_first + 1) / 2; k.S = (S - k.s_first + 1) / 2;
-      k.pad_h = (ph + pad - k.r_first) / 2; k.pad_w = (pw + pad - k.s_first) / 2;
-      k.H = (H - ph + 1) / 2; k.W = (W - pw + 1) / 2;
-      hp.R = k.R > hp.R ? k.R : hp.R;
-      hp.S = k.S > hp.S ? k.S : hp.S;
-    }
-    const int blocks = (Cout + kb_channels - 1) / kb_channels;
-    hp.k_last = blocks - 1;
-    const int left = view.a_channels - hp.k_last * kb_channels, per_mma = kb_channels / 4;
-    hp.last_mmas = left < kb_channels ? (left + per_mma - 1) / per_mma : 4;
+  HaloParams hp4;
+  TileShape shapes4[6];
+  if (!fused && plan_parities(sparse, view, B, H, W, Cin, Cout, R, S, stride, pad, conv_groups, &hp4, shapes4)) {
+    hp4.f16 = dtype == SDGP_FP16 ? 1 : 0;
     view.d.base = (uint8_t*)dD;
     view.d.sw = 2 * (int64_t)Cd * 2;
     view.d.sh = 2 * (int64_t)W * Cd * 2;
     view.d.sb = (int64_t)H * W * Cd * 2;
     view.d.aligned32 = 0;
-    struct Shape { int bn, nt; double cost; } shapes[] = {{64, 1, 0}, {64, 2, 0}, {128, 1, 0}, {128, 2, 0}, {192, 1, 0}, {256, 1, 0}};
-    for (Shape& s : shapes) {
-      const double cost = halo_cost_classes(B, hp.H, hp.W, R, S, pad, s.bn, s.nt, sparse, (view.d.channels + s.bn - 1) / s.bn,
-                                            k_window(s.bn, view.d.channels, blocks, kb_channels, Cout, conv_groups));
-      s.cost = cost > 0.0 ? cost : 1e9;
-    }
-    std::sort(std::begin(shapes), std::end(shapes), [](const Shape& a, const Shape& b) { return a.cost < b.cost; });
-    for (const Shape& s : shapes) {
-      hp.tiles_n = (view.d.channels + s.bn - 1) / s.bn;
-      hp.k_blocks = k_window(s.bn, view.d.channels, blocks, kb_channels, Cout, conv_groups);
-      hp.diag_cin_g = hp.diag_cout_g = hp.diag_last = 0;
-      if (hp.k_blocks < blocks) {
-        hp.diag_cin_g = conv_groups->cin_g; hp.diag_cout_g = conv_groups->cout_g;
-        hp.diag_last = blocks - hp.k_blocks;
-      }
-      const sdgp_status st = sparse ? launch_halo_sparse(s.bn, s.nt, A, meta, Wt, view, hp, stream) : launch_halo_dense(s.bn, s.nt, A, Wt, view, hp, stream);
+    for (const TileShape& s : shapes4) {
+      set_width(&hp4, s.bn, view.d.channels, kb_channels, conv_groups);
+      const sdgp_status st = sparse ? launch_halo_sparse(s.bn, s.nt, A, meta, Wt, view, hp4, stream) : launch_halo_dense(s.bn, s.nt, A, Wt, view, hp4, stream);
       if (st != SDGP_ERR_UNSUPPORTED) return st;
     }
   }
@@ -365,7 +395,7 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
   int last_class = 0;  // of those that launch a kernel
   const int all_blocks = (Cout + kb_channels - 1) / kb_channels;
   // Tile shapes of the strip kernel, one for all classes of the call (kernels that alternate between shapes measured up to 10 % slower).
-  struct Shape { int bn, nt; double cost; } shapes[] = {{64, 1, 0}, {64, 2, 0}, {128, 1, 0}, {128, 2, 0}, {192, 1, 0}, {256, 1, 0}};
+  TileShape shapes[] = {{64, 1, 0}, {64, 2, 0}, {128, 1, 0}, {128, 2, 0}, {192, 1, 0}, {256, 1, 0}};
   for (int ph = 0; ph < stride; ++ph)
     for (int pw = 0; pw < stride; ++pw) {
       const int r0 = (ph + pad) % stride, s0 = (pw + pad) % stride;
@@ -375,14 +405,14 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
       const int Hs = (H - ph + stride - 1) / stride, Ws = (W - pw + stride - 1) / stride;
       const int Rs = (R - r0 + stride - 1) / stride, Ss = (S - s0 + stride - 1) / stride;
       if (!halo_applies(Hs, Ws, Rs * Ss, sparse, fused != nullptr)) continue;
-      for (Shape& s : shapes) {
+      for (TileShape& s : shapes) {
         const int tiles_n = (view.d.channels + s.bn - 1) / s.bn;
         const double cost = halo_cost(B, Hs, Ws, Rs, Ss, s.bn, s.nt, sparse, tiles_n,
                                       k_window(s.bn, view.d.channels, all_blocks, kb_channels, Cout, conv_groups), fused);
         s.cost += cost > 0.0 ? cost : 1e9;  // (does not exist for this class: tried last)
       }
     }
-  std::sort(std::begin(shapes), std::end(shapes), [](const Shape& a, const Shape& b) { return a.cost < b.cost; });
+  std::sort(std::begin(shapes), std::end(shapes), [](const TileShape& a, const TileShape& b) { return a.cost < b.cost; });
   if (any_empty && cudaMemsetAsync(dD, 0, (size_t)B * H * W * Cd * 2, stream) != cudaSuccess) return SDGP_ERR_CUDA;
   for (int ph = 0; ph < stride; ++ph) {
     for (int pw = 0; pw < stride; ++pw) {
@@ -446,7 +476,7 @@ sdgp_status launch_dgrad(bool sparse, const void* A, const void* meta, const voi
           hp.fused_n = p.fused_n; hp.fused_m = p.fused_m; hp.fused_scheme = p.fused_scheme; hp.seed_lo = p.seed_lo; hp.seed_hi = p.seed_hi;
         }
         // from the cheapest on, until one fits shared memory (a large filter's box and a wide tile may not)
-        for (const Shape& s : shapes) {
+        for (const TileShape& s : shapes) {
           set_width(s.bn);
           hp.tiles_n = p.tiles_n; hp.k_blocks = p.k_blocks;
           hp.diag_cin_g = p.diag_cin_g; hp.diag_cout_g = p.diag_cout_g; hp.diag_last = p.diag_last;
@@ -495,6 +525,52 @@ bool rows_fused_pays(int64_t rows, int K, int N, int m, int scheme, RowsPlan* pl
 }
 
 }  // namespace
+
+// Prune kernel, block-diagonal filters and contraction of a grouped layer. Constants fitted to the same layers as estimate_grouped()'s: within 10 % for
+// nineteen in twenty.
+double estimate_block_diagonal(int B, int H, int W, int C, int groups, int R, int S, int pad, const FusedPrune& prune) {
+  const int P = H + 2 * pad - R + 1, Q = W + 2 * pad - S + 1, Ck = (C + 63) / 64 * 64, blocks = (Ck + 127) / 128;
+  const ConvGroups cg = {C / groups, C / groups};
+  const double e = (double)B * P * Q * C, filters = 2.0 * Ck * R * S * Ck;
+  const double prune_mem = 3.125 * e / 6.4e6, prune_alu = e * prune_cost(prune.m, prune.scheme).ps * 1e-6;
+  const double before = 6.7 + 1.37 * (prune_mem > prune_alu ? prune_mem : prune_alu) + 0.25e-6 * filters;
+  if (halo_applies(H, W, R * S, true, false)) {
+    double best = 0.0;
+    const TileShape all[] = {{64, 1, 0}, {64, 2, 0}, {128, 1, 0}, {128, 2, 0}, {192, 1, 0}, {256, 1, 0}};
+    for (const TileShape& s : all) {
+      const double cost = halo_cost(B, H, W, R, S, s.bn, s.nt, true, (C + s.bn - 1) / s.bn, k_window(s.bn, C, blocks, 128, Ck, &cg), nullptr);
+      if (cost > 0.0 && (best == 0.0 || cost < best)) best = cost;
+    }
+    if (best > 0.0) return before + 0.187 * best;
+  }
+  int64_t m_tiles;
+  if (R == 1 && S == 1 && pad == 0) {
+    m_tiles = ((int64_t)B * H * W + kBM - 1) / kBM;
+  } else {
+    int TW, TH, TB;
+    choose_patch(B, H, W, &TW, &TH, &TB);
+    m_tiles = (int64_t)((W + TW - 1) / TW) * ((H + TH - 1) / TH) * ((B + TB - 1) / TB);
+  }
+  const int bn = choose_bn(m_tiles, C, blocks, 128, Ck, &cg);
+  const int64_t tiles = (m_tiles + 1) / 2 * ((C + bn - 1) / bn), pairs = sm_count() / 2;
+  return before + 0.5 + 1.8 * (double)((tiles + pairs - 1) / pairs) * (256.0 + (double)k_window(bn, C, blocks, 128, Ck, &cg) * R * S * (256 + 2 * bn)) / 1900.0;
+}
+
+bool query_parities(bool sparse, int B, int H, int W, int Cin, int Cout, int R, int S, int stride, int pad, const StoredChannels* stored,
+                    const ConvGroups* conv_groups, int* plan) {
+  const DgradView view = dgrad_view(B, H, W, Cin, Cout, R, S, stride, pad, stored);
+  HaloParams hp;
+  TileShape shapes[6];
+  if (!plan_parities(sparse, view, B, H, W, Cin, Cout, R, S, stride, pad, conv_groups, &hp, shapes)) return false;
+  for (const TileShape& s : shapes) {
+    set_width(&hp, s.bn, view.d.channels, sparse ? 128 : 64, conv_groups);
+    HaloParams p = hp;
+    if (!(sparse ? plan_halo_sparse(s.bn, s.nt, &p) : plan_halo_dense(s.bn, s.nt, &p))) continue;
+    plan[0] = 2; plan[1] = p.units; plan[2] = p.split_from; plan[3] = pairs_for(p.units); plan[4] = s.bn; plan[5] = s.nt; plan[6] = p.tb;
+    return true;
+  }
+  return false;
+}
 
 sdgp_status try_rows_fused(const void* dO, const void* W, void* dD, int64_t rows, int K, int N, const FusedPrune& prune, int dtype,
                            cudaStream_t stream, bool* taken) {

@@ -894,5 +894,17 @@ sdgp_status launch_halo(int bn, int nt, const void* A, const void* meta, const v
   }
 }
 
+template <bool SPARSE>
+bool plan_halo_shape(int bn, int nt, HaloParams* p) {
+  if (nt < 1 || nt > 2) return false;
+  switch (bn) {
+    case 64: return plan_halo<SPARSE, 64, false>(p, nt);
+    case 128: return plan_halo<SPARSE, 128, false>(p, nt);
+    case 192: return plan_halo<SPARSE, 192, false>(p, nt);
+    case 256: return plan_halo<SPARSE, 256, false>(p, nt);
+    default: return false;
+  }
+}
+
 }  // namespace
 }  // namespace sdgp

@@ -97,6 +97,9 @@ struct HaloOutMaps {
 sdgp_status launch_halo_sparse(int bn, int nt, const void* A, const void* meta, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream);
 sdgp_status launch_halo_dense(int bn, int nt, const void* A, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream);
 sdgp_status launch_halo_fused(int bn, int nt, const void* dO, const void* Wt, const DgradView& view, const HaloParams& p, cudaStream_t stream);
+// The same plans without a launch.
+bool plan_halo_sparse(int bn, int nt, HaloParams* p);
+bool plan_halo_dense(int bn, int nt, HaloParams* p);
 cudaError_t take_error_halo_sparse(unsigned int* word);
 cudaError_t take_error_halo_dense(unsigned int* word);
 cudaError_t take_error_halo_fused(unsigned int* word);

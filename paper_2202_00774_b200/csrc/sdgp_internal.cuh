@@ -100,10 +100,19 @@ cudaError_t launch_expand_grouped_weights(const void* Wg, int Cout, int taps, in
                                           void* Wfull, cudaStream_t stream);
 
 // Data gradient of a grouped convolution with C channels on both sides, pruned inside the kernel (n <= 2); Wg [C, R, S, C / groups].
-// SDGP_ERR_UNSUPPORTED (nothing launched): groups of other widths than 16 or 32 channels, filters or images that no plan fits.
+// SDGP_ERR_UNSUPPORTED (nothing launched): groups of other widths than 16 or 32 channels, filters or images that no plan fits or that the
+// path over block-diagonal filters is faster on.
 sdgp_status launch_grouped_fused(const void* dO, const void* Wg, void* dD, int B, int H, int W, int C, int groups, int R, int S, int stride,
                                  int pad, const FusedPrune& prune, int dtype, cudaStream_t stream);
 cudaError_t take_error_grouped(unsigned int* word);
+// Estimated time, us, of that other path at stride 1: prune kernel, block-diagonal filters, contraction.
+double estimate_block_diagonal(int B, int H, int W, int C, int groups, int R, int S, int pad, const FusedPrune& prune);
+
+// For sdgp_selftest_plan(): whether a call takes the kernel for narrow groups, or the four output parities of a stride-2 layer in one launch, and its
+// plan (eight ints). Arguments as launch_grouped_fused's and launch_dgrad's.
+bool query_grouped(int B, int H, int W, int C, int groups, int R, int S, int stride, int pad, const FusedPrune& prune, int* plan);
+bool query_parities(bool sparse, int B, int H, int W, int Cin, int Cout, int R, int S, int stride, int pad, const StoredChannels* stored,
+                    const ConvGroups* conv_groups, int* plan);
 
 // Launches a one-CTA kernel whose only wait can never be satisfied (50 ms limit).
 sdgp_status launch_bounded_wait_selftest(cudaStream_t stream);

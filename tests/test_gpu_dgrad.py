@@ -11,6 +11,7 @@ import numpy as np
 import pytest
 
 import oracle
+import plan_cases
 from paper_2202_00774_b200 import inputs
 
 torch = pytest.importorskip("torch")
@@ -485,20 +486,11 @@ def test_whole_filter_reuse_kernel(case, mode):
     assert_close(got, *conv_ref(src, W, H, Wd, stride, pad))
 
 
-# The four output parities of a strided layer in one launch: classes of unequal size whose last strips lie outside the smaller ones, filters
-# of two to five rows and columns, no padding, images of less than a strip, several column tiles and channel blocks (the last
-# one half full), several rounds of units with a split last one.
-STRIDE2_CLASS_CASES = [
-    # B, H, W, Cin, Cout, R, S, pad
-    (1, 33, 20, 64, 128, 3, 3, 1),
-    (2, 18, 49, 128, 192, 3, 3, 1),
-    (3, 12, 12, 192, 64, 3, 3, 0),
-    (1, 40, 24, 64, 64, 5, 5, 2),
-    (2, 22, 30, 128, 128, 2, 3, 1),
-    (5, 14, 14, 320, 256, 3, 3, 1),
-    (1, 9, 64, 64, 128, 3, 3, 1),
-    (24, 56, 56, 64, 128, 3, 3, 1),
-]
+# The four output parities of a strided layer in one launch (test_plan_host.py checks that they are): classes of unequal size, a row of strips that
+# lies outside the smaller ones, filters of two to five rows and columns, no padding, images of less than a strip, several column tiles and channel
+# blocks (the last one half full), several rounds of units, a last one that is dealt out strip by strip. The first one is four launches: its
+# strips cover three times the images.
+STRIDE2_CLASS_CASES = [(1, 33, 20, 64, 128, 3, 3, 1)] + [c for c, _, _ in plan_cases.PARITIES]
 
 
 @pytest.mark.parametrize("mode", ["dense", "two_pass"])

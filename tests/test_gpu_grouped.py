@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 import oracle
+import plan_cases
 from paper_2202_00774_b200 import inputs
 
 torch = pytest.importorskip("torch")
@@ -25,29 +26,37 @@ def magnitudes(bits):
     return (np.asarray(bits).view(np.uint16) & np.uint16(0x7FFF)).astype(np.uint16)
 
 
-def check(got, src, W, layer, what):
-    ref = oracle.dgrad_conv2d_grouped(src, W, layer.H, layer.W, layer.groups, layer.stride, layer.pad)
-    absdot = oracle.dgrad_conv2d_grouped(magnitudes(src), magnitudes(W), layer.H, layer.W, layer.groups, layer.stride, layer.pad)
+def to_f16_f64(t):
+    return inputs.f16_bits_to_f32(t.cpu().numpy().view(np.uint16)).astype(np.float64)
+
+
+def check(got, src, W, layer, what, dtype=oracle.BF16):
+    ref = oracle.dgrad_conv2d_grouped(src, W, layer.H, layer.W, layer.groups, layer.stride, layer.pad, dtype=dtype)
+    absdot = oracle.dgrad_conv2d_grouped(magnitudes(src), magnitudes(W), layer.H, layer.W, layer.groups, layer.stride, layer.pad, dtype=dtype)
     assert np.linalg.norm(got - ref) <= TOL * max(np.linalg.norm(ref), 1e-30), what
-    bad = np.abs(got - ref) > 2.0 ** -7 * np.abs(ref) + 2.0 ** -16 * absdot
+    # one rounding to the 16-bit type, with a factor two to spare (binary16: 2^-11 of the value, 2^-25 below 2^-14)
+    unit, least = (2.0 ** -10, 2.0 ** -24) if dtype == oracle.FP16 else (2.0 ** -7, 0.0)
+    bad = ~(np.abs(got - ref) <= unit * np.abs(ref) + 2.0 ** -16 * absdot + least)
     assert not bad.any(), "%s: %d elements off, first at %s" % (what, int(bad.sum()), np.argwhere(bad)[0])
 
 
-def run(layer, n, m, scheme, flags, seed=9):
+def run(layer, n, m, scheme, flags, seed=9, dtype=oracle.BF16):
     import paper_2202_00774_b200 as sdgp
     dO, W = inputs.conv_layer_tensors(layer, seed=seed)
+    if dtype == oracle.FP16:
+        dO, W = inputs.bf16_bits_as_f16_bits(dO), inputs.bf16_bits_as_f16_bits(W)
     size = sdgp.sdgp_workspace_size_conv2d_grouped(layer.B, layer.H, layer.W, layer.Cin, layer.Cout, layer.R, layer.S,
                                                    layer.stride, layer.pad, layer.groups, flags)
     ws = torch.empty(size, dtype=torch.uint8, device="cuda")
     dD = torch.full(layer.dD_shape(), -1, dtype=torch.int16, device="cuda")
     sdgp.sdgp_dgrad_conv2d_grouped(dev16(dO), dev16(W), dD, layer.stride, layer.pad, layer.groups, n, m, scheme, seed=77,
-                                   workspace=ws, flags=flags)
+                                   dtype=dtype, workspace=ws, flags=flags)
     assert sdgp.sdgp_last_device_error() == 0
     if flags == sdgp.FLAG_DENSE or n == m:
         src = dO
     else:
-        src = oracle.prune(dO.reshape(-1, layer.Cout), n, m, scheme, 77, want=("dense",))["dense"].reshape(dO.shape)
-    check(to_f64(dD), src, W, layer, "%s flags=%d %d:%d" % (layer.name, flags, n, m))
+        src = oracle.prune(dO.reshape(-1, layer.Cout), n, m, scheme, 77, want=("dense",), dtype=dtype)["dense"].reshape(dO.shape)
+    check(to_f16_f64(dD) if dtype == oracle.FP16 else to_f64(dD), src, W, layer, "%s flags=%d %d:%d" % (layer.name, flags, n, m), dtype)
 
 
 REGNETX = {l.name: l for l in inputs.regnetx_400mf_layers(batch=3)}
@@ -127,11 +136,11 @@ def test_argument_errors():
     (1, 4, 4, 32, 3, 3, 1, 1, 2, 2, 4, oracle.MAGNITUDE),       # one unit, one block that is half empty
     (1, 5, 3, 48, 1, 3, 1, 0, 3, 1, 8, oracle.RESCALED),        # three slices of a block, one row of taps
     (3, 13, 27, 112, 3, 3, 2, 1, 7, 2, 4, oracle.RANDOM),       # four classes of uneven size
-    (2, 9, 12, 96, 5, 5, 1, 2, 3, 2, 32, oracle.RESCALED),      # groups of 32 on both sides of the pruning, 25 taps
+    (2, 9, 12, 96, 5, 5, 1, 2, 3, 2, 32, oracle.RESCALED),      # 25 taps of groups of 32 do not fit: the other path
     (2, 10, 7, 64, 3, 3, 1, 2, 4, 2, 16, oracle.RANDOM),        # padding of a whole filter: dL/dO is larger than dD
     (2, 11, 11, 160, 3, 3, 1, 0, 5, 2, 32, oracle.MAGNITUDE),   # no padding: dL/dO is smaller; groups of 32, two blocks and a half
     (1, 3, 260, 32, 3, 3, 1, 1, 2, 2, 4, oracle.MAGNITUDE),     # rows too long for a box: the other path
-    (170, 14, 14, 176, 3, 3, 1, 1, 11, 2, 4, oracle.RESCALED),  # several units of every multiprocessor, a last block of 48 channels
+    (170, 14, 14, 176, 3, 3, 1, 1, 11, 2, 4, oracle.RESCALED),  # four units of every multiprocessor, a last block of 48 channels
 ])
 def test_narrow_groups(B, H, Wd, C, R, S, stride, pad, groups, n, m, scheme):
     import paper_2202_00774_b200 as sdgp
@@ -148,3 +157,82 @@ def test_last_channel_block_of_the_strip_kernel(B, Cout, mode):
     import paper_2202_00774_b200 as sdgp
     layer = inputs.ConvLayer("last", B, 16, 16, 64, Cout, 3, 3, 1, 1, 1)
     run(layer, 2, 4, oracle.MAGNITUDE, {"two_pass": sdgp.FLAG_TWO_PASS, "fused": sdgp.FLAG_FUSED, "dense": sdgp.FLAG_DENSE, "masked": sdgp.FLAG_MASKED}[mode])
+
+
+# Plans and element types of the kernel for narrow groups (test_plan_host.py checks that these layers take it, and how): rings and accumulators
+# that are used again, units of one to four accumulators, binary16 under every function
+@pytest.mark.parametrize("case", [c for c, _ in plan_cases.NARROW])
+def test_narrow_groups_plans(case):
+    import paper_2202_00774_b200 as sdgp
+    B, H, Wd, C, R, S, stride, pad, groups, n, m, scheme, fp16 = case
+    run(inputs.ConvLayer("narrow", B, H, Wd, C, C, R, S, stride, pad, groups), n, m, scheme, sdgp.FLAG_TWO_PASS, dtype=oracle.FP16 if fp16 else oracle.BF16)
+
+
+@pytest.mark.parametrize("case", [c for c in plan_cases.NARROW_ELSEWHERE if c[0] * c[1] * c[2] * c[3] < 3e6])
+def test_narrow_groups_on_the_other_path(case):
+    import paper_2202_00774_b200 as sdgp
+    B, H, Wd, C, R, S, stride, pad, groups, n, m, scheme = case
+    run(inputs.ConvLayer("elsewhere", B, H, Wd, C, C, R, S, stride, pad, groups), n, m, scheme, sdgp.FLAG_TWO_PASS)
+
+
+@pytest.mark.parametrize("fp16", [False, True])
+@pytest.mark.parametrize("case", [c for c, _ in plan_cases.BLOCK_DIAGONAL])
+def test_block_diagonal_filters(case, fp16):
+    import paper_2202_00774_b200 as sdgp
+    B, H, Wd, Cin, Cout, R, S, stride, pad, groups, n, m, scheme = case
+    run(inputs.ConvLayer("diagonal", B, H, Wd, Cin, Cout, R, S, stride, pad, groups), n, m, scheme, sdgp.FLAG_TWO_PASS,
+        dtype=oracle.FP16 if fp16 else oracle.BF16)
+
+
+# Infinities and NaN in dL/dO through the narrow-group kernel's own pruning: kept, pruned and rescaled as the oracle does, and felt by their group and
+# the pixels under their taps only. (Filters are finite: a pruned position is a zero that meets its filter like any other.)
+@pytest.mark.parametrize("fp16", [False, True])
+@pytest.mark.parametrize("n,m,scheme", [(2, 4, oracle.MAGNITUDE), (1, 4, oracle.RESCALED), (2, 8, oracle.RESCALED), (2, 32, oracle.RESCALED), (2, 4, oracle.RANDOM)])
+@pytest.mark.parametrize("stride,groups", [(1, 6), (2, 3)])
+def test_narrow_groups_non_finite_gradients(n, m, scheme, stride, groups, fp16):
+    import paper_2202_00774_b200 as sdgp
+    dtype = oracle.FP16 if fp16 else oracle.BF16
+    layer = inputs.ConvLayer("special", 2, 12, 11, 96, 96, 3, 3, stride, 1, groups)
+    dO, W = inputs.conv_layer_tensors(layer, seed=5)
+    if fp16:
+        dO, W = inputs.bf16_bits_as_f16_bits(dO), inputs.bf16_bits_as_f16_bits(W)
+    rng = np.random.Generator(np.random.PCG64(m + n))
+    flat = dO.reshape(-1)
+    for pattern in (0x7C00, 0xFC00, 0xFE01) if fp16 else (0x7F80, 0xFF80, 0xFFC1):
+        flat[rng.integers(0, flat.size, 10)] = pattern
+    src = oracle.prune(dO.reshape(-1, 96), n, m, scheme, 3, want=("dense",), dtype=dtype)["dense"].reshape(dO.shape)
+    ref = oracle.dgrad_conv2d_grouped(src, W, layer.H, layer.W, groups, stride, 1, dtype=dtype)
+    dD = torch.full(layer.dD_shape(), -1, dtype=torch.int16, device="cuda")
+    ws = torch.empty(sdgp.sdgp_workspace_size_conv2d_grouped(2, 12, 11, 96, 96, 3, 3, stride, 1, groups, sdgp.FLAG_TWO_PASS), dtype=torch.uint8, device="cuda")
+    sdgp.sdgp_dgrad_conv2d_grouped(dev16(dO), dev16(W), dD, stride, 1, groups, n, m, scheme, seed=3, dtype=dtype, workspace=ws)
+    assert sdgp.sdgp_last_device_error() == 0
+    got = to_f16_f64(dD) if fp16 else to_f64(dD)
+    finite = np.isfinite(ref)
+    assert (~finite).any() and finite.sum() > finite.size / 2
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    assert np.array_equal(got[np.isinf(ref)], ref[np.isinf(ref)])
+    special = magnitudes(src) >= (0x7C00 if fp16 else 0x7F80)
+    absdot = oracle.dgrad_conv2d_grouped(np.where(special, 0, magnitudes(src)).astype(np.uint16), magnitudes(W), layer.H, layer.W, groups, stride, 1, dtype=dtype)
+    bound = (2.0 ** -10 if fp16 else 2.0 ** -7) * np.abs(ref[finite]) + 2.0 ** -16 * absdot[finite] + (2.0 ** -24 if fp16 else 0.0)  # as in check()
+    assert (np.abs(got[finite] - ref[finite]) <= bound).all()
+
+
+# dD on a 16-byte boundary that is not a 32-byte one (rows leave in halves of a sector), nothing written outside it
+@pytest.mark.parametrize("stride,C,groups", [(1, 96, 6), (2, 96, 3), (1, 64, 4)])
+def test_narrow_groups_dD_on_a_16_byte_boundary(stride, C, groups):
+    import paper_2202_00774_b200 as sdgp
+    layer = inputs.ConvLayer("aligned", 3, 15, 10, C, C, 3, 3, stride, 1, groups)
+    dO, W = inputs.conv_layer_tensors(layer, seed=4)
+    size = int(np.prod(layer.dD_shape()))
+    ws = torch.empty(sdgp.sdgp_workspace_size_conv2d_grouped(3, 15, 10, C, C, 3, 3, stride, 1, groups, sdgp.FLAG_TWO_PASS), dtype=torch.uint8, device="cuda")
+    around = torch.full((size + 16,), -1, dtype=torch.int16, device="cuda")
+    dD = around[8:8 + size].view(layer.dD_shape())
+    assert dD.data_ptr() % 32 == 16
+    aligned = torch.empty(layer.dD_shape(), dtype=torch.int16, device="cuda")
+    for out in (dD, aligned):
+        sdgp.sdgp_dgrad_conv2d_grouped(dev16(dO), dev16(W), out, stride, 1, groups, 2, 4, sdgp.MAGNITUDE, workspace=ws)
+    assert sdgp.sdgp_last_device_error() == 0
+    assert torch.equal(dD, aligned)
+    assert bool((around[:8] == -1).all()) and bool((around[8 + size:] == -1).all())
+    src = oracle.prune(dO.reshape(-1, C), 2, 4, oracle.MAGNITUDE, 0, want=("dense",))["dense"].reshape(dO.shape)
+    check(to_f64(dD), src, W, layer, "16-byte dD")

@@ -226,6 +226,8 @@ sdgp_status sdgp_maxpool_relu_backward_prune(const void* dYp, const void* dSkipP
  * way into shared memory and reads the filters as they are. All others first write the filters as the block-diagonal filters of an ordinary convolution,
  * channel counts rounded up to multiples of 64, into the workspace (read again by the contraction on `stream`), then run the
  * ordinary kernels on them. dL/dO and dD are used as stored, without padded copies, either way.
+ * Filters that are not finite: the one-kernel path and SDGP_FLAG_MASKED multiply pruned positions as the zeros they are (zero times infinity is
+ * NaN), the paths over the compressed form skip them. With finite filters all paths agree.
  * Workspace: sdgp_workspace_size_conv2d_grouped() bytes (every mode needs one), 256-byte aligned, owned by the caller. */
 size_t sdgp_workspace_size_conv2d_grouped(int B, int H, int Wd, int Cin, int Cout, int R, int S, int stride, int pad,
                                           int groups, uint32_t flags);

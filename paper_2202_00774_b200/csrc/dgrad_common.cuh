@@ -12,7 +12,7 @@
 namespace sdgp {
 
 // Where dD goes: element (b, h, w, channel 0) of the launch's output grid is at base + b * sb + h * sh + w * sw (bytes;
-// stride-2 convolutions write one output parity per launch), `channels` elements of 16 bits per pixel (a store is clipped there).
+// stride-2 convolutions: of one output parity, (0, 0) where a launch holds all four), `channels` elements of 16 bits per pixel (a store is clipped there).
 struct OutView {
   uint8_t* base;
   int64_t sw, sh, sb;

@@ -16,9 +16,11 @@
 // and warp 2 the filters by TMA, warp 1 issues the MMAs (128 x width x 16, one group at a time), warps 4..7 are the epilogue, the other
 // seventeen prune: a thread takes two vectors of 8 channels out of the stage that TMA filled and puts them back pruned, dense, for the
 // tensor core. Dense, because the MMA's time is reading its 128 rows of A (4 KB: 41 clocks at best) for either kind and 16 columns leave the
-// tensor pipe idle anyway. (Loading dL/dO into the pruning warps' registers instead
-// measured the same within 3 %.) 256 images of 14 x 14, 10 groups of 16, rescaled, us: three kernels 32.8, this 22.8; 124 x 4 x 4, 11 groups, 11.2 and
-// 5.2; 60 x 32 x 32, 15 groups, 31.7 and 26.5. What bounds it: the MMAs at 51 to 59 clocks each, the pruning close behind.
+// tensor pipe idle anyway. A pruned position is thus a zero that meets its filter, where the compressed form skips it: with filters that are not
+// finite the two differ. (Loading dL/dO into the pruning warps' registers instead measured the same within 3 %.) 256 images of 14 x 14, 10 groups of 16, rescaled, us: three kernels 32.8, this 22.8; 124 x 4 x 4, 11 groups, 11.2 and
+// 5.2; 60 x 32 x 32, 15 groups, 31.7 and 26.5. What bounds it: the pruning of the random and rescaled functions - the first layer's units take some 4600
+// clocks of it, halo positions (a fifth there, 40 % at 32 x 32) and the absent half of the last block of 32 channels included - beside MMAs of
+// 51 to 59 clocks each, 4000 a unit, half of that in the last block. 80 registers are the most 24 warps can have; the pruning spills 32 to 40 bytes.
 #include "dgrad_prune.cuh"
 
 namespace sdgp {
@@ -493,7 +495,7 @@ bool plan_grouped(GroupedParams* p, int R, int S, int pad, int tiles, int* smem_
 
 // Estimated time of a plan, us. MMAs and pruning overlap but for a third of the shorter one; every unit has a fixed part, the first unit's pruning
 // and the last one's stores are in nobody's shadow. A pruning pass is 8 positions of 64 channels; an MMA takes 16 channels (the last block may
-// have fewer than four). Constants fitted to 330 layers of stride 1: within 10 % for four in five.
+// have fewer than four). Constants fitted to 330 layers of stride 1; over 1088 others within 12 % for nine in ten.
 double estimate_grouped(const GroupedParams& p, int m, int scheme) {
   const double pass = scheme == SDGP_MAGNITUDE ? (m == 4 ? 48.0 : 70.0) : scheme == SDGP_RANDOM ? (m == 4 ? 112.0 : 132.0) : (m == 4 ? 100.0 : 105.0);
   const double mma = 53.0 * (p.C / 16.0 / p.k_blocks) * p.taps * p.tiles, prune = (p.span + p.reach + p.chunk_pos) / 8.0 * pass;
@@ -502,10 +504,12 @@ double estimate_grouped(const GroupedParams& p, int m, int scheme) {
   return (rounds * (longer + 0.36 * shorter + 805.0) + prune + 1700.0 * p.tiles * p.classes) / 1900.0 + 2.3;
 }
 
-// The fastest plan, if there is one and the call should take it. Stride 2 always does (211 layers drawn: none slower, 0.38 x the time in the
-// median). At stride 1 the other path can be the faster one: every unit prunes its halo anew, so that filters and images with a long reach in
+// The fastest plan, if there is one and the call should take it. Stride 2 always does: 488 layers drawn, wide images among them, take 0.52 x the time in
+// the mean; seven are 6 to 15 % slower, most wider than 130 pixels, where most others still gain, and neither estimates nor the reach told
+// them apart (25 x 15 x 175, 8 groups, 2 x 2, 12.0 us and 13.9; 1 x 57 x 198, 26 groups of 32, 17.1 and 16.8). At stride 1 the other path can be the faster one: every unit prunes its halo anew, so that filters and images with a long reach in
 // the line (tall filters, wide images) prune a position two to five times, and filters of 16 taps and more are bound by the MMAs of one group
-// each. The rule compares the two estimates: of 379 layers drawn, 14 had been slower here, up to 2.4 x. Us, the other path and this: 5 x 76 x 76 images,
+// each. The rule compares the two estimates: of 1088 layers drawn, tall and wide filters and images among them, 124 are more than 5 % slower here, up
+// to 2.7 x; the rule leaves 6 of these, up to 1.15 x, and sends 24 to the other path that were more than 5 % faster here (mean 0.4 % behind the best). Us, the other path and this: 5 x 76 x 76 images,
 // 26 groups of 16, 7 x 1, random 2:4, 31.1 and 75.5; 12 x 75 x 144, 15 groups, 3 x 3, random, 68.1 and 105.4; 237 x 16 x 16, 5 groups, 5 x 5,
 // random, 31.3 and 40.0; 256 x 14 x 14, 10 groups, 3 x 3, rescaled, 30.1 and 21.9.
 bool choose_grouped(int B, int H, int W, int C, int groups, int R, int S, int stride, int pad, const FusedPrune& prune, GroupedParams* best,
